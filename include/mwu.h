@@ -59,10 +59,10 @@ typedef enum {
 
 /* How mwu_project organises its kernels.  Every choice gives the same bits. */
 typedef enum {
-    MWU_ALGO_AUTO = 0,       /* one pass from 8192 blocks on, multi pass below                 */
+    MWU_ALGO_AUTO = 0,       /* by size: multi pass up to about 600 000 blocks, one pass above */
     MWU_ALGO_ONE_PASS = 1,   /* outputs written in one sweep over W with thresholds estimated
                                 from a sample, then the few blocks near a threshold corrected */
-    MWU_ALGO_MULTI_PASS = 2  /* statistics pass, exact thresholds, emit pass                  */
+    MWU_ALGO_MULTI_PASS = 2  /* block keys first, exact thresholds, then the outputs: one launch */
 } mwu_proj_algo;
 
 typedef struct {

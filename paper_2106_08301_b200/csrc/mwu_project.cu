@@ -2,48 +2,31 @@
 //
 // Two pipelines give the same bits (all on the caller's stream, no host synchronisation).
 //
-// One-pass pipeline (MWU_ALGO_ONE_PASS; the default from ONE_PASS_MIN_BLOCKS blocks on):
-//   sample_kernel   one CTA sorts the keys of <= 4096 evenly spaced blocks; for each selection
-//                   (prune key, L_u of the survivors) it takes the sample quantile as a provisional
-//                   threshold and the sample keys 4 sigma of rank to either side as a window.
-//   pass_kernel     streams W (+U) once, evaluates the fp64 keys of every block (Section 3.1) and
-//                   writes every output -- Q, u, sign plane, bitmaps -- with the class the
-//                   provisional thresholds give.  A block whose key lies outside the window has
-//                   its final class (as long as the exact threshold lies inside, which the counts
-//                   prove afterwards); the few per cent inside go to a candidate list with their
-//                   bin codes and into the window histograms.
-//   list_select_kernel
-//                   exact prune threshold (key, block index) from the window histogram and the
-//                   list; the listed survivors complete the L_u histogram.
-//   list_finish_kernel
-//                   exact unify threshold; rewrites the outputs of the listed blocks whose
-//                   class changed.
-//   If a count shows that a threshold lies outside its window (or a tie group overflows the
-//   sort buffer, or the list overflows) a flag is set and the multi-pass kernels, which are
-//   always enqueued behind and otherwise return at once, redo the projection.
+// Exact pipeline (exact_kernel; small tensors, and every tensor with MWU_ALGO_MULTI_PASS): one launch.
+// A team of CTAs reads W (+U) once, keeps the fp64 keys of its blocks (Section 3.1: q = mean|v|,
+// L_u = sum(|v|-q)^2, L_p = sum v^2, fixed pairwise trees) in shared memory, finds both exact
+// thresholds (mwu_select.cuh) and writes every output.  Tensors whose keys do not fit evaluate them
+// again in every phase (exact_walk_kernel).
 //
-// Multi-pass pipeline (MWU_ALGO_MULTI_PASS; small tensors, and the fallback):
-//   sample_kernel   as above.  The window only steers efficiency; any window gives the same result.
-//   stats_kernel    streams W (+U) once; every thread owns 64 contiguous bytes (four 128-bit
-//                   loads in flight) and evaluates the fp64 keys of its blocks (Section 3.1:
-//                   q = mean|v|, L_u = sum(|v|-q)^2, L_p = sum v^2) with the fixed pairwise
-//                   tree; writes a 2x16-bit bin code per block, the prune-key histogram, the
-//                   sign plane and q of every block (into u).
-//   prune_select_kernel  locates the bin of the k_prune-th key, then one pass over the bin codes:
-//                   blocks of that bin become candidates (normally a few dozen to a few hundred),
-//                   blocks above it are counted in the L_u histogram.  The last CTA sorts the
-//                   candidates: the result is the exact threshold element (key, block index); it
-//                   adds the surviving candidates to the L_u histogram and locates the bin of the
-//                   unify threshold.
-//   collect_kernel  gathers the blocks of that bin that were not pruned; the last CTA sorts them.
-//   emit_kernel     classifies every block from its bin code (exact key only for blocks in a
-//                   threshold bin), writes Q, both bitmaps and the final u (0 unless unified).  W
-//                   is read again only for the 64-byte units that hold a block keeping its values:
-//                   unified blocks are rebuilt from q and the sign plane, pruned ones are zeros.
-// When a threshold bin holds more than 2048 blocks (massive ties, e.g. re-projecting an already
-// projected tensor) the last CTA narrows the range of the 96-bit composite key (key, index) by
-// itself, pass by pass, until the candidates fit: slow but exact.
-#include "mwu_common.cuh"
+// One-pass pipeline (MWU_ALGO_ONE_PASS; the default for larger tensors):
+//   sample_keys_kernel, sample_kernel
+//                   rank the keys of <= 4096 evenly spaced blocks; for each selection (prune key, L_u
+//                   of the survivors) the sample quantile is a provisional threshold and the sample
+//                   keys 4 sigma of rank to either side a window.
+//   pass_kernel     streams W (+U) once, evaluates the fp64 keys of every block and writes every
+//                   output -- Q, u, sign plane, bitmaps -- with the class the provisional
+//                   thresholds give.  A block whose key lies outside the window has its final class
+//                   (as long as the exact threshold lies inside, which the counts prove afterwards);
+//                   the few per cent inside go to a candidate list with their bin codes and into
+//                   the window histograms.
+//   resolve_kernel  exact thresholds from the window histograms and the list; rewrites the outputs of
+//                   the listed blocks whose class changed.
+//   If a count shows that a threshold lies outside its window (or a tie group overflows the
+//   sort buffer, or the list overflows) a flag is set and the same launch redoes the projection with
+//   the exact pipeline's phases.
+#include <type_traits>
+
+#include "mwu_select.cuh"
 
 namespace mwu {
 namespace proj {
@@ -56,8 +39,6 @@ constexpr int SAMP_THREADS = 1024;
 constexpr int SAMP_PER = NSAMP / SAMP_THREADS;
 static_assert(SAMP_PER == 4, "sample_select ranks one level-A key with the four threads that hold 16 samples");
 constexpr int STAGE_ENTRIES = 64;  // per-warp staging of candidate-list entries in pass_kernel
-constexpr long long ONE_PASS_MIN_BLOCKS = 8192;    // below: launch latency decides, multi-pass has fewer launches
-constexpr int PASS_LOADS = 4;      // 16-byte loads of bin codes a thread keeps in flight in the selection passes
 constexpr int FIN_THREADS = 1024;   // block size of the kernels whose last CTA finalises
 static_assert(NB_MAX / FIN_THREADS <= 64, "scan_hist searches one thread's bins with one warp, two per lane");
 
@@ -79,16 +60,14 @@ struct Sel {
 
 struct Work {
     Sel sel[2];                 // 0: prune, 1: unify
-    unsigned cand_count[2];
-    unsigned ticket[4];         // [1]: prune_select, [3]: collect<1>
     // one-pass pipeline
     unsigned fcand_count[2];    // threshold-bin candidates of the two halves of resolve_kernel
     unsigned fticket[2];
     unsigned list_count;        // entries appended to the candidate list
-    unsigned failed;            // != 0: the one-pass result is void, the multi-pass kernel runs
+    unsigned failed;            // != 0: the one-pass result is void, the exact phases run
     u64 That[2];                // provisional thresholds (key bit patterns)
     unsigned release;           // resolve_kernel: the prune threshold and the unify bin are published
-    unsigned bar;               // multipass_kernel: arrivals at its grid barriers (only ever grows)
+    unsigned bar;               // resolve_kernel: arrivals at its grid barriers (only ever grows)
     unsigned pad1[2];
 };
 
@@ -101,12 +80,10 @@ struct Params {
     int use_l1;
     Work *work;
     int nb;                     // level-0 bins in use (NB_SMALL or NB_MAX)
-    unsigned *hist;             // [3][nb]: prune, unify, refine scratch (multi-pass kernels)
+    sel::XWork *xwork;          // team state of the exact phases
     unsigned *fhist;            // [2][nb]: prune, unify (one-pass kernels)
     uint2 *list;                // [list_cap] candidate list: (block index, bin codes)
     unsigned list_cap;
-    int gated;                  // the multi-pass kernel returns at once unless work->failed is set
-    int run_sample;             // the multi-pass kernel also chooses the windows (no sample_kernel before it)
     // grouped pruning: the prune class of a block is the bit of its group (nullptr: pruning by key)
     const unsigned *gprune;     // [ceil(n_groups / 32)]
     unsigned group_rows, group_cols;     // extent of a prune group in rows and columns of W
@@ -119,7 +96,6 @@ struct Params {
     unsigned *cand_idx;         // [2 * CAP]
     unsigned *cand_aux;         // [2 * CAP] what resolve_kernel wants to know about a candidate besides its key
     u64 *samp_kp, *samp_ku;     // [NSAMP] each: keys of the sample blocks (one-pass pipeline)
-    unsigned *bins;             // [n_blocks]
     unsigned *dev_status;
 };
 
@@ -283,8 +259,8 @@ __device__ __forceinline__ void load_block(const float *W, const float *U, long 
 // window gives the same result), so its keys need no more than a few good digits, and sample_kernel,
 // a single CTA, has one SM's fp64 units.
 template <int B>
-__device__ __forceinline__ void block_keys_sample(const float *W, const float *U, long long j, int use_l1, u64 *kp,
-                                                  u64 *ku) {
+__device__ __forceinline__ void block_keys_sample(const float *W, const float *U, long long j, int use_l1, float *kp,
+                                                  float *ku) {
     float v[B];
     load_block<B>(W, U, j, v);
     float S = 0.f, sq = 0.f;
@@ -294,8 +270,8 @@ __device__ __forceinline__ void block_keys_sample(const float *W, const float *U
     float lu = 0.f;
 #pragma unroll
     for (int l = 0; l < B; ++l) { const float d = fabsf(v[l]) - q; lu = fmaf(d, d, lu); }
-    *kp = key_bits((double)(use_l1 ? S : sq));
-    *ku = key_bits((double)lu);
+    *kp = use_l1 ? S : sq;
+    *ku = lu;
 }
 
 // exact keys of block j, read from global memory (threshold-bin blocks)
@@ -518,7 +494,10 @@ __global__ void __launch_bounds__(128) sample_keys_kernel(Params p, unsigned *ze
         unsigned in_group = 0;
         if (i < ns) {
             const long long j = sample_block(i, mb, ns);
-            block_keys_sample<B>(p.W, p.U, j, p.use_l1, &kp, &ku);
+            float fp, fu;
+            block_keys_sample<B>(p.W, p.U, j, p.use_l1, &fp, &fu);
+            kp = key_bits((double)fp);
+            ku = key_bits((double)fu);
             if (p.gprune) in_group = group_pruned(p, (unsigned)j) ? 1u : 0u;
         }
         p.samp_kp[i] = kp;
@@ -530,9 +509,8 @@ __global__ void __launch_bounds__(128) sample_keys_kernel(Params p, unsigned *ze
 }
 
 // Run by one whole CTA of SAMP_THREADS threads: windows and provisional thresholds of the two
-// selections, written into p.work.  from_keys: the sample keys were computed by sample_keys_kernel.
-template <int B>
-__device__ void sample_body(const Params &p, bool from_keys = false) {
+// selections from the keys sample_keys_kernel computed, written into p.work.
+__device__ void sample_body(const Params &p) {
     const long long k_unify = p.k_unify, k_prune = p.k_prune;
     const long long mb = p.n_blocks;
     const bool by_group = p.gprune != nullptr;
@@ -546,15 +524,11 @@ __device__ void sample_body(const Params &p, bool from_keys = false) {
         ku[t] = ~0ull;
         valid[t] = i < ns;
         in_group[t] = false;
-        if (i < ns && from_keys) {
+        if (i < ns) {
             kp[t] = p.samp_kp[i];
             const u64 x = p.samp_ku[i];
             ku[t] = x & (~0ull >> 1);
             in_group[t] = (x >> 63) != 0ull;
-        } else if (i < ns) {
-            const long long j = sample_block(i, mb, ns);
-            block_keys_sample<B>(p.W, p.U, j, p.use_l1, &kp[t], &ku[t]);
-            if (by_group) in_group[t] = group_pruned(p, (unsigned)j);
         }
     }
     Sel *sp = &p.work->sel[0];
@@ -597,14 +571,13 @@ __device__ void sample_body(const Params &p, bool from_keys = false) {
 // Second kernel of the one-pass pipeline (one CTA): clears the selection state and chooses the
 // windows from the sample keys.  Launched with programmatic stream serialization behind
 // sample_keys_kernel, and itself lets pass_kernel's CTAs start early.
-template <int B>
 __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     unsigned *w = reinterpret_cast<unsigned *>(p.work);
     for (unsigned i = threadIdx.x; i < sizeof(Work) / 4; i += blockDim.x) w[i] = 0u;
     asm volatile("griddepcontrol.wait;" ::: "memory");     // the sample keys are complete and visible
     __syncthreads();
-    sample_body<B>(p, true);
+    sample_body(p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -798,17 +771,6 @@ __device__ __forceinline__ SelView view_of(const Sel *s) {
     return v;
 }
 
-// the same, for state written earlier in the running kernel (read by one CTA only)
-__device__ __forceinline__ SelView view_vol(const Sel *s) {
-    SelView v;
-    v.mode = ld_vol(&s->mode);
-    v.B = ld_vol(&s->B);
-    v.T_key = ld_vol(&s->T_key);
-    v.T_idx = ld_vol(&s->T_idx);
-    return v;
-}
-
-
 template <int B>
 __device__ __forceinline__ bool selected(const Params &p, const SelView &s, long long j, unsigned bin,
                                          int which) {
@@ -821,120 +783,6 @@ __device__ __forceinline__ bool selected(const Params &p, const SelView &s, long
     return key < s.T_key || (key == s.T_key && (u64)j <= s.T_idx);
 }
 
-// ---------------------------------------------------------------------------------------------
-// stats_kernel
-// ---------------------------------------------------------------------------------------------
-template <int B>
-__device__ void stats_body(const Params &p, const Work &w, double *loss_u, double *loss_p, float *u_out,
-                           unsigned *sign_bits) {
-    if (p.gated && p.resid && blockIdx.x == 0 && threadIdx.x == 0) *p.resid = 0.0;   // emit_body sums afresh
-    constexpr int NBT = 16 / B;                         // blocks per thread and step
-    const Sel *sp = &w.sel[0];
-    const Sel *su = &w.sel[1];
-    const u64 plo = sp->lo0, phi = sp->hi0, ulo = su->lo0, uhi = su->hi0;
-    const unsigned psh = sp->shift0, ush = su->shift0;
-    const unsigned nb = (unsigned)p.nb;
-    unsigned cnt_under = 0, cnt_over = 0;
-    unsigned nonfinite = 0;
-    const long long n = p.n_floats;
-    const long long n_units = (n + 15) / 16;
-    const long long ustride = (long long)gridDim.x * blockDim.x;
-    long long unit = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    float nxt[16];
-    if (unit < n_units) load16(p.W, p.U, unit * 16, n, nxt);
-    for (; unit < n_units; unit += ustride) {
-        float v[16];
-#pragma unroll
-        for (int l = 0; l < 16; ++l) v[l] = nxt[l];
-        // the next unit's 64 bytes travel while this one is evaluated
-        if (unit + ustride < n_units) load16(p.W, p.U, (unit + ustride) * 16, n, nxt);
-        unsigned ex = 0;
-#pragma unroll
-        for (int l = 0; l < 16; ++l) ex = max(ex, __float_as_uint(v[l]) & 0x7fffffffu);
-        nonfinite |= (ex >= 0x7f800000u) ? 1u : 0u;
-        // sign plane (final): bit l of this unit's half word = (v[l] < 0)
-        {
-            unsigned sb = 0;
-#pragma unroll
-            for (int l = 0; l < 16; ++l) sb |= (v[l] < 0.f ? 1u : 0u) << l;
-            unsigned short *halves = reinterpret_cast<unsigned short *>(sign_bits);
-            halves[unit] = (unsigned short)sb;
-            if (unit == n_units - 1 && (n_units & 1)) halves[unit + 1] = 0;
-        }
-        unsigned code[NBT];
-        float qv[NBT];                                   // q = mean|v| of every block; emit keeps the unified ones
-#pragma unroll
-        for (int e = 0; e < NBT; ++e) {
-            double S, Lu, Kp;
-            block_keys<B>(v + e * B, p.use_l1, &S, &Lu, &Kp);
-            qv[e] = __double2float_rn(__dmul_rn(S, 1.0 / (double)B));
-            const long long j = unit * NBT + e;
-            const unsigned bu = bin_of(key_bits(Lu), ulo, uhi, ush, nb);
-            const unsigned bp = bin_of(key_bits(Kp), plo, phi, psh, nb);
-            code[e] = bp | (bu << 16);
-            if (j < p.n_blocks) {
-                if (bp == 0) ++cnt_under;
-                else if (bp == nb - 1u) ++cnt_over;
-                else atomicAdd(&p.hist[bp], 1u);
-                if (loss_u) loss_u[j] = Lu;
-                if (loss_p) loss_p[j] = Kp;
-            }
-        }
-        const long long j0 = unit * NBT;
-        if (j0 + NBT <= p.n_blocks) {
-            if (NBT == 1) { p.bins[j0] = code[0]; u_out[j0] = qv[0]; }
-            else if (NBT == 2) {
-                *reinterpret_cast<uint2 *>(p.bins + j0) = make_uint2(code[0], code[1 % NBT]);
-                *reinterpret_cast<float2 *>(u_out + j0) = make_float2(qv[0], qv[1 % NBT]);
-            } else {
-#pragma unroll
-                for (int e = 0; e < NBT; e += 4) {
-                    *reinterpret_cast<uint4 *>(p.bins + j0 + e) =
-                        make_uint4(code[e % NBT], code[(e + 1) % NBT], code[(e + 2) % NBT], code[(e + 3) % NBT]);
-                    *reinterpret_cast<float4 *>(u_out + j0 + e) =
-                        make_float4(qv[e % NBT], qv[(e + 1) % NBT], qv[(e + 2) % NBT], qv[(e + 3) % NBT]);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int e = 0; e < NBT; ++e)
-                if (j0 + e < p.n_blocks) { p.bins[j0 + e] = code[e]; u_out[j0 + e] = qv[e]; }
-        }
-    }
-    // block-level totals of the two catch-all bins
-    __shared__ unsigned s_under, s_over;
-    if (threadIdx.x == 0) { s_under = 0; s_over = 0; }
-    __syncthreads();
-    for (int m = 16; m > 0; m >>= 1) {
-        cnt_under += __shfl_xor_sync(0xffffffffu, cnt_under, m);
-        cnt_over += __shfl_xor_sync(0xffffffffu, cnt_over, m);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (cnt_under) atomicAdd(&s_under, cnt_under);
-        if (cnt_over) atomicAdd(&s_over, cnt_over);
-    }
-    if (nonfinite) atomicOr(p.dev_status, (unsigned)MWU_DEV_NONFINITE);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (s_under) atomicAdd(&p.hist[0], s_under);
-        if (s_over) atomicAdd(&p.hist[nb - 1u], s_over);
-    }
-}
-
-// four consecutive bin codes starting at j4 (j4 % 4 == 0); codes beyond n read as 0
-__device__ __forceinline__ void load_codes4(const unsigned *bins, long long j4, long long n, unsigned (&c)[4]) {
-    if (j4 + 4 <= n) {
-        const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(bins + j4));
-        c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
-    } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) c[e] = (j4 + e < n) ? __ldcg(bins + j4 + e) : 0u;
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
-// collect_kernel: exact threshold element of one selection
-// ---------------------------------------------------------------------------------------------
 __device__ void sort_candidates(u64 *key, unsigned *idx, int n_pow2) {
     for (int k = 2; k <= n_pow2; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
@@ -953,479 +801,319 @@ __device__ void sort_candidates(u64 *key, unsigned *idx, int n_pow2) {
     }
 }
 
-// Exact threshold element of selection KIND.  w: this phase's copy of the selection state;
-// c_key / c_idx: CAP entries of shared memory each.
-template <int KIND, int B>
-__device__ void collect_body(const Params &p, const Work &w, u64 *c_key, unsigned *c_idx) {
-    Sel *s = &p.work->sel[KIND];
-    const Sel *sw = &w.sel[KIND];
-    if (sw->mode != 0u) return;                       // the same in every CTA
-    __shared__ unsigned s_bin, s_err, s_n;
-    __shared__ u64 s_r, s_cnt;
-    const SelView pv = view_of(&w.sel[0]);
-    const unsigned Bsel = sw->B;
-    const bool too_many = sw->cnt > (u64)CAP;
-    const long long stride = (long long)gridDim.x * blockDim.x;
+// ---------------------------------------------------------------------------------------------
+// exact pipeline
+// ---------------------------------------------------------------------------------------------
+struct Outs {
+    float *Q;
+    double *loss_u, *loss_p;
+    float *u;
+    unsigned *pruned_bitmap, *unified_bitmap, *sign_bits;
+};
 
-    if (!too_many) {
-        const u128 lo = from_halves(sw->lo_hi, sw->lo_lo);
-        const u128 hi = from_halves(sw->hi_hi, sw->hi_lo);
-        for (long long j0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4; j0 < p.n_blocks;
-             j0 += stride * 4 * PASS_LOADS) {
-            unsigned codes[PASS_LOADS][4];
-#pragma unroll
-            for (int q = 0; q < PASS_LOADS; ++q) load_codes4(p.bins, j0 + q * stride * 4, p.n_blocks, codes[q]);
-#pragma unroll
-            for (int q = 0; q < PASS_LOADS; ++q) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const long long j = j0 + q * stride * 4 + e;
-                    const unsigned code = codes[q][e];
-                    const unsigned bin = KIND ? (code >> 16) : (code & 0xffffu);
-                    if (j >= p.n_blocks || bin != Bsel) continue;
-                    if (KIND == 1 && selected<B>(p, pv, j, code & 0xffffu, 0)) continue;
-                    const u64 key = exact_key<B>(p, j, KIND);
-                    const u128 c = make_c(key, (u64)j);
-                    if (c >= lo && c < hi) {
-                        const unsigned slot = atomicAdd(&p.work->cand_count[KIND], 1u);
-                        if (slot < (unsigned)CAP) { p.cand_key[slot] = key; p.cand_idx[slot] = (unsigned)j; }
-                    }
-                }
-            }
-        }
-    }
-    if (!last_block_done(&p.work->ticket[KIND ? 3 : 1])) return;
+constexpr u64 NO_KEY = ~0ull;                            // of a slot without a block
 
-    // ---- last CTA only ----
-    if (too_many) {
-        // massive ties: narrow the composite range pass by pass with this CTA alone
-        unsigned *rhist = p.hist + (size_t)2 * p.nb;
-        for (int level = 0; level < 10; ++level) {
-            if (ld_vol(&s->cnt) <= (u64)CAP) break;
-            for (int i = threadIdx.x; i < p.nb; i += blockDim.x) rhist[i] = 0;
-            __syncthreads();
-            const u128 lo = from_halves(ld_vol(&s->lo_hi), ld_vol(&s->lo_lo));
-            const u128 hi = from_halves(ld_vol(&s->hi_hi), ld_vol(&s->hi_lo));
-            unsigned shift = 0;
-            while (((hi - lo - 1) >> shift) >= (u128)p.nb) ++shift;
-            for (long long j = threadIdx.x; j < p.n_blocks; j += blockDim.x) {
-                const unsigned code = ld_vol(p.bins + j);
-                const unsigned bin = KIND ? (code >> 16) : (code & 0xffffu);
-                if (bin != Bsel) continue;
-                if (KIND == 1 && selected<B>(p, pv, j, code & 0xffffu, 0)) continue;
-                const u128 c = make_c(exact_key<B>(p, j, KIND), (u64)j);
-                if (c >= lo && c < hi) atomicAdd(&rhist[(unsigned)((c - lo) >> shift)], 1u);
-            }
-            __threadfence();
-            __syncthreads();
-            if (threadIdx.x == 0) s_err = 0;
-            __syncthreads();
-            scan_hist(rhist, p.nb, ld_vol(&s->r), &s_bin, &s_r, &s_cnt, &s_err);
-            if (threadIdx.x == 0) {
-                if (s_err) atomicOr(p.dev_status, (unsigned)MWU_DEV_SELECT);
-                u128 nlo = lo + ((u128)s_bin << shift);
-                u128 nhi = nlo + ((u128)1 << shift);
-                if (nhi > hi) nhi = hi;
-                s->r = s_r;
-                s->cnt = s_cnt;
-                s->lo_hi = (u64)(nlo >> 64); s->lo_lo = (u64)nlo;
-                s->hi_hi = (u64)(nhi >> 64); s->hi_lo = (u64)nhi;
-                __threadfence();
-            }
-            __syncthreads();
-        }
-        // collect inside the narrowed range
-        if (threadIdx.x == 0) s_n = 0;
-        __syncthreads();
-        const u128 lo = from_halves(ld_vol(&s->lo_hi), ld_vol(&s->lo_lo));
-        const u128 hi = from_halves(ld_vol(&s->hi_hi), ld_vol(&s->hi_lo));
-        for (long long j = threadIdx.x; j < p.n_blocks; j += blockDim.x) {
-            const unsigned code = ld_vol(p.bins + j);
-            const unsigned bin = KIND ? (code >> 16) : (code & 0xffffu);
-            if (bin != Bsel) continue;
-            if (KIND == 1 && selected<B>(p, pv, j, code & 0xffffu, 0)) continue;
-            const u64 key = exact_key<B>(p, j, KIND);
-            const u128 c = make_c(key, (u64)j);
-            if (c >= lo && c < hi) {
-                const unsigned slot = atomicAdd(&s_n, 1u);
-                if (slot < (unsigned)CAP) { p.cand_key[slot] = key; p.cand_idx[slot] = (unsigned)j; }
-            }
-        }
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) p.work->cand_count[KIND] = s_n;
-        __syncthreads();
-    }
-    const unsigned n = ld_vol(&p.work->cand_count[KIND]);
-    const u64 r = ld_vol(&s->r);
-    const unsigned m = n < (unsigned)CAP ? n : (unsigned)CAP;
-    for (int i = threadIdx.x; i < CAP; i += blockDim.x) {
-        c_key[i] = (i < (int)m) ? ld_vol(&p.cand_key[i]) : ~0ull;
-        c_idx[i] = (i < (int)m) ? ld_vol(&p.cand_idx[i]) : ~0u;
-    }
-    __syncthreads();
-    int np2 = 2;
-    while (np2 < (int)m) np2 <<= 1;
-    sort_candidates(c_key, c_idx, np2);
-    if (threadIdx.x == 0) {
-        if (n > (unsigned)CAP || r == 0 || r > (u64)m) {
-            atomicOr(p.dev_status, (unsigned)MWU_DEV_SELECT);
-            s->T_key = 0; s->T_idx = 0;
-        } else {
-            s->T_key = c_key[r - 1];
-            s->T_idx = (u64)c_idx[r - 1];
-        }
-    }
+// keys of block j with values v; both NO_KEY beyond the tensor.  Sets *bad when a value is not finite.
+template <int B>
+__device__ __forceinline__ void keys_of(const Params &p, unsigned j, const float *v, u64 *kp, u64 *ku, const Outs &o,
+                                        unsigned *bad) {
+    double S, Lu, Kp;
+    block_keys<B>(v, p.use_l1, &S, &Lu, &Kp);
+    const bool there = j < (unsigned)p.n_blocks;
+    *bad |= ((unsigned)__double2hiint(S) >= 0x7ff00000u) ? 1u : 0u;
+    *kp = there ? key_bits(Kp) : NO_KEY;
+    *ku = there ? key_bits(Lu) : NO_KEY;
+    if (there && o.loss_u) o.loss_u[j] = Lu;
+    if (there && o.loss_p) o.loss_p[j] = Kp;
 }
 
-// ---------------------------------------------------------------------------------------------
-// prune_select_kernel: exact prune threshold and the L_u histogram of the survivors in one pass
-// ---------------------------------------------------------------------------------------------
-// Every CTA first locates the prune threshold bin from the finished histogram (all write the same
-// values).  The pass over the bin codes then needs no exact key outside that bin: blocks below it
-// are pruned, blocks above it survive and are counted in the L_u histogram, blocks inside it become
-// candidates.  The last CTA sorts the candidates, which fixes the threshold element, counts the
-// L_u bins of the candidates that survive, and locates the unify threshold bin.
+// Every output of one unit from its values and classes (bit e of cls_p / cls_u: block e); all lanes of
+// the warp call it, units beyond the tensor included.  ws: 128 float4 of shared memory of the warp.
+// Returns the unit's share of ||V - Q||^2.
 template <int B>
-__device__ void prune_select_body(const Params &p, const Work &w, u64 *c_key, unsigned *c_idx) {
-    Sel *sp = &p.work->sel[0];
-    Sel *su = &p.work->sel[1];
-    const unsigned mode_p = w.sel[0].mode, mode_u = w.sel[1].mode;
-    if (mode_p != 0u && mode_u != 0u) return;         // the same in every CTA
-    __shared__ unsigned s_bin, s_err, s_n;
-    __shared__ u64 s_r, s_cnt;
-    __shared__ BinSel s_sel;
-    unsigned *hist_u = p.hist + p.nb;
-    if (threadIdx.x == 0) { s_sel.B = 0; s_sel.r = 0; s_sel.cnt = 0; s_sel.lo_hi = s_sel.lo_lo = s_sel.hi_hi = s_sel.hi_lo = 0; }
-    __syncthreads();
-    if (mode_p == 0u) select_bin(p, &w.sel[0], sp, p.hist, &s_sel, true);
-    const unsigned Bp = s_sel.B;
-    const bool too_many = mode_p == 0u && s_sel.cnt > (u64)CAP;
-    const u128 lo0 = from_halves(s_sel.lo_hi, s_sel.lo_lo);
-    const u128 hi0 = from_halves(s_sel.hi_hi, s_sel.hi_lo);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    unsigned under = 0, over = 0;
-    if (mode_p != 2u) {                                   // mode 2: everything is pruned, nothing survives
-        // PASS_LOADS 16-byte loads are in flight per thread before their codes are looked at
-        for (long long j0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4; j0 < p.n_blocks;
-             j0 += stride * 4 * PASS_LOADS) {
-            unsigned codes[PASS_LOADS][4];
-#pragma unroll
-            for (int q = 0; q < PASS_LOADS; ++q) load_codes4(p.bins, j0 + q * stride * 4, p.n_blocks, codes[q]);
-#pragma unroll
-            for (int q = 0; q < PASS_LOADS; ++q) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const long long j = j0 + q * stride * 4 + e;
-                    if (j >= p.n_blocks) break;
-                    const unsigned bp = codes[q][e] & 0xffffu, bu = codes[q][e] >> 16;
-                    if (mode_p == 0u) {
-                        if (bp < Bp) continue;                // pruned
-                        if (bp == Bp) {                       // decided by the last CTA
-                            if (!too_many) {
-                                const u64 key = exact_key<B>(p, j, 0);
-                                const u128 c = make_c(key, (u64)j);
-                                if (c >= lo0 && c < hi0) {
-                                    const unsigned slot = atomicAdd(&p.work->cand_count[0], 1u);
-                                    if (slot < (unsigned)CAP) { p.cand_key[slot] = key; p.cand_idx[slot] = (unsigned)j; }
-                                }
-                            }
-                            continue;
-                        }
-                    } else if (mode_p == 3u) {
-                        if (group_pruned(p, (unsigned)j)) continue;
-                    }
-                    if (mode_u != 0u) continue;
-                    if (bu == 0) ++under;
-                    else if (bu == (unsigned)p.nb - 1u) ++over;
-                    else atomicAdd(&hist_u[bu], 1u);
-                }
-            }
-        }
-    }
-    for (int m = 16; m > 0; m >>= 1) {
-        under += __shfl_xor_sync(0xffffffffu, under, m);
-        over += __shfl_xor_sync(0xffffffffu, over, m);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (under) atomicAdd(&hist_u[0], under);
-        if (over) atomicAdd(&hist_u[p.nb - 1], over);
-    }
-    if (!last_block_done(&p.work->ticket[1])) return;
-
-    // ---- last CTA only ----
-    if (mode_p == 0u) {
-        if (too_many) {
-            // massive ties: narrow the composite range pass by pass with this CTA alone
-            unsigned *rhist = p.hist + (size_t)2 * p.nb;
-            for (int level = 0; level < 10; ++level) {
-                if (ld_vol(&sp->cnt) <= (u64)CAP) break;
-                for (int i = threadIdx.x; i < p.nb; i += blockDim.x) rhist[i] = 0;
-                __syncthreads();
-                const u128 lo = from_halves(ld_vol(&sp->lo_hi), ld_vol(&sp->lo_lo));
-                const u128 hi = from_halves(ld_vol(&sp->hi_hi), ld_vol(&sp->hi_lo));
-                unsigned shift = 0;
-                while (((hi - lo - 1) >> shift) >= (u128)p.nb) ++shift;
-                for (long long j = threadIdx.x; j < p.n_blocks; j += blockDim.x) {
-                    if ((ld_vol(p.bins + j) & 0xffffu) != Bp) continue;
-                    const u128 c = make_c(exact_key<B>(p, j, 0), (u64)j);
-                    if (c >= lo && c < hi) atomicAdd(&rhist[(unsigned)((c - lo) >> shift)], 1u);
-                }
-                __threadfence();
-                __syncthreads();
-                if (threadIdx.x == 0) s_err = 0;
-                __syncthreads();
-                scan_hist(rhist, p.nb, ld_vol(&sp->r), &s_bin, &s_r, &s_cnt, &s_err);
-                if (threadIdx.x == 0) {
-                    if (s_err) atomicOr(p.dev_status, (unsigned)MWU_DEV_SELECT);
-                    u128 nlo = lo + ((u128)s_bin << shift);
-                    u128 nhi = nlo + ((u128)1 << shift);
-                    if (nhi > hi) nhi = hi;
-                    sp->r = s_r;
-                    sp->cnt = s_cnt;
-                    sp->lo_hi = (u64)(nlo >> 64); sp->lo_lo = (u64)nlo;
-                    sp->hi_hi = (u64)(nhi >> 64); sp->hi_lo = (u64)nhi;
-                    __threadfence();
-                }
-                __syncthreads();
-            }
-            if (threadIdx.x == 0) s_n = 0;
-            __syncthreads();
-            const u128 lo = from_halves(ld_vol(&sp->lo_hi), ld_vol(&sp->lo_lo));
-            const u128 hi = from_halves(ld_vol(&sp->hi_hi), ld_vol(&sp->hi_lo));
-            for (long long j = threadIdx.x; j < p.n_blocks; j += blockDim.x) {
-                if ((ld_vol(p.bins + j) & 0xffffu) != Bp) continue;
-                const u64 key = exact_key<B>(p, j, 0);
-                const u128 c = make_c(key, (u64)j);
-                if (c >= lo && c < hi) {
-                    const unsigned slot = atomicAdd(&s_n, 1u);
-                    if (slot < (unsigned)CAP) { p.cand_key[slot] = key; p.cand_idx[slot] = (unsigned)j; }
-                }
-            }
-            __threadfence();
-            __syncthreads();
-            if (threadIdx.x == 0) p.work->cand_count[0] = s_n;
-            __syncthreads();
-        }
-        const unsigned n = ld_vol(&p.work->cand_count[0]);
-        const u64 r = ld_vol(&sp->r);
-        const unsigned m = n < (unsigned)CAP ? n : (unsigned)CAP;
-        for (int i = threadIdx.x; i < CAP; i += blockDim.x) {
-            c_key[i] = (i < (int)m) ? ld_vol(&p.cand_key[i]) : ~0ull;
-            c_idx[i] = (i < (int)m) ? ld_vol(&p.cand_idx[i]) : ~0u;
-        }
-        __syncthreads();
-        int np2 = 2;
-        while (np2 < (int)m) np2 <<= 1;
-        sort_candidates(c_key, c_idx, np2);
-        const bool bad = n > (unsigned)CAP || r == 0 || r > (u64)m;
-        if (threadIdx.x == 0) {
-            if (bad) {
-                atomicOr(p.dev_status, (unsigned)MWU_DEV_SELECT);
-                sp->T_key = 0; sp->T_idx = 0;
-            } else {
-                sp->T_key = c_key[r - 1];
-                sp->T_idx = (u64)c_idx[r - 1];
-            }
-            __threadfence();
-        }
-        __syncthreads();
-        // the blocks of the threshold bin that survive join the L_u histogram
-        if (mode_u == 0u && !bad) {
-            if (!too_many) {
-                for (unsigned i = (unsigned)r + threadIdx.x; i < m; i += blockDim.x)
-                    atomicAdd(&hist_u[ld_vol(p.bins + c_idx[i]) >> 16], 1u);
-            } else {
-                const SelView pv = view_vol(sp);
-                for (long long j = threadIdx.x; j < p.n_blocks; j += blockDim.x) {
-                    const unsigned code = ld_vol(p.bins + j);
-                    if ((code & 0xffffu) != Bp) continue;
-                    if (!selected<B>(p, pv, j, Bp, 0)) atomicAdd(&hist_u[code >> 16], 1u);
-                }
-            }
-        }
-        __threadfence();
-        __syncthreads();
-    }
-    if (mode_u == 0u) select_bin(p, &w.sel[1], su, hist_u, &s_sel, true);
-}
-
-// ---------------------------------------------------------------------------------------------
-// emit_body
-// ---------------------------------------------------------------------------------------------
-// s_stage: 128 float4 of shared memory per warp of the CTA
-template <int B>
-__device__ void emit_body(const Params &p, const Work &w, float *Q, float *u_out, unsigned *pruned_bitmap,
-                          unsigned *unified_bitmap, unsigned *sign_bits, float4 *s_stage) {
+__device__ __forceinline__ double store_unit(const Params &p, const Outs &o, unsigned unit, const float (&v)[16],
+                                             unsigned cls_p, unsigned cls_u, float4 *ws) {
     constexpr int NBT = 16 / B;
-    const SelView vp = view_of(&w.sel[0]);
-    const SelView vu = view_of(&w.sel[1]);
-    const long long n = p.n_floats;
     const int lane = threadIdx.x & 31;
-    const long long n_units = (n + 15) / 16;
-    const long long n_iter = (n_units + 31) / 32 * 32;      // whole warps take part in every step
-    const long long n_bm_words = (p.n_blocks + 31) / 32;
-    float4 *ws = s_stage + (threadIdx.x >> 5) * 128;         // one warp step of Q per warp
-    double resid_acc = 0.0;
-
-    for (long long unit = (long long)blockIdx.x * blockDim.x + threadIdx.x; unit < n_iter;
-         unit += (long long)gridDim.x * blockDim.x) {
-        const long long f = unit * 16;
-        const bool warp_full = (unit - lane + 32) * 16 <= n;      // all 512 floats of this warp step exist
-        unsigned code[NBT];
-        const long long j0 = unit * NBT;
-        if (j0 + NBT <= p.n_blocks) {
-            if (NBT == 1) code[0] = __ldcg(p.bins + j0);
-            else if (NBT == 2) { const uint2 c = __ldcg(reinterpret_cast<const uint2 *>(p.bins + j0)); code[0] = c.x; code[1 % NBT] = c.y; }
-            else {
+    const long long n = p.n_floats, f = (long long)unit * 16;
+    const unsigned n_units = (unsigned)((n + 15) / 16), n_blocks = (unsigned)p.n_blocks;
+    const bool warp_full = (long long)(unit - lane + 32u) * 16 <= n;      // all 512 floats of this warp step exist
+    const unsigned j0 = unit * NBT;
+    double resid = 0.0;
+    if (unit < n_units) {
+        unsigned sb = 0;
 #pragma unroll
-                for (int e = 0; e < NBT; e += 4) {
-                    const uint4 c = __ldcg(reinterpret_cast<const uint4 *>(p.bins + j0 + e));
-                    code[e % NBT] = c.x; code[(e + 1) % NBT] = c.y; code[(e + 2) % NBT] = c.z; code[(e + 3) % NBT] = c.w;
-                }
-            }
-        } else {
-#pragma unroll
-            for (int e = 0; e < NBT; ++e) code[e] = (j0 + e < p.n_blocks) ? __ldcg(p.bins + j0 + e) : 0u;
-        }
-        unsigned cls_p = 0, cls_u = 0;                       // bit e: block e of this thread
-        constexpr unsigned ALL = (1u << NBT) - 1u;
-        unsigned valid = 0;
+        for (int l = 0; l < 16; ++l) sb |= (v[l] < 0.f ? 1u : 0u) << l;
+        unsigned short *halves = reinterpret_cast<unsigned short *>(o.sign_bits);
+        halves[unit] = (unsigned short)sb;
+        if (unit == n_units - 1 && (n_units & 1)) halves[unit + 1] = 0;
+        float uo[NBT], q[16];
 #pragma unroll
         for (int e = 0; e < NBT; ++e) {
-            const long long j = j0 + e;
-            bool pr = false, un = false;
-            if (j < p.n_blocks) {
-                valid |= 1u << e;
-                pr = selected<B>(p, vp, j, code[e] & 0xffffu, 0);
-                un = !pr && selected<B>(p, vu, j, code[e] >> 16, 1);
+            const bool pr = (cls_p >> e) & 1u, un = (cls_u >> e) & 1u;
+            double a[B];
+#pragma unroll
+            for (int l = 0; l < B; ++l) a[l] = (double)fabsf(v[e * B + l]);
+            const double qd = __dmul_rn(tree_sum<B>(a), 1.0 / (double)B);
+            uo[e] = un ? __double2float_rn(qd) : 0.f;
+            if (p.resid && (pr || un)) {
+                // the loss of the block's class: distance to zero or to the unified block
+                double t[B];
+#pragma unroll
+                for (int l = 0; l < B; ++l) {
+                    const double d = pr ? a[l] : __dsub_rn(a[l], qd);
+                    t[l] = __dmul_rn(d, d);
+                }
+                resid += tree_sum<B>(t);
             }
-            cls_p |= (pr ? 1u : 0u) << e;
-            cls_u |= (un ? 1u : 0u) << e;
-        }
-        // q of the unified blocks and the sign plane come from stats_kernel; W is read again
-        // only where a block keeps its own values (everywhere for the dual update: it needs v)
-        float uo[NBT];
 #pragma unroll
-        for (int e = 0; e < NBT; ++e) uo[e] = 0.f;
-        if (cls_u) {
-#pragma unroll
-            for (int e = 0; e < NBT; ++e)
-                if ((cls_u >> e) & 1u) uo[e] = u_out[j0 + e];
-        }
-        if (unit < n_units) {
-            if (Q || p.U_next || p.resid) {
-                float v[16];
-                const bool admm = p.U_next != nullptr || p.resid != nullptr;
-                const bool need_v = admm || ((~cls_p & ~cls_u) & valid & ALL) != 0u;
-                if (need_v) load16(p.W, p.U, f, n, v);
-                else {
-#pragma unroll
-                    for (int l = 0; l < 16; ++l) v[l] = 0.f;
-                }
-                unsigned sb = 0;
-                if (cls_u) sb = reinterpret_cast<const unsigned short *>(sign_bits)[unit];
-                float q[16];
-#pragma unroll
-                for (int e = 0; e < NBT; ++e) {
-                    const bool pr = (cls_p >> e) & 1u, un = (cls_u >> e) & 1u;
-#pragma unroll
-                    for (int l = 0; l < B; ++l) {
-                        const bool neg = (sb >> (e * B + l)) & 1u;
-                        q[e * B + l] = pr ? 0.f : (un ? (neg ? -uo[e] : uo[e]) : v[e * B + l]);
-                    }
-                }
-                if (admm) {
-                    // dual update V - Q and ||V - Q||^2 (loss of the block's class)
-#pragma unroll
-                    for (int e = 0; e < NBT; ++e) {
-                        const bool pr = (cls_p >> e) & 1u, un = (cls_u >> e) & 1u;
-                        if (p.resid && (pr || un)) {
-                            double S, Lu, Kp;
-                            block_keys<B>(v + e * B, 0, &S, &Lu, &Kp);
-                            resid_acc += pr ? Kp : Lu;
-                        }
-                    }
-                    if (p.U_next) {
-                        if (f + 16 <= n) {
-                            float4 *dst = reinterpret_cast<float4 *>(p.U_next + f);
-#pragma unroll
-                            for (int c = 0; c < 4; ++c)
-                                dst[c] = make_float4(__fsub_rn(v[4 * c], q[4 * c]), __fsub_rn(v[4 * c + 1], q[4 * c + 1]),
-                                                     __fsub_rn(v[4 * c + 2], q[4 * c + 2]), __fsub_rn(v[4 * c + 3], q[4 * c + 3]));
-                        } else {
-#pragma unroll
-                            for (int l = 0; l < 16; ++l)
-                                if (f + l < n) p.U_next[f + l] = __fsub_rn(v[l], q[l]);
-                        }
-                    }
-                }
-                if (Q) {
-                if (!warp_full) {
-                    if (f + 16 <= n) {
-                        float4 *dst = reinterpret_cast<float4 *>(Q + f);
-                        dst[0] = make_float4(q[0], q[1], q[2], q[3]);
-                        dst[1] = make_float4(q[4], q[5], q[6], q[7]);
-                        dst[2] = make_float4(q[8], q[9], q[10], q[11]);
-                        dst[3] = make_float4(q[12], q[13], q[14], q[15]);
-                    } else {
-#pragma unroll
-                        for (int l = 0; l < 16; ++l)
-                            if (f + l < n) Q[f + l] = q[l];
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        ws[lane * 4 + (c ^ ((lane >> 1) & 3))] = make_float4(q[4 * c], q[4 * c + 1], q[4 * c + 2], q[4 * c + 3]);
-                }
-                }
+            for (int l = 0; l < B; ++l) {
+                const int k = e * B + l;
+                q[k] = pr ? 0.f : (un ? (((sb >> k) & 1u) ? -uo[e] : uo[e]) : v[k]);
             }
-            if (j0 + NBT <= p.n_blocks) {
-                if (NBT == 1) u_out[j0] = uo[0];
-                else if (NBT == 2) *reinterpret_cast<float2 *>(u_out + j0) = make_float2(uo[0], uo[1 % NBT]);
-                else {
+        }
+        if (p.U_next) {
+            // dual update: one fp32 subtraction per entry (v for a pruned block, +0 for a kept one)
+            if (f + 16 <= n) {
+                float4 *dst = reinterpret_cast<float4 *>(p.U_next + f);
 #pragma unroll
-                    for (int e = 0; e < NBT; e += 4)
-                        *reinterpret_cast<float4 *>(u_out + j0 + e) =
-                            make_float4(uo[e % NBT], uo[(e + 1) % NBT], uo[(e + 2) % NBT], uo[(e + 3) % NBT]);
-                }
+                for (int c = 0; c < 4; ++c)
+                    dst[c] = make_float4(__fsub_rn(v[4 * c], q[4 * c]), __fsub_rn(v[4 * c + 1], q[4 * c + 1]),
+                                         __fsub_rn(v[4 * c + 2], q[4 * c + 2]), __fsub_rn(v[4 * c + 3], q[4 * c + 3]));
             } else {
 #pragma unroll
-                for (int e = 0; e < NBT; ++e)
-                    if (j0 + e < p.n_blocks) u_out[j0 + e] = uo[e];
+                for (int l = 0; l < 16; ++l)
+                    if (f + l < n) p.U_next[f + l] = __fsub_rn(v[l], q[l]);
             }
         }
-        // Q of a whole warp step (2 KB): 16-byte stores at a 64-byte stride reach L2 as four partial
-        // writes per 64 bytes, so the step goes through shared memory and leaves as four stores of
-        // 512 contiguous bytes.  Thread t keeps piece c at slot c ^ ((t >> 1) & 3): no bank conflicts.
-        if (Q && warp_full) {
-            __syncwarp();
-            float4 *dst = reinterpret_cast<float4 *>(Q + (unit - lane) * 16);
+        if (o.Q && !warp_full) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int t = 8 * k + (lane >> 2), c = lane & 3;
-                dst[k * 32 + lane] = ws[t * 4 + (c ^ ((t >> 1) & 3))];
-            }
-            __syncwarp();
+            for (int l = 0; l < 16; ++l)
+                if (f + l < n) o.Q[f + l] = q[l];
+        } else if (o.Q) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                ws[lane * 4 + (c ^ ((lane >> 1) & 3))] = make_float4(q[4 * c], q[4 * c + 1], q[4 * c + 2], q[4 * c + 3]);
         }
-        // class bitmaps: the warp's 32 * NBT blocks make NBT words
-        {
-            const long long word0 = ((unit - lane) * NBT) >> 5;
 #pragma unroll
-            for (int w = 0; w < NBT; ++w) {
-                const int blk = w * 32 + lane;               // block of this warp step that lane reports
-                const unsigned sp = __shfl_sync(0xffffffffu, cls_p, blk / NBT);
-                const unsigned su = __shfl_sync(0xffffffffu, cls_u, blk / NBT);
-                const unsigned wp = __ballot_sync(0xffffffffu, (sp >> (blk % NBT)) & 1u);
-                const unsigned wu = __ballot_sync(0xffffffffu, (su >> (blk % NBT)) & 1u);
-                if (lane == 0 && word0 + w < n_bm_words) {
-                    pruned_bitmap[word0 + w] = wp;
-                    unified_bitmap[word0 + w] = wu;
-                }
+        for (int e = 0; e < NBT; ++e)
+            if (j0 + e < n_blocks) o.u[j0 + e] = uo[e];
+    }
+    // Q of a whole warp step (2 KB): 16-byte stores at a 64-byte stride reach L2 as four partial writes
+    // per 64 bytes, so the step goes through shared memory and leaves as four stores of 512 contiguous
+    // bytes.  Thread t keeps piece c at slot c ^ ((t >> 1) & 3): no bank conflicts.
+    if (o.Q && warp_full) {
+        __syncwarp();
+        float4 *dst = reinterpret_cast<float4 *>(o.Q + (long long)(unit - lane) * 16);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int t = 8 * k + (lane >> 2), c = lane & 3;
+            dst[k * 32 + lane] = ws[t * 4 + (c ^ ((t >> 1) & 3))];
+        }
+        __syncwarp();
+    }
+    // class bitmaps: the warp's 32 * NBT blocks make NBT words
+    const unsigned word0 = ((unit - lane) * NBT) >> 5, n_bm_words = (n_blocks + 31u) / 32u;
+#pragma unroll
+    for (int w = 0; w < NBT; ++w) {
+        const int blk = w * 32 + lane;                   // block of this warp step that lane reports
+        const unsigned xp = __shfl_sync(0xffffffffu, cls_p, blk / NBT);
+        const unsigned xu = __shfl_sync(0xffffffffu, cls_u, blk / NBT);
+        const unsigned wp = __ballot_sync(0xffffffffu, (xp >> (blk % NBT)) & 1u);
+        const unsigned wu = __ballot_sync(0xffffffffu, (xu >> (blk % NBT)) & 1u);
+        if (lane == 0 && word0 + w < n_bm_words) {
+            o.pruned_bitmap[word0 + w] = wp;
+            o.unified_bitmap[word0 + w] = wu;
+        }
+    }
+    return resid;
+}
+
+// class bits of block j from its keys
+__device__ __forceinline__ void add_class(const Params &p, const sel::Thresholds &T, unsigned j, unsigned e, u64 kp, u64 ku,
+                                          unsigned *cls_p, unsigned *cls_u) {
+    if (kp == NO_KEY) return;
+    const bool pr = T.pruned(kp, j, T.mode_p == 3u && group_pruned(p, j));
+    *cls_p |= (pr ? 1u : 0u) << e;
+    *cls_u |= (!pr && T.unified(ku, j) ? 1u : 0u) << e;
+}
+
+// What select_exact sees of a tensor: this thread's blocks with their keys in shared memory (slot t * NBT + e
+// holds block e of unit first + t * stride) ...
+template <int B, int NT>
+struct HeldKeys {
+    static constexpr int NBT = 16 / B;
+    const Params &p;
+    unsigned first, stride, units;
+    u64 *keys;                                           // this thread's column: prune key, then L_u, of each slot
+    template <class F>
+    __device__ __forceinline__ void for_blocks(F f) const {
+        const u64 *k = keys;
+        unsigned j0 = first * NBT;
+#pragma unroll 1
+        for (unsigned t = 0; t < units; ++t, j0 += stride * NBT) {
+#pragma unroll(NBT < 2 ? NBT : 2)
+            for (int e = 0; e < NBT; ++e, k += 2 * NT) f(j0 + e, k[0], k[NT]);
+        }
+    }
+    __device__ __forceinline__ bool in_group(unsigned j) const { return group_pruned(p, j); }
+};
+
+// ... or evaluated again in every phase
+template <int B>
+struct WalkedKeys {
+    static constexpr int NBT = 16 / B;
+    const Params &p;
+    unsigned first, stride;
+    template <class F>
+    __device__ __forceinline__ void for_blocks(F f) const {
+        const unsigned n_units = (unsigned)((p.n_floats + 15) / 16);
+        const Outs none = {};
+        unsigned bad = 0;
+        for (unsigned unit = first; unit < n_units; unit += stride) {
+            float v[16];
+            load16(p.W, p.U, (long long)unit * 16, p.n_floats, v);
+#pragma unroll
+            for (int e = 0; e < NBT; ++e) {
+                u64 kp, ku;
+                keys_of<B>(p, unit * NBT + e, v + e * B, &kp, &ku, none, &bad);
+                f(unit * NBT + e, kp, ku);
             }
         }
     }
-    if (p.resid) block_add_double(resid_acc, p.resid);
+    __device__ __forceinline__ bool in_group(unsigned j) const { return group_pruned(p, j); }
+};
+
+// approximate keys of this thread's sample block; false: it has none, or the block lies in a pruned group
+template <int B, int NT>
+__device__ __forceinline__ bool sample_of(const Params &p, const sel::Problem &pb, float *kp, float *ku) {
+    unsigned j;
+    *kp = *ku = 0.f;
+    if (!sel::sample_block_of<NT>(pb, threadIdx.x, &j)) return false;
+    block_keys_sample<B>(p.W, p.U, (long long)j, p.use_l1, kp, ku);
+    return !pb.by_group || !group_pruned(p, j);
+}
+
+// one CTA's shared memory of the exact phases: candidates while selecting, Q staging afterwards
+template <int NT>
+union ExactSmem {
+    sel::SelSmem sel;
+    float4 stage[NT / 32][128];
+};
+
+// The projection with keys evaluated in every phase, by all CTAs of a cooperative launch.  `team` has
+// its counters cleared.
+template <int B, int NT>
+__device__ __noinline__ void exact_walk(const Params &p, const Outs &o, const sel::Problem &pb, sel::GridTeam &team, ExactSmem<NT> &sm) {
+    constexpr int NBT = 16 / B;
+    const WalkedKeys<B> src = {p, team.cta * NT + threadIdx.x, team.n_cta * NT};
+    if (p.resid && team.cta == 0 && threadIdx.x == 0) *p.resid = 0.0;
+    sel::Thresholds T;
+    float sp, su;
+    const bool samp_ok = sample_of<B, NT>(p, pb, &sp, &su);
+    // (a barrier before the emit phase orders the cleared residual even when nothing is selected)
+    if (!sel::select_exact<NT>(src, team, sm.sel, pb, sp, su, samp_ok, p.dev_status, T) || !team.sync()) {
+        if (threadIdx.x == 0) atomicOr(p.dev_status, (unsigned)MWU_DEV_TIMEOUT);
+        return;
+    }
+    const unsigned n_units = (unsigned)((p.n_floats + 15) / 16);
+    double resid = 0.0;
+    unsigned bad = 0;
+    for (unsigned unit = src.first; unit < (n_units + 31u) / 32u * 32u; unit += src.stride) {
+        float v[16];
+        unsigned cp = 0, cu = 0;
+        load16(p.W, p.U, (long long)unit * 16, p.n_floats, v);
+#pragma unroll
+        for (int e = 0; e < NBT; ++e) {
+            u64 kp, ku;
+            keys_of<B>(p, unit * NBT + e, v + e * B, &kp, &ku, o, &bad);
+            add_class(p, T, unit * NBT + e, e, kp, ku, &cp, &cu);
+        }
+        resid += store_unit<B>(p, o, unit, v, cp, cu, sm.stage[threadIdx.x >> 5]);
+    }
+    if (bad) atomicOr(p.dev_status, (unsigned)MWU_DEV_NONFINITE);
+    if (p.resid) block_add_double(resid, p.resid);
+}
+
+constexpr int CL_THREADS = 512;                          // cluster form
+constexpr int GR_THREADS = 512;                          // grid form
+constexpr int EX_SLOTS = 8192;                           // most blocks a CTA holds: 16 bytes of keys each
+
+// The whole projection in one launch, keys held in shared memory: `units` units of 64 bytes a thread.
+// CLUSTER: one cluster of eight CTAs; otherwise a cooperative grid over a counter that the host has
+// cleared.
+template <int B, bool CLUSTER>
+__global__ void __launch_bounds__(CLUSTER ? CL_THREADS : GR_THREADS) exact_kernel(Params p, Outs o, sel::Problem pb, unsigned units) {
+    constexpr int NBT = 16 / B, NT = CLUSTER ? CL_THREADS : GR_THREADS;
+    extern __shared__ __align__(16) unsigned char mp_smem[];
+    __shared__ ExactSmem<NT> sm;
+    typename std::conditional<CLUSTER, sel::ClusterTeam, sel::GridTeam>::type team;
+    team.cta = blockIdx.x;
+    team.s = &sm.sel;
+    if constexpr (CLUSTER) {
+        __shared__ sel::ClusterCounts counts;
+        team.mine = &counts;
+        team.begin();
+    } else {
+        team.n_cta = gridDim.x;
+        team.x = p.xwork;
+        team.k = 0;
+    }
+    float v[16];
+    const unsigned first = blockIdx.x * NT + threadIdx.x;
+    load16(p.W, p.U, (long long)first * 16, p.n_floats, v);              // in flight beside the sample's loads
+    float sp, su;
+    const bool samp_ok = sample_of<B, NT>(p, pb, &sp, &su);
+    if (p.resid && blockIdx.x == 0 && threadIdx.x == 0) *p.resid = 0.0;
+    HeldKeys<B, NT> src = {p, first, gridDim.x * NT, units,
+                           reinterpret_cast<u64 *>(mp_smem) + threadIdx.x};
+    const unsigned n_units = (unsigned)((p.n_floats + 15) / 16);
+    unsigned bad = 0;
+    {
+        u64 *k = src.keys;
+#pragma unroll 1
+        for (unsigned t = 0; t < units; ++t) {
+            const unsigned unit = src.first + t * src.stride;
+            if (t) load16(p.W, p.U, (long long)unit * 16, p.n_floats, v);
+#pragma unroll
+            for (int e = 0; e < NBT; ++e, k += 2 * NT)
+                keys_of<B>(p, unit * NBT + e, v + e * B, k, k + NT, o, &bad);
+        }
+    }
+    if (bad) atomicOr(p.dev_status, (unsigned)MWU_DEV_NONFINITE);
+    if constexpr (CLUSTER) team.wait();                  // every CTA's counts are cleared
+    sel::Thresholds T;
+    bool ok = sel::select_exact<NT>(src, team, sm.sel, pb, sp, su, samp_ok, p.dev_status, T);
+    // with nothing to select there has been no barrier yet between the cleared residual and its sums
+    if (ok && p.resid && T.mode_p != 0u && T.mode_u != 0u) ok = team.sync();
+    if (!ok) {
+        if (threadIdx.x == 0) atomicOr(p.dev_status, (unsigned)MWU_DEV_TIMEOUT);
+        return;
+    }
+    __syncthreads();                                     // the candidates' memory becomes the staging buffer
+    double resid = 0.0;
+    const u64 *k = src.keys;
+#pragma unroll 1
+    for (unsigned t = 0; t < units; ++t) {
+        const unsigned unit = src.first + t * src.stride;
+        if (unit - (threadIdx.x & 31u) >= n_units) break;                // the whole warp is beyond the tensor
+        unsigned cp = 0, cu = 0;
+        if (units > 1u) load16(p.W, p.U, (long long)unit * 16, p.n_floats, v);
+#pragma unroll
+        for (int e = 0; e < NBT; ++e, k += 2 * NT) add_class(p, T, unit * NBT + e, e, k[0], k[NT], &cp, &cu);
+        resid += store_unit<B>(p, o, unit, v, cp, cu, sm.stage[threadIdx.x >> 5]);
+    }
+    if (p.resid) block_add_double(resid, p.resid);
+}
+
+// MWU_ALGO_MULTI_PASS on tensors whose keys do not fit
+constexpr int WALK_THREADS = 512;
+template <int B>
+__global__ void __launch_bounds__(WALK_THREADS) exact_walk_kernel(const __grid_constant__ Params p, const __grid_constant__ Outs o,
+                                                                  const __grid_constant__ sel::Problem pb) {
+    __shared__ ExactSmem<WALK_THREADS> sm;
+    sel::GridTeam team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u};
+    exact_walk<B, WALK_THREADS>(p, o, pb, team, sm);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1769,45 +1457,10 @@ __device__ __forceinline__ double apply_class(const Params &p, float *Q, float *
     return (pr ? sq : (un ? Lu : 0.0)) - (pr0 ? sq : (un0 ? Lu : 0.0));
 }
 
-constexpr int MP_SMEM_BYTES = (FIN_THREADS / 32) * 128 * 16;     // emit staging: 2 KB per warp
+constexpr int RES_SMEM_BYTES = (int)sizeof(ExactSmem<FIN_THREADS>);
 constexpr int CHG_PER_THREAD = 3;                    // list entries a thread classifies before the changed ones are applied
-static_assert(MP_SMEM_BYTES >= CAP * 20 + CHG_PER_THREAD * FIN_THREADS * 8,
+static_assert(RES_SMEM_BYTES >= CAP * 20 + CHG_PER_THREAD * FIN_THREADS * 8,
               "candidate buffers, corrections and the compaction buffer share the staging memory");
-
-// The multi-pass projection as a sequence of phases separated by grid barriers (cooperative launch):
-// [windows from a sample] -> statistics -> prune threshold -> unify threshold -> emit.  k counts the
-// barriers of the running kernel that have been passed.
-template <int B>
-__device__ void multipass_phases(const Params &p, Work &w, unsigned &k, bool run_sample, unsigned char *smem, float *Q,
-                                 double *loss_u, double *loss_p, float *u_out, unsigned *pruned_bitmap,
-                                 unsigned *unified_bitmap, unsigned *sign_bits) {
-    u64 *c_key = reinterpret_cast<u64 *>(smem);
-    unsigned *c_idx = reinterpret_cast<unsigned *>(smem + CAP * sizeof(u64));
-    bool ok = true;
-    if (run_sample) {
-        if (blockIdx.x == 0) sample_body<B>(p);
-        ok = grid_sync(&p.work->bar, ++k);
-    }
-    if (ok) {
-        load_work(p.work, &w);
-        stats_body<B>(p, w, loss_u, loss_p, u_out, sign_bits);
-        ok = grid_sync(&p.work->bar, ++k);
-    }
-    if (ok) {
-        prune_select_body<B>(p, w, c_key, c_idx);
-        ok = grid_sync(&p.work->bar, ++k);
-    }
-    if (ok) {
-        load_work(p.work, &w);
-        collect_body<1, B>(p, w, c_key, c_idx);
-        ok = grid_sync(&p.work->bar, ++k);
-    }
-    if (ok) {
-        load_work(p.work, &w);
-        emit_body<B>(p, w, Q, u_out, pruned_bitmap, unified_bitmap, sign_bits, reinterpret_cast<float4 *>(smem));
-    }
-    if (!ok && threadIdx.x == 0) atomicOr(p.dev_status, (unsigned)MWU_DEV_TIMEOUT);
-}
 
 // rank the m candidates in shared memory (c_key, c_idx) by (key, index); m <= CAP
 // c_aux (when the candidates fit one per thread: the return value) receives g_aux in the same order
@@ -1864,9 +1517,10 @@ __device__ bool rank_candidates(const Params &p, const u64 *g_key, const unsigne
 //      the CTA that finishes last, which fixes the threshold element and their classes.
 //      -- grid barrier --
 //   4  if any step gave the one-pass result up (a threshold outside its window, a threshold bin or
-//      tie group too large to rank, a full list), the multi-pass phases redo the projection here.
+//      tie group too large to rank, a full list), the exact phases redo the projection here.
 template <int B>
-__global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(Params p, float *Q, double *loss_u, double *loss_p,
+__global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_constant__ Params p,
+                                                              const __grid_constant__ sel::Problem pb, float *Q, double *loss_u, double *loss_p,
                                                               float *u_out, unsigned *pruned_bitmap,
                                                               unsigned *unified_bitmap, unsigned *sign_bits) {
     extern __shared__ __align__(16) unsigned char mp_smem[];
@@ -2088,22 +1742,10 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(Params p, float *Q
     }
     load_work(p.work, &w);
     if (w.failed == 0u) return;
-    multipass_phases<B>(p, w, k, false, mp_smem, Q, loss_u, loss_p, u_out, pruned_bitmap, unified_bitmap, sign_bits);
-}
-
-// ---------------------------------------------------------------------------------------------
-// multipass_kernel (cooperative launch): the whole multi-pass projection in one launch.  It is the
-// projection of small tensors (launch latency decides there) and of MWU_ALGO_MULTI_PASS.
-// ---------------------------------------------------------------------------------------------
-template <int B>
-__global__ void __launch_bounds__(FIN_THREADS) multipass_kernel(Params p, float *Q, double *loss_u, double *loss_p,
-                                                                float *u_out, unsigned *pruned_bitmap,
-                                                                unsigned *unified_bitmap, unsigned *sign_bits) {
-    extern __shared__ __align__(16) unsigned char mp_smem[];
-    __shared__ Work w;
-    unsigned k = 0;
-    multipass_phases<B>(p, w, k, p.run_sample != 0, mp_smem, Q, loss_u, loss_p, u_out, pruned_bitmap, unified_bitmap,
-                        sign_bits);
+    ExactSmem<FIN_THREADS> &sm = *reinterpret_cast<ExactSmem<FIN_THREADS> *>(mp_smem);
+    sel::GridTeam team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u};
+    const Outs o = {Q, loss_u, loss_p, u_out, pruned_bitmap, unified_bitmap, sign_bits};
+    exact_walk<B, FIN_THREADS>(p, o, pb, team, sm);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2251,28 +1893,58 @@ __global__ void __launch_bounds__(FIN_THREADS) group_select_kernel(const double 
 // ---------------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------------
-static size_t ws_off_hist() { return align_up(sizeof(proj::Work)); }
-static size_t ws_off_cand_key() { return align_up(ws_off_hist() + 5 * proj::NB_MAX * sizeof(unsigned)); }
+static size_t ws_off_xwork() { return align_up(sizeof(proj::Work)); }
+static size_t ws_off_hist() { return align_up(ws_off_xwork() + sizeof(sel::XWork)); }
+static size_t ws_off_cand_key() { return align_up(ws_off_hist() + 2 * proj::NB_MAX * sizeof(unsigned)); }
 // two sets of candidates: the two halves of resolve_kernel each keep their own
 static size_t ws_off_cand_idx() { return align_up(ws_off_cand_key() + 2 * proj::CAP * sizeof(proj::u64)); }
 static size_t ws_off_cand_aux() { return align_up(ws_off_cand_idx() + 2 * proj::CAP * sizeof(unsigned)); }
 static size_t ws_off_samp() { return align_up(ws_off_cand_aux() + 2 * proj::CAP * sizeof(unsigned)); }
-static size_t ws_off_bins() { return align_up(ws_off_samp() + 2 * proj::NSAMP * sizeof(proj::u64)); }
-static size_t ws_off_list(size_t mb) { return align_up(ws_off_bins() + (mb + 8) * sizeof(unsigned)); }
-// candidate list of the one-pass pipeline: a quarter of the blocks (the windows hold a few per cent)
-static size_t list_capacity(size_t mb) { return mb / 4 + 4096; }
-static size_t ws_off_gkey(size_t mb) { return align_up(ws_off_list(mb) + list_capacity(mb) * sizeof(uint2)); }
+static size_t ws_off_list() { return align_up(ws_off_samp() + 2 * proj::NSAMP * sizeof(proj::u64)); }
+// candidate list of the one-pass pipeline: a quarter of the blocks (the windows hold a few per cent;
+// of a small tensor they may hold more)
+static size_t list_capacity(size_t mb) { return mb / 4 + 65536; }
+static size_t ws_off_gkey(size_t mb) { return align_up(ws_off_list() + list_capacity(mb) * sizeof(uint2)); }
 static size_t n_groups_of(const mwu_proj_desc *d) {
     return grouped(d) ? (size_t)(d->rows / d->prune_group_rows) * (size_t)(d->cols / d->prune_group_cols) : 0;
 }
 static size_t ws_off_gprune(const mwu_proj_desc *d, size_t mb) { return align_up(ws_off_gkey(mb) + n_groups_of(d) * sizeof(double)); }
 
-static bool use_one_pass(const mwu_proj_desc *desc) {
-    const long long mb = desc->rows * desc->cols / desc->block;
-    if (mb >= (1ll << 30)) return false;               // list entries keep two class bits above the block index
-    if (desc->algo == MWU_ALGO_ONE_PASS) return true;
-    if (desc->algo == MWU_ALGO_MULTI_PASS) return false;
-    return mb >= proj::ONE_PASS_MIN_BLOCKS;
+// Which pipeline, and how many units of 64 bytes a thread of the exact kernel holds.
+//
+// Both lines were measured on whole mwu_project calls (50 % / 25 %, us).  Up to 32768 blocks a cluster
+// beats the grid (256 x 256, b = 4: 18.7 against 27.2; 256 x 1024, b = 16: 23.1 / 27.1; at the line, b = 8:
+// 29.0 / 28.1): its barriers cost half, but its eight SMs also have all the arithmetic.  Up to 4096 blocks a
+// CTA on every SM (606208 on 148) the exact kernel beats the one-pass pipeline's four launches (512 x 1152,
+// b = 8: 24 against 39; 2048 x 2048, b = 8, 524288 blocks: 45 / 52; 1024 x 2048, b = 4: 42 / 46), beyond it
+// does not (1024 x 2048, b = 2, 1048576 blocks: 67 / 54): the phases' L2 counts grow with the blocks.
+constexpr long long EX_CLUSTER_BLOCKS = 32768, EX_AUTO_BLOCKS_PER_CTA = 4096;
+struct Route {
+    bool one_pass, cluster;         // else the exact kernel: as one cluster or as a cooperative grid
+    int grid, held;                 // its CTAs and units per thread (0: keys evaluated in every phase)
+};
+static Route route_of(const mwu_proj_desc *desc, int sm_count) {
+    const long long mb = desc->rows * desc->cols / desc->block, units = (desc->rows * desc->cols + 15) / 16;
+    Route r = {false, false, 0, 0};
+    if (desc->algo == MWU_ALGO_ONE_PASS && mb < (1ll << 30)) {      // list entries keep two class bits above the block index
+        r.one_pass = true;
+        return r;
+    }
+    if (desc->algo == MWU_ALGO_AUTO && mb > EX_AUTO_BLOCKS_PER_CTA * sm_count && mb < (1ll << 30)) {
+        r.one_pass = true;
+        return r;
+    }
+    r.cluster = mb <= EX_CLUSTER_BLOCKS;
+    const long long threads = r.cluster ? proj::CL_THREADS : proj::GR_THREADS;
+    const long long ctas = (units + threads - 1) / threads;          // with one unit a thread
+    r.grid = r.cluster ? sel::CLUSTER_CTAS : (int)(ctas < sm_count ? ctas : sm_count);
+    const long long held = (ctas + r.grid - 1) / r.grid;
+    if (held * threads * (16 / desc->block) <= proj::EX_SLOTS) r.held = (int)held;
+    else {
+        r.cluster = false;
+        r.one_pass = desc->algo == MWU_ALGO_AUTO && mb < (1ll << 30);
+    }
+    return r;
 }
 
 }  // namespace mwu
@@ -2301,10 +1973,36 @@ static cudaError_t launch_cooperative(void (*kern)(Args...), int grid, int threa
 }
 
 template <int B>
-static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_desc *desc, float *Q,
-                                  float *u, unsigned *pb, unsigned *ub, unsigned *sb, double *loss_u,
-                                  double *loss_p, int sm_count, bool one_pass, double *gkey, unsigned *gprune,
-                                  cudaStream_t st) {
+static cudaError_t launch_exact_held(const mwu::proj::Params &p, const mwu::proj::Outs &o, const mwu::Route &route, int sm_count,
+                                     cudaStream_t st) {
+    using namespace mwu::proj;
+    const int threads = route.cluster ? CL_THREADS : GR_THREADS;
+    const int smem = route.held * (16 / B) * threads * 16;
+    const mwu::sel::Problem pb = mwu::sel::problem_of(p.n_blocks, p.k_prune, p.k_unify, p.gprune != nullptr, threads);
+    auto kern = route.cluster ? exact_kernel<B, true> : exact_kernel<B, false>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, EX_SLOTS * 16);
+    if (e != cudaSuccess) return e;
+    if (!route.cluster)
+        return launch_cooperative(kern, route.grid, threads, (size_t)smem, sm_count, st, p, o, pb, (unsigned)route.held);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)route.grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)route.grid;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    mwu::count_launch();
+    return cudaLaunchKernelEx(&cfg, kern, p, o, pb, (unsigned)route.held);
+}
+
+template <int B>
+static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_desc *desc, const mwu::proj::Outs &o,
+                                  int sm_count, const mwu::Route &route, double *gkey, unsigned *gprune, cudaStream_t st) {
     using namespace mwu::proj;
     cudaError_t e;
     if (p.gprune) {
@@ -2321,6 +2019,15 @@ static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_des
         mwu::count_launch(2);
     }
     const long long n_units = (p.n_floats + 15) / 16;
+    if (!route.one_pass) {
+        // the grid form's barrier counter and counts start at zero; a cluster clears them itself
+        if (!route.cluster && cudaMemsetAsync(p.xwork, 0, mwu::sel::XWORK_ZERO_BYTES, st) != cudaSuccess) return cudaErrorUnknown;
+        if (route.held) return launch_exact_held<B>(p, o, route, sm_count, st);
+        const long long want = (n_units + WALK_THREADS - 1) / WALK_THREADS;
+        return launch_cooperative(exact_walk_kernel<B>, (int)(want < 2ll * sm_count ? want : 2ll * sm_count), WALK_THREADS, 0,
+                                  sm_count, st, p, o,
+                                  mwu::sel::problem_of(p.n_blocks, p.k_prune, p.k_unify, p.gprune != nullptr, WALK_THREADS));
+    }
     const long long want = (n_units + 255) / 256;
     const long long cap_blocks = (long long)sm_count * 8;
     const int grid_stream = (int)(want < cap_blocks ? (want > 0 ? want : 1) : cap_blocks);
@@ -2328,53 +2035,44 @@ static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_des
     const bool need_p = !p.gprune && desc->k_prune > 0 && desc->k_prune < mb;
     const long long ksel_u = desc->k_unify - desc->k_prune;
     const bool need_u = ksel_u > 0 && ksel_u < mb - desc->k_prune;
-    const long long want_mp = (n_units + FIN_THREADS - 1) / FIN_THREADS;
-    const int grid_mp = (int)(want_mp < (long long)sm_count ? (want_mp > 0 ? want_mp : 1) : (long long)sm_count);
-    static bool smem_set = false;                       // per instantiation: the attribute sticks to the function
-    if (!smem_set) {
-        e = cudaFuncSetAttribute(multipass_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, MP_SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(resolve_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, MP_SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        smem_set = true;
-    }
-
-    if (one_pass) {
-        // the sample keys (and the cleared histograms) from 32 SMs, then one CTA ranks the sample; the two
-        // kernels behind are launched with programmatic stream serialization, so their CTAs are in place
-        // (and the sweep's first loads in flight) when their predecessor ends
-        const unsigned n_zero = 5u * (unsigned)p.nb;
-        sample_keys_kernel<B><<<NSAMP / 128, 128, 0, st>>>(p, p.hist, n_zero);
-        {
-            cudaLaunchConfig_t cfg = {};
-            cfg.stream = st;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            cfg.gridDim = dim3(1);
-            cfg.blockDim = dim3(SAMP_THREADS);
-            e = cudaLaunchKernelEx(&cfg, sample_kernel<B>, p);
-            if (e != cudaSuccess) return e;
-            cfg.gridDim = dim3((unsigned)grid_stream);
-            cfg.blockDim = dim3(256);
-            if (p.U_next || p.resid) e = cudaLaunchKernelEx(&cfg, pass_kernel<B, true>, p, Q, loss_u, loss_p, u, pb, ub, sb);
-            else e = cudaLaunchKernelEx(&cfg, pass_kernel<B, false>, p, Q, loss_u, loss_p, u, pb, ub, sb);
-            if (e != cudaSuccess) return e;
-        }
-        mwu::count_launch(3);
-        if (!need_p && !need_u) return cudaGetLastError();       // no threshold: every class is final
-        // the list holds a few per cent of the blocks: a thread per expected entry, one CTA per SM at most.
-        // Should the one-pass result be given up (once in thousands of calls), the same kernel redoes the
-        // projection with the multi-pass phases.
-        const long long lb = (mb / 8 + FIN_THREADS - 1) / FIN_THREADS;
-        const int grid_list = (int)(lb < (long long)sm_count ? (lb > 16 ? lb : 16) : (long long)sm_count);
-        return launch_cooperative(resolve_kernel<B>, grid_list, FIN_THREADS, (size_t)MP_SMEM_BYTES, sm_count, st, p, Q,
-                                  loss_u, loss_p, u, pb, ub, sb);
-    }
-    return launch_cooperative(multipass_kernel<B>, grid_mp, FIN_THREADS, (size_t)MP_SMEM_BYTES, sm_count, st, p, Q, loss_u,
-                              loss_p, u, pb, ub, sb);
+    e = cudaFuncSetAttribute(resolve_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    // the sample keys (and the cleared histograms) from 32 SMs, then one CTA ranks the sample; the two
+    // kernels behind are launched with programmatic stream serialization, so their CTAs are in place
+    // (and the sweep's first loads in flight) when their predecessor ends
+    unsigned *zero = reinterpret_cast<unsigned *>(p.xwork);
+    const unsigned n_zero = (unsigned)(p.fhist - zero) + 2u * (unsigned)p.nb;
+    sample_keys_kernel<B><<<NSAMP / 128, 128, 0, st>>>(p, zero, n_zero);
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(SAMP_THREADS);
+    e = cudaLaunchKernelEx(&cfg, sample_kernel, p);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3((unsigned)grid_stream);
+    cfg.blockDim = dim3(256);
+    if (p.U_next || p.resid)
+        e = cudaLaunchKernelEx(&cfg, pass_kernel<B, true>, p, o.Q, o.loss_u, o.loss_p, o.u, o.pruned_bitmap, o.unified_bitmap,
+                               o.sign_bits);
+    else
+        e = cudaLaunchKernelEx(&cfg, pass_kernel<B, false>, p, o.Q, o.loss_u, o.loss_p, o.u, o.pruned_bitmap,
+                               o.unified_bitmap, o.sign_bits);
+    if (e != cudaSuccess) return e;
+    mwu::count_launch(3);
+    if (!need_p && !need_u) return cudaGetLastError();       // no threshold: every class is final
+    // the list holds a few per cent of the blocks: a thread per expected entry, one CTA per SM at most.
+    // Should the one-pass result be given up (once in thousands of calls), the same kernel redoes the
+    // projection with the exact phases.
+    const long long lb = (mb / 8 + FIN_THREADS - 1) / FIN_THREADS;
+    const int grid_list = (int)(lb < (long long)sm_count ? (lb > 16 ? lb : 16) : (long long)sm_count);
+    return launch_cooperative(resolve_kernel<B>, grid_list, FIN_THREADS, (size_t)RES_SMEM_BYTES, sm_count, st, p,
+                              mwu::sel::problem_of(p.n_blocks, p.k_prune, p.k_unify, p.gprune != nullptr, FIN_THREADS), o.Q,
+                              o.loss_u, o.loss_p, o.u, o.pruned_bitmap, o.unified_bitmap, o.sign_bits);
 }
 
 // mwu_project and mwu_admm_step: the latter also wants U_next and / or residual_sq
@@ -2403,7 +2101,7 @@ static int project_impl(const mwu_proj_desc *desc, const float *W, const float *
     if (shape_of(desc).shaped)                          // 2- and 3-dim blocks: the block-by-block path
         return shapes::project(desc, W, U_dual, Q, U_next, residual_sq, u, pruned_bitmap, unified_bitmap, sign_bits,
                                loss_u, loss_p, dev_status, workspace, sm_count, st);
-    const bool one_pass = use_one_pass(desc);
+    const Route route = route_of(desc, sm_count);
     proj::Params p;
     p.W = W;
     p.U = U_dual;
@@ -2413,18 +2111,15 @@ static int project_impl(const mwu_proj_desc *desc, const float *W, const float *
     p.use_l1 = desc->prune_key == MWU_PRUNE_KEY_L1;
     p.work = (proj::Work *)ws;
     p.nb = p.n_blocks <= (8ll << 20) ? proj::NB_SMALL : proj::NB_MAX;
-    p.hist = (unsigned *)(ws + ws_off_hist());
-    p.fhist = p.hist + 3 * (size_t)p.nb;
+    p.xwork = (sel::XWork *)(ws + ws_off_xwork());
+    p.fhist = (unsigned *)(ws + ws_off_hist());
     p.cand_key = (proj::u64 *)(ws + ws_off_cand_key());
     p.cand_idx = (unsigned *)(ws + ws_off_cand_idx());
     p.cand_aux = (unsigned *)(ws + ws_off_cand_aux());
     p.samp_kp = (proj::u64 *)(ws + ws_off_samp());
     p.samp_ku = p.samp_kp + proj::NSAMP;
-    p.bins = (unsigned *)(ws + ws_off_bins());
-    p.list = (uint2 *)(ws + ws_off_list((size_t)p.n_blocks));
+    p.list = (uint2 *)(ws + ws_off_list());
     p.list_cap = (unsigned)list_capacity((size_t)p.n_blocks);
-    p.gated = one_pass ? 1 : 0;
-    p.run_sample = one_pass ? 0 : 1;
     p.dev_status = dev_status;
     p.U_next = U_next;
     p.resid = residual_sq;
@@ -2444,17 +2139,13 @@ static int project_impl(const mwu_proj_desc *desc, const float *W, const float *
         p.groups_per_row = (unsigned)(desc->cols / desc->prune_group_cols);
     }
 
-    // The one-pass pipeline clears its selection state and histograms in its first kernel; the
-    // multi-pass kernel, launched alone, needs them (and its barrier counter) cleared beforehand.
-    if (!one_pass &&
-        cudaMemsetAsync(ws, 0, ws_off_hist() + 5 * (size_t)p.nb * sizeof(unsigned), st) != cudaSuccess)
-        return MWU_ERR_CUDA;
+    const proj::Outs o = {Q, loss_u, loss_p, u, pruned_bitmap, unified_bitmap, sign_bits};
     cudaError_t e;
     switch (desc->block) {
-        case 2: e = launch_project<2>(p, desc, Q, u, pruned_bitmap, unified_bitmap, sign_bits, loss_u, loss_p, sm_count, one_pass, gkey, gprune, st); break;
-        case 4: e = launch_project<4>(p, desc, Q, u, pruned_bitmap, unified_bitmap, sign_bits, loss_u, loss_p, sm_count, one_pass, gkey, gprune, st); break;
-        case 8: e = launch_project<8>(p, desc, Q, u, pruned_bitmap, unified_bitmap, sign_bits, loss_u, loss_p, sm_count, one_pass, gkey, gprune, st); break;
-        default: e = launch_project<16>(p, desc, Q, u, pruned_bitmap, unified_bitmap, sign_bits, loss_u, loss_p, sm_count, one_pass, gkey, gprune, st); break;
+        case 2: e = launch_project<2>(p, desc, o, sm_count, route, gkey, gprune, st); break;
+        case 4: e = launch_project<4>(p, desc, o, sm_count, route, gkey, gprune, st); break;
+        case 8: e = launch_project<8>(p, desc, o, sm_count, route, gkey, gprune, st); break;
+        default: e = launch_project<16>(p, desc, o, sm_count, route, gkey, gprune, st); break;
     }
     return e == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
 }

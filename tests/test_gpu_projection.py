@@ -304,3 +304,25 @@ def test_projection_largest_sweep_size_properties():
     assert float(Lu[unified].max()) <= float(Lu[kept].min()) * (1 + 1e-12)
     # the unified value is the mean magnitude
     assert torch.allclose(u[unified].double(), q[unified, 0], rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("b,rows,cols,permille", [(2, 256, 256, (500, 250)),      # 32768 blocks: the last one-cluster size
+                                                  (2, 256, 258, (500, 250)),      # just above: a cooperative grid
+                                                  (16, 512, 1024, (900, 0)),      # one cluster, eight units a thread
+                                                  (16, 513, 1024, (0, 0)),
+                                                  (4, 2368, 1024, (600, 300)),    # 606208 blocks: all SMs full
+                                                  (8, 3, 8, (700, 300)), (16, 1, 16, (1000, 0))])
+def test_projection_exact_kernel_size_edges(b, rows, cols, permille):
+    W = inputs.normal_weights(rows, cols, 0.02, 6000 + b)
+    Mb = rows * cols // b
+    check_against_oracle(W, b, O.count_from_permille(Mb, permille[0]), O.count_from_permille(Mb, permille[1]),
+                         algos=(B.MWU_ALGO_AUTO, B.MWU_ALGO_MULTI_PASS))
+
+
+@pytest.mark.parametrize("rows,k_prune,k_unify", [(64, 5, 3000), (640, 40000, 81000), (640, 0, 81919)])
+def test_projection_exact_kernel_ties_beyond_the_candidate_list(rows, k_prune, k_unify):
+    """Thousands of blocks with one key: the threshold is found by block index (cluster and grid form)."""
+    blk = torch.tensor([0.5, -0.25, 0.125, 1.0, -0.5, 0.75, 0.25, -0.125])
+    W = blk.repeat(rows * 128).reshape(rows, 1024).contiguous()
+    W[:, 512:516] += 0.01
+    check_against_oracle(W, 8, k_unify, k_prune, algos=(B.MWU_ALGO_AUTO,))
