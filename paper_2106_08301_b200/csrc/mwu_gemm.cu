@@ -1,7 +1,7 @@
 // mwu_gemm / mwu_conv_implicit: Y = X . W_hat^T on the packed weights (Section 3.2).
 //
-// One persistent CTA per SM works on tiles of 256 activation rows x 256 weight rows (128
-// activation rows when the problem has no more).  A 64-wide k stage of the weight
+// One persistent CTA per SM works on tiles of 256 activation rows x 256 weight rows (128 rows for a
+// convolution with no more pixels; a GEMM of few rows takes mwu_gemm4.cu).  A 64-wide k stage of the weight
 // tile is decoded once into shared memory and multiplied with both 128-row halves of the
 // activation tile, which halves decode work, shared-memory stores and slot hand-shakes per FLOP.
 // Warp roles:
@@ -30,6 +30,10 @@ namespace gemm {
 // pair kernel (two CTAs per tile), defined in mwu_gemm2.cu
 bool pair_eligible(const Params &p);
 cudaError_t launch_pair(int bw, const CUtensorMap &tmap, const Params &p, int sm_count, cudaStream_t st);
+// few activation rows, defined in mwu_gemm4.cu
+bool stream_eligible(const Params &p, int sm_count);
+int stream_box_rows(const Params &p, int sm_count);
+cudaError_t launch_stream(int bw, const CUtensorMap &tmap_x, const Params &p, int sm_count, cudaStream_t st);
 // decode-once path, defined in mwu_gemm3.cu
 cudaError_t launch_decode(int bw, const Params &p, __nv_bfloat16 *Wd, long long ldw, cudaStream_t st);
 cudaError_t launch_dense(const CUtensorMap &tmap_x, const CUtensorMap &tmap_w, const CUtensorMap &tmap_y,
@@ -622,6 +626,13 @@ extern "C" int mwu_gemm_ws(const mwu_proj_desc *desc, const void *packed, const 
     p.ldy = ldy;
     if (p.n_stages > MAX_STAGES_K) return MWU_ERR_SHAPE;
 
+    if (stream_eligible(p, sm_count)) {
+        CUtensorMap tmap_x;
+        if (!encode_bf16_2d(encode, &tmap_x, X, desc->cols, M, ldx, stream_box_rows(p, sm_count)))
+            return MWU_ERR_CUDA;
+        return launch_stream(desc->block, tmap_x, p, sm_count, st) == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
+    }
+
     // decode once into the caller's workspace, then a two-operand GEMM over it
     const size_t need = mwu_gemm_workspace_bytes(desc, M);
     if (workspace && need && workspace_bytes >= need) {
@@ -643,28 +654,24 @@ extern "C" int mwu_gemm_ws(const mwu_proj_desc *desc, const void *packed, const 
         return launch_dense(tmap_x, tmap_w, tmap_y, p, sm_count, st) == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
     }
 
-    // tiles of 256 activation rows unless the problem has no second half to fill
-    const int mt = (M > BMH) ? 2 : 1;
-    const int bm = mt * BMH;
+    // more than 256 rows (fewer take the streaming kernel): tiles of 256 activation rows
+    constexpr int bm = 2 * BMH;
     CUtensorMap tmap;
     if (!encode_bf16_2d(encode, &tmap, X, desc->cols, M, ldx, bm)) return MWU_ERR_CUDA;
     const int nrec = p.n_rec_tiles >= 2 ? 2 : 1;
     const long long tiles = ((M + bm - 1) / bm) * ((p.n_rec_tiles + nrec - 1) / nrec);
     const int grid = (int)(tiles < sm_count ? tiles : sm_count);
-    size_t smem = smem_bytes(nrec, mt, p.n_stages, 0);
+    size_t smem = smem_bytes(nrec, 2, p.n_stages, 0);
     if (smem > 227 * 1024) return MWU_ERR_SHAPE;
-    cudaError_t e;
     // bf16 rows are 16-byte aligned (checked above), which the staged epilogue stores need
     if (!y_dtype && smem + NEPI_WARPS * 2048 <= 227 * 1024) {
         p.stage_epi = 1;
         smem += NEPI_WARPS * 2048;
     }
-    if (mt == 2 && pair_eligible(p))
+    if (pair_eligible(p))
         return launch_pair(desc->block, tmap, p, sm_count, st) == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
-    if (mt == 2) e = (nrec == 2) ? launch_bw<0, 2, 2>(desc->block, tmap, p, grid, smem, st)
-                                 : launch_bw<0, 1, 2>(desc->block, tmap, p, grid, smem, st);
-    else e = (nrec == 2) ? launch_bw<0, 2, 1>(desc->block, tmap, p, grid, smem, st)
-                         : launch_bw<0, 1, 1>(desc->block, tmap, p, grid, smem, st);
+    const cudaError_t e = (nrec == 2) ? launch_bw<0, 2, 2>(desc->block, tmap, p, grid, smem, st)
+                                      : launch_bw<0, 1, 2>(desc->block, tmap, p, grid, smem, st);
     return e == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
 }
 

@@ -1,0 +1,446 @@
+// mwu_gemm for few activation rows: the packed weights streamed through the tensor cores once.
+//
+// With few activation rows the product is bound by the packed bytes (16384 x 4096, b = 16, 80 % / 60 %,
+// 16 rows: 41 MB, 6.3 us at the copy bandwidth).  Expanding the weights first writes and reads them again
+// as 134 MB of bf16, so here a record is decoded in shared memory and multiplied there, and nothing but
+// the output leaves the SM.  The weights are the M operand (128 rows of a record on the 128
+// tensor-memory lanes), the activation rows the N operand, so 16 rows cost an MMA of N = 16.
+//
+// One CTA: one 128-row weight tile, up to 128 activation rows, a range of the 64-wide k stages; the CTAs
+// that share a tile's stages form a cluster (`split` of them) and add up their partial sums through
+// distributed shared memory, in rank order.  Roles:
+//   decode     groups of two warps, each with a weight tile and a box of X of its own, take the records in
+//              turn.  A record is a chain of short waits (list entries from L2, the tile's last MMA, zeroing,
+//              scattering, the proxy fence, the next MMA), about 2000 cycles however many threads share
+//              it, so 6 to 12 groups an SM work on as many records at a time: two groups of eight warps an SM
+//              took 38 us for the call above.  The lists of a group's next record are brought to L2 one turn
+//              ahead.  The tile is zeroed first, so pruned blocks need neither their list nor a store.
+//   MMA        one warp: tensor memory, the MMAs in record order, a commit per record frees its group.
+// Two CTAs to an SM.
+// Every wait on an mbarrier is bounded; when one runs out the kernel raises MWU_DEV_TIMEOUT, waits for
+// its copies in flight, frees tensor memory and returns.  Tensor memory is given back before the cluster
+// barrier, so holding it never depends on another CTA.
+#include "mwu_gemm_dev.cuh"
+
+namespace mwu {
+namespace gemm {
+
+constexpr int ST_GROUP = 64;                        // threads of a decode group
+constexpr int ST_MAX_GROUPS = 6;
+constexpr int ST_MAX_THREADS = ST_MAX_GROUPS * ST_GROUP + 32;
+constexpr int ST_MAX_ROWS = 128;                    // activation rows of a CTA
+constexpr int ST_SMEM_CTA = 227 * 512 - 1024;       // two CTAs an SM; each costs 1 KB besides
+
+struct StreamParams {
+    int mpad;                   // activation rows of a CTA, a multiple of 16
+    int m_tiles;
+    int split;                  // CTAs of a cluster
+    int stages_per;             // k stages of a CTA (the last one of a cluster may have fewer)
+    int groups;
+    unsigned tmem_cols;
+};
+
+struct StreamSmem {
+    unsigned long long x_full[ST_MAX_GROUPS], tile_full[ST_MAX_GROUPS], tile_empty[ST_MAX_GROUPS], tfull;
+    unsigned tmem_base;
+    int abort;
+    int drain_abort;
+};
+
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, unsigned (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ float4 ld_cluster_f4(unsigned addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+// barrier over the 64 threads of one decode group; true when `pred` held in any of them
+__device__ __forceinline__ bool group_any(int group, bool pred) {
+    unsigned r;
+    __syncwarp();
+    asm volatile(
+        "{\n\t.reg .pred a, b;\n\t"
+        "setp.ne.u32 a, %1, 0;\n\t"
+        "bar.red.or.pred b, %2, %3, a;\n\t"
+        "selp.u32 %0, 1, 0, b;\n\t}"
+        : "=r"(r) : "r"(pred ? 1u : 0u), "r"(1 + group), "n"(ST_GROUP) : "memory");
+    return r != 0u;
+}
+
+__device__ __forceinline__ void group_sync(int group) {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(ST_GROUP) : "memory");
+}
+
+// the lines of `bytes` bytes from p on, spread over a decode group
+__device__ __forceinline__ void prefetch_span(const unsigned char *p, unsigned bytes, unsigned t0) {
+    for (unsigned l = t0 * 128u; l < bytes; l += ST_GROUP * 128u) prefetch_l2(p + l);
+}
+
+template <int BW>
+__global__ void __launch_bounds__(ST_MAX_THREADS)
+mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ Params p,
+                       const __grid_constant__ StreamParams q) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched while the kernel before may still run
+    MWU_CHECK_HEADER(p);
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *base = reinterpret_cast<unsigned char *>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *tiles = base;
+    unsigned char *xbuf = tiles + q.groups * REC_BYTES;
+    const unsigned x_bytes = (unsigned)q.mpad * (BK * 2);
+    StreamSmem *sm = reinterpret_cast<StreamSmem *>(xbuf + q.groups * x_bytes);
+    uint4 *srec = reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(sm) + ((sizeof(StreamSmem) + 15) & ~(size_t)15));
+    float *part = reinterpret_cast<float *>(base);          // partial sums [mpad][128], once everything is multiplied
+    volatile int *abort = &sm->abort;
+
+    const int n_threads = q.groups * ST_GROUP + 32, mma_warp = q.groups * (ST_GROUP / 32);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const unsigned rank = blockIdx.x % (unsigned)q.split, unit = blockIdx.x / (unsigned)q.split;
+    const unsigned mt = unit % (unsigned)q.m_tiles;
+    const long long rt = unit / (unsigned)q.m_tiles;
+    const int k0 = (int)rank * q.stages_per;
+    int n_st = (int)p.n_stages - k0;
+    n_st = n_st < 0 ? 0 : (n_st > q.stages_per ? q.stages_per : n_st);
+
+    if (tid == 0) {
+        for (int g = 0; g < ST_MAX_GROUPS; ++g) {
+            mbar_init(smem_u32(&sm->x_full[g]), 1);
+            mbar_init(smem_u32(&sm->tile_full[g]), ST_GROUP / 32);
+            mbar_init(smem_u32(&sm->tile_empty[g]), 1);
+        }
+        mbar_init(smem_u32(&sm->tfull), 1);
+        sm->abort = 0;
+        sm->drain_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    if (warp == mma_warp) tmem_alloc(smem_u32(&sm->tmem_base), q.tmem_cols);
+    // the record table of this CTA's stages
+    if (n_st > 0) {
+        const uint4 *recs = reinterpret_cast<const uint4 *>(p.packed + p.off_rec) + rt * p.n_stages + k0;
+        for (int i = tid; i <= n_st; i += n_threads) srec[i] = __ldg(recs + i);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const unsigned tmem_base = *reinterpret_cast<volatile unsigned *>(&sm->tmem_base);
+    // a record whose ranges do not lie inside the sections is not touched
+    for (int i = tid; i < n_st; i += n_threads) {
+        const uint4 a = srec[i], b = srec[i + 1];
+        if (a.x > b.x || b.x > p.n_unified || a.y > b.y || b.y > p.n_dense ||
+            (b.x - a.x) + (b.y - a.y) > (unsigned)(kTileRows * BK / BW)) {
+            atomicOr(p.dev_status, (unsigned)MWU_DEV_BOUNDS);
+            srec[i].w = 0u;
+        }
+    }
+    __syncthreads();
+    bool any = false;
+    for (int i = 0; i < n_st; ++i) any = any || (srec[i].w & 0xFu) != 0u;
+
+    if (warp == mma_warp) {
+        // ---------------- MMA issuer ----------------
+        const unsigned idesc = make_idesc(q.mpad);
+        unsigned n = 0, g = 0, phase = 0;
+        bool ok = true;
+        for (int i = 0; i < n_st; ++i) {
+            const unsigned live = srec[i].w & 0xFu;
+            if (!live) continue;
+            if (!mbar_wait_spin(smem_u32(&sm->tile_full[g]), phase, abort) ||
+                !mbar_wait_spin(smem_u32(&sm->x_full[g]), phase, abort)) ok = false;
+            if (!__all_sync(0xffffffffu, ok)) break;
+            tc_fence_after();
+            const unsigned long long adesc = make_desc(smem_u32(tiles + g * REC_BYTES));
+            const unsigned long long bdesc = make_desc(smem_u32(xbuf + g * x_bytes));
+            if (elect_one()) {
+                bool first = n == 0;
+#pragma unroll
+                for (int k4 = 0; k4 < 4; ++k4) {
+                    if ((live >> k4) & 1u) {
+                        umma_bf16(tmem_base, adesc + (unsigned long long)(k4 * 2), bdesc + (unsigned long long)(k4 * 2), idesc,
+                                  first ? 0u : 1u);
+                        first = false;
+                    }
+                }
+                umma_commit(smem_u32(&sm->tile_empty[g]));
+            }
+            __syncwarp();
+            ++n;
+            if (++g == (unsigned)q.groups) { g = 0; phase ^= 1u; }
+        }
+        if (n) {
+            if (elect_one()) umma_commit(smem_u32(&sm->tfull));
+            __syncwarp();
+            // nothing this warp issued may be running when tensor memory is freed
+            mbar_wait(smem_u32(&sm->tfull), 0, &sm->drain_abort);
+        }
+        __syncwarp();
+    } else {
+        // ---------------- decode: this group takes every q.groups-th live record ----------------
+        constexpr unsigned OFF_MASK = DecodeCfg<BW, ST_GROUP>::OFF_MASK;
+        constexpr int WORDS = BW / 2;
+        constexpr unsigned BATCH = 4;                       // entries a thread reads before it stores any
+        constexpr unsigned PIECES = BW == 16 ? 2 : 1;       // 16-byte pieces of a dense block (or the block, if smaller)
+        constexpr unsigned PIECE_BYTES = BW >= 8 ? 16 : 2 * BW;
+        const int group = warp / (ST_GROUP / 32);
+        const unsigned t0 = (unsigned)tid & (ST_GROUP - 1u);
+        unsigned char *tile = tiles + group * REC_BYTES;
+        const unsigned char *ulist = p.packed + p.off_ulist, *dposl = p.packed + p.off_dpos, *dpayl = p.packed + p.off_dpay;
+        int turn = group;                                   // live records until this group's next one
+        unsigned mine = 0;
+        bool ok = true;
+        for (int i = 0; i < n_st; ++i) {
+            const uint4 a = srec[i];
+            if (!(a.w & 0xFu)) continue;
+            if (turn == 0) {
+                turn = q.groups;
+                const uint4 b = srec[i + 1];
+                const unsigned n_u = b.x - a.x, n_p = (b.y - a.y) * PIECES;
+                const uint2 *ul = reinterpret_cast<const uint2 *>(ulist) + a.x;
+                const unsigned short *dpos = reinterpret_cast<const unsigned short *>(dposl) + a.y;
+                const unsigned char *pay = dpayl + (unsigned long long)a.y * (2 * BW);
+                // the first entries travel while the tile is waited for and zeroed
+                uint2 ent[BATCH];                           // x: spread signs, y: off | bf16(u) << 16
+                unsigned off[BATCH];
+                uint4 v[BATCH];
+                auto read_u = [&](unsigned e0) {
+#pragma unroll
+                    for (unsigned k = 0; k < BATCH; ++k)
+                        if (e0 + k * ST_GROUP < n_u) ent[k] = __ldg(ul + e0 + k * ST_GROUP);
+                };
+                auto read_d = [&](unsigned e0) {
+#pragma unroll
+                    for (unsigned k = 0; k < BATCH; ++k) {
+                        const unsigned e = e0 + k * ST_GROUP;
+                        if (e >= n_p) continue;
+                        off[k] = (__ldg(dpos + e / PIECES) & OFF_MASK) ^ (PIECES == 2 ? (e & 1u) << 4 : 0u);
+                        if (BW >= 8) v[k] = __ldg(reinterpret_cast<const uint4 *>(pay + (size_t)e * PIECE_BYTES));
+                        if (BW == 4) { const uint2 h = __ldg(reinterpret_cast<const uint2 *>(pay + (size_t)e * PIECE_BYTES)); v[k].x = h.x; v[k].y = h.y; }
+                        if (BW == 2) v[k].x = __ldg(reinterpret_cast<const unsigned *>(pay + (size_t)e * PIECE_BYTES));
+                    }
+                };
+                auto write_u = [&](unsigned e0) {
+#pragma unroll
+                    for (unsigned k = 0; k < BATCH; ++k) {
+                        if (e0 + k * ST_GROUP >= n_u) break;
+                        const unsigned at = ent[k].y & OFF_MASK, u2 = __byte_perm(ent[k].y, 0u, 0x3232);
+                        unsigned w[8];
+#pragma unroll
+                        for (int t = 0; t < 8; ++t)         // weights 2t, 2t+1: sign bits t and 16+t
+                            w[t] = (t < WORDS) ? (((ent[k].x << (15 - t)) & 0x80008000u) ^ u2) : 0u;
+                        if (BW >= 8) *reinterpret_cast<uint4 *>(tile + at) = make_uint4(w[0], w[1], w[2], w[3]);
+                        if (BW == 16) *reinterpret_cast<uint4 *>(tile + (at ^ 16u)) = make_uint4(w[4], w[5], w[6], w[7]);
+                        if (BW == 4) *reinterpret_cast<uint2 *>(tile + at) = make_uint2(w[0], w[1]);
+                        if (BW == 2) *reinterpret_cast<unsigned *>(tile + at) = w[0];
+                    }
+                };
+                auto write_d = [&](unsigned e0) {
+#pragma unroll
+                    for (unsigned k = 0; k < BATCH; ++k) {
+                        if (e0 + k * ST_GROUP >= n_p) break;
+                        if (BW >= 8) *reinterpret_cast<uint4 *>(tile + off[k]) = v[k];
+                        if (BW == 4) *reinterpret_cast<uint2 *>(tile + off[k]) = make_uint2(v[k].x, v[k].y);
+                        if (BW == 2) *reinterpret_cast<unsigned *>(tile + off[k]) = v[k].x;
+                    }
+                };
+                read_u(t0);
+                read_d(t0);
+                // lists of this group's next record (its stage if none between is dead)
+                if (i + q.groups < n_st) {
+                    const uint4 na = srec[i + q.groups], nb = srec[i + q.groups + 1];
+                    if (na.w & 0xFu) {
+                        prefetch_span(ulist + (size_t)na.x * 8u, (nb.x - na.x) * 8u, t0);
+                        prefetch_span(dpayl + (size_t)na.y * (2u * BW), (nb.y - na.y) * (2u * BW), t0);
+                        prefetch_span(dposl + (size_t)na.y * 2u, (nb.y - na.y) * 2u, t0);
+                    }
+                }
+                // tile and box are free once the group's last record is multiplied
+                if (mine && !mbar_wait(smem_u32(&sm->tile_empty[group]), (mine - 1u) & 1u, abort)) ok = false;
+                if (group_any(group, !ok)) { ok = false; break; }          // the same decision in every thread of the group
+                if (t0 == 0) {
+                    mbar_expect_tx(smem_u32(&sm->x_full[group]), x_bytes);
+                    tma_load_2d(smem_u32(xbuf + group * x_bytes), &tmap_x, smem_u32(&sm->x_full[group]), (k0 + i) * BK, (int)mt * q.mpad);
+                }
+                uint4 *z = reinterpret_cast<uint4 *>(tile) + t0;
+#pragma unroll
+                for (int t = 0; t < REC_BYTES / 16 / ST_GROUP; ++t) z[t * ST_GROUP] = make_uint4(0, 0, 0, 0);
+                group_sync(group);
+                write_u(t0);
+                write_d(t0);
+                for (unsigned e0 = t0 + BATCH * ST_GROUP; e0 < n_u; e0 += BATCH * ST_GROUP) { read_u(e0); write_u(e0); }
+                for (unsigned e0 = t0 + BATCH * ST_GROUP; e0 < n_p; e0 += BATCH * ST_GROUP) { read_d(e0); write_d(e0); }
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&sm->tile_full[group]));
+                ++mine;
+            }
+            --turn;
+        }
+        // a box of X that is still on its way must land before this CTA's shared memory goes away
+        if (t0 == 0 && mine) mbar_wait(smem_u32(&sm->x_full[group]), (mine - 1u) & 1u, &sm->drain_abort);
+        __syncwarp();
+        if (any && ok) mbar_wait(smem_u32(&sm->tfull), 0, abort);
+        __syncwarp();
+    }
+    __syncthreads();
+    // ---------------- epilogue: partial sums to shared memory, tensor memory given back ----------------
+    const bool sums = any && *abort == 0;
+    const int readers = mma_warp >= 8 ? 2 : 1;              // warps to a quarter of the lanes
+    if (warp < 4 * readers) {
+        tc_fence_after();
+        const int quarter = warp & 3;                       // tensor-memory lanes (weight rows) this warp may read
+        for (int c = (warp >> 2) * 16; c < q.mpad; c += 16 * readers) {
+            unsigned v[16];
+            if (sums) tmem_ld16(tmem_base + ((unsigned)(quarter * 32) << 16) + (unsigned)c, v);
+            else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) part[(c + j) * 128 + quarter * 32 + lane] = __uint_as_float(v[j]);
+        }
+        tc_fence_before();
+    }
+    __syncthreads();
+    if (warp == mma_warp) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, q.tmem_cols);
+    }
+    if ((*abort || sm->drain_abort) && tid == 0) atomicOr(p.dev_status, (unsigned)MWU_DEV_TIMEOUT);
+    __syncwarp();
+    if (q.split > 1) cluster_sync_all();
+    // rows rank, rank + split, ... of the tile: a warp adds up one row of 128 columns
+    const long long m0 = (long long)mt * q.mpad;
+    const long long n0 = rt * kTileRows + lane * 4;
+    for (int m = (int)rank + warp * q.split; m < q.mpad && m0 + m < p.M; m += (n_threads / 32) * q.split) {
+        const unsigned at = smem_u32(part + m * 128 + lane * 4);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (q.split == 1) acc = *reinterpret_cast<const float4 *>(part + m * 128 + lane * 4);
+        else {
+#pragma unroll 4
+            for (int c = 0; c < q.split; ++c) {
+                const float4 v = ld_cluster_f4(mbar_addr_in_cta(at, (unsigned)c));
+                acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+            }
+        }
+        const float r[4] = {acc.x, acc.y, acc.z, acc.w};
+        if (p.y_fp32) {
+            float *dst = reinterpret_cast<float *>(p.Y) + (m0 + m) * p.ldy + n0;
+            if (n0 + 4 <= p.N) *reinterpret_cast<float4 *>(dst) = acc;
+            else
+                for (int j = 0; j < 4; ++j)
+                    if (n0 + j < p.N) dst[j] = r[j];
+        } else {
+            __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(p.Y) + (m0 + m) * p.ldy + n0;
+            if (n0 + 4 <= p.N) {
+                const __nv_bfloat162 h0 = __floats2bfloat162_rn(acc.x, acc.y), h1 = __floats2bfloat162_rn(acc.z, acc.w);
+                *reinterpret_cast<uint2 *>(dst) = make_uint2(*reinterpret_cast<const unsigned *>(&h0), *reinterpret_cast<const unsigned *>(&h1));
+            } else {
+                for (int j = 0; j < 4; ++j)
+                    if (n0 + j < p.N) dst[j] = __float2bfloat16_rn(r[j]);
+            }
+        }
+    }
+    __syncwarp();
+    if (q.split > 1) cluster_sync_all();                    // nobody leaves while its sums are still being read
+}
+
+// ------------------------------------------------------------------------------------------
+// host
+// ------------------------------------------------------------------------------------------
+// Shape of a launch: rows per CTA, CTAs per cluster, decode groups.  `cost` estimates the call in record times of
+// one CTA: waves of resident CTAs, each its stages plus a fixed part.
+struct StreamPlan {
+    StreamParams q;
+    size_t smem;
+    long long grid;
+    long long cost;
+};
+
+static StreamPlan plan_with(const Params &p, int split, int sm_count) {
+    StreamPlan s;
+    s.q.m_tiles = (int)((p.M + ST_MAX_ROWS - 1) / ST_MAX_ROWS);
+    s.q.mpad = (int)(((p.M + s.q.m_tiles - 1) / s.q.m_tiles + 15) / 16 * 16);
+    s.q.split = split;
+    s.q.stages_per = (int)((p.n_stages + split - 1) / split);
+    s.q.tmem_cols = s.q.mpad <= 32 ? 32u : (s.q.mpad <= 64 ? 64u : 128u);
+    // as many groups as tiles and boxes of X fit: six up to 16 rows, three at 128
+    const size_t x = (size_t)s.q.mpad * BK * 2;
+    const size_t fixed = 1024 + sizeof(StreamSmem) + 16 + (size_t)(s.q.stages_per + 1) * 16;
+    size_t groups = ((size_t)ST_SMEM_CTA - fixed) / (REC_BYTES + x);
+    if (groups > (size_t)ST_MAX_GROUPS) groups = ST_MAX_GROUPS;
+    if (groups > (size_t)s.q.stages_per) groups = s.q.stages_per < 2 ? 2 : s.q.stages_per;
+    s.q.groups = (int)groups;
+    s.smem = fixed + groups * (REC_BYTES + x);
+    const int resident = 2;
+    const long long units = p.n_rec_tiles * s.q.m_tiles;
+    s.grid = units * split;
+    const long long waves = (s.grid + (long long)resident * sm_count - 1) / ((long long)resident * sm_count);
+    s.cost = waves * (s.q.stages_per + 4 + split / 2);
+    return s;
+}
+
+template <int BW>
+static cudaError_t launch_stream_bw(const CUtensorMap &tmap_x, const Params &p, const StreamPlan &s, cudaStream_t st) {
+    auto kern = mwu_gemm_stream_kernel<BW>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM_CTA);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)s.grid);
+    cfg.blockDim = dim3((unsigned)(s.q.groups * ST_GROUP + 32));
+    cfg.dynamicSmemBytes = s.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)s.q.split;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = s.q.split > 1 ? 2 : 1;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, kern, tmap_x, p, s.q);
+}
+
+static StreamPlan plan_of(const Params &p, int sm_count) {
+    StreamPlan best = plan_with(p, 1, sm_count);
+    for (int split = 2; split <= 8 && split <= p.n_stages; split *= 2) {
+        const StreamPlan s = plan_with(p, split, sm_count);
+        if (s.cost < best.cost) best = s;
+    }
+    return best;
+}
+
+// activation rows of the TMA box of X
+int stream_box_rows(const Params &p, int sm_count) { return plan_of(p, sm_count).q.mpad; }
+
+// A record is decoded once per activation tile of 128 rows, so the path that expands the weights once
+// overtakes this one as rows are added.  Measured (us, this kernel / expanding): 16384 x 4096, b = 16:
+// 27 / 66 at 16 rows, 41 / 68 at 128, 67 / 68 at 256, 131 / 89 at 512; 4096 x 4096, b = 8: 26 / 37 at 256, 41 / 37 at
+// 512; b = 2: 43 / 50 at 256, 72 / 52 at 512.  A small weight stays here longer, while the decodes are few to an
+// SM: 1000 x 1216, b = 8, 1024 rows (1216 decodes): 15 / 19; 4096 x 1024, b = 4, 512 rows (2048): 22 / 19.
+bool stream_eligible(const Params &p, int sm_count) {
+    return p.M <= 256 || p.n_rec_tiles * p.n_stages * ((p.M + ST_MAX_ROWS - 1) / ST_MAX_ROWS) <= 9ll * sm_count;
+}
+
+cudaError_t launch_stream(int bw, const CUtensorMap &tmap_x, const Params &p, int sm_count, cudaStream_t st) {
+    const StreamPlan s = plan_of(p, sm_count);
+    switch (bw) {
+        case 2: return launch_stream_bw<2>(tmap_x, p, s, st);
+        case 4: return launch_stream_bw<4>(tmap_x, p, s, st);
+        case 8: return launch_stream_bw<8>(tmap_x, p, s, st);
+        default: return launch_stream_bw<16>(tmap_x, p, s, st);
+    }
+}
+
+}  // namespace gemm
+}  // namespace mwu

@@ -276,3 +276,19 @@ def test_gemm_pair_tiles_resident_weights(K, b):
     W = inputs.normal_weights(512, K, 0.02, 95 + b)
     Mb = W.numel() // b
     check_gemm(W, b, Mb * 3 // 4, Mb // 2, 77000 + 37, seed=31 + b)
+
+
+@pytest.mark.parametrize("b,rows,cols,M,ku,kp", [(2, 136, 64, 1, 7, 3),           # one stage, one row, a padded weight tile
+                                                 (2, 128, 320, 16, 10, 0),        # every block unified: the longest u lists
+                                                 (4, 200, 448, 17, 0, 0),         # every block dense: the longest payloads
+                                                 (8, 384, 1088, 48, 6, 3),        # 17 stages over a cluster, the last CTA with fewer
+                                                 (16, 256, 2304, 128, 8, 6),      # the most rows of one CTA
+                                                 (16, 1000, 4096, 65, 9, 8),
+                                                 (4, 128, 192, 100, 10, 10)])     # everything pruned: no MMA at all
+def test_gemm_few_rows(b, rows, cols, M, ku, kp):
+    """Few activation rows: the streaming kernel, with and without dead stages (ku, kp in tenths)."""
+    W = inputs.normal_weights(rows, cols, 0.02, 300 + b)
+    if cols > 256 and kp < ku:
+        W[:, 64:144] = 0.0                       # a dead stage and a dead slice wherever blocks of zeros are pruned
+    Mb = W.numel() // b
+    check_gemm(W, b, Mb * ku // 10, Mb * kp // 10, M, seed=40 + b)
