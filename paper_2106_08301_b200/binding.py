@@ -109,16 +109,25 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+# The marshalling of a call is a good part of a small layer's time, so it does no more than it must:
+# addresses go through ctypes as plain integers, and the current stream is asked for by its raw handle
+# (torch.cuda.current_stream() builds a Stream object, about 4 us, as long as the rest of a call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
     assert t.is_cuda and t.is_contiguous(), "device-resident contiguous tensors only"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream: Optional[torch.cuda.Stream]):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def status_string(status: int) -> str:
