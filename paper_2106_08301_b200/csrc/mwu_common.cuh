@@ -114,6 +114,31 @@ inline bool aligned_to(const void *p, size_t a) { return (reinterpret_cast<uintp
 // MWU_OK when the current device is compute capability 10.x; also reports its SM count.
 int check_device(int *sm_count);
 
+// Launch with programmatic stream serialization: the kernel may start while its predecessor on the stream
+// still drains.  The rule all of the library's kernels follow: such a kernel executes griddepcontrol.wait
+// before it touches memory of anyone else, and griddepcontrol.launch_dependents, if at all, only behind that
+// wait (or behind the trigger of a kernel that has itself waited), so whatever ran before the chain is
+// complete when any kernel of the chain reads its inputs.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                  int cluster, Args... args) {
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // adds n to the process-wide count of kernels launched (mwu_kernel_launches)
 void count_launch(int n = 1);
 

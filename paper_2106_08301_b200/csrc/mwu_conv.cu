@@ -155,6 +155,7 @@ template <int BW>
 __global__ void __launch_bounds__(PREP_THREADS) conv_prep_kernel(const Params p, unsigned short *Wd, int taps, int C,
                                                                  unsigned n_rec, const unsigned short *x,
                                                                  unsigned short *xt, int HW, int tiles_hw, int tiles_c) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tensor-core kernel may set itself up meanwhile
     if (blockIdx.x < n_rec) {
         MWU_CHECK_HEADER(p);
@@ -466,18 +467,9 @@ static int run_taps(ConvParams &p, const void *X_nchw, int n, int c, int h, int 
         return MWU_ERR_CUDA;
     const long long tiles = (long long)n * p.tiles_per_img * p.n_ntiles;
     const int grid = (int)(tiles < sm_count ? tiles : sm_count);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(C_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     count_launch();
-    if (cudaLaunchKernelEx(&cfg, mwu_conv_taps_kernel, tmap_x, tmap_w, p) != cudaSuccess) return MWU_ERR_CUDA;
+    if (launch_chained(mwu_conv_taps_kernel, dim3((unsigned)grid), dim3(C_THREADS), smem, st, 1, tmap_x, tmap_w, p) != cudaSuccess)
+        return MWU_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
 }
 
@@ -528,10 +520,10 @@ extern "C" int mwu_conv_implicit_ws(const mwu_proj_desc *desc, const void *packe
                     [&](const unsigned short *x, unsigned short *xo, int HW, int tiles_hw, int tiles_c, unsigned n_tiles) {
         const unsigned grid = n_rec + n_tiles;
         switch (bw) {
-            case 2: conv_prep_kernel<2><<<grid, PREP_THREADS, 0, st>>>(g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
-            case 4: conv_prep_kernel<4><<<grid, PREP_THREADS, 0, st>>>(g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
-            case 8: conv_prep_kernel<8><<<grid, PREP_THREADS, 0, st>>>(g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
-            default: conv_prep_kernel<16><<<grid, PREP_THREADS, 0, st>>>(g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
+            case 2: launch_chained(conv_prep_kernel<2>, dim3(grid), dim3(PREP_THREADS), 0, st, 1, g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
+            case 4: launch_chained(conv_prep_kernel<4>, dim3(grid), dim3(PREP_THREADS), 0, st, 1, g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
+            case 8: launch_chained(conv_prep_kernel<8>, dim3(grid), dim3(PREP_THREADS), 0, st, 1, g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
+            default: launch_chained(conv_prep_kernel<16>, dim3(grid), dim3(PREP_THREADS), 0, st, 1, g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
         }
         count_launch();
     });

@@ -39,6 +39,7 @@ constexpr int DEC_THREADS = 128;
 template <int BW>
 __global__ void __launch_bounds__(DEC_THREADS)
 mwu_decode_kernel(const Params p, __nv_bfloat16 *Wd, long long ldw) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the GEMM behind may set itself up meanwhile
     MWU_CHECK_HEADER(p);
     __shared__ __align__(1024) unsigned char tile[REC_BYTES];
@@ -72,9 +73,8 @@ mwu_decode_kernel(const Params p, __nv_bfloat16 *Wd, long long ldw) {
 template <int BW>
 static cudaError_t launch_decode_bw(const Params &p, __nv_bfloat16 *Wd, long long ldw, cudaStream_t st) {
     const long long n_rec = p.n_rec_tiles * p.n_stages;
-    mwu_decode_kernel<BW><<<(unsigned)n_rec, DEC_THREADS, 0, st>>>(p, Wd, ldw);
     count_launch();
-    return cudaGetLastError();
+    return launch_chained(mwu_decode_kernel<BW>, dim3((unsigned)n_rec), dim3(DEC_THREADS), 0, st, 1, p, Wd, ldw);
 }
 
 cudaError_t launch_decode(int bw, const Params &p, __nv_bfloat16 *Wd, long long ldw, cudaStream_t st) {
@@ -454,22 +454,8 @@ cudaError_t launch_dense(const CUtensorMap &tmap_x, const CUtensorMap &tmap_w, c
     if (tiles >= (1ll << 31)) return cudaErrorInvalidValue;
     long long pairs = sm_count / 2;
     if (tiles < pairs) pairs = tiles;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * pairs));
-    cfg.blockDim = dim3(D_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
     count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, tmap_x, tmap_w, tmap_y, p);
+    return launch_chained(kern, dim3((unsigned)(2 * pairs)), dim3(D_THREADS), smem, st, 2, tmap_x, tmap_w, tmap_y, p);
 }
 
 }  // namespace gemm

@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(ST_MAX_THREADS)
 mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ Params p,
                        const __grid_constant__ StreamParams q) {
     asm volatile("griddepcontrol.wait;" ::: "memory");      // launched while the kernel before may still run
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     MWU_CHECK_HEADER(p);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
@@ -393,22 +394,9 @@ static cudaError_t launch_stream_bw(const CUtensorMap &tmap_x, const Params &p, 
     auto kern = mwu_gemm_stream_kernel<BW>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM_CTA);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)s.grid);
-    cfg.blockDim = dim3((unsigned)(s.q.groups * ST_GROUP + 32));
-    cfg.dynamicSmemBytes = s.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)s.q.split;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = s.q.split > 1 ? 2 : 1;
     count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, tmap_x, p, s.q);
+    return launch_chained(kern, dim3((unsigned)s.grid), dim3((unsigned)(s.q.groups * ST_GROUP + 32)), s.smem, st, s.q.split, tmap_x,
+                          p, s.q);
 }
 
 static StreamPlan plan_of(const Params &p, int sm_count) {

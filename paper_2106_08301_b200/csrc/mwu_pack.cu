@@ -2,10 +2,11 @@
 // magnitude per unified block, nothing but its position for a pruned block, one sign bit per
 // weight of a unified block, bf16 values for the rest), arranged per GEMM tile.
 //
-//   count_kernel  one CTA per tile of 128 rows, a lane per record (128 rows x 64 columns) walking the
-//                 rows: number of unified / dense / pruned blocks and the record's live-slice mask.
-//   scan_kernel   one CTA: exclusive scan of the per-record counts over all records (1024 records
-//                 at a time, read and written as whole lines), header.
+//   count_kernel  a CTA per tile of 128 rows and 32 records, a lane per record (128 rows x 64 columns)
+//                 walking the rows: number of unified / dense / pruned blocks and the record's live-slice
+//                 mask.  Only for weights of many records; a few are counted by scan_kernel itself.
+//   scan_kernel   one cluster of eight CTAs: exclusive scan of the per-record counts (each CTA its eighth,
+//                 totals through distributed shared memory), header.
 //   fill_kernel   one CTA per record.  First one thread per row: class masks, then a scan over the
 //                 rows of the number of blocks per (class, store slot), which gives every block its
 //                 place in the round-robin order of its class list; the places go to shared memory.
@@ -91,17 +92,21 @@ __device__ __forceinline__ unsigned live_of(unsigned P, int b) {
 
 constexpr int COUNT_WARPS = 16;                         // each takes 8 of the tile's 128 rows
 
-__global__ void __launch_bounds__(32 * COUNT_WARPS) count_kernel(Params p) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+struct CountSmem {
+    unsigned cu[COUNT_WARPS][32], cp[COUNT_WARPS][32], live[COUNT_WARPS][32];
+};
+
+// Counts of one unit (a tile and 32 of its stages), by COUNT_WARPS warps (warp: 0 .. COUNT_WARPS-1) that all
+// call it together; the first of them writes them to the record table.  `sync` joins these warps.
+template <class Sync>
+__device__ __forceinline__ void count_unit(const Params &p, unsigned unit, int warp, int lane, CountSmem &s, Sync sync) {
     const unsigned chunks = (p.n_stages + 31u) / 32u;       // 32 records of a tile at a time: lane = record (stage)
-    const long long tile = blockIdx.x / chunks;
-    const long long stage = (long long)(blockIdx.x % chunks) * 32 + lane;
+    const long long tile = unit / chunks;
+    const long long stage = (long long)(unit % chunks) * 32 + lane;
     const int nb = kStageK / p.b;
     const unsigned mask = (nb >= 32) ? 0xffffffffu : ((1u << nb) - 1u);
     const long long bpr = p.bpr;                            // blocks per row
     constexpr int RPW = kTileRows / COUNT_WARPS;
-    __shared__ unsigned s_cu[COUNT_WARPS][32], s_cp[COUNT_WARPS][32], s_live[COUNT_WARPS][32];
     unsigned cu = 0, cp = 0, live = 0;
     if (stage < p.L.n_stages) {
         unsigned P[RPW], U[RPW];
@@ -124,36 +129,108 @@ __global__ void __launch_bounds__(32 * COUNT_WARPS) count_kernel(Params p) {
             live |= live_of(Pm, p.b);
         }
     }
-    s_cu[warp][lane] = cu; s_cp[warp][lane] = cp; s_live[warp][lane] = live;
-    __syncthreads();
+    s.cu[warp][lane] = cu; s.cp[warp][lane] = cp; s.live[warp][lane] = live;
+    sync();
     if (warp == 0 && stage < p.L.n_stages) {
         unsigned tu = 0, tp = 0, tl = 0;
 #pragma unroll
-        for (int w = 0; w < COUNT_WARPS; ++w) { tu += s_cu[w][lane]; tp += s_cp[w][lane]; tl |= s_live[w][lane]; }
+        for (int w = 0; w < COUNT_WARPS; ++w) { tu += s.cu[w][lane]; tp += s.cp[w][lane]; tl |= s.live[w][lane]; }
         // counts for now (ubase, dbase, pbase, live); scan_kernel makes bases
         uint4 *recs = reinterpret_cast<uint4 *>(p.packed + p.L.off_rec);
         recs[tile * p.L.n_stages + stage] = make_uint4(tu, (unsigned)(kTileRows * nb) - tu - tp, tp, tl);
     }
 }
 
-__global__ void __launch_bounds__(1024) scan_kernel(Params p) {
+// launched with programmatic stream serialization: the projection may still be running
+__global__ void __launch_bounds__(32 * COUNT_WARPS) count_kernel(Params p) {
+    __shared__ CountSmem s;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long long n_rec = p.L.n_tiles * p.L.n_stages;
-    uint4 *recs = reinterpret_cast<uint4 *>(p.packed + p.L.off_rec);     // ubase, dbase, pbase, live
+    count_unit(p, blockIdx.x, threadIdx.x >> 5, threadIdx.x & 31, s, [] { __syncthreads(); });
+}
+
+constexpr int SCAN_CTAS = 8, SCAN_THREADS = 1024, SCAN_PER = 4;      // consecutive records a thread takes at a time
+
+__device__ __forceinline__ void scan_cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Bound by latency: a handful of dependent L2 round trips and cluster barriers (8192 records on one CTA, in
+// two rounds, took 13 us).  Counts the records itself when count_kernel has not (`counted` == 0).
+__global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(Params p, int counted) {
+    __shared__ CountSmem s_count[SCAN_THREADS / (32 * COUNT_WARPS)];
     __shared__ unsigned s_w[3][32];
+    __shared__ unsigned long long s_tot[3];                 // this CTA's totals, read by all
+    __shared__ unsigned long long s_before[2][3];           // totals of the CTAs before this one, and of all
+    const unsigned n_rec = (unsigned)(p.L.n_tiles * p.L.n_stages);
+    uint4 *recs = reinterpret_cast<uint4 *>(p.packed + p.L.off_rec);     // ubase, dbase, pbase, live
+    const unsigned cta = blockIdx.x;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // fill_kernel reads the projection's outputs before it waits for this kernel, so it may start only once
+    // the projection is complete: after count_kernel's own wait, or after this one
+    if (!counted) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");      // the counts are complete and visible
-    unsigned long long cu = 0, cd = 0, cp = 0;              // totals of the chunks before this one
-    constexpr int PER = 4;                                  // consecutive records per thread; a chunk is 4096 records
-    for (long long g0 = 0; g0 < n_rec; g0 += PER * 1024) {
-        const long long i0 = g0 + (long long)threadIdx.x * PER;
-        uint4 held[PER];
-        unsigned su = 0, sd = 0, sp = 0;                    // a chunk's counts fit 32 bits (at most 4096 blocks a record)
-#pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            held[k] = (i0 + k < n_rec) ? recs[i0 + k] : make_uint4(0, 0, 0, 0);
-            su += held[k].x; sd += held[k].y; sp += held[k].z;
+    if (!counted) {
+        constexpr int TEAMS = SCAN_THREADS / (32 * COUNT_WARPS);
+        const int team = wid / COUNT_WARPS;
+        const unsigned units = (unsigned)p.L.n_tiles * ((p.n_stages + 31u) / 32u);
+        for (unsigned unit = cta * TEAMS + team; unit < units; unit += SCAN_CTAS * TEAMS) {
+            auto join = [team] { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(32 * COUNT_WARPS) : "memory"); };
+            count_unit(p, unit, wid % COUNT_WARPS, lane, s_count[team], join);
+            join();                                         // the counts have been read
         }
+        scan_cluster_sync();
+    }
+    const unsigned per = (n_rec + SCAN_CTAS - 1) / SCAN_CTAS;
+    const unsigned r0 = min(cta * per, n_rec), r1 = min(r0 + per, n_rec);
+    constexpr unsigned STEP = SCAN_PER * SCAN_THREADS;
+    uint4 held[SCAN_PER];
+    auto read = [&](unsigned i0) {
+#pragma unroll
+        for (int k = 0; k < SCAN_PER; ++k) held[k] = (i0 + k < r1) ? __ldcg(recs + i0 + k) : make_uint4(0, 0, 0, 0);
+    };
+    // totals of this CTA's records
+    unsigned long long tot[3] = {0, 0, 0};
+    for (unsigned g0 = r0; g0 < r1; g0 += STEP) {
+        read(g0 + threadIdx.x * SCAN_PER);
+#pragma unroll
+        for (int k = 0; k < SCAN_PER; ++k) { tot[0] += held[k].x; tot[1] += held[k].y; tot[2] += held[k].z; }
+    }
+    if (threadIdx.x < 3) s_tot[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        // a thread's share fits 32 bits (counts of up to 4096 blocks); CTAs hold fewer than 2^31 blocks in all
+        const unsigned t = __reduce_add_sync(0xffffffffu, (unsigned)tot[c]);
+        if (lane == 0 && t) atomicAdd(&s_tot[c], (unsigned long long)t);
+    }
+    scan_cluster_sync();
+    if (threadIdx.x < 3) {
+        const unsigned at = (unsigned)__cvta_generic_to_shared(&s_tot[threadIdx.x]);
+        unsigned long long before = 0, all = 0;
+#pragma unroll
+        for (unsigned c = 0; c < SCAN_CTAS; ++c) {
+            unsigned long long t;
+            unsigned remote;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(at), "r"(c));
+            asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(t) : "r"(remote) : "memory");
+            before += c < cta ? t : 0ull;
+            all += t;
+        }
+        s_before[0][threadIdx.x] = before;
+        s_before[1][threadIdx.x] = all;
+    }
+    __syncthreads();
+    unsigned long long cu = s_before[0][0], cd = s_before[0][1], cp = s_before[0][2];
+    for (unsigned g0 = r0; g0 < r1; g0 += STEP) {
+        const unsigned i0 = g0 + threadIdx.x * SCAN_PER;
+        if (per > STEP) read(i0);                           // else this thread still holds them
+        unsigned su = 0, sd = 0, sp = 0;                    // a step's counts fit 32 bits
+#pragma unroll
+        for (int k = 0; k < SCAN_PER; ++k) { su += held[k].x; sd += held[k].y; sp += held[k].z; }
         // inclusive scan of the thread sums: inside a warp, then over the 32 warp totals
         unsigned iu = su, id = sd, ip = sp;
 #pragma unroll
@@ -163,39 +240,40 @@ __global__ void __launch_bounds__(1024) scan_kernel(Params p) {
             const unsigned ap = __shfl_up_sync(0xffffffffu, ip, off);
             if (lane >= off) { iu += au; id += ad; ip += ap; }
         }
-        __syncthreads();                                    // the previous chunk's warp totals have been read
+        __syncthreads();                                    // the previous step's warp totals have been read
         if (lane == 31) { s_w[0][wid] = iu; s_w[1][wid] = id; s_w[2][wid] = ip; }
         __syncthreads();
-        unsigned wu = s_w[0][lane], wd = s_w[1][lane], wp = s_w[2][lane];     // every warp scans the 32 totals
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned au = __shfl_up_sync(0xffffffffu, wu, off);
-            const unsigned ad = __shfl_up_sync(0xffffffffu, wd, off);
-            const unsigned ap = __shfl_up_sync(0xffffffffu, wp, off);
-            if (lane >= off) { wu += au; wd += ad; wp += ap; }
-        }
-        const unsigned tu = __shfl_sync(0xffffffffu, wu, 31), td = __shfl_sync(0xffffffffu, wd, 31),
-                       tp = __shfl_sync(0xffffffffu, wp, 31);
-        const unsigned bu = __shfl_sync(0xffffffffu, wu - s_w[0][lane], wid);  // totals of the warps before this one
-        const unsigned bd = __shfl_sync(0xffffffffu, wd - s_w[1][lane], wid);
-        const unsigned bp = __shfl_sync(0xffffffffu, wp - s_w[2][lane], wid);
+        const unsigned wu = s_w[0][lane], wd = s_w[1][lane], wp = s_w[2][lane];
+        const unsigned bu = __reduce_add_sync(0xffffffffu, lane < wid ? wu : 0u);      // totals of the warps before this one
+        const unsigned bd = __reduce_add_sync(0xffffffffu, lane < wid ? wd : 0u);
+        const unsigned bp = __reduce_add_sync(0xffffffffu, lane < wid ? wp : 0u);
         unsigned long long ru = cu + bu + (iu - su), rd = cd + bd + (id - sd), rp = cp + bp + (ip - sp);
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            if (i0 + k < n_rec) recs[i0 + k] = make_uint4((unsigned)ru, (unsigned)rd, (unsigned)rp, held[k].w);
+        for (int k = 0; k < SCAN_PER; ++k) {
+            if (i0 + k < r1) recs[i0 + k] = make_uint4((unsigned)ru, (unsigned)rd, (unsigned)rp, held[k].w);
             ru += held[k].x; rd += held[k].y; rp += held[k].z;
         }
-        cu += tu; cd += td; cp += tp;
+        if (per > STEP) {                                   // the totals of this step, for the next one
+            cu += __reduce_add_sync(0xffffffffu, wu);
+            cd += __reduce_add_sync(0xffffffffu, wd);
+            cp += __reduce_add_sync(0xffffffffu, wp);
+        }
     }
-    if (threadIdx.x == 1023) {
-        if (cu != (unsigned long long)p.L.n_unified || cd != (unsigned long long)p.L.n_dense ||
-            cp != (unsigned long long)p.L.n_plist)
+    scan_cluster_sync();                                    // nobody leaves while its totals are still being read
+    if (cta != 0) return;
+    if (threadIdx.x == SCAN_THREADS - 1) {
+        const unsigned long long au = s_before[1][0], ad = s_before[1][1], ap = s_before[1][2];
+        if (au != (unsigned long long)p.L.n_unified || ad != (unsigned long long)p.L.n_dense ||
+            ap != (unsigned long long)p.L.n_plist)
             atomicOr(p.dev_status, (unsigned)MWU_DEV_BOUNDS);
-        recs[n_rec] = make_uint4((unsigned)cu, (unsigned)cd, (unsigned)cp, 0u);
+        recs[n_rec] = make_uint4((unsigned)au, (unsigned)ad, (unsigned)ap, 0u);
     }
     // the padding between the sections must read as zero (each gap is shorter than the alignment)
-    for (int g = 0; g < 5; ++g)
-        for (unsigned long long a = p.gap[g][0] + threadIdx.x; a < p.gap[g][1]; a += blockDim.x) p.packed[a] = 0;
+    {
+        const int g = wid - 1;                              // a warp to a gap; the first warp writes the header
+        if (g >= 0 && g < 5)
+            for (unsigned long long a = p.gap[g][0] + lane; a < p.gap[g][1]; a += 32) p.packed[a] = 0;
+    }
     if (threadIdx.x < 32) {
         unsigned long long *h = reinterpret_cast<unsigned long long *>(p.packed);
         unsigned long long v = 0;
@@ -239,6 +317,7 @@ __global__ void __launch_bounds__(128) fill_kernel(Params p) {
     constexpr int STORE = (B >= 8) ? 16 : 2 * B;            // bytes of one shared-memory store
     constexpr int G = 128 / STORE;                          // store slots of a 128-byte row
     constexpr int LPB = (B >= 4) ? B / 4 : 1;               // lanes that share a dense block's run of W
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned rec = blockIdx.x;
     const unsigned tile_u = rec / p.n_stages;
     const long long tile = tile_u, stage = rec - tile_u * p.n_stages;
@@ -443,30 +522,25 @@ extern "C" int mwu_pack(const mwu_proj_desc *desc, const float *W, const float *
         {p.L.off_dpay + 2 * (size_t)desc->block * p.L.n_dense, p.L.off_ppos},
         {p.L.off_ppos + 2 * (size_t)p.L.n_plist, p.L.total}};
     for (int g = 0; g < 5; ++g) { p.gap[g][0] = gaps[g][0]; p.gap[g][1] = gaps[g][1] > gaps[g][0] ? gaps[g][1] : gaps[g][0]; }
-    pack::count_kernel<<<(unsigned)(p.L.n_tiles * ((p.L.n_stages + 31) / 32)), 32 * pack::COUNT_WARPS, 0, st>>>(p);
-    // the next two start while their predecessor drains (programmatic stream serialization) and wait
-    // for its memory themselves
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3(1024);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, pack::scan_kernel, p);
-    cfg.gridDim = dim3((unsigned)n_rec);
-    cfg.blockDim = dim3(128);
+    // All three start while their predecessor drains (programmatic stream serialization) and wait for its
+    // memory themselves.  Up to two units for every team of the scan cluster it counts them itself, in two
+    // rounds of loads at most; beyond that a grid of CTAs is faster.
+    const long long units = p.L.n_tiles * ((p.L.n_stages + 31) / 32);
+    const int counted = units > 2 * pack::SCAN_CTAS * (pack::SCAN_THREADS / (32 * pack::COUNT_WARPS)) ? 1 : 0;
+    cudaError_t e = cudaSuccess;
+    if (counted) e = launch_chained(pack::count_kernel, dim3((unsigned)units), dim3(32 * pack::COUNT_WARPS), 0, st, 1, p);
+    if (e == cudaSuccess)
+        e = launch_chained(pack::scan_kernel, dim3(pack::SCAN_CTAS), dim3(pack::SCAN_THREADS), 0, st, pack::SCAN_CTAS, p, counted);
     if (e == cudaSuccess) {
+        const dim3 grid((unsigned)n_rec), block(128);
         switch (desc->block) {
-            case 2: e = cudaLaunchKernelEx(&cfg, pack::fill_kernel<2>, p); break;
-            case 4: e = cudaLaunchKernelEx(&cfg, pack::fill_kernel<4>, p); break;
-            case 8: e = cudaLaunchKernelEx(&cfg, pack::fill_kernel<8>, p); break;
-            default: e = cudaLaunchKernelEx(&cfg, pack::fill_kernel<16>, p); break;
+            case 2: e = launch_chained(pack::fill_kernel<2>, grid, block, 0, st, 1, p); break;
+            case 4: e = launch_chained(pack::fill_kernel<4>, grid, block, 0, st, 1, p); break;
+            case 8: e = launch_chained(pack::fill_kernel<8>, grid, block, 0, st, 1, p); break;
+            default: e = launch_chained(pack::fill_kernel<16>, grid, block, 0, st, 1, p); break;
         }
     }
     if (e != cudaSuccess) return MWU_ERR_CUDA;
-    count_launch(3);
+    count_launch(2 + counted);
     return cudaGetLastError() == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
 }

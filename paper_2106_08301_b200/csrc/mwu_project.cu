@@ -485,6 +485,7 @@ __device__ __forceinline__ long long sample_block(int i, long long mb, int ns) {
 // 9 us; over 32 SMs they take one memory round trip).  The same launch clears the histograms.
 template <int B>
 __global__ void __launch_bounds__(128) sample_keys_kernel(Params p, unsigned *zero_base, unsigned n_zero) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const long long mb = p.n_blocks;
     const int ns = (int)(mb < (long long)NSAMP ? mb : (long long)NSAMP);
@@ -1054,6 +1055,8 @@ __global__ void __launch_bounds__(CLUSTER ? CL_THREADS : GR_THREADS) exact_kerne
         __shared__ sel::ClusterCounts counts;
         team.mine = &counts;
         team.begin();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     } else {
         team.n_cta = gridDim.x;
         team.x = p.xwork;
@@ -1984,20 +1987,9 @@ static cudaError_t launch_exact_held(const mwu::proj::Params &p, const mwu::proj
     if (e != cudaSuccess) return e;
     if (!route.cluster)
         return launch_cooperative(kern, route.grid, threads, (size_t)smem, sm_count, st, p, o, pb, (unsigned)route.held);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)route.grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)route.grid;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     mwu::count_launch();
-    return cudaLaunchKernelEx(&cfg, kern, p, o, pb, (unsigned)route.held);
+    return mwu::launch_chained(kern, dim3((unsigned)route.grid), dim3((unsigned)threads), (size_t)smem, st, route.grid, p, o, pb,
+                               (unsigned)route.held);
 }
 
 template <int B>
@@ -2042,26 +2034,15 @@ static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_des
     // (and the sweep's first loads in flight) when their predecessor ends
     unsigned *zero = reinterpret_cast<unsigned *>(p.xwork);
     const unsigned n_zero = (unsigned)(p.fhist - zero) + 2u * (unsigned)p.nb;
-    sample_keys_kernel<B><<<NSAMP / 128, 128, 0, st>>>(p, zero, n_zero);
-    cudaLaunchConfig_t cfg = {};
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3(SAMP_THREADS);
-    e = cudaLaunchKernelEx(&cfg, sample_kernel, p);
+    e = mwu::launch_chained(sample_keys_kernel<B>, dim3(NSAMP / 128), dim3(128), 0, st, 1, p, zero, n_zero);
+    if (e == cudaSuccess) e = mwu::launch_chained(sample_kernel, dim3(1), dim3(SAMP_THREADS), 0, st, 1, p);
     if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3((unsigned)grid_stream);
-    cfg.blockDim = dim3(256);
     if (p.U_next || p.resid)
-        e = cudaLaunchKernelEx(&cfg, pass_kernel<B, true>, p, o.Q, o.loss_u, o.loss_p, o.u, o.pruned_bitmap, o.unified_bitmap,
-                               o.sign_bits);
+        e = mwu::launch_chained(pass_kernel<B, true>, dim3((unsigned)grid_stream), dim3(256), 0, st, 1, p, o.Q, o.loss_u, o.loss_p,
+                                o.u, o.pruned_bitmap, o.unified_bitmap, o.sign_bits);
     else
-        e = cudaLaunchKernelEx(&cfg, pass_kernel<B, false>, p, o.Q, o.loss_u, o.loss_p, o.u, o.pruned_bitmap,
-                               o.unified_bitmap, o.sign_bits);
+        e = mwu::launch_chained(pass_kernel<B, false>, dim3((unsigned)grid_stream), dim3(256), 0, st, 1, p, o.Q, o.loss_u, o.loss_p,
+                                o.u, o.pruned_bitmap, o.unified_bitmap, o.sign_bits);
     if (e != cudaSuccess) return e;
     mwu::count_launch(3);
     if (!need_p && !need_u) return cudaGetLastError();       // no threshold: every class is final
