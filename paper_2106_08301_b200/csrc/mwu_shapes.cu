@@ -1,230 +1,227 @@
 // Projection for 2- and 3-dim block shapes (Section 3.1; Table 1: [2,2], [2,2,2]).
 //
 // A block spans dk input channels x dr rows x dt kernel taps of W[rows][cin * taps]; its weights are
-// not contiguous in memory, so this path works block by block instead of streaming 64-byte units:
-//   shape_stats_kernel     one thread per block gathers its weights and evaluates the fp64 keys of
-//                          Section 3.1 (same pairwise tree as the 1-dim kernels, members in
-//                          (row, channel, tap) order) into two key arrays.
-//   sign_plane_kernel      one bit per weight, v < 0.
-//   select_smallest_kernel exact selection of the k smallest (key, index) among the eligible
-//                          entries of a key array, as a bitmap: radix selection on the keys' bit
-//                          patterns, then the entries holding exactly the threshold key in index order.
-//                          Run twice: prune keys of all blocks, then L_u of the blocks not pruned.
-//   shape_emit_kernel      one thread per block writes Q, u and, for mwu_admm_step, the dual update
-//                          and the residual.
+// not contiguous in memory, so this path works block by block instead of streaming 64-byte units.
+// One launch: a team of CTAs gathers every block once, evaluates the fp64 keys (the pairwise trees of
+// the 1-dim kernels, members in (row, channel, tap) order), selects exactly (mwu_select.cuh) and writes
+// every output.  The keys stay in shared memory while they fit (1.2 million blocks on 148 SMs) and are
+// gathered again in every phase beyond that.  A chain of latencies, like the exact kernel of the 1-dim
+// blocks; the 3x3 convolution weight 128 x 1152
+// with 2x2x2 blocks (20480) takes 25 us, and took 145 with five launches, two of them radix selections by a
+// single CTA; 1024 x 1024 with 2x2 blocks 36 us against 1516.
+//
 // lower_kernel turns the result of a shape whose blocks are runs of dk entries in each of their rows
 // (dt = 1, taps = 1) into the per-row 1-dim arrays mwu_pack reads.
-#include "mwu_common.cuh"
+#include <type_traits>
+
+#include "mwu_blocks.cuh"
+#include "mwu_select.cuh"
 
 namespace mwu {
 namespace shapes {
 
 typedef unsigned long long u64;
-constexpr int SEL_THREADS = 1024;
+using proj::key_bits;
 
 struct SParams {
     const float *W;
     const float *U;
     long long rows, cols;
-    int dk, dr, dt, taps;
-    long long cin_groups, ntg, mb;
+    int ldk, ldr, ldt;          // log2 of the block's extents
+    unsigned taps, ntg, cin_groups, mb;
     int use_l1;
+    sel::XWork *xwork;
+    float *Q, *u, *U_next;
+    double *resid, *loss_u, *loss_p;
+    unsigned *pruned_bitmap, *unified_bitmap, *sign_bits, *dev_status;
 };
 
-// flat indices of block j's weights in (row, channel, tap) order; returns their number
-__device__ __forceinline__ int block_members(const SParams &p, long long j, long long (&idx)[16]) {
-    const long long gt = j % p.ntg, gc = (j / p.ntg) % p.cin_groups, gi = j / (p.ntg * p.cin_groups);
-    const int t_cnt = (int)((p.taps - gt * p.dt) < p.dt ? (p.taps - gt * p.dt) : p.dt);
-    int n = 0;
-    for (int r = 0; r < p.dr; ++r)
-        for (int c = 0; c < p.dk; ++c)
-            for (int t = 0; t < t_cnt; ++t)
-                idx[n++] = (gi * p.dr + r) * p.cols + (gc * p.dk + c) * p.taps + gt * p.dt + t;
-    return n;
+// where block j starts, and whether it lies in the short last tap group (half as many weights)
+__device__ __forceinline__ long long block_base(const SParams &p, unsigned j, bool *is_short) {
+    const unsigned gt = j % p.ntg, g = j / p.ntg, gc = g % p.cin_groups, gi = g / p.cin_groups;
+    const unsigned t0 = gt << p.ldt;
+    *is_short = p.taps - t0 < (1u << p.ldt);
+    return ((long long)gi << p.ldr) * p.cols + ((long long)gc << p.ldk) * p.taps + t0;
 }
-
-__device__ __forceinline__ double tree(double (&t)[16], int n) {
-    for (int w = 1; w < n; w <<= 1)
-        for (int i = 0; i < n; i += 2 * w) t[i] = __dadd_rn(t[i], t[i + w]);
-    return t[0];
+// distance of weight l from the block's start; ldt: log2 of the taps the block really has
+__device__ __forceinline__ long long member(const SParams &p, int l, int ldt) {
+    const int r = l >> (p.ldk + ldt), c = (l >> ldt) & ((1 << p.ldk) - 1), t = l & ((1 << ldt) - 1);
+    return (long long)r * p.cols + (long long)((unsigned)c * p.taps + (unsigned)t);
 }
-
-// S = sum|v|, q = S / n, Lu = sum(|v| - q)^2, sumsq = sum v^2: every operation rounded on its own
-__device__ __forceinline__ void keys_of(const float (&v)[16], int n, double *S, double *q, double *Lu, double *sumsq) {
-    double a[16], t[16];
-    for (int l = 0; l < n; ++l) { a[l] = (double)fabsf(v[l]); t[l] = a[l]; }
-    *S = tree(t, n);
-    *q = __dmul_rn(*S, 1.0 / (double)n);               // n is a power of two: exact scaling
-    for (int l = 0; l < n; ++l) { const double d = __dsub_rn(a[l], *q); t[l] = __dmul_rn(d, d); }
-    *Lu = tree(t, n);
-    for (int l = 0; l < n; ++l) t[l] = __dmul_rn(a[l], a[l]);
-    *sumsq = tree(t, n);
-}
-
-__device__ __forceinline__ int load_members(const SParams &p, long long j, long long (&idx)[16], float (&v)[16]) {
-    const int n = block_members(p, j, idx);
-    for (int l = 0; l < n; ++l) {
-        float w = __ldg(p.W + idx[l]);
-        if (p.U) w = __fadd_rn(w, __ldg(p.U + idx[l]));
-        v[l] = w;
+template <int N>
+__device__ __forceinline__ void gather(const SParams &p, long long base, int ldt, float (&v)[N]) {
+#pragma unroll
+    for (int l = 0; l < N; ++l) {
+        const long long f = base + member(p, l, ldt);
+        v[l] = __ldg(p.W + f);
+        if (p.U) v[l] = __fadd_rn(v[l], __ldg(p.U + f));
     }
-    return n;
 }
 
-__global__ void __launch_bounds__(256) shape_stats_kernel(SParams p, double *key_p, double *key_u, double *loss_u,
-                                                          double *loss_p, unsigned *dev_status) {
-    unsigned bad = 0;
-    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < p.mb; j += (long long)gridDim.x * blockDim.x) {
-        long long idx[16];
-        float v[16];
-        const int n = load_members(p, j, idx, v);
-        double S, q, Lu, sq;
-        keys_of(v, n, &S, &q, &Lu, &sq);
-        bad |= ((unsigned)__double2hiint(S) >= 0x7ff00000u) ? 1u : 0u;       // Inf or NaN among the weights
-        const double kp = p.use_l1 ? S : sq;
-        key_p[j] = kp;
-        key_u[j] = Lu;
-        if (loss_u) loss_u[j] = Lu;
-        if (loss_p) loss_p[j] = kp;
+struct Keys {
+    u64 kp, ku;
+    bool bad;                   // a weight is not finite
+};
+template <int N>
+__device__ __forceinline__ Keys keys_n(const SParams &p, long long base, int ldt) {
+    float v[N];
+    gather<N>(p, base, ldt, v);
+    double S, Lu, Kp;
+    proj::block_keys<N>(v, p.use_l1, &S, &Lu, &Kp);
+    Keys k = {key_bits(Kp), key_bits(Lu), (unsigned)__double2hiint(S) >= 0x7ff00000u};
+    return k;
+}
+template <int N>
+struct Half { static constexpr int value = N / 2 < 2 ? 2 : N / 2; };      // blocks of two weights have no short form
+template <int N>
+__device__ __forceinline__ Keys keys_of(const SParams &p, unsigned j) {
+    bool is_short;
+    const long long base = block_base(p, j, &is_short);
+    return is_short ? keys_n<Half<N>::value>(p, base, p.ldt - 1) : keys_n<N>(p, base, p.ldt);
+}
+
+// outputs of block j in its class; returns its share of ||V - Q||^2
+template <int N>
+__device__ __forceinline__ double emit_n(const SParams &p, unsigned j, long long base, int ldt, bool pr, bool un) {
+    float v[N];
+    gather<N>(p, base, ldt, v);
+    double S, Lu, Kp;
+    proj::block_keys<N>(v, 1, &S, &Lu, &Kp);
+    const float qf = __double2float_rn(__dmul_rn(S, 1.0 / (double)N));
+    p.u[j] = un ? qf : 0.f;
+#pragma unroll
+    for (int l = 0; l < N; ++l) {
+        const long long f = base + member(p, l, ldt);
+        const float q = pr ? 0.f : (un ? (v[l] < 0.f ? -qf : qf) : v[l]);
+        if (p.Q) p.Q[f] = q;
+        if (p.U_next) p.U_next[f] = __fsub_rn(v[l], q);
     }
-    if (bad) atomicOr(dev_status, (unsigned)MWU_DEV_NONFINITE);
+    if (!p.resid || !(pr || un)) return 0.0;
+    return pr ? proj::block_sumsq<N>(v) : Lu;
 }
 
-__global__ void __launch_bounds__(256) sign_plane_kernel(const float *W, const float *U, long long n, unsigned *sign_bits) {
-    const long long n_words = (n + 31) / 32;
-    for (long long wi = (long long)blockIdx.x * blockDim.x + threadIdx.x; wi < n_words; wi += (long long)gridDim.x * blockDim.x) {
-        unsigned word = 0;
-        for (int b = 0; b < 32; ++b) {
-            const long long f = wi * 32 + b;
+constexpr u64 NO_KEY = ~0ull;
+constexpr int SH_THREADS = 512;
+constexpr int SH_SLOTS = 8192;                           // most blocks a CTA holds: 16 bytes of keys each
+enum Form { CLUSTER, GRID, WALK };                       // WALK: a grid that gathers the keys again in every phase
+
+// what select_exact sees: block first + t * stride in slot t of this thread's column ...
+struct Held {
+    const SParams &p;
+    unsigned first, stride, per;
+    const u64 *keys;
+    template <class F>
+    __device__ __forceinline__ void for_blocks(F f) const {
+        const u64 *k = keys;
+#pragma unroll 1
+        for (unsigned t = 0; t < per; ++t, k += 2 * SH_THREADS) f(first + t * stride, k[0], k[SH_THREADS]);
+    }
+    __device__ __forceinline__ bool in_group(unsigned) const { return false; }
+};
+// ... or evaluated each time
+template <int N>
+struct Walked {
+    const SParams &p;
+    unsigned first, stride;
+    template <class F>
+    __device__ __forceinline__ void for_blocks(F f) const {
+        for (unsigned j = first; j < p.mb; j += stride) {
+            const Keys k = keys_of<N>(p, j);
+            f(j, k.kp, k.ku);
+        }
+    }
+    __device__ __forceinline__ bool in_group(unsigned) const { return false; }
+};
+
+template <int N, int FORM>
+__global__ void __launch_bounds__(SH_THREADS) shape_kernel(const __grid_constant__ SParams p,
+                                                           const __grid_constant__ sel::Problem pb, unsigned per) {
+    extern __shared__ __align__(16) unsigned char key_smem[];
+    __shared__ sel::SelSmem sm;
+    typename std::conditional<FORM == CLUSTER, sel::ClusterTeam, sel::GridTeam>::type team;
+    team.cta = blockIdx.x;
+    team.s = &sm;
+    if constexpr (FORM == CLUSTER) {
+        __shared__ sel::ClusterCounts counts;
+        team.mine = &counts;
+        team.begin();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    } else {
+        team.n_cta = gridDim.x;
+        team.x = p.xwork;
+        team.k = 0;
+    }
+    const unsigned first = blockIdx.x * SH_THREADS + threadIdx.x, stride = gridDim.x * SH_THREADS;
+    const int lane = threadIdx.x & 31;
+    if (p.resid && first == 0u) *p.resid = 0.0;
+    float sp = 0.f, su = 0.f;
+    unsigned sj;
+    const bool samp_ok = sel::sample_block_of<SH_THREADS>(pb, threadIdx.x, &sj);
+    if (samp_ok) {
+        const Keys k = keys_of<N>(p, sj);
+        sp = (float)__longlong_as_double((long long)k.kp);
+        su = (float)__longlong_as_double((long long)k.ku);
+    }
+    u64 *keys = reinterpret_cast<u64 *>(key_smem) + threadIdx.x;
+    bool bad = false;
+    // keys of this thread's blocks
+    for (unsigned t = 0, j = first; FORM == WALK ? j < p.mb : t < per; ++t, j += stride) {
+        Keys k = {NO_KEY, NO_KEY, false};
+        if (j < p.mb) {
+            k = keys_of<N>(p, j);
+            bad = bad || k.bad;
+            if (p.loss_u) p.loss_u[j] = __longlong_as_double((long long)k.ku);
+            if (p.loss_p) p.loss_p[j] = __longlong_as_double((long long)k.kp);
+        }
+        if (FORM != WALK) { keys[2 * t * SH_THREADS] = k.kp; keys[(2 * t + 1) * SH_THREADS] = k.ku; }
+    }
+    if (bad) atomicOr(p.dev_status, (unsigned)MWU_DEV_NONFINITE);
+    // sign plane: a warp to a word
+    {
+        const long long n = p.rows * p.cols, n_words = (n + 31) / 32;
+#pragma unroll 4
+        for (long long wi = first >> 5; wi < n_words; wi += stride >> 5) {
+            const long long f = wi * 32 + lane;
+            float v = 0.f;
             if (f < n) {
-                float w = __ldg(W + f);
-                if (U) w = __fadd_rn(w, __ldg(U + f));
-                word |= (w < 0.f ? 1u : 0u) << b;
+                v = __ldg(p.W + f);
+                if (p.U) v = __fadd_rn(v, __ldg(p.U + f));
             }
-        }
-        sign_bits[wi] = word;
-    }
-}
-
-__device__ __forceinline__ unsigned block_scan_incl(unsigned x, unsigned *s_warp) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int m = 1; m < 32; m <<= 1) {
-        const unsigned y = __shfl_up_sync(0xffffffffu, x, m);
-        if (lane >= m) x += y;
-    }
-    if (lane == 31) s_warp[w] = x;
-    __syncthreads();
-    if (w == 0) {
-        unsigned t = s_warp[lane];
-        for (int m = 1; m < 32; m <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, t, m);
-            if (lane >= m) t += y;
-        }
-        s_warp[lane] = t;
-    }
-    __syncthreads();
-    const unsigned add = w ? s_warp[w - 1] : 0u;
-    __syncthreads();
-    return x + add;
-}
-
-// One CTA: bit i of `out` is set for the k entries with the smallest (key, index) among the entries
-// whose bit in `exclude` is clear (exclude may be null).  Keys are non-negative doubles, compared
-// through their bit patterns.  k larger than the eligible count selects all eligible entries.
-__global__ void __launch_bounds__(SEL_THREADS) select_smallest_kernel(const double *key, unsigned n, unsigned k,
-                                                                      const unsigned *exclude, unsigned *out) {
-    __shared__ unsigned s_hist[256];
-    __shared__ u64 s_prefix;
-    __shared__ unsigned s_r, s_all;
-    __shared__ unsigned s_warp[32];
-    const u64 *keys = reinterpret_cast<const u64 *>(key);
-    const unsigned n_words = (n + 31u) / 32u;
-    auto eligible = [&](unsigned i) -> bool { return !exclude || !((exclude[i >> 5] >> (i & 31u)) & 1u); };
-    if (threadIdx.x == 0) { s_prefix = 0; s_r = k; s_all = 0; }
-    __syncthreads();
-    u64 mask = 0;
-    if (k > 0u) {
-        for (int shift = 56; shift >= 0; shift -= 8) {
-            for (unsigned i = threadIdx.x; i < 256u; i += blockDim.x) s_hist[i] = 0;
-            __syncthreads();
-            const u64 prefix = s_prefix;
-            for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
-                const u64 kk = keys[i];
-                if ((kk & mask) == prefix && eligible(i)) atomicAdd(&s_hist[(unsigned)(kk >> shift) & 255u], 1u);
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                unsigned r = s_r, d = 0;
-                while (d < 256u && s_hist[d] < r) { r -= s_hist[d]; ++d; }
-                if (d == 256u) { s_all = 1; d = 255; }  // fewer than k eligible entries under this prefix: take everything
-                s_r = r;
-                s_prefix = prefix | ((u64)d << shift);
-            }
-            mask |= (u64)255 << shift;
-            __syncthreads();
-            if (s_all) break;
+            const unsigned word = __ballot_sync(0xffffffffu, v < 0.f);
+            if (lane == 0) p.sign_bits[wi] = word;
         }
     }
-    const bool all = s_all != 0u;
-    const u64 T = s_prefix;
-    const unsigned r_ties = s_r;
-    const unsigned words_per = (n_words + blockDim.x - 1u) / blockDim.x;
-    const unsigned w0 = threadIdx.x * words_per, w1 = w0 + words_per < n_words ? w0 + words_per : n_words;
-    unsigned ties = 0;
-    if (k > 0u && !all)
-        for (unsigned wi = w0; wi < w1; ++wi)
-            for (unsigned bit = 0; bit < 32u; ++bit) {
-                const unsigned i = wi * 32u + bit;
-                if (i < n && keys[i] == T && eligible(i)) ++ties;
-            }
-    const unsigned incl = block_scan_incl(ties, s_warp);
-    unsigned ordinal = incl - ties;
-    for (unsigned wi = w0; wi < w1; ++wi) {
-        unsigned wv = 0;
-        for (unsigned bit = 0; bit < 32u; ++bit) {
-            const unsigned i = wi * 32u + bit;
-            if (i >= n) break;
-            if (k == 0u || !eligible(i)) continue;
-            bool take = all;
-            if (!all) {
-                const u64 kk = keys[i];
-                take = kk < T;
-                if (kk == T) { take = ordinal < r_ties; ++ordinal; }
-            }
-            wv |= (take ? 1u : 0u) << bit;
-        }
-        out[wi] = wv;
+    if constexpr (FORM == CLUSTER) team.wait();          // every CTA's counts are cleared
+    typename std::conditional<FORM == WALK, Walked<N>, Held>::type src = [&]() {
+        if constexpr (FORM == WALK) return Walked<N>{p, first, stride};
+        else return Held{p, first, stride, per, keys};
+    }();
+    sel::Thresholds T;
+    bool ok = sel::select_exact<SH_THREADS>(src, team, sm, pb, sp, su, samp_ok, p.dev_status, T);
+    // with nothing to select there has been no barrier yet between the cleared residual and its sums
+    if (ok && p.resid && T.mode_p != 0u && T.mode_u != 0u) ok = team.sync();
+    if (!ok) {
+        if (threadIdx.x == 0) atomicOr(p.dev_status, (unsigned)MWU_DEV_TIMEOUT);
+        return;
     }
-}
-
-__global__ void __launch_bounds__(256) shape_emit_kernel(SParams p, const unsigned *pruned_bitmap,
-                                                         const unsigned *unified_bitmap, float *Q, float *u_out,
-                                                         float *U_next, double *resid) {
-    double acc = 0.0;
-    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < p.mb; j += (long long)gridDim.x * blockDim.x) {
-        long long idx[16];
-        float v[16];
-        const int n = load_members(p, j, idx, v);
-        const bool pr = (pruned_bitmap[j >> 5] >> (j & 31)) & 1u;
-        const bool un = !pr && ((unified_bitmap[j >> 5] >> (j & 31)) & 1u);
-        float qf = 0.f;
-        if (un || (resid && pr)) {
-            double S, q, Lu, sq;
-            keys_of(v, n, &S, &q, &Lu, &sq);
-            qf = __double2float_rn(q);
-            if (resid) acc += pr ? sq : Lu;
+    double resid = 0.0;
+    for (unsigned t = 0, j = first; j - (unsigned)lane < p.mb; ++t, j += stride) {      // whole warps stay together
+        bool pr = false, un = false;
+        if (j < p.mb) {
+            u64 kp, ku;
+            if (FORM == WALK) { const Keys k = keys_of<N>(p, j); kp = k.kp; ku = k.ku; }
+            else { kp = keys[2 * t * SH_THREADS]; ku = keys[(2 * t + 1) * SH_THREADS]; }
+            pr = T.pruned(kp, j, false);
+            un = !pr && T.unified(ku, j);
+            bool is_short;
+            const long long base = block_base(p, j, &is_short);
+            resid += is_short ? emit_n<Half<N>::value>(p, j, base, p.ldt - 1, pr, un) : emit_n<N>(p, j, base, p.ldt, pr, un);
         }
-        u_out[j] = un ? qf : 0.f;
-        for (int l = 0; l < n; ++l) {
-            const float q = pr ? 0.f : (un ? (v[l] < 0.f ? -qf : qf) : v[l]);
-            if (Q) Q[idx[l]] = q;
-            if (U_next) U_next[idx[l]] = __fsub_rn(v[l], q);
-        }
+        const unsigned wp = __ballot_sync(0xffffffffu, pr), wu = __ballot_sync(0xffffffffu, un);
+        if (lane == 0) { p.pruned_bitmap[j >> 5] = wp; p.unified_bitmap[j >> 5] = wu; }
     }
-    if (resid) {
-        for (int m = 16; m > 0; m >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, m);
-        if ((threadIdx.x & 31) == 0 && acc != 0.0) atomicAdd(resid, acc);
-    }
+    if (p.resid) proj::block_add_double(resid, p.resid);
 }
 
 // 1-dim run jb = row * (cols / dk) + kb belongs to block (row / dr, kb): its class and magnitude
@@ -251,34 +248,63 @@ static int grid_for(long long items, int sm_count) {
     return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 
-// bytes of scratch the shape path needs: the two key arrays
-size_t workspace_bytes(const mwu_proj_desc *desc) {
-    const ShapeInfo sh = shape_of(desc);
-    return align_up((size_t)sh.mb * sizeof(double)) * 2 + 256;
+// scratch of the shape path: the team's state
+size_t workspace_bytes(const mwu_proj_desc *) { return align_up(sizeof(sel::XWork)); }
+
+template <int N>
+static cudaError_t launch(const SParams &p, const mwu_proj_desc *desc, int sm_count, cudaStream_t st) {
+    const long long mb = p.mb, ctas = (mb + SH_THREADS - 1) / SH_THREADS;
+    const sel::Problem pb = sel::problem_of(mb, desc->k_prune, desc->k_unify, false, SH_THREADS);
+    // One cluster up to 8192 blocks (two a thread): gathering is most of the work, and a grid has more SMs for
+    // it than the cluster's barriers save (20480 blocks: 34 us as a cluster, 25 as a grid; 5120: 18).  Keys
+    // held while a CTA's fit.
+    if (mb <= 2ll * sel::CLUSTER_CTAS * SH_THREADS) {
+        const unsigned per = (unsigned)((ctas + sel::CLUSTER_CTAS - 1) / sel::CLUSTER_CTAS);
+        const size_t smem = (size_t)per * SH_THREADS * 16;
+        const cudaError_t e = cudaFuncSetAttribute(shape_kernel<N, CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * SH_THREADS * 16);
+        if (e != cudaSuccess) return e;
+        count_launch();
+        return launch_chained(shape_kernel<N, CLUSTER>, dim3(sel::CLUSTER_CTAS), dim3(SH_THREADS), smem, st, sel::CLUSTER_CTAS, p, pb, per);
+    }
+    if (cudaMemsetAsync(p.xwork, 0, sel::XWORK_ZERO_BYTES, st) != cudaSuccess) return cudaErrorUnknown;
+    const int grid = (int)(ctas < sm_count ? ctas : sm_count);
+    unsigned per = (unsigned)((ctas + grid - 1) / grid);
+    const bool held = (long long)per * SH_THREADS <= SH_SLOTS;
+    auto kern = held ? shape_kernel<N, GRID> : shape_kernel<N, WALK>;
+    if (held) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SH_SLOTS * 16);
+        if (e != cudaSuccess) return e;
+    }
+    const size_t smem = held ? (size_t)per * SH_THREADS * 16 : 0;
+    SParams pc = p;
+    sel::Problem pbc = pb;
+    void *argv[] = {&pc, &pbc, &per};
+    count_launch();
+    return cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)grid), dim3(SH_THREADS), argv, smem, st);
 }
 
 int project(const mwu_proj_desc *desc, const float *W, const float *U_dual, float *Q, float *U_next,
             double *residual_sq, float *u, uint32_t *pruned_bitmap, uint32_t *unified_bitmap, uint32_t *sign_bits,
             double *loss_u, double *loss_p, uint32_t *dev_status, void *workspace, int sm_count, cudaStream_t st) {
     const ShapeInfo sh = shape_of(desc);
+    auto log2_of = [](int x) { int l = 0; while ((1 << l) < x) ++l; return l; };
     SParams p;
     p.W = W; p.U = U_dual;
     p.rows = desc->rows; p.cols = desc->cols;
-    p.dk = sh.dk; p.dr = sh.dr; p.dt = sh.dt; p.taps = sh.taps;
-    p.cin_groups = sh.cin_groups; p.ntg = sh.ntg; p.mb = sh.mb;
+    p.ldk = log2_of(sh.dk); p.ldr = log2_of(sh.dr); p.ldt = log2_of(sh.dt);
+    p.taps = (unsigned)sh.taps; p.ntg = (unsigned)sh.ntg; p.cin_groups = (unsigned)sh.cin_groups; p.mb = (unsigned)sh.mb;
     p.use_l1 = desc->prune_key == MWU_PRUNE_KEY_L1;
-    double *key_p = (double *)workspace;
-    double *key_u = (double *)((char *)workspace + align_up((size_t)sh.mb * sizeof(double)));
-    if (residual_sq && cudaMemsetAsync(residual_sq, 0, sizeof(double), st) != cudaSuccess) return MWU_ERR_CUDA;
-    shape_stats_kernel<<<grid_for(sh.mb, sm_count), 256, 0, st>>>(p, key_p, key_u, loss_u, loss_p, dev_status);
-    const long long n = desc->rows * desc->cols;
-    sign_plane_kernel<<<grid_for((n + 31) / 32, sm_count), 256, 0, st>>>(W, U_dual, n, sign_bits);
-    select_smallest_kernel<<<1, SEL_THREADS, 0, st>>>(key_p, (unsigned)sh.mb, (unsigned)desc->k_prune, nullptr, pruned_bitmap);
-    select_smallest_kernel<<<1, SEL_THREADS, 0, st>>>(key_u, (unsigned)sh.mb, (unsigned)(desc->k_unify - desc->k_prune),
-                                                      pruned_bitmap, unified_bitmap);
-    shape_emit_kernel<<<grid_for(sh.mb, sm_count), 256, 0, st>>>(p, pruned_bitmap, unified_bitmap, Q, u, U_next, residual_sq);
-    count_launch(5);
-    return cudaGetLastError() == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
+    p.xwork = (sel::XWork *)workspace;
+    p.Q = Q; p.u = u; p.U_next = U_next; p.resid = residual_sq; p.loss_u = loss_u; p.loss_p = loss_p;
+    p.pruned_bitmap = pruned_bitmap; p.unified_bitmap = unified_bitmap; p.sign_bits = sign_bits; p.dev_status = dev_status;
+    cudaError_t e;
+    switch (sh.dk * sh.dr * sh.dt) {
+        case 2: e = launch<2>(p, desc, sm_count, st); break;
+        case 4: e = launch<4>(p, desc, sm_count, st); break;
+        case 8: e = launch<8>(p, desc, sm_count, st); break;
+        default: e = launch<16>(p, desc, sm_count, st); break;
+    }
+    return e == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
 }
 
 // scratch mwu_pack needs behind the packed bytes for a shaped descriptor: lowered u and bitmaps

@@ -158,3 +158,13 @@ def test_shape_descriptors_are_validated():
     assert B.mwu_project_workspace_bytes(shaped_desc(64, 72, O.BlockShape(2, 2, 2, taps=9), 10, 5)) > 0
     d = shaped_desc(64, 72, O.BlockShape(2, 2, 2, taps=9), 64 * 4 * 5 // 2 + 1, 0)                   # k_unify > blocks
     assert B.mwu_project_workspace_bytes(d) == 0
+
+
+@pytest.mark.parametrize("shape,rows,cols", [(O.BlockShape(2, 2, 2, taps=9), 128, 576),      # 10240 blocks: a grid with spare SMs
+                                             (O.BlockShape(2, 2, 2, taps=9), 64, 36),        # 160 blocks: one cluster, mostly empty
+                                             (O.BlockShape(2, 4, 2, taps=9), 512, 576),      # 16 weights to a block, short tap groups
+                                             (O.BlockShape(2, 2), 4096, 1280)])              # 1.3 M blocks: keys gathered again in every phase
+def test_block_shape_projection_size_edges(shape, rows, cols):
+    W = inputs.normal_weights(rows, cols, 0.02, 1900 + rows + cols)
+    W[:: max(rows // 16, 1)] = 0.0                       # equal keys across many blocks
+    check_shape(W, shape, 600, 300)
