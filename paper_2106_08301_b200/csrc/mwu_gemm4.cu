@@ -93,8 +93,7 @@ mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     MWU_CHECK_HEADER(p);
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *base = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *base = smem_raw + smem_pad_1024(smem_raw);
     unsigned char *tiles = base;
     unsigned char *xbuf = tiles + q.groups * REC_BYTES;
     const unsigned x_bytes = (unsigned)q.mpad * (BK * 2);

@@ -82,6 +82,9 @@ __device__ __forceinline__ bool header_matches(const Params &p) {
 __device__ __forceinline__ unsigned smem_u32(const void *p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
+// bytes from p to the next 1024-byte boundary of shared memory.  (Rounding the pointer itself up through an
+// integer would hide from the compiler that it points to shared memory: every access would become generic.)
+__device__ __forceinline__ unsigned smem_pad_1024(const void *p) { return (1024u - (smem_u32(p) & 1023u)) & 1023u; }
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
 }

@@ -292,3 +292,19 @@ def test_gemm_few_rows(b, rows, cols, M, ku, kp):
         W[:, 64:144] = 0.0                       # a dead stage and a dead slice wherever blocks of zeros are pruned
     Mb = W.numel() // b
     check_gemm(W, b, Mb * ku // 10, Mb * kp // 10, M, seed=40 + b)
+
+
+@pytest.mark.parametrize("filters,cin,h,w,k,stride,pad,n,b", [(128, 64, 13, 11, 3, 2, 1, 2, 4),    # four planes, odd sizes
+                                                              (136, 128, 9, 9, 3, 1, 1, 1, 8),     # two chunks over a cluster, ragged filters
+                                                              (256, 64, 30, 29, 3, 1, 1, 24, 16),  # several tiles to a CTA, two filter tiles
+                                                              (128, 80, 12, 10, 2, 2, 0, 3, 2),    # a chunk of 16 channels, four taps
+                                                              (128, 64, 7, 8, 1, 2, 0, 2, 4),      # 1x1 with a stride: one plane of four
+                                                              (128, 64, 9, 7, 3, 1, 4, 2, 4),      # more padding than kernel
+                                                              (128, 64, 6, 700, 3, 1, 1, 1, 8),    # long rows: one gather per kernel row
+                                                              (128, 64, 10, 9, 3, 3, 1, 2, 16)])
+def test_conv_fused_shapes(filters, cin, h, w, k, stride, pad, n, b):
+    """The kernel without scratch memory: strides, planes, halos and chunks at their edges."""
+    W = inputs.normal_weights(filters, cin * k * k, 0.05, 780 + filters + cin + k + h)
+    x = inputs.normal_activations_bf16((n, cin, h, w), 781 + h)
+    Mb = W.numel() // b
+    conv_case(W, b, Mb * 6 // 10, Mb * 3 // 10, x, k, k, stride, pad)
