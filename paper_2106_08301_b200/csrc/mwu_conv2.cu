@@ -53,6 +53,9 @@ struct HaloParams {
 
 struct HaloSmem {
     unsigned long long a_full[2], a_empty[2], w_full, w_empty, t_full, t_empty;
+    int4 group[CV_TAPS];                // of every gather: see TapGroup
+    int4 group2[CV_TAPS];
+    uint4 rec[CV_TAPS + 1];             // record table of the chunk being decoded
     unsigned tmem_base;
     int abort;
 };
@@ -72,10 +75,10 @@ __device__ __forceinline__ bool named_any(int id, bool pred) {
 }
 
 // One gather: the taps (di0 + s * i, dj0 + s * j), i < ni, j < nj, of one plane; tap (i, j) reads the rows
-// i * Wp + j further on than the tile's own, counted from `base`.
+// i * Wp + j further on than the tile's own, counted from `base`.  A pixel (y, x) of the plane's line is the
+// image's (y * s + dy, x * s + dx).
 struct TapGroup {
-    int di0, dj0, ni, nj;
-    long long base;
+    int di0, dj0, ni, nj, base, dy, dx;
 };
 __device__ __forceinline__ int tap_groups(const HaloParams &p) {
     const int pa = p.stride < p.KH ? p.stride : p.KH, pb = p.stride < p.KW ? p.stride : p.KW;
@@ -88,10 +91,19 @@ __device__ __forceinline__ TapGroup tap_group(const HaloParams &p, int g) {
     else { t.di0 = g / pb; t.dj0 = g - t.di0 * pb; }
     t.ni = p.group_mode == 0 ? (p.KH - 1 - t.di0) / s + 1 : 1;
     t.nj = p.group_mode == 2 ? 1 : (p.KW - 1 - t.dj0) / s + 1;
-    t.base = (long long)(t.di0 / s) * p.Wp + t.dj0 / s;
-    if (p.shared_pad) t.base -= (long long)p.pad * p.Wp + p.pad;
+    t.base = (t.di0 / s) * p.Wp + t.dj0 / s;
+    if (p.shared_pad) t.base -= p.pad * p.Wp + p.pad;
+    t.dy = p.shared_pad ? 0 : t.di0 % s - p.pad;
+    t.dx = p.shared_pad ? 0 : t.dj0 % s - p.pad;
     return t;
 }
+// (their divisions take longer than a gather's loads: worked out once per CTA)
+__device__ __forceinline__ TapGroup load_group(const int4 *a, const int4 *b, int g) {
+    const int4 x = a[g], y = b[g];
+    TapGroup t = {x.x, x.y, x.z, x.w, y.x, y.y, y.z};
+    return t;
+}
+
 // n / d for n < 2^31, with m = floor(2^32 / d) + 1: the product's high word is the quotient or one too many
 __device__ __forceinline__ unsigned divide(unsigned n, unsigned d, unsigned m, unsigned *rem) {
     unsigned q = d == 1u ? n : __umulhi(n, m);
@@ -204,28 +216,34 @@ __device__ __noinline__ void permute_rows(unsigned w_s, int warp, int lane) {
 
 // The records of one chunk of 64 channels -> one 128 x 64 tile per tap, by all workers.
 template <int BW>
-__device__ __forceinline__ void weights_to_taps(const HaloParams &p, unsigned char *w, int nt, int chunk, int taps, int tid) {
+__device__ __forceinline__ void weights_to_taps(const HaloParams &p, unsigned char *w, uint4 *s_rec, int nt, int chunk, int taps, int tid) {
     const uint4 *recs = reinterpret_cast<const uint4 *>(p.g.packed + p.g.off_rec) + (long long)nt * p.g.n_stages;
     const int s0 = chunk * taps;
     const int n = s0 + taps < (int)p.g.n_stages ? taps : (int)p.g.n_stages - s0;        // at least one
     constexpr unsigned ROUND = Entries<BW>::BATCH * CV_WORK_THREADS;
+    if (tid <= n) s_rec[tid] = __ldg(recs + s0 + tid);
+    uint4 *z = reinterpret_cast<uint4 *>(w);
+    for (int i = tid; i < taps * (REC_BYTES / 16); i += CV_WORK_THREADS) z[i] = make_uint4(0, 0, 0, 0);
+    named_any<CV_WORK_THREADS>(1, false);
     // a record whose ranges do not lie inside the sections counts as empty
-    auto check = [&](const uint4 &a, uint4 &b) {
+    auto ends = [&](int i, uint4 &a, uint4 &b) {
+        a = s_rec[i];
+        b = s_rec[i + 1];
         if (a.x > b.x || b.x > p.g.n_unified || a.y > b.y || b.y > p.g.n_dense) {
             if (tid == 0) atomicOr(p.g.dev_status, (unsigned)MWU_DEV_BOUNDS);
             b.x = a.x; b.y = a.y;
         }
     };
-    uint4 a = __ldg(recs + s0), b = __ldg(recs + s0 + 1), b_raw = b;
-    check(a, b);
+    // The CTAs of a launch mostly decode the same records at the same time; each starts with another one, so that
+    // they do not all ask for the same lines of L2 at once.
+    int cur_i = (int)(blockIdx.x % (unsigned)n);
+    uint4 a, b, na, nb;
+    ends(cur_i, a, b);
     Entries<BW> x;
     read_entries<BW>(p.g, a, b, (unsigned)tid, x);
-    uint4 *z = reinterpret_cast<uint4 *>(w);
-    for (int i = tid; i < taps * (REC_BYTES / 16); i += CV_WORK_THREADS) z[i] = make_uint4(0, 0, 0, 0);
-    named_any<CV_WORK_THREADS>(1, false);
     for (int i = 0; i < n; ++i) {
-        uint4 na = b_raw, nb = make_uint4(0, 0, 0, 0), nb_raw = nb;
-        if (i + 1 < n) { nb = __ldg(recs + s0 + i + 2); nb_raw = nb; check(na, nb); }
+        const int next_i = cur_i + 1 == n ? 0 : cur_i + 1;
+        if (i + 1 < n) ends(next_i, na, nb);
         const unsigned most = max(b.x - a.x, b.y - a.y);
         for (unsigned r0 = 0;; r0 += ROUND) {
             const bool last = r0 + ROUND >= most;
@@ -233,10 +251,10 @@ __device__ __forceinline__ void weights_to_taps(const HaloParams &p, unsigned ch
             // the next round's entries travel while this one's are stored
             if (!last) read_entries<BW>(p.g, a, b, r0 + ROUND + (unsigned)tid, x);
             else if (i + 1 < n) read_entries<BW>(p.g, na, nb, (unsigned)tid, x);
-            write_blocks<BW>(w + i * REC_BYTES, a, b, r0 + (unsigned)tid, cur);
+            write_blocks<BW>(w + cur_i * REC_BYTES, a, b, r0 + (unsigned)tid, cur);
             if (last) break;
         }
-        a = na; b = nb; b_raw = nb_raw;
+        a = na; b = nb; cur_i = next_i;
     }
     named_any<CV_WORK_THREADS>(1, false);
     const int warp = tid >> 5, lane = tid & 31;
@@ -261,8 +279,7 @@ __device__ __forceinline__ void gather_rows(const HaloParams &p, unsigned char *
     const int rows = CV_TILE + (tgp.ni - 1) * p.Wp + tgp.nj - 1;
     const long long plane = (long long)p.H * p.W;
     const int oct = warp & 7, c0 = chunk * BK + oct * 8, n_ch = p.C - c0 < 8 ? p.C - c0 : 8;
-    const int dy = p.shared_pad ? 0 : tgp.di0 % p.stride - p.pad, dx = p.shared_pad ? 0 : tgp.dj0 % p.stride - p.pad;
-    const int sy = p.shared_pad ? 1 : p.stride;
+    const int sy = p.stride;                                // 1 where zero pixels are shared
     constexpr int U = 3, STEP = 32 * (CV_WORKERS / 8);
     for (int r0 = (warp >> 3) * 32 + lane; r0 - lane < rows; r0 += U * STEP) {
         const unsigned short *src[U];
@@ -274,8 +291,8 @@ __device__ __forceinline__ void gather_rows(const HaloParams &p, unsigned char *
             int img = 0, y = 0, x = 0;
             in[k] = r < rows && P >= 0 && P < p.M && n_ch > 0;
             split_pixel(p, in[k] ? P : 0, &img, &y, &x);
-            y = y * sy + dy;
-            x = x * sy + dx;
+            y = y * sy + tgp.dy;
+            x = x * sy + tgp.dx;
             in[k] = in[k] && (unsigned)y < (unsigned)p.H && (unsigned)x < (unsigned)p.W;
             src[k] = in[k] ? p.X + ((long long)img * p.C + c0) * plane + (y * p.W + x) : p.X;
         }
@@ -329,6 +346,12 @@ __global__ void __launch_bounds__(CV_THREADS, 1) mwu_conv_halo_kernel(const __gr
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
+    if (warp == 1 && lane < n_groups) {
+        const TapGroup t = tap_group(p, lane);
+        sm->group[lane] = make_int4(t.di0, t.dj0, t.ni, t.nj);
+        sm->group2[lane] = make_int4(t.base, t.dy, t.dx, 0);
+    }
+    __syncwarp();
     if (warp == CV_MMA_WARP) tmem_alloc(smem_u32(&sm->tmem_base), p.tmem_cols);
     tc_fence_before();
     __syncthreads();
@@ -347,7 +370,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) mwu_conv_halo_kernel(const __gr
             for (int chunk = rank; chunk < p.chunks; chunk += p.split) {
                 if (ok && !mbar_wait(smem_u32(&sm->w_empty), w_phase ^ 1u, abort)) ok = false;
                 if (named_any<CV_WORK_THREADS>(1, !ok)) { ok = false; break; }          // the same decision in every worker
-                weights_to_taps<BW>(p, sW, nt, chunk, taps, (int)threadIdx.x);
+                weights_to_taps<BW>(p, sW, sm->rec, nt, chunk, taps, (int)threadIdx.x);
                 fence_proxy_async();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&sm->w_full));
@@ -358,7 +381,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) mwu_conv_halo_kernel(const __gr
                         if (!mbar_wait(smem_u32(&sm->a_empty[ab]), a_phase ^ 1u, abort)) ok = false;
                         ok = __all_sync(0xffffffffu, ok);
                         if (!ok) break;
-                        gather_rows(p, sA + ab * a_bytes, tap_group(p, g), p0, chunk, warp, lane);
+                        gather_rows(p, sA + ab * a_bytes, load_group(sm->group, sm->group2, g), p0, chunk, warp, lane);
                         fence_proxy_async();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&sm->a_full[ab]));
@@ -399,13 +422,13 @@ __global__ void __launch_bounds__(CV_THREADS, 1) mwu_conv_halo_kernel(const __gr
                     if (p.g.y_fp32) {
                         float *dst = reinterpret_cast<float *>(p.g.Y) + at + o0 * out_plane;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (o0 + j < p.g.N) dst[j * out_plane] = __uint_as_float(v[j]);
+                        for (int j = 0; j < 32; ++j, dst += out_plane)
+                            if (o0 + j < p.g.N) *dst = __uint_as_float(v[j]);
                     } else {
                         __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(p.g.Y) + at + o0 * out_plane;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (o0 + j < p.g.N) dst[j * out_plane] = __float2bfloat16_rn(__uint_as_float(v[j]));
+                        for (int j = 0; j < 32; ++j, dst += out_plane)
+                            if (o0 + j < p.g.N) *dst = __float2bfloat16_rn(__uint_as_float(v[j]));
                     }
                 }
                 __syncwarp();
@@ -429,7 +452,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) mwu_conv_halo_kernel(const __gr
                 for (int q = 0; ok && q < CV_BATCH && t0 + q * step < n_tiles; ++q) {
                     bool fresh = chunk == rank;          // the tile's first MMA overwrites
                     for (int g = 0; ok && g < n_groups; ++g) {
-                        const TapGroup tgp = tap_group(p, g);
+                        const TapGroup tgp = load_group(sm->group, sm->group2, g);
                         if (!mbar_wait_spin(smem_u32(&sm->a_full[ab]), a_phase, abort)) ok = false;
                         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
                         tc_fence_after();
