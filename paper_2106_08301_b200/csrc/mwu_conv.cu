@@ -1,24 +1,19 @@
-// mwu_conv_implicit_ws: the convolution as an implicit GEMM over weights expanded once per call.
+// mwu_conv_implicit_ws and mwu_conv_dense: the convolution over operands laid out once per call in the
+// caller's workspace.
 //
-// The fused kernel behind mwu_conv_implicit decodes every weight record again for each activation
-// tile and assembles its im2col rows element by element.  With a workspace the work is split:
-//   conv_prep_kernel        one launch, two jobs side by side: image tiles are copied into
-//                           pixel-major order (channels innermost, so that the 64 channels of a
-//                           pixel are one 128-byte line), and the packed weights are expanded once,
-//                           as mwu_decode does, but with the reduction axis tap-major: column
-//                           (i*kw + j) * cin + c instead of c * kh*kw + i*kw + j (the same products,
-//                           summed tap by tap);
-//   mwu_conv_taps_kernel    one CTA per tile of R output rows x OW pixels (R * OW <= 128) and 128
-//                           filters.  A k stage is one filter tap and 64 channels: its activation
-//                           operand is a box of the pixel-major image shifted by the tap's offset,
-//                           fetched by ONE tiled TMA load whose out-of-range rows and columns read
-//                           as zero (the padding costs nothing and no im2col row is ever built);
-//                           its weight operand is a 128 x 64 box of the expanded weights.
-//                           tcgen05.mma 128 x 128 x 16, fp32 accumulators double-buffered in
-//                           tensor memory, so the epilogue of a tile runs under the next tile's loop.
-// Roles (6 warps): warp 0 issues the TMA loads, warp 1 owns tensor memory and issues the MMAs,
-// warps 2-5 read the accumulators and store NCHW output (a lane is a pixel, so the 32 lanes of a
-// warp write 32 neighbouring pixels of one filter: one 64-byte run).
+//   conv_prep_kernel      one launch, two jobs side by side.  The image becomes a line of pixels, 64 channels of
+//                         a pixel to a 128-byte row, with enough zero pixels between image rows and images that
+//                         a tap never reaches into a neighbour.  The weights (packed records, or a plain matrix)
+//                         get a tap-major reduction axis: column (i*kw + j) * cin + c instead of c * kh*kw + i*kw + j.
+//   mwu_conv_line_kernel  for every tap the activation operand of 128 consecutive pixels of the line is 128 rows
+//                         of it, shifted by a constant.  So a CTA fetches a tile's rows with their halo once per 64
+//                         channels (plain TMA boxes), and every tap's MMAs read them through a descriptor that
+//                         starts the tap's shift further on; the weights arrive as one 128 x 64 box per tap.
+//                         Fetching a box per tap instead (the image nine times) bound the kernel: 576 KB from L2
+//                         for a tile of 112 pixels and 18 taps x chunks, against 360 KB for 256 pixels.
+// Roles (11 warps): warp 0 fetches halo rows, warp 10 weights, warp 1 owns tensor memory and issues the MMAs
+// (128 x 128 x 16; a tile of 256 pixels is two accumulators that share every weight box), warps 2-9 store NCHW
+// output (a tensor-memory lane is a pixel).  Accumulators are double-buffered.
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises MWU_DEV_TIMEOUT, waits
 // for the loads it has in flight, frees its tensor memory and returns.
 #include "mwu_gemm_dev.cuh"
@@ -28,26 +23,31 @@ namespace gemm {
 
 EncodeTiledFn get_encode_fn();          // mwu_gemm.cu
 
-constexpr int C_STAGES = 6;
-constexpr int C_A_BYTES = 128 * 128;    // up to 128 pixels x 64 channels
-constexpr int C_B_BYTES = REC_BYTES;    // 128 filters x 64 channels
-constexpr int C_THREADS = 32 * 6;
+constexpr int L_THREADS = 32 * 11;
+constexpr int L_B_WARP = 10;
+constexpr int L_MAX_STAGES = 8;         // weight boxes in flight
+constexpr int L_SMEM = 227 * 1024;
 
 struct ConvParams {
     Params g;                           // packed weights, N = filters, K = cin*kh*kw, Y, y_fp32, dev_status
     int C, H, W, KH, KW, pad, OH, OW, NIMG;
-    int R;                              // output rows per tile
-    int tiles_per_img;
+    int Hp, Wp, shift;                  // the line of pixels: image rows, pitch, and how far the taps start before a pixel
+    long long M;                        // its pixels: NIMG * Hp * Wp
+    unsigned img_magic, row_magic;
+    int tm;                             // pixels of a tile: 128 or 256
+    int rows_apart;                     // 1: a fetch serves one kernel row, not all taps
+    int a_rows, a_bufs, box_rows;       // rows of a fetch, buffers, rows of a TMA box
+    int b_stages;
     int n_ntiles;                       // 128-filter tiles
-    unsigned a_bytes;                   // bytes one activation load delivers
     long long wait_limit;               // cycles a wait may take
-    long long withhold;                 // testing aid: running number of a stage whose loads are left out (-1: none)
+    long long withhold;                 // testing aid: running number of a weight box that is left out (-1: none)
 };
 
 struct ConvSmem {
-    unsigned long long full[C_STAGES], empty[C_STAGES], tfull[2], tempty[2], drain;
+    unsigned long long a_full[2], a_empty[2], b_full[L_MAX_STAGES], b_empty[L_MAX_STAGES], tfull[2], tempty[2], drain;
     unsigned tmem_base;
     int abort;
+    int no_abort;
 };
 
 __device__ __forceinline__ bool mbar_wait_lim(unsigned bar, unsigned parity, volatile int *abort, long long limit) {
@@ -64,58 +64,55 @@ __device__ __forceinline__ bool mbar_wait_lim(unsigned bar, unsigned parity, vol
     }
 }
 
-__device__ __forceinline__ void tma_load_4d(unsigned dst, const CUtensorMap *map, unsigned bar, int c0, int c1,
-                                            int c2, int c3) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-        ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+
+// n / d for n < 2^31, with m = floor(2^32 / d) + 1: the product's high word is the quotient or one too many
+__device__ __forceinline__ unsigned line_divide(unsigned n, unsigned d, unsigned m, unsigned *rem) {
+    unsigned q = d == 1u ? n : __umulhi(n, m);
+    unsigned r = n - q * d;
+    if ((int)r < 0) { --q; r += d; }
+    *rem = r;
+    return q;
+}
+// (image, row, column) of a pixel of the line
+__device__ __forceinline__ void line_pixel(const ConvParams &p, unsigned P, int *img, int *y, int *x) {
+    unsigned rem, col;
+    *img = (int)line_divide(P, (unsigned)p.Hp * (unsigned)p.Wp, p.img_magic, &rem);
+    *y = (int)line_divide(rem, (unsigned)p.Wp, p.row_magic, &col);
+    *x = (int)col;
 }
 
 // ------------------------------------------------------------------------------------------
-// preparation, one launch: the input image [n][c][h*w] -> [n][h*w][c], and the weights
+// preparation
 // ------------------------------------------------------------------------------------------
-constexpr int PREP_THREADS = 512;
+constexpr int PREP_THREADS = 256;
 
-// one CTA: a tile of 64 pixels x 64 channels of one image, read as pixel pairs, written as channel pairs
-__device__ __forceinline__ void nchw_to_nhwc_tile(const unsigned short *x, unsigned short *xt, int C, int HW,
-                                                  int tile, int tiles_hw, int tiles_c) {
-    __shared__ unsigned short s_t[64][66];
-    const int img = tile / (tiles_hw * tiles_c), rem = tile % (tiles_hw * tiles_c);
-    const int hw0 = (rem % tiles_hw) * 64, c0 = (rem / tiles_hw) * 64;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;            // 32 x 16
-    const long long base = (long long)img * C * HW;
+// a warp: 32 pixels x 16 channels, read along the image rows, written as 32 bytes of each pixel's row
+__device__ __forceinline__ void image_to_line(const ConvParams &p, const unsigned short *x, unsigned short *xt, long long task) {
+    const int lane = threadIdx.x & 31;
+    const unsigned n_c = (unsigned)p.C / 16u;
+    const long long pix0 = (task / n_c) * 32;
+    const int c0 = (int)(task % n_c) * 16;
+    const long long P = pix0 + lane;
+    if (P >= p.M) return;
+    int img, y, xx;
+    line_pixel(p, (unsigned)P, &img, &y, &xx);
+    y -= p.pad - p.shift;                                   // shift: zero pixels follow an image row, else they surround it
+    xx -= p.pad - p.shift;
+    const bool in = (unsigned)y < (unsigned)p.H && (unsigned)xx < (unsigned)p.W;
+    const long long plane = (long long)p.H * p.W;
+    const unsigned short *src = x + ((long long)img * p.C + c0) * plane + (in ? y * p.W + xx : 0);
+    unsigned v[16];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int c = c0 + ty + 16 * i, hw = hw0 + 2 * tx;
-        unsigned short a = 0, b = 0;
-        if (c < C) {
-            if (hw + 1 < HW && (HW & 1) == 0) {
-                const unsigned v = *reinterpret_cast<const unsigned *>(x + base + (long long)c * HW + hw);
-                a = (unsigned short)v; b = (unsigned short)(v >> 16);
-            } else {
-                if (hw < HW) a = x[base + (long long)c * HW + hw];
-                if (hw + 1 < HW) b = x[base + (long long)c * HW + hw + 1];
-            }
-        }
-        s_t[ty + 16 * i][2 * tx] = a;
-        s_t[ty + 16 * i][2 * tx + 1] = b;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int hw = hw0 + ty + 16 * i, c = c0 + 2 * tx;
-        if (hw < HW && c + 1 < C + 1) {
-            unsigned short *dst = xt + ((long long)img * HW + hw) * C + c;
-            const unsigned short a = s_t[2 * tx][ty + 16 * i], b = s_t[2 * tx + 1][ty + 16 * i];
-            if (c + 1 < C) *reinterpret_cast<unsigned *>(dst) = (unsigned)a | ((unsigned)b << 16);     // C is even
-            else if (c < C) dst[0] = a;
-        }
-    }
+    for (int e = 0; e < 16; ++e) v[e] = in ? (unsigned)__ldg(src + e * plane) : 0u;
+    uint4 *dst = reinterpret_cast<uint4 *>(xt + P * p.C + c0);
+    dst[0] = make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
+    dst[1] = make_uint4(v[8] | (v[9] << 16), v[10] | (v[11] << 16), v[12] | (v[13] << 16), v[14] | (v[15] << 16));
 }
 
-// one CTA: a packed 128 x 64 record -> row-major bf16 with the reduction axis in tap-major order
+// a packed 128 x 64 record -> tap-major rows; `part` of `parts` CTAs that decode it alike and write its share of rows
+// (the scattered 2-byte stores take longer than the decoding)
 template <int BW>
-__device__ __forceinline__ void decode_taps_record(const Params &p, unsigned short *Wd, int taps, int C, long long rec) {
+__device__ __forceinline__ void record_to_taps(const Params &p, unsigned short *Wd, int taps, int C, long long rec, int part, int parts) {
     __shared__ __align__(1024) unsigned char tile[REC_BYTES];
     constexpr int ENT = DecodeCfg<BW, PREP_THREADS>::ENT;
     const PackedRec *recs = reinterpret_cast<const PackedRec *>(p.packed + p.off_rec);
@@ -133,222 +130,257 @@ __device__ __forceinline__ void decode_taps_record(const Params &p, unsigned sho
     write_entries<BW, PREP_THREADS>(tile, r0, r1, p, tid, m0, m1);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-#pragma unroll
-    for (int i = 0; i < (REC_BYTES / 16) / PREP_THREADS; ++i) {
-        const int q = tid + i * PREP_THREADS;               // 16-byte piece: row q / 8, piece q % 8
-        const int r = q >> 3, j = q & 7;
+    const int rows = kTileRows / parts;
+    for (int q = tid; q < rows * 8; q += PREP_THREADS) {
+        const int r = part * rows + (q >> 3), j = q & 7;    // 16-byte piece j of row r
         const uint4 v = *reinterpret_cast<const uint4 *>(tile + r * 128 + ((j ^ (r & 7)) << 4));
         const unsigned wds[4] = {v.x, v.y, v.z, v.w};
         unsigned short *row = Wd + (rt * kTileRows + r) * p.K;
+        const int k0 = (int)ks * BK + j * 8;                // columns in [c][tap] order
+        int c = k0 / taps, tap = k0 - c * taps;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const int k = (int)ks * BK + j * 8 + e;         // column in [c][tap] order
-            const int c = k / taps, tap = k - c * taps;
             row[(long long)tap * C + c] = (unsigned short)(wds[e >> 1] >> (16 * (e & 1)));
+            if (++tap == taps) { tap = 0; ++c; }
         }
     }
 }
 
-// CTAs [0, n_rec): weight records; the rest: image tiles.  The two jobs do not depend on each other,
-// so one launch runs them side by side.
+// CTAs [0, n_w): weights; the rest: image.  BW 0: a plain weight matrix [rows][ldw] in [c][tap] column order
 template <int BW>
-__global__ void __launch_bounds__(PREP_THREADS) conv_prep_kernel(const Params p, unsigned short *Wd, int taps, int C,
-                                                                 unsigned n_rec, const unsigned short *x,
-                                                                 unsigned short *xt, int HW, int tiles_hw, int tiles_c) {
+__global__ void __launch_bounds__(PREP_THREADS) conv_prep_kernel(const __grid_constant__ ConvParams p, const unsigned short *Wd,
+                                                                 long long ldw, long long n_pad, unsigned short *wt, unsigned n_w,
+                                                                 int parts, const unsigned short *x, unsigned short *xt) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the tensor-core kernel may set itself up meanwhile
-    if (blockIdx.x < n_rec) {
-        MWU_CHECK_HEADER(p);
-        decode_taps_record<BW>(p, Wd, taps, C, blockIdx.x);
+    const int taps = p.KH * p.KW;
+    if (blockIdx.x < n_w) {
+        if constexpr (BW == 0) {
+            const long long K = p.g.K, total = n_pad * K;
+            for (long long i = (long long)blockIdx.x * PREP_THREADS + threadIdx.x; i < total; i += (long long)n_w * PREP_THREADS) {
+                const long long row = i / K;
+                const int kk = (int)(i - row * K), tap = kk / p.C, c = kk - tap * p.C;
+                wt[i] = row < p.g.N ? Wd[row * ldw + (long long)c * taps + tap] : (unsigned short)0;     // rows past the last: zeros
+            }
+        } else {
+            MWU_CHECK_HEADER(p.g);
+            record_to_taps<BW>(p.g, wt, taps, p.C, blockIdx.x / (unsigned)parts, (int)(blockIdx.x % (unsigned)parts), parts);
+        }
     } else {
-        nchw_to_nhwc_tile(x, xt, C, HW, (int)(blockIdx.x - n_rec), tiles_hw, tiles_c);
-    }
-}
-
-// the image alone (weights come from somewhere else)
-__global__ void __launch_bounds__(PREP_THREADS) nchw_to_nhwc_kernel(const unsigned short *x, unsigned short *xt, int C,
-                                                                    int HW, int tiles_hw, int tiles_c) {
-    nchw_to_nhwc_tile(x, xt, C, HW, (int)blockIdx.x, tiles_hw, tiles_c);
-}
-
-// a plain dense weight matrix [rows][ldw] in [c][tap] column order -> [n_pad][c * taps] tap-major
-// (rows beyond `rows` are written as zeros)
-__global__ void __launch_bounds__(256) permute_taps_kernel(const unsigned short *Wd, long long ldw, long long rows,
-                                                           long long n_pad, int taps, int C, unsigned short *out) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long long K = (long long)taps * C, total = n_pad * K;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const long long row = i / K, kk = i - row * K;
-        const int tap = (int)(kk / C), c = (int)(kk - (long long)tap * C);
-        out[i] = row < rows ? Wd[row * ldw + (long long)c * taps + tap] : (unsigned short)0;
+        image_to_line(p, x, xt, (long long)(blockIdx.x - n_w) * (PREP_THREADS / 32) + (threadIdx.x >> 5));
     }
 }
 
 // ------------------------------------------------------------------------------------------
 // the tensor-core kernel
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(C_THREADS, 1)
-mwu_conv_taps_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
-                     const ConvParams p) {
+__global__ void __launch_bounds__(L_THREADS, 1)
+mwu_conv_line_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
+                     const __grid_constant__ ConvParams p) {
     if (!p.g.all_live) MWU_CHECK_HEADER(p.g);
     extern __shared__ unsigned char smem_raw[];
-    unsigned char *base = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    unsigned char *sA = base;
-    unsigned char *sB = base + C_STAGES * C_A_BYTES;
-    ConvSmem *sm = reinterpret_cast<ConvSmem *>(sB + C_STAGES * C_B_BYTES);
+    unsigned char *sA = smem_raw + smem_pad_1024(smem_raw);
+    const unsigned a_bytes = (unsigned)p.a_rows * 128u;
+    unsigned char *sB = sA + (size_t)p.a_bufs * a_bytes;
+    __shared__ ConvSmem sm_;
+    ConvSmem *sm = &sm_;
     volatile int *abort = &sm->abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int chunks = p.C / BK;                            // 64-channel chunks
-    const int n_ks = p.KH * p.KW * chunks;                  // k stages per tile
-    const long long total_tiles = (long long)p.NIMG * p.tiles_per_img * p.n_ntiles;
+    const int chunks = p.C / BK;                            // of 64 channels
+    const int fetches = p.rows_apart ? p.KH : 1, taps_per = p.KH * p.KW / fetches;
+    const int m_tiles = (int)((p.M + p.tm - 1) / p.tm);
+    const long long total_tiles = (long long)m_tiles * p.n_ntiles;
     const long long limit = p.wait_limit;
+    const int halves = p.tm / 128;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < C_STAGES; ++s) {
-            mbar_init(smem_u32(&sm->full[s]), 1);
-            mbar_init(smem_u32(&sm->empty[s]), 1);
-        }
         for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&sm->a_full[b]), 1);
+            mbar_init(smem_u32(&sm->a_empty[b]), 1);
             mbar_init(smem_u32(&sm->tfull[b]), 1);
-            mbar_init(smem_u32(&sm->tempty[b]), 4);
+            mbar_init(smem_u32(&sm->tempty[b]), 8);
+        }
+        for (int s = 0; s < L_MAX_STAGES; ++s) {
+            mbar_init(smem_u32(&sm->b_full[s]), 1);
+            mbar_init(smem_u32(&sm->b_empty[s]), 1);
         }
         mbar_init(smem_u32(&sm->drain), 1);
         sm->abort = 0;
+        sm->no_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(smem_u32(&sm->tmem_base), 256);
+    __syncwarp();
+    if (warp == 1) tmem_alloc(smem_u32(&sm->tmem_base), 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     // launched with programmatic stream serialization: the set-up above ran while the kernel that
     // prepares the operands was still finishing; its memory is complete from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned tmem_base = *reinterpret_cast<volatile unsigned *>(&sm->tmem_base);
 
     if (warp == 0) {
-        // ---------------- TMA producer ----------------
-        int stage = 0;
-        unsigned phase = 0;
+        // ---------------- halo rows ----------------
+        unsigned buf = 0, phase = 0, issued = 0, last_phase = 0;
         bool ok = true;
-        long long seq = 0;                                  // stages issued so far
-        unsigned issued = 0, last_phase = 0;                // per slot: a load was issued; parity of its phase
         for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
-            const long long nt = t % p.n_ntiles, mt = t / p.n_ntiles;
-            const int img = (int)(mt / p.tiles_per_img), oh0 = (int)(mt % p.tiles_per_img) * p.R;
-            for (int ks = 0; ks < n_ks; ++ks) {
-                if (!mbar_wait_lim(smem_u32(&sm->empty[stage]), phase ^ 1u, abort, limit)) ok = false;
+            const int p0 = (int)(t / p.n_ntiles) * p.tm;
+            for (int f = 0; ok && f < chunks * fetches; ++f) {
+                const int chunk = f / fetches, di = f - chunk * fetches;
+                if (!mbar_wait_lim(smem_u32(&sm->a_empty[buf]), phase ^ 1u, abort, limit)) ok = false;
                 if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-                if (seq != p.withhold && elect_one()) {
-                    const int tap = ks / chunks, cc = ks - tap * chunks;
-                    const int di = tap / p.KW, dj = tap - di * p.KW;
-                    const unsigned bar = smem_u32(&sm->full[stage]);
-                    mbar_expect_tx(bar, p.a_bytes + C_B_BYTES);
-                    tma_load_4d(smem_u32(sA + stage * C_A_BYTES), &tmap_x, bar, cc * BK, dj - p.pad, oh0 + di - p.pad, img);
-                    tma_load_2d(smem_u32(sB + stage * C_B_BYTES), &tmap_w, bar, ks * BK, (int)(nt * kTileRows));
+                if (elect_one()) {
+                    const unsigned bar = smem_u32(&sm->a_full[buf]);
+                    mbar_expect_tx(bar, a_bytes);
+                    // a box may start before the first pixel or end after the last: zeros there
+                    const int row = p0 - p.shift * (p.Wp + 1) + (p.rows_apart ? di * p.Wp : 0);
+                    for (int b = 0; b * p.box_rows < p.a_rows; ++b)
+                        tma_load_2d(smem_u32(sA + buf * a_bytes + (unsigned)(b * p.box_rows) * 128u), &tmap_x, bar, chunk * BK,
+                                    row + b * p.box_rows);
                 }
                 __syncwarp();
-                if (seq != p.withhold) {
-                    issued |= 1u << stage;
-                    last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
-                }
-                ++seq;
-                if (++stage == C_STAGES) { stage = 0; phase ^= 1u; }
+                issued |= 1u << buf;
+                last_phase = (last_phase & ~(1u << buf)) | (phase << buf);
+                if (++buf == (unsigned)p.a_bufs) { buf = 0; phase ^= 1u; }
             }
         }
-        if (!ok) {
-            // leaving early: the loads already issued must have landed before the CTA goes away.  Their
-            // barriers need nothing but the loads' own bytes, so these waits end (and are bounded anyway).
-            __shared__ int s_no_abort;
-            if (lane == 0) s_no_abort = 0;
-            __syncwarp();
-            for (int s = 0; s < C_STAGES; ++s)
-                if ((issued >> s) & 1u) mbar_wait_lim(smem_u32(&sm->full[s]), (last_phase >> s) & 1u, &s_no_abort, limit);
+        // leaving early: the loads already issued must have landed before the CTA goes away.  Their
+        // barriers need nothing but the loads' own bytes, so these waits end (and are bounded anyway).
+        if (!ok)
+            for (int b = 0; b < 2; ++b)
+                if ((issued >> b) & 1u) mbar_wait_lim(smem_u32(&sm->a_full[b]), (last_phase >> b) & 1u, &sm->no_abort, limit);
+        __syncwarp();
+    } else if (warp == L_B_WARP) {
+        // ---------------- weights ----------------
+        unsigned stage = 0, phase = 0, issued = 0, last_phase = 0;
+        long long seq = 0;                                  // boxes so far
+        bool ok = true;
+        for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
+            const int nt = (int)(t % p.n_ntiles);
+            for (int f = 0; ok && f < chunks * fetches; ++f) {
+                const int chunk = f / fetches, tap0 = (f - chunk * fetches) * taps_per;
+                for (int q = 0; q < taps_per; ++q) {
+                    if (!mbar_wait_lim(smem_u32(&sm->b_empty[stage]), phase ^ 1u, abort, limit)) ok = false;
+                    if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+                    if (seq != p.withhold) {
+                        if (elect_one()) {
+                            const unsigned bar = smem_u32(&sm->b_full[stage]);
+                            mbar_expect_tx(bar, REC_BYTES);
+                            tma_load_2d(smem_u32(sB + stage * REC_BYTES), &tmap_w, bar, (tap0 + q) * p.C + chunk * BK, nt * kTileRows);
+                        }
+                        issued |= 1u << stage;
+                        last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
+                    }
+                    __syncwarp();
+                    ++seq;
+                    if (++stage == (unsigned)p.b_stages) { stage = 0; phase ^= 1u; }
+                }
+            }
         }
+        if (!ok)
+            for (int s = 0; s < p.b_stages; ++s)
+                if ((issued >> s) & 1u) mbar_wait_lim(smem_u32(&sm->b_full[s]), (last_phase >> s) & 1u, &sm->no_abort, limit);
+        __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        int stage = 0;
-        unsigned phase = 0;
+        unsigned buf = 0, a_phase = 0, stage = 0, b_phase = 0;
         bool ok = true, issued_any = false;
         const unsigned idesc = make_idesc(128);
         long long k = 0;
         for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x, ++k) {
-            const unsigned buf = (unsigned)(k & 1), use_phase = (unsigned)((k >> 1) & 1);
-            if (!mbar_wait_lim(smem_u32(&sm->tempty[buf]), use_phase ^ 1u, abort, limit)) ok = false;
+            const unsigned acc = (unsigned)(k & 1), use_phase = (unsigned)((k >> 1) & 1);
+            if (!mbar_wait_lim(smem_u32(&sm->tempty[acc]), use_phase ^ 1u, abort, limit)) ok = false;
             if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
             tc_fence_after();
-            for (int ks = 0; ks < n_ks; ++ks) {
-                if (!mbar_wait_lim(smem_u32(&sm->full[stage]), phase, abort, limit)) ok = false;
+            const unsigned d = tmem_base + acc * 256u;
+            for (int f = 0; ok && f < chunks * fetches; ++f) {
+                if (!mbar_wait_lim(smem_u32(&sm->a_full[buf]), a_phase, abort, limit)) ok = false;
                 if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-                tc_fence_after();
-                const unsigned long long adesc = make_desc(smem_u32(sA + stage * C_A_BYTES));
-                const unsigned long long bdesc = make_desc(smem_u32(sB + stage * C_B_BYTES));
-                if (elect_one()) {
+                const unsigned a_s = smem_u32(sA + buf * a_bytes);
+                int i = 0, j = 0;
+                for (int q = 0; q < taps_per; ++q) {
+                    if (!mbar_wait_lim(smem_u32(&sm->b_full[stage]), b_phase, abort, limit)) ok = false;
+                    if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+                    tc_fence_after();
+                    const unsigned long long bdesc = make_desc(smem_u32(sB + stage * REC_BYTES));
+                    const unsigned long long adesc = make_desc(a_s + (unsigned)(i * p.Wp + j) * 128u);
+                    if (elect_one()) {
+                        for (int h = 0; h < halves; ++h)
 #pragma unroll
-                    for (int k4 = 0; k4 < 4; ++k4)
-                        umma_bf16(tmem_base + buf * 128u, adesc + (unsigned long long)(k4 * 2),
-                                  bdesc + (unsigned long long)(k4 * 2), idesc, (ks | k4) ? 1u : 0u);
-                    umma_commit(smem_u32(&sm->empty[stage]));
+                            for (int k4 = 0; k4 < 4; ++k4)
+                                umma_bf16(d + (unsigned)h * 128u, adesc + (unsigned long long)(h * (128 * 128 >> 4) + k4 * 2),
+                                          bdesc + (unsigned long long)(k4 * 2), idesc, (f | q | k4) ? 1u : 0u);
+                        umma_commit(smem_u32(&sm->b_empty[stage]));
+                    }
+                    issued_any = true;
+                    __syncwarp();
+                    if (++j == p.KW) { j = 0; ++i; }
+                    if (++stage == (unsigned)p.b_stages) { stage = 0; b_phase ^= 1u; }
                 }
-                issued_any = true;
+                if (!ok) break;
+                if (elect_one()) umma_commit(smem_u32(&sm->a_empty[buf]));
                 __syncwarp();
-                if (++stage == C_STAGES) { stage = 0; phase ^= 1u; }
+                if (++buf == (unsigned)p.a_bufs) { buf = 0; a_phase ^= 1u; }
             }
             if (!ok) break;
-            if (elect_one()) umma_commit(smem_u32(&sm->tfull[buf]));
+            if (elect_one()) umma_commit(smem_u32(&sm->tfull[acc]));
             __syncwarp();
         }
         // everything this warp issued must have retired before tensor memory is freed
-        if (lane == 0 && issued_any) {
-            __shared__ int s_no_abort2;
-            s_no_abort2 = 0;
-            umma_commit(smem_u32(&sm->drain));
-            mbar_wait_lim(smem_u32(&sm->drain), 0, &s_no_abort2, limit);
+        if (issued_any) {
+            if (elect_one()) umma_commit(smem_u32(&sm->drain));
+            __syncwarp();
+            mbar_wait_lim(smem_u32(&sm->drain), 0, &sm->no_abort, limit);
         }
         __syncwarp();
     } else {
-        // ---------------- epilogue: TMEM lanes are pixels, columns are filters ----------------
-        const int quarter = warp & 3;
-        const int m = quarter * 32 + lane;                  // pixel of the tile
+        // ---------------- output: tensor-memory lanes are pixels, columns are filters ----------------
+        const int quarter = warp & 3, second = (warp - 2) >> 2;
+        // two warps to a quarter: a half of the pixels each, or of the filters
+        const int half = halves == 2 ? second : 0, c_from = halves == 2 ? 0 : second * 64, c_to = halves == 2 ? 128 : c_from + 64;
         bool ok = true;
         long long k = 0;
         const long long plane = (long long)p.OH * p.OW;
         for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x, ++k) {
-            const long long nt = t % p.n_ntiles, mt = t / p.n_ntiles;
-            const long long img = mt / p.tiles_per_img;
-            const int oh0 = (int)(mt % p.tiles_per_img) * p.R;
-            const unsigned buf = (unsigned)(k & 1), use_phase = (unsigned)((k >> 1) & 1);
-            if (!mbar_wait_lim(smem_u32(&sm->tfull[buf]), use_phase, abort, limit)) ok = false;
+            const long long nt = t % p.n_ntiles, P = (t / p.n_ntiles) * p.tm + half * 128 + quarter * 32 + lane;
+            const unsigned acc = (unsigned)(k & 1), use_phase = (unsigned)((k >> 1) & 1);
+            int img = 0, oh = 0, ow = 0;
+            bool px = P < p.M;
+            if (px) {
+                line_pixel(p, (unsigned)P, &img, &oh, &ow);
+                px = oh < p.OH && ow < p.OW;                // the others are zero pixels
+            }
+            if (!mbar_wait_lim(smem_u32(&sm->tfull[acc]), use_phase, abort, limit)) ok = false;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            const int rows_here = (p.OH - oh0) < p.R ? (p.OH - oh0) : p.R;
-            const bool px_ok = m < rows_here * p.OW;
-            const unsigned trow = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * 128u;
-            const long long pix = (long long)oh0 * p.OW + m;
+            const unsigned trow = tmem_base + ((unsigned)(quarter * 32) << 16) + acc * 256u + (unsigned)half * 128u;
 #pragma unroll 1
-            for (int c0 = 0; c0 < 128; c0 += 32) {
+            for (int c0 = c_from; c0 < c_to; c0 += 32) {
                 const long long o0 = nt * kTileRows + c0;
                 if (o0 >= p.g.N) break;
                 unsigned v[32];
                 tmem_ld32(trow + (unsigned)c0, v);
-                if (px_ok) {
+                const long long at = (img * p.g.N + o0) * plane + (long long)oh * p.OW + ow;
+                if (px) {
                     if (p.g.y_fp32) {
-                        float *dst = reinterpret_cast<float *>(p.g.Y) + (img * p.g.N + o0) * plane + pix;
+                        float *dst = reinterpret_cast<float *>(p.g.Y) + at;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (o0 + j < p.g.N) dst[j * plane] = __uint_as_float(v[j]);
+                        for (int j = 0; j < 32; ++j, dst += plane)
+                            if (o0 + j < p.g.N) *dst = __uint_as_float(v[j]);
                     } else {
-                        __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(p.g.Y) + (img * p.g.N + o0) * plane + pix;
+                        __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(p.g.Y) + at;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (o0 + j < p.g.N) dst[j * plane] = __float2bfloat16_rn(__uint_as_float(v[j]));
+                        for (int j = 0; j < 32; ++j, dst += plane)
+                            if (o0 + j < p.g.N) *dst = __float2bfloat16_rn(__uint_as_float(v[j]));
                     }
                 }
+                __syncwarp();
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sm->tempty[buf]));
+            if (lane == 0) mbar_arrive(smem_u32(&sm->tempty[acc]));
         }
     }
 
@@ -359,33 +391,117 @@ mwu_conv_taps_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_co
     if (*abort && threadIdx.x == 0) atomicOr(p.g.dev_status, (unsigned)MWU_DEV_TIMEOUT);
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 256);
+        tmem_dealloc(tmem_base, 512);
     }
 }
 
-static size_t conv_smem_bytes() { return 1024 + (size_t)C_STAGES * (C_A_BYTES + C_B_BYTES) + sizeof(ConvSmem); }
-
-// shape served by the workspace path?  Fills the tile geometry when it is.
-static bool taps_path(const mwu_proj_desc *desc, int n, int c, int h, int w, int kh, int kw, int stride, int pad,
-                      int *OH, int *OW, int *R) {
-    if (validate_desc(desc, true) != MWU_OK) return false;
-    if (n <= 0 || c <= 0 || h <= 0 || w <= 0 || kh <= 0 || kw <= 0 || stride != 1 || pad < 0) return false;
-    if ((int64_t)c * kh * kw != desc->cols || c % BK != 0) return false;
-    if (h + 2 * pad < kh || w + 2 * pad < kw || pad > 32767) return false;
-    const int oh = h + 2 * pad - kh + 1, ow = w + 2 * pad - kw + 1;
-    if (ow > 128 || w > 65535 || h > 65535) return false;
-    int r = 128 / ow;
-    if (r > oh) r = oh;
-    if (r > 256) r = 256;
-    *OH = oh; *OW = ow; *R = r;
-    return true;
-}
-
-static size_t x_bytes_aligned(int n, int c, int h, int w) { return align_up((size_t)n * c * h * w * 2, 1024); }
-
-// testing aid (see mwu.h): limit of the bounded waits and a stage to leave out
+// ------------------------------------------------------------------------------------------
+// host
+// ------------------------------------------------------------------------------------------
+// testing aid (see mwu.h): limit of the bounded waits and a weight box to leave out
 static long long g_wait_limit = WAIT_LIMIT_CYCLES;
 static long long g_withhold = -1;
+
+// shapes this path serves: stride 1, channels in chunks of 64, at most 128 output pixels per row
+static bool line_shape(int n, int c, int h, int w, int kh, int kw, int stride, int pad) {
+    if (n <= 0 || c <= 0 || h <= 0 || w <= 0 || kh <= 0 || kw <= 0 || stride != 1 || pad < 0) return false;
+    if (c % BK != 0 || h + 2 * pad < kh || w + 2 * pad < kw || pad > 32767) return false;
+    return w + 2 * pad - kw + 1 <= 128 && w <= 65535 && h <= 65535;
+}
+
+// The line of pixels.  With pad < kernel a run of `pad` zero pixels after every image row and `pad` such rows after
+// every image serve both neighbours; a wider padding is laid out in full.
+static void line_of(int n, int h, int w, int kh, int kw, int pad, int *Hp, int *Wp, int *shift, long long *M) {
+    const bool shared = pad < kh && pad < kw;
+    *Hp = h + (shared ? pad : 2 * pad);
+    *Wp = w + (shared ? pad : 2 * pad);
+    *shift = shared ? pad : 0;
+    *M = (long long)n * *Hp * *Wp;
+}
+static size_t line_bytes(int n, int c, int h, int w, int kh, int kw, int pad) {
+    int Hp, Wp, shift;
+    long long M;
+    line_of(n, h, w, kh, kw, pad, &Hp, &Wp, &shift, &M);
+    return align_up((size_t)M * c * 2, 1024);
+}
+static size_t conv_workspace(int64_t rows, int n, int c, int h, int w, int kh, int kw, int pad) {
+    const int64_t n_pad = (rows + kTileRows - 1) / kTileRows * kTileRows;
+    return line_bytes(n, c, h, w, kh, kw, pad) + (size_t)n_pad * (size_t)c * kh * kw * 2;
+}
+
+// p.g is filled; bw 0: plain weights Wd
+static int run_line(ConvParams &p, int bw, const void *Wd, long long ldw, const void *X_nchw, int n, int c, int h, int w, int kh,
+                    int kw, int pad, void *workspace, int sm_count, cudaStream_t st) {
+    EncodeTiledFn encode = get_encode_fn();
+    if (!encode) return MWU_ERR_CUDA;
+    p.C = c; p.H = h; p.W = w; p.KH = kh; p.KW = kw; p.pad = pad; p.NIMG = n;
+    p.OH = h + 2 * pad - kh + 1;
+    p.OW = w + 2 * pad - kw + 1;
+    line_of(n, h, w, kh, kw, pad, &p.Hp, &p.Wp, &p.shift, &p.M);
+    if (p.M + 256 >= (1ll << 31)) return MWU_ERR_SHAPE;
+    p.img_magic = (unsigned)((1ull << 32) / ((unsigned)p.Hp * (unsigned)p.Wp)) + 1u;
+    p.row_magic = (unsigned)((1ull << 32) / (unsigned)p.Wp) + 1u;
+    const int64_t n_pad = (p.g.N + kTileRows - 1) / kTileRows * kTileRows;
+    p.n_ntiles = (int)(n_pad / kTileRows);
+    p.wait_limit = g_wait_limit;
+    p.withhold = g_withhold;
+    // Tiles of 256 pixels share a weight box between two accumulators; of 128 where those would leave SMs idle.
+    // All taps from one fetch where two buffers of it fit beside four weight boxes, else a fetch per kernel row.
+    const long long room = L_SMEM - 2048;
+    p.tm = (p.M + 255) / 256 * p.n_ntiles * 10 >= 6ll * sm_count ? 256 : 128;
+    for (p.rows_apart = 0;; p.rows_apart = 1) {
+        const long long rows = p.tm + (p.rows_apart ? 0 : (long long)(kh - 1) * p.Wp) + kw - 1;
+        const long long boxes = (rows + 255) / 256;
+        p.box_rows = (int)(((rows + boxes - 1) / boxes + 7) / 8 * 8);
+        const long long a_rows = boxes * p.box_rows;
+        p.a_bufs = a_rows * 256 + 4 * REC_BYTES <= room ? 2 : 1;
+        const long long left = room - p.a_bufs * a_rows * 128;
+        p.a_rows = (int)a_rows;
+        p.b_stages = left / REC_BYTES > L_MAX_STAGES ? L_MAX_STAGES : (int)(left / REC_BYTES);
+        if (left >= 2 * REC_BYTES) break;
+        if (p.rows_apart) return MWU_ERR_SHAPE;
+    }
+    unsigned short *xt = (unsigned short *)workspace;
+    unsigned short *wt = (unsigned short *)((char *)workspace + line_bytes(n, c, h, w, kh, kw, pad));
+    auto map_2d = [&](CUtensorMap *tm, void *ptr, long long inner, long long outer, int rows) {
+        const cuuint64_t dim[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
+        const cuuint64_t str[1] = {(cuuint64_t)inner * 2};
+        const cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)rows};
+        const cuuint32_t est[2] = {1, 1};
+        return encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, dim, str, box, est, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    CUtensorMap tmap_x, tmap_w;
+    if (!map_2d(&tmap_x, xt, c, p.M, p.box_rows) || !map_2d(&tmap_w, wt, p.g.K, n_pad, kTileRows)) return MWU_ERR_CUDA;
+    // weights: a record to a CTA, or to four that share its rows while the records are few
+    unsigned n_w;
+    int parts = 1;
+    if (bw == 0) {
+        const long long want = (n_pad * p.g.K + 4 * PREP_THREADS - 1) / (4 * PREP_THREADS);
+        n_w = (unsigned)(want < 16ll * sm_count ? want : 16ll * sm_count);
+    } else {
+        const long long n_rec = p.g.n_rec_tiles * p.g.n_stages;
+        while (parts < 4 && n_rec * parts * 2 <= 2ll * sm_count) parts *= 2;
+        if (n_rec * parts >= (1ll << 30)) return MWU_ERR_SHAPE;
+        n_w = (unsigned)(n_rec * parts);
+    }
+    const long long tasks = (p.M + 31) / 32 * (c / 16), img_ctas = (tasks + PREP_THREADS / 32 - 1) / (PREP_THREADS / 32);
+    if (img_ctas >= (1ll << 30)) return MWU_ERR_SHAPE;
+    auto prep = bw == 0 ? conv_prep_kernel<0> : bw == 2 ? conv_prep_kernel<2> : bw == 4 ? conv_prep_kernel<4>
+              : bw == 8 ? conv_prep_kernel<8> : conv_prep_kernel<16>;
+    count_launch(2);
+    if (launch_chained(prep, dim3(n_w + (unsigned)img_ctas), dim3(PREP_THREADS), 0, st, 1, p, (const unsigned short *)Wd, ldw,
+                       (long long)n_pad, wt, n_w, parts, (const unsigned short *)X_nchw, xt) != cudaSuccess)
+        return MWU_ERR_CUDA;
+    const size_t smem = (size_t)p.a_bufs * p.a_rows * 128 + (size_t)p.b_stages * REC_BYTES + 1024;
+    if (cudaFuncSetAttribute(mwu_conv_line_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L_SMEM - 1024) != cudaSuccess)
+        return MWU_ERR_CUDA;
+    const long long tiles = (p.M + p.tm - 1) / p.tm * p.n_ntiles;
+    const int grid = (int)(tiles < sm_count ? tiles : sm_count);
+    return launch_chained(mwu_conv_line_kernel, dim3((unsigned)grid), dim3(L_THREADS), smem, st, 1, tmap_x, tmap_w, p) == cudaSuccess
+               ? MWU_OK : MWU_ERR_CUDA;
+}
 
 }  // namespace gemm
 }  // namespace mwu
@@ -398,83 +514,10 @@ extern "C" void mwu_debug_conv_wait(int64_t limit_cycles, int64_t withhold_stage
 extern "C" size_t mwu_conv_workspace_bytes(const mwu_proj_desc *desc, int32_t n, int32_t c, int32_t h,
                                            int32_t w, int32_t kh, int32_t kw, int32_t stride, int32_t pad) {
     using namespace mwu;
-    int OH, OW, R;
-    if (!gemm::taps_path(desc, n, c, h, w, kh, kw, stride, pad, &OH, &OW, &R)) return 0;
-    const PackedLayout L = packed_layout(desc);
-    return gemm::x_bytes_aligned(n, c, h, w) + (size_t)L.n_pad * (size_t)desc->cols * 2;
+    if (validate_desc(desc, true) != MWU_OK || !gemm::line_shape(n, c, h, w, kh, kw, stride, pad)) return 0;
+    if ((int64_t)c * kh * kw != desc->cols) return 0;
+    return gemm::conv_workspace(desc->rows, n, c, h, w, kh, kw, pad);
 }
-
-namespace mwu {
-namespace gemm {
-
-// shape of the convolution alone (no descriptor): stride 1, channels in chunks of 64, at most 128
-// output pixels per row
-static bool taps_geometry(int n, int c, int h, int w, int kh, int kw, int stride, int pad, int *OH, int *OW, int *R) {
-    if (n <= 0 || c <= 0 || h <= 0 || w <= 0 || kh <= 0 || kw <= 0 || stride != 1 || pad < 0) return false;
-    if (c % BK != 0 || h + 2 * pad < kh || w + 2 * pad < kw || pad > 32767) return false;
-    const int oh = h + 2 * pad - kh + 1, ow = w + 2 * pad - kw + 1;
-    if (ow > 128 || w > 65535 || h > 65535) return false;
-    int r = 128 / ow;
-    if (r > oh) r = oh;
-    if (r > 256) r = 256;
-    *OH = oh; *OW = ow; *R = r;
-    return true;
-}
-
-// tensor maps, the preparation (`prepare` enqueues the image copy and whatever puts the tap-major
-// weights into `wd`) and the tensor-core kernel
-template <typename F>
-static int run_taps(ConvParams &p, const void *X_nchw, int n, int c, int h, int w, int kh, int kw, int pad,
-                    unsigned short *xt, unsigned short *wd, long long n_pad, int sm_count, cudaStream_t st,
-                    F prepare) {
-    EncodeTiledFn encode = get_encode_fn();
-    if (!encode) return MWU_ERR_CUDA;
-    int OH, OW, R;
-    if (!taps_geometry(n, c, h, w, kh, kw, 1, pad, &OH, &OW, &R)) return MWU_ERR_SHAPE;
-    const long long K = (long long)c * kh * kw;
-    p.C = c; p.H = h; p.W = w; p.KH = kh; p.KW = kw; p.pad = pad; p.OH = OH; p.OW = OW; p.NIMG = n;
-    p.R = R;
-    p.tiles_per_img = (OH + R - 1) / R;
-    p.n_ntiles = (int)(n_pad / kTileRows);
-    p.a_bytes = (unsigned)(R * OW * 128);
-    p.wait_limit = g_wait_limit;
-    p.withhold = g_withhold;
-    // tensor maps: the pixel-major image as [n][h][w][c] (innermost first: c, w, h, n), and the weights
-    CUtensorMap tmap_x, tmap_w;
-    {
-        const cuuint64_t gdim[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
-        const cuuint64_t gstr[3] = {(cuuint64_t)c * 2, (cuuint64_t)w * c * 2, (cuuint64_t)h * w * c * 2};
-        const cuuint32_t box[4] = {(cuuint32_t)BK, (cuuint32_t)OW, (cuuint32_t)R, 1};
-        const cuuint32_t estr[4] = {1, 1, 1, 1};
-        if (encode(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, xt, gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return MWU_ERR_CUDA;
-        const cuuint64_t wdim[2] = {(cuuint64_t)K, (cuuint64_t)n_pad};
-        const cuuint64_t wstr[1] = {(cuuint64_t)K * 2};
-        const cuuint32_t wbox[2] = {(cuuint32_t)BK, (cuuint32_t)kTileRows};
-        const cuuint32_t west[2] = {1, 1};
-        if (encode(&tmap_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, wd, wdim, wstr, wbox, west, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return MWU_ERR_CUDA;
-    }
-    const int HW = h * w;
-    const int tiles_hw = (HW + 63) / 64, tiles_c = (c + 63) / 64;
-    prepare((const unsigned short *)X_nchw, xt, HW, tiles_hw, tiles_c, (unsigned)(n * tiles_hw * tiles_c));
-    const size_t smem = conv_smem_bytes();
-    if (cudaFuncSetAttribute(mwu_conv_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return MWU_ERR_CUDA;
-    const long long tiles = (long long)n * p.tiles_per_img * p.n_ntiles;
-    const int grid = (int)(tiles < sm_count ? tiles : sm_count);
-    count_launch();
-    if (launch_chained(mwu_conv_taps_kernel, dim3((unsigned)grid), dim3(C_THREADS), smem, st, 1, tmap_x, tmap_w, p) != cudaSuccess)
-        return MWU_ERR_CUDA;
-    return cudaGetLastError() == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
-}
-
-}  // namespace gemm
-}  // namespace mwu
 
 extern "C" int mwu_conv_implicit_ws(const mwu_proj_desc *desc, const void *packed, const void *X_nchw,
                                     int32_t n, int32_t c, int32_t h, int32_t w, int32_t kh, int32_t kw,
@@ -511,31 +554,14 @@ extern "C" int mwu_conv_implicit_ws(const mwu_proj_desc *desc, const void *packe
     p.g.Y = Y_nchw;
     p.g.y_fp32 = y_dtype;
     p.g.dev_status = dev_status;
-    unsigned short *xt = (unsigned short *)workspace;
-    unsigned short *wd = (unsigned short *)((char *)workspace + x_bytes_aligned(n, c, h, w));
-    const unsigned n_rec = (unsigned)(L.n_tiles * L.n_stages);
-    const int taps = kh * kw, bw = desc->block;
-    const Params g = p.g;
-    return run_taps(p, X_nchw, n, c, h, w, kh, kw, pad, xt, wd, L.n_pad, sm_count, st,
-                    [&](const unsigned short *x, unsigned short *xo, int HW, int tiles_hw, int tiles_c, unsigned n_tiles) {
-        const unsigned grid = n_rec + n_tiles;
-        switch (bw) {
-            case 2: launch_chained(conv_prep_kernel<2>, dim3(grid), dim3(PREP_THREADS), 0, st, 1, g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
-            case 4: launch_chained(conv_prep_kernel<4>, dim3(grid), dim3(PREP_THREADS), 0, st, 1, g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
-            case 8: launch_chained(conv_prep_kernel<8>, dim3(grid), dim3(PREP_THREADS), 0, st, 1, g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
-            default: launch_chained(conv_prep_kernel<16>, dim3(grid), dim3(PREP_THREADS), 0, st, 1, g, wd, taps, c, n_rec, x, xo, HW, tiles_hw, tiles_c); break;
-        }
-        count_launch();
-    });
+    return run_line(p, desc->block, nullptr, 0, X_nchw, n, c, h, w, kh, kw, pad, workspace, sm_count, st);
 }
 
 extern "C" size_t mwu_conv_dense_workspace_bytes(int64_t rows, int32_t n, int32_t c, int32_t h, int32_t w,
                                                  int32_t kh, int32_t kw, int32_t stride, int32_t pad) {
     using namespace mwu;
-    int OH, OW, R;
-    if (rows <= 0 || !gemm::taps_geometry(n, c, h, w, kh, kw, stride, pad, &OH, &OW, &R)) return 0;
-    const int64_t n_pad = (rows + kTileRows - 1) / kTileRows * kTileRows;
-    return gemm::x_bytes_aligned(n, c, h, w) + (size_t)n_pad * (size_t)c * kh * kw * 2;
+    if (rows <= 0 || !gemm::line_shape(n, c, h, w, kh, kw, stride, pad)) return 0;
+    return gemm::conv_workspace(rows, n, c, h, w, kh, kw, pad);
 }
 
 extern "C" int mwu_conv_dense(int64_t rows, const void *Wd, int64_t ldw, const void *X_nchw, int32_t n, int32_t c,
@@ -563,18 +589,5 @@ extern "C" int mwu_conv_dense(int64_t rows, const void *Wd, int64_t ldw, const v
     p.g.Y = Y_nchw;
     p.g.y_fp32 = y_dtype;
     p.g.dev_status = dev_status;
-    const long long n_pad = (rows + kTileRows - 1) / kTileRows * kTileRows;
-    unsigned short *xt = (unsigned short *)workspace;
-    unsigned short *wd = (unsigned short *)((char *)workspace + x_bytes_aligned(n, c, h, w));
-    const int taps = kh * kw;
-    const long long K = p.g.K;
-    return run_taps(p, X_nchw, n, c, h, w, kh, kw, pad, xt, wd, n_pad, sm_count, st,
-                    [&](const unsigned short *x, unsigned short *xo, int HW, int tiles_hw, int tiles_c, unsigned n_tiles) {
-        nchw_to_nhwc_kernel<<<n_tiles, PREP_THREADS, 0, st>>>(x, xo, c, HW, tiles_hw, tiles_c);
-        const long long total = n_pad * K;
-        const long long want = (total + 255) / 256, cap = (long long)sm_count * 16;
-        permute_taps_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>((const unsigned short *)Wd, ldw, rows,
-                                                                                  n_pad, taps, c, wd);
-        count_launch(2);
-    });
+    return run_line(p, 0, Wd, ldw, X_nchw, n, c, h, w, kh, kw, pad, workspace, sm_count, st);
 }

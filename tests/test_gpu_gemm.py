@@ -308,3 +308,31 @@ def test_conv_fused_shapes(filters, cin, h, w, k, stride, pad, n, b):
     x = inputs.normal_activations_bf16((n, cin, h, w), 781 + h)
     Mb = W.numel() // b
     conv_case(W, b, Mb * 6 // 10, Mb * 3 // 10, x, k, k, stride, pad)
+
+
+@pytest.mark.parametrize("filters,cin,h,w,k,pad,n,b", [(128, 64, 17, 120, 11, 5, 1, 8),     # a halo too large for one fetch: a fetch per kernel row
+                                                       (128, 64, 5, 6, 3, 3, 2, 4),         # padding as wide as the kernel
+                                                       (256, 128, 56, 55, 3, 1, 8, 16),     # tiles of 256 pixels
+                                                       (130, 64, 31, 33, 5, 2, 2, 2)])
+def test_conv_line_shapes(filters, cin, h, w, k, pad, n, b):
+    W = inputs.normal_weights(filters, cin * k * k, 0.05, 790 + filters + cin + k + h)
+    x = inputs.normal_activations_bf16((n, cin, h, w), 791 + h)
+    Mb = W.numel() // b
+    if k * k <= 9:
+        conv_case(W, b, Mb * 6 // 10, Mb * 3 // 10, x, k, k, 1, pad, expect_ws=True)
+        return
+    # plain weights: the projection is beside the point here
+    desc, bufs, packed, p = project_and_pack(W, b, Mb * 6 // 10, Mb * 3 // 10)
+    What = O.decoded_weights(p)
+    ref = O.conv2d_direct(x.to(torch.float64).numpy(), What, k, k, 1, pad)
+    ws = torch.empty(B.mwu_conv_dense_workspace_bytes(filters, n, cin, h, w, k, k, 1, pad), dtype=torch.uint8, device="cuda")
+    Wd = torch.from_numpy(What).to(torch.bfloat16).cuda()
+    for call in ("dense", "packed"):
+        Y = torch.full(ref.shape, float("nan"), dtype=torch.float32, device="cuda")
+        if call == "dense":
+            B.mwu_conv_dense(filters, Wd, cin * k * k, x.cuda(), n, cin, h, w, k, k, 1, pad, Y, 1, ws, bufs.dev_status)
+        else:
+            B.mwu_conv_implicit_ws(desc, packed, x.cuda(), n, cin, h, w, k, k, 1, pad, Y, 1, ws, bufs.dev_status)
+        torch.cuda.synchronize()
+        assert int(bufs.dev_status.item()) == 0
+        assert errors(Y.cpu().numpy(), ref)[0] <= 1e-5, call
