@@ -50,11 +50,13 @@ struct ConvSmem {
     int no_abort;
 };
 
+// Bounded wait with this kernel's own limit.  The producers and the MMA issuer poll for a while (a waiter
+// suspended in try_wait wakes a few hundred cycles late, once per 64 x 128 step), the others sleep at once.
+template <bool POLL>
 __device__ __forceinline__ bool mbar_wait_lim(unsigned bar, unsigned parity, volatile int *abort, long long limit) {
-    if (mbar_test(bar, parity)) return true;
 #pragma unroll 1
-    for (int i = 0; i < 128; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
+    for (int i = 0; i < (POLL ? 4096 : 1); ++i)
+        if (mbar_test(bar, parity)) return true;
     const long long t0 = clock64();
 #pragma unroll 1
     while (true) {
@@ -63,7 +65,6 @@ __device__ __forceinline__ bool mbar_wait_lim(unsigned bar, unsigned parity, vol
         if (clock64() - t0 > limit) { *abort = 1; return false; }
     }
 }
-
 
 // n / d for n < 2^31, with m = floor(2^32 / d) + 1: the product's high word is the quotient or one too many
 __device__ __forceinline__ unsigned line_divide(unsigned n, unsigned d, unsigned m, unsigned *rem) {
@@ -216,21 +217,24 @@ mwu_conv_line_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_co
     tc_fence_after();
     // launched with programmatic stream serialization: the set-up above ran while the kernel that
     // prepares the operands was still finishing; its memory is complete from here on
+    // No trigger for the kernel behind: its small CTAs would crowd, eight to an SM, on the SMs that have no tile, and
+    // run there while the others stand idle (384 x 192 x 14 x 14, 5x5, n 16, call after call: 82 us with it, 48 without).
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned tmem_base = *reinterpret_cast<volatile unsigned *>(&sm->tmem_base);
 
+    // The three roles below are one thread each: a step then holds no warp vote or barrier (a quarter of a 128 x 128
+    // step's time), and a wait that runs out leaves no other lane behind.
     if (warp == 0) {
         // ---------------- halo rows ----------------
-        unsigned buf = 0, phase = 0, issued = 0, last_phase = 0;
-        bool ok = true;
-        for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
-            const int p0 = (int)(t / p.n_ntiles) * p.tm;
-            for (int f = 0; ok && f < chunks * fetches; ++f) {
-                const int chunk = f / fetches, di = f - chunk * fetches;
-                if (!mbar_wait_lim(smem_u32(&sm->a_empty[buf]), phase ^ 1u, abort, limit)) ok = false;
-                if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-                if (elect_one()) {
+        if (elect_one()) {
+            unsigned buf = 0, phase = 0, issued = 0, last_phase = 0;
+            bool ok = true;
+            for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
+                const int p0 = (int)(t / p.n_ntiles) * p.tm;
+                for (int f = 0; f < chunks * fetches; ++f) {
+                    const int chunk = f / fetches, di = f - chunk * fetches;
+                    ok = mbar_wait_lim<true>(smem_u32(&sm->a_empty[buf]), phase ^ 1u, abort, limit);
+                    if (!ok) break;
                     const unsigned bar = smem_u32(&sm->a_full[buf]);
                     mbar_expect_tx(bar, a_bytes);
                     // a box may start before the first pixel or end after the last: zeros there
@@ -238,100 +242,97 @@ mwu_conv_line_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_co
                     for (int b = 0; b * p.box_rows < p.a_rows; ++b)
                         tma_load_2d(smem_u32(sA + buf * a_bytes + (unsigned)(b * p.box_rows) * 128u), &tmap_x, bar, chunk * BK,
                                     row + b * p.box_rows);
+                    issued |= 1u << buf;
+                    last_phase = (last_phase & ~(1u << buf)) | (phase << buf);
+                    if (++buf == (unsigned)p.a_bufs) { buf = 0; phase ^= 1u; }
                 }
-                __syncwarp();
-                issued |= 1u << buf;
-                last_phase = (last_phase & ~(1u << buf)) | (phase << buf);
-                if (++buf == (unsigned)p.a_bufs) { buf = 0; phase ^= 1u; }
             }
+            // leaving early: the loads already issued must have landed before the CTA goes away.  Their
+            // barriers need nothing but the loads' own bytes, so these waits end (and are bounded anyway).
+            if (!ok)
+                for (int b = 0; b < 2; ++b)
+                    if ((issued >> b) & 1u) mbar_wait_lim<true>(smem_u32(&sm->a_full[b]), (last_phase >> b) & 1u, &sm->no_abort, limit);
         }
-        // leaving early: the loads already issued must have landed before the CTA goes away.  Their
-        // barriers need nothing but the loads' own bytes, so these waits end (and are bounded anyway).
-        if (!ok)
-            for (int b = 0; b < 2; ++b)
-                if ((issued >> b) & 1u) mbar_wait_lim(smem_u32(&sm->a_full[b]), (last_phase >> b) & 1u, &sm->no_abort, limit);
         __syncwarp();
     } else if (warp == L_B_WARP) {
         // ---------------- weights ----------------
-        unsigned stage = 0, phase = 0, issued = 0, last_phase = 0;
-        long long seq = 0;                                  // boxes so far
-        bool ok = true;
-        for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
-            const int nt = (int)(t % p.n_ntiles);
-            for (int f = 0; ok && f < chunks * fetches; ++f) {
-                const int chunk = f / fetches, tap0 = (f - chunk * fetches) * taps_per;
-                for (int q = 0; q < taps_per; ++q) {
-                    if (!mbar_wait_lim(smem_u32(&sm->b_empty[stage]), phase ^ 1u, abort, limit)) ok = false;
-                    if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-                    if (seq != p.withhold) {
-                        if (elect_one()) {
+        if (elect_one()) {
+            unsigned stage = 0, phase = 0, issued = 0, last_phase = 0;
+            long long seq = 0;                              // boxes so far
+            bool ok = true;
+            for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
+                const int nt = (int)(t % p.n_ntiles);
+                for (int f = 0; ok && f < chunks * fetches; ++f) {
+                    const int chunk = f / fetches, tap0 = (f - chunk * fetches) * taps_per;
+                    for (int q = 0; q < taps_per; ++q) {
+                        ok = mbar_wait_lim<true>(smem_u32(&sm->b_empty[stage]), phase ^ 1u, abort, limit);
+                        if (!ok) break;
+                        if (seq++ != p.withhold) {
                             const unsigned bar = smem_u32(&sm->b_full[stage]);
                             mbar_expect_tx(bar, REC_BYTES);
                             tma_load_2d(smem_u32(sB + stage * REC_BYTES), &tmap_w, bar, (tap0 + q) * p.C + chunk * BK, nt * kTileRows);
+                            issued |= 1u << stage;
+                            last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
                         }
-                        issued |= 1u << stage;
-                        last_phase = (last_phase & ~(1u << stage)) | (phase << stage);
+                        if (++stage == (unsigned)p.b_stages) { stage = 0; phase ^= 1u; }
                     }
-                    __syncwarp();
-                    ++seq;
-                    if (++stage == (unsigned)p.b_stages) { stage = 0; phase ^= 1u; }
                 }
             }
+            if (!ok)
+                for (int s = 0; s < p.b_stages; ++s)
+                    if ((issued >> s) & 1u) mbar_wait_lim<true>(smem_u32(&sm->b_full[s]), (last_phase >> s) & 1u, &sm->no_abort, limit);
         }
-        if (!ok)
-            for (int s = 0; s < p.b_stages; ++s)
-                if ((issued >> s) & 1u) mbar_wait_lim(smem_u32(&sm->b_full[s]), (last_phase >> s) & 1u, &sm->no_abort, limit);
         __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        unsigned buf = 0, a_phase = 0, stage = 0, b_phase = 0;
-        bool ok = true, issued_any = false;
-        const unsigned idesc = make_idesc(128);
-        long long k = 0;
-        for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x, ++k) {
-            const unsigned acc = (unsigned)(k & 1), use_phase = (unsigned)((k >> 1) & 1);
-            if (!mbar_wait_lim(smem_u32(&sm->tempty[acc]), use_phase ^ 1u, abort, limit)) ok = false;
-            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-            tc_fence_after();
-            const unsigned d = tmem_base + acc * 256u;
-            for (int f = 0; ok && f < chunks * fetches; ++f) {
-                if (!mbar_wait_lim(smem_u32(&sm->a_full[buf]), a_phase, abort, limit)) ok = false;
-                if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-                const unsigned a_s = smem_u32(sA + buf * a_bytes);
-                int i = 0, j = 0;
-                for (int q = 0; q < taps_per; ++q) {
-                    if (!mbar_wait_lim(smem_u32(&sm->b_full[stage]), b_phase, abort, limit)) ok = false;
-                    if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-                    tc_fence_after();
-                    const unsigned long long bdesc = make_desc(smem_u32(sB + stage * REC_BYTES));
-                    const unsigned long long adesc = make_desc(a_s + (unsigned)(i * p.Wp + j) * 128u);
-                    if (elect_one()) {
-                        for (int h = 0; h < halves; ++h)
+        if (elect_one()) {
+            unsigned buf = 0, a_phase = 0, stage = 0, b_phase = 0;
+            bool ok = true, issued_any = false;
+            const unsigned idesc = make_idesc(128);
+            long long k = 0;
+            for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x, ++k) {
+                const unsigned acc = (unsigned)(k & 1), use_phase = (unsigned)((k >> 1) & 1);
+                ok = mbar_wait_lim<true>(smem_u32(&sm->tempty[acc]), use_phase ^ 1u, abort, limit);
+                if (!ok) break;
+                tc_fence_after();
+                const unsigned d = tmem_base + acc * 256u;
+                for (int f = 0; f < chunks * fetches; ++f) {
+                    ok = mbar_wait_lim<true>(smem_u32(&sm->a_full[buf]), a_phase, abort, limit);
+                    if (!ok) break;
+                    const unsigned a_s = smem_u32(sA + buf * a_bytes);
+                    int i = 0, j = 0;
+                    for (int q = 0; q < taps_per; ++q) {
+                        ok = mbar_wait_lim<true>(smem_u32(&sm->b_full[stage]), b_phase, abort, limit);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const unsigned long long bdesc = make_desc(smem_u32(sB + stage * REC_BYTES));
+                        const unsigned long long adesc = make_desc(a_s + (unsigned)(i * p.Wp + j) * 128u);
+#pragma unroll
+                        for (int k4 = 0; k4 < 4; ++k4)
+                            umma_bf16(d, adesc + (unsigned long long)(k4 * 2), bdesc + (unsigned long long)(k4 * 2), idesc,
+                                      (f | q | k4) ? 1u : 0u);
+                        if (halves == 2) {
 #pragma unroll
                             for (int k4 = 0; k4 < 4; ++k4)
-                                umma_bf16(d + (unsigned)h * 128u, adesc + (unsigned long long)(h * (128 * 128 >> 4) + k4 * 2),
+                                umma_bf16(d + 128u, adesc + (unsigned long long)((128 * 128 >> 4) + k4 * 2),
                                           bdesc + (unsigned long long)(k4 * 2), idesc, (f | q | k4) ? 1u : 0u);
+                        }
                         umma_commit(smem_u32(&sm->b_empty[stage]));
+                        issued_any = true;
+                        if (++j == p.KW) { j = 0; ++i; }
+                        if (++stage == (unsigned)p.b_stages) { stage = 0; b_phase ^= 1u; }
                     }
-                    issued_any = true;
-                    __syncwarp();
-                    if (++j == p.KW) { j = 0; ++i; }
-                    if (++stage == (unsigned)p.b_stages) { stage = 0; b_phase ^= 1u; }
+                    if (!ok) break;
+                    umma_commit(smem_u32(&sm->a_empty[buf]));
+                    if (++buf == (unsigned)p.a_bufs) { buf = 0; a_phase ^= 1u; }
                 }
-                if (!ok) break;
-                if (elect_one()) umma_commit(smem_u32(&sm->a_empty[buf]));
-                __syncwarp();
-                if (++buf == (unsigned)p.a_bufs) { buf = 0; a_phase ^= 1u; }
+                if (ok) umma_commit(smem_u32(&sm->tfull[acc]));
             }
-            if (!ok) break;
-            if (elect_one()) umma_commit(smem_u32(&sm->tfull[acc]));
-            __syncwarp();
-        }
-        // everything this warp issued must have retired before tensor memory is freed
-        if (issued_any) {
-            if (elect_one()) umma_commit(smem_u32(&sm->drain));
-            __syncwarp();
-            mbar_wait_lim(smem_u32(&sm->drain), 0, &sm->no_abort, limit);
+            // everything issued must have retired before tensor memory is freed
+            if (issued_any) {
+                umma_commit(smem_u32(&sm->drain));
+                mbar_wait_lim<true>(smem_u32(&sm->drain), 0, &sm->no_abort, limit);
+            }
         }
         __syncwarp();
     } else {
@@ -351,7 +352,7 @@ mwu_conv_line_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_co
                 line_pixel(p, (unsigned)P, &img, &oh, &ow);
                 px = oh < p.OH && ow < p.OW;                // the others are zero pixels
             }
-            if (!mbar_wait_lim(smem_u32(&sm->tfull[acc]), use_phase, abort, limit)) ok = false;
+            if (!mbar_wait_lim<false>(smem_u32(&sm->tfull[acc]), use_phase, abort, limit)) ok = false;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
