@@ -10,7 +10,7 @@
 //
 // One-pass pipeline (MWU_ALGO_ONE_PASS; the default for larger tensors):
 //   sample_keys_kernel, sample_kernel
-//                   rank the keys of <= 4096 evenly spaced blocks; for each selection (prune key, L_u
+//                   rank the keys of <= 65536 evenly spaced blocks; for each selection (prune key, L_u
 //                   of the survivors) the sample quantile is a provisional threshold and the sample
 //                   keys 4 sigma of rank to either side a window.
 //   pass_kernel     streams W (+U) once, evaluates the fp64 keys of every block and writes every
@@ -33,12 +33,14 @@ namespace mwu {
 namespace proj {
 
 constexpr int NB_MAX = 65536;   // level-0 bins (codes fit 16 bits): bin 0 = below the window, nb-1 = above it
-constexpr int NB_SMALL = 8192;  // used up to 8M blocks: fewer bins to clear and scan
+constexpr int NB_SMALL = 8192;  // used up to NB_SMALL_BLOCKS blocks: fewer bins to clear and scan
+constexpr long long NB_SMALL_BLOCKS = 1ll << 27;    // about 1.4 % of them in a window: at most 450 to a bin
 constexpr int CAP = 2048;       // candidates sorted by the last step
-constexpr int NSAMP = 4096;        // sample blocks ranked by sample_kernel
-constexpr int SAMP_THREADS = 1024;
-constexpr int SAMP_PER = NSAMP / SAMP_THREADS;
-static_assert(SAMP_PER == 4, "sample_select ranks one level-A key with the four threads that hold 16 samples");
+// sample blocks ranked by sample_kernel: at most NSAMP_MAX, SAMP_PER to a thread
+constexpr int SAMP_CTAS = 8, SAMP_THREADS = 1024, SAMP_PER = 8;
+constexpr int NSAMP_MAX = SAMP_CTAS * SAMP_THREADS * SAMP_PER;
+constexpr int NSAMP_SMALL_LG = 14, NSAMP_LG = 16;
+static_assert(NSAMP_MAX == 1 << NSAMP_LG, "the larger sample fills the cluster");
 constexpr int STAGE_ENTRIES = 64;  // per-warp staging of candidate-list entries in pass_kernel
 constexpr int FIN_THREADS = 1024;   // block size of the kernels whose last CTA finalises
 static_assert(NB_MAX / FIN_THREADS <= 64, "scan_hist searches one thread's bins with one warp, two per lane");
@@ -96,7 +98,8 @@ struct Params {
     u64 *cand_key;              // [CAP]
     unsigned *cand_idx;         // [2 * CAP]
     unsigned *cand_aux;         // [2 * CAP] what resolve_kernel wants to know about a candidate besides its key
-    u64 *samp_kp, *samp_ku;     // [NSAMP] each: keys of the sample blocks (one-pass pipeline)
+    float2 *samp;               // [n_samp] prune key and L_u of the sample blocks (one-pass pipeline; in the list's memory)
+    int n_samp, samp_lg;        // their number; its logarithm, or -1: every block is a sample
     unsigned *dev_status;
 };
 
@@ -263,18 +266,8 @@ __device__ __forceinline__ unsigned block_scan_incl(unsigned x, unsigned *s_warp
     }
     if (lane == 31) s_warp[w] = x;
     __syncthreads();
-    if (w == 0) {
-        unsigned t = s_warp[lane];
-        for (int m = 1; m < 32; m <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, t, m);
-            if (lane >= m) t += y;
-        }
-        s_warp[lane] = t;
-    }
-    __syncthreads();
-    const unsigned add = w ? s_warp[w - 1] : 0u;
-    __syncthreads();
-    return x + add;
+    const unsigned t = lane < w ? s_warp[lane] : 0u;
+    return x + __reduce_add_sync(0xffffffffu, t);
 }
 
 // Window around the `frac` quantile of n sample keys: +-4 sigma (binomial) in rank.  Returns the
@@ -290,36 +283,35 @@ __device__ __forceinline__ void window_ranks_f(int n, float frac, int *il, int *
     *il = a; *ih = b; *ipos = c;
 }
 
-// One selection of sample_kernel.  key[t] / valid[t]: this thread's sample keys; `frac` of the
-// valid ones are to be selected.  Level A ranks a 1-in-16 subsample (<= 256 keys) to get a coarse
-// window; level B counts all valid samples in SAMP_THREADS bins across that window and reads the
-// final window [lo, hi) and the provisional threshold from the bin edges.
-__device__ void sample_select(const u64 (&key)[SAMP_PER], const bool (&valid)[SAMP_PER], float frac,
-                              u64 *lo_out, u64 *hi_out, u64 *t_out) {
-    constexpr int NA = NSAMP / 16;
+// Level-B counts of one selection; the cluster adds its eight up
+struct SampCounts {
+    unsigned bins[SAMP_THREADS];
+    unsigned under, n_valid;
+};
+
+// One selection of sample_kernel, by all CTAs of the cluster alike.  key[t] / valid[t]: this thread's
+// sample keys (bits of non-negative floats); a_key / a_valid: the level-A key that this thread and its
+// three neighbours rank.  `frac` of the valid ones are to be selected.  Level A ranks 256 of the sample
+// keys to get a coarse window; level B counts all valid ones in SAMP_THREADS bins across that window and
+// reads the final window [lo, hi) and the provisional threshold from the bin edges.  c: cleared before a
+// cluster barrier.
+__device__ void sample_select(const unsigned (&key)[SAMP_PER], const unsigned (&valid)[SAMP_PER], unsigned a_key, bool a_valid,
+                              float frac, SampCounts *c, unsigned *lo_out, unsigned *hi_out, unsigned *t_out) {
+    constexpr int NA = SAMP_THREADS / 4;
     // level-A keys, shortened to the top 24 bits below the (clear) sign bit, with the key's index in
     // the low byte: distinct words, one 32-bit compare per pair; invalid keys rank last
     __shared__ __align__(16) unsigned s_a[NA];
     __shared__ unsigned s_edge[2];                    // shortened keys at the coarse window's ranks
-    __shared__ unsigned s_hist[SAMP_THREADS + 2];     // [0] under, [1 .. SAMP_THREADS] window, [+1] over
     __shared__ unsigned s_warp[32];
-    __shared__ unsigned s_nvalid;
-    __shared__ u64 s_res[3];
+    __shared__ unsigned s_res[3];
     static_assert(NA == 256, "the index of a level-A key fills the low byte of its shortened form");
-    const int tid = threadIdx.x;
-    if (tid == 0) s_nvalid = 0;
-    for (int i = tid; i < SAMP_THREADS + 2; i += SAMP_THREADS) s_hist[i] = 0;
-    // level A: sample index 16 * a is slot 0 of thread 4 * a
+    const int tid = threadIdx.x, lane = tid & 31;
     const bool is_a = (tid % 4) == 0;
     const int a = tid / 4;
-    const bool a_valid = is_a && valid[0];
-    if (is_a) s_a[a] = a_valid ? ((unsigned)(key[0] >> 39) << 8) | (unsigned)a : 0xffffffffu;
-    int nv = 0;
-#pragma unroll
-    for (int t = 0; t < SAMP_PER; ++t) nv += valid[t] ? 1 : 0;
-    for (int m = 16; m > 0; m >>= 1) nv += __shfl_xor_sync(0xffffffffu, nv, m);
-    const int na_raw = __syncthreads_count(a_valid);           // also orders the stores above
-    if ((tid & 31) == 0 && nv) atomicAdd(&s_nvalid, (unsigned)nv);
+    a_valid = a_valid && is_a;
+    __syncthreads();                                  // an earlier call's shared words are no longer read
+    if (is_a) s_a[a] = a_valid ? ((a_key >> 7) << 8) | (unsigned)a : 0xffffffffu;
+    const int na_raw = __syncthreads_count(a_valid);  // also orders the stores above
     const int na = na_raw > 0 ? na_raw : 1;
     int il, ih, ipos;
     window_ranks_f(na, frac, &il, &ih, &ipos);
@@ -343,40 +335,47 @@ __device__ void sample_select(const u64 (&key)[SAMP_PER], const bool (&valid)[SA
         }
     }
     __syncthreads();
-    const int n_valid = (int)s_nvalid > 0 ? (int)s_nvalid : 1;
-    // back to full keys: the low 39 bits of the edges are zero (any window is a valid window)
-    u64 clo = (u64)(s_edge[0] >> 8) << 39;
-    u64 chi = (u64)(s_edge[1] >> 8) << 39;
-    if (s_edge[0] == 0xffffffffu) clo = ~0ull >> 1;
-    if (s_edge[1] == 0xffffffffu) chi = ~0ull >> 1;
+    // back to full keys: the low 7 bits of the edges are zero (any window is a valid window)
+    unsigned clo = (s_edge[0] >> 8) << 7, chi = (s_edge[1] >> 8) << 7;
+    if (s_edge[0] == 0xffffffffu) clo = 0x7fffffffu;
+    if (s_edge[1] == 0xffffffffu) chi = 0x7fffffffu;
     if (chi < clo) chi = clo;
     // smallest shift with ((chi - clo) >> shift) < SAMP_THREADS (a power of two)
-    const int width = 64 - __clzll((long long)(chi - clo));            // bits of chi - clo
+    const int width = 32 - __clz((int)(chi - clo));                    // bits of chi - clo
     const unsigned shift = width > 10 ? (unsigned)(width - 10) : 0u;
     static_assert(SAMP_THREADS == 1024, "ten bits of bin index");
     // level B
-    unsigned n_under = 0, n_over = 0;                 // the two catch-all counts stay in registers
+    unsigned n_under = 0, n_valid = 0;
 #pragma unroll
     for (int t = 0; t < SAMP_PER; ++t) {
         if (!valid[t]) continue;
-        const u64 k = key[t];
+        ++n_valid;
+        const unsigned k = key[t];
         if (k < clo) ++n_under;
-        else if (k >= chi) ++n_over;
-        else atomicAdd(&s_hist[1u + (unsigned)((k - clo) >> shift)], 1u);
+        else if (k < chi) atomicAdd(&c->bins[(k - clo) >> shift], 1u);
     }
-    for (int m = 16; m > 0; m >>= 1) {
-        n_under += __shfl_xor_sync(0xffffffffu, n_under, m);
-        n_over += __shfl_xor_sync(0xffffffffu, n_over, m);
+    n_under = __reduce_add_sync(0xffffffffu, n_under);
+    n_valid = __reduce_add_sync(0xffffffffu, n_valid);
+    if (lane == 0) {
+        if (n_under) atomicAdd(&c->under, n_under);
+        if (n_valid) atomicAdd(&c->n_valid, n_valid);
     }
-    if ((tid & 31) == 0) {
-        if (n_under) atomicAdd(&s_hist[0], n_under);
-        if (n_over) atomicAdd(&s_hist[SAMP_THREADS + 1], n_over);
+    sel::ClusterTeam::arrive();
+    sel::ClusterTeam::wait();
+    unsigned mine = 0, under = 0, total = 0;
+#pragma unroll
+    for (unsigned r = 0; r < SAMP_CTAS; ++r) {
+        unsigned x, y, z;
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x) : "r"(sel::ClusterTeam::in_cta(sel::ClusterTeam::addr(&c->bins[tid]), r)) : "memory");
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(y) : "r"(sel::ClusterTeam::in_cta(sel::ClusterTeam::addr(&c->under), r)) : "memory");
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(z) : "r"(sel::ClusterTeam::in_cta(sel::ClusterTeam::addr(&c->n_valid), r)) : "memory");
+        mine += x;
+        under += y;
+        total += z;
     }
-    __syncthreads();
-    const unsigned mine = s_hist[1 + tid];
-    const unsigned incl = block_scan_incl(mine, s_warp) + s_hist[0];
+    const unsigned incl = block_scan_incl(mine, s_warp) + under;
     const unsigned excl = incl - mine;
-    window_ranks_f(n_valid, frac, &il, &ih, &ipos);
+    window_ranks_f(total > 0u ? (int)total : 1, frac, &il, &ih, &ipos);
     if (tid == 0) {
         // ranks outside the coarse window keep its edge
         s_res[0] = clo;
@@ -384,8 +383,8 @@ __device__ void sample_select(const u64 (&key)[SAMP_PER], const bool (&valid)[SA
         s_res[2] = clo;
     }
     __syncthreads();
-    const u64 edge_lo = clo + ((u64)tid << shift);
-    u64 edge_hi = clo + ((u64)(tid + 1) << shift);
+    const unsigned edge_lo = clo + ((unsigned)tid << shift);
+    unsigned edge_hi = clo + ((unsigned)(tid + 1) << shift);
     if (edge_hi > chi) edge_hi = chi;
     if (mine) {
         if (excl <= (unsigned)il && (unsigned)il < incl) s_res[0] = edge_lo < chi ? edge_lo : chi;
@@ -393,121 +392,119 @@ __device__ void sample_select(const u64 (&key)[SAMP_PER], const bool (&valid)[SA
         if (excl <= (unsigned)ipos && (unsigned)ipos < incl) s_res[2] = edge_lo < chi ? edge_lo : chi;
     }
     __syncthreads();
-    u64 lo = s_res[0], hi = s_res[1], That = s_res[2];
+    const unsigned lo = s_res[0], hi = s_res[1];
+    unsigned That = s_res[2];
     if (That < lo) That = lo;
     if (hi > lo && That >= hi) That = hi - 1;         // the provisional threshold lies inside [lo, hi)
     *lo_out = lo;
     *hi_out = hi;
     *t_out = That;
-    __syncthreads();
 }
 
-// block of the i-th of ns evenly spaced samples: i * mb / ns without a division (ns is either
-// NSAMP, a power of two, or mb itself); i < 2^12 and mb < 2^31, so the product fits 64 bits
-__device__ __forceinline__ long long sample_block(int i, long long mb, int ns) {
-    static_assert((NSAMP & (NSAMP - 1)) == 0, "NSAMP is a power of two");
-    return ns == NSAMP ? (long long)(((u64)i * (u64)mb) / (u64)NSAMP) : (long long)i;
+// block of the i-th of the evenly spaced samples, without a division (their number is a power of
+// two, or that of all blocks); i < 2^16 and n_blocks < 2^31, so the product fits 64 bits
+__device__ __forceinline__ long long sample_block(const Params &p, int i) {
+    return p.samp_lg >= 0 ? (long long)(((u64)i * (u64)p.n_blocks) >> p.samp_lg) : (long long)i;
 }
 
-// sample_keys_kernel: approximate keys of the NSAMP evenly spaced sample blocks, one block per
-// thread, spread over many SMs (4096 scattered 64-byte reads issued by a single SM take about
-// 9 us; over 32 SMs they take one memory round trip).  The same launch clears the histograms.
+// sample_keys_kernel: approximate keys of the evenly spaced sample blocks, one block per thread,
+// spread over the SMs: scattered 64-byte reads take one memory round trip (4096 of them issued by a
+// single SM take about 9 us).  The same launch clears the histograms.
 template <int B>
 __global__ void __launch_bounds__(128) sample_keys_kernel(Params p, unsigned *zero_base, unsigned n_zero) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const long long mb = p.n_blocks;
-    const int ns = (int)(mb < (long long)NSAMP ? mb : (long long)NSAMP);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < NSAMP) {
-        u64 kp = ~0ull, ku = ~0ull;
-        unsigned in_group = 0;
-        if (i < ns) {
-            const long long j = sample_block(i, mb, ns);
-            float fp, fu;
-            block_keys_sample<B>(p.W, p.U, j, p.use_l1, &fp, &fu);
-            kp = key_bits((double)fp);
-            ku = key_bits((double)fu);
-            if (p.gprune) in_group = group_pruned(p, (unsigned)j) ? 1u : 0u;
-        }
-        p.samp_kp[i] = kp;
-        p.samp_ku[i] = ku | ((u64)in_group << 63);       // keys are non-negative doubles: bit 63 is free
+    if (i < p.n_samp) {
+        const long long j = sample_block(p, i);
+        float kp, ku;
+        block_keys_sample<B>(p.W, p.U, j, p.use_l1, &kp, &ku);
+        // keys are not negative: the sign bit of L_u tells that the block lies in a pruned group
+        if (p.gprune && group_pruned(p, (unsigned)j)) ku = __uint_as_float(__float_as_uint(ku) | 0x80000000u);
+        p.samp[i] = make_float2(kp, ku);
     }
     uint4 *z = reinterpret_cast<uint4 *>(zero_base);
     for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < n_zero / 4; q += gridDim.x * blockDim.x)
         z[q] = make_uint4(0, 0, 0, 0);
 }
 
-// Run by one whole CTA of SAMP_THREADS threads: windows and provisional thresholds of the two
-// selections from the keys sample_keys_kernel computed, written into p.work.
-__device__ void sample_body(const Params &p) {
+// Second kernel of the one-pass pipeline (one cluster): clears the selection state and chooses windows
+// and provisional thresholds of the two selections from the sample keys.  Launched with programmatic stream
+// serialization behind sample_keys_kernel, and itself lets pass_kernel's CTAs start early.
+//
+// Why a cluster: a window is +-4 sigma of rank, so the share of blocks that pass_kernel has to list, and
+// resolve_kernel to go through, falls with the root of the sample's size.  With 4096 samples (one CTA) 11 % of the
+// blocks of a 50 % / 25 % projection were listed, with 65536 it is 3 %.
+__global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
+    __shared__ SampCounts s_counts[2];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (blockIdx.x == 0) {
+        unsigned *w = reinterpret_cast<unsigned *>(p.work);
+        for (unsigned i = threadIdx.x; i < sizeof(Work) / 4; i += blockDim.x) w[i] = 0u;
+    }
+    unsigned *zc = reinterpret_cast<unsigned *>(s_counts);
+    for (unsigned i = threadIdx.x; i < sizeof(s_counts) / 4; i += blockDim.x) zc[i] = 0u;
+    asm volatile("griddepcontrol.wait;" ::: "memory");     // the sample keys are complete and visible
+    __syncthreads();
     const long long k_unify = p.k_unify, k_prune = p.k_prune;
     const long long mb = p.n_blocks;
     const bool by_group = p.gprune != nullptr;
-    const int ns = (int)(mb < (long long)NSAMP ? mb : (long long)NSAMP);
-    u64 kp[SAMP_PER], ku[SAMP_PER];
-    bool valid[SAMP_PER], in_group[SAMP_PER];
+    const int ns = p.n_samp;
+    constexpr unsigned SIGN = 0x80000000u;
+    unsigned kp[SAMP_PER], ku[SAMP_PER], valid[SAMP_PER];
 #pragma unroll
     for (int t = 0; t < SAMP_PER; ++t) {
-        const int i = threadIdx.x * SAMP_PER + t;
-        kp[t] = ~0ull;
-        ku[t] = ~0ull;
-        valid[t] = i < ns;
-        in_group[t] = false;
-        if (i < ns) {
-            kp[t] = p.samp_kp[i];
-            const u64 x = p.samp_ku[i];
-            ku[t] = x & (~0ull >> 1);
-            in_group[t] = (x >> 63) != 0ull;
-        }
+        const int i = (t * SAMP_CTAS + (int)blockIdx.x) * SAMP_THREADS + (int)threadIdx.x;
+        const float2 x = i < ns ? __ldg(&p.samp[i]) : make_float2(0.f, 0.f);
+        kp[t] = __float_as_uint(x.x);
+        ku[t] = __float_as_uint(x.y) & ~SIGN;
+        valid[t] = i < ns && !(by_group && (__float_as_uint(x.y) & SIGN)) ? 1u : 0u;
     }
+    const int a = (int)threadIdx.x / 4;
+    const int ia = p.samp_lg >= 8 ? a << (p.samp_lg - 8) : a;      // 256 of the samples, evenly spaced
+    const float2 xa = ia < ns ? __ldg(&p.samp[ia]) : make_float2(0.f, 0.f);
+    bool a_valid = ia < ns && !(by_group && (__float_as_uint(xa.y) & SIGN));
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     Sel *sp = &p.work->sel[0];
     Sel *su = &p.work->sel[1];
     const long long ksel_u = k_unify - k_prune;
-    u64 lo, hi, That = 0;
-    if (threadIdx.x == 0 && p.resid) *p.resid = 0.0;  // the kernels that follow add to it
+    unsigned lo, hi, That = 0;
+    auto key64 = [](unsigned x) { return key_bits((double)__uint_as_float(x < 0x7f800000u ? x : 0x7f800000u)); };
+    if (lead && p.resid) *p.resid = 0.0;              // the kernels that follow add to it
+    sel::ClusterTeam::arrive();                       // every CTA's counts are cleared
+    sel::ClusterTeam::wait();
     if (by_group) {
         // the prune classes are known (bit of the block's group): nothing to estimate
-        if (threadIdx.x == 0) {
+        if (lead) {
             set_window(sp, 0, 0, p.nb);
             sp->mode = 3u;
             sp->k = (u64)k_prune;
             p.work->That[0] = 0;
         }
-#pragma unroll
-        for (int t = 0; t < SAMP_PER; ++t) valid[t] = valid[t] && !in_group[t];
     } else {
-        sample_select(kp, valid, (float)((double)k_prune / (double)mb), &lo, &hi, &That);
-        if (threadIdx.x == 0) {
-            set_window(sp, lo, hi, p.nb);
+        sample_select(kp, valid, __float_as_uint(xa.x), a_valid, (float)((double)k_prune / (double)mb), &s_counts[0], &lo, &hi, &That);
+        if (lead) {
+            set_window(sp, key64(lo), key64(hi), p.nb);
             sp->mode = (k_prune == 0) ? 1u : (k_prune == mb ? 2u : 0u);
             sp->k = (u64)k_prune;
-            p.work->That[0] = That;
+            p.work->That[0] = key64(That);
         }
         // the sample blocks that survive the (estimated) prune threshold
 #pragma unroll
-        for (int t = 0; t < SAMP_PER; ++t) valid[t] = valid[t] && (k_prune == 0 || kp[t] > That);
+        for (int t = 0; t < SAMP_PER; ++t) valid[t] = valid[t] && (k_prune == 0 || kp[t] > That) ? 1u : 0u;
+        a_valid = a_valid && (k_prune == 0 || __float_as_uint(xa.x) > That);
     }
     const long long elig = mb - k_prune;
-    sample_select(ku, valid, elig > 0 ? (float)((double)ksel_u / (double)elig) : 0.f, &lo, &hi, &That);
-    if (threadIdx.x == 0) {
-        set_window(su, lo, hi, p.nb);
+    sample_select(ku, valid, __float_as_uint(xa.y) & ~SIGN, a_valid, elig > 0 ? (float)((double)ksel_u / (double)elig) : 0.f,
+                  &s_counts[1], &lo, &hi, &That);
+    if (lead) {
+        set_window(su, key64(lo), key64(hi), p.nb);
         su->mode = (ksel_u == 0) ? 1u : (ksel_u == elig ? 2u : 0u);
         su->k = (u64)ksel_u;
-        p.work->That[1] = That;
+        p.work->That[1] = key64(That);
     }
-}
-
-// Second kernel of the one-pass pipeline (one CTA): clears the selection state and chooses the
-// windows from the sample keys.  Launched with programmatic stream serialization behind
-// sample_keys_kernel, and itself lets pass_kernel's CTAs start early.
-__global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    unsigned *w = reinterpret_cast<unsigned *>(p.work);
-    for (unsigned i = threadIdx.x; i < sizeof(Work) / 4; i += blockDim.x) w[i] = 0u;
-    asm volatile("griddepcontrol.wait;" ::: "memory");     // the sample keys are complete and visible
-    __syncthreads();
-    sample_body(p);
+    sel::ClusterTeam::arrive();                       // nobody leaves while its counts are still read
+    sel::ClusterTeam::wait();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1831,11 +1828,11 @@ static size_t ws_off_cand_key() { return align_up(ws_off_hist() + 2 * proj::NB_M
 // two sets of candidates: the two halves of resolve_kernel each keep their own
 static size_t ws_off_cand_idx() { return align_up(ws_off_cand_key() + 2 * proj::CAP * sizeof(proj::u64)); }
 static size_t ws_off_cand_aux() { return align_up(ws_off_cand_idx() + 2 * proj::CAP * sizeof(unsigned)); }
-static size_t ws_off_samp() { return align_up(ws_off_cand_aux() + 2 * proj::CAP * sizeof(unsigned)); }
-static size_t ws_off_list() { return align_up(ws_off_samp() + 2 * proj::NSAMP * sizeof(proj::u64)); }
+static size_t ws_off_list() { return align_up(ws_off_cand_aux() + 2 * proj::CAP * sizeof(unsigned)); }
 // candidate list of the one-pass pipeline: a quarter of the blocks (the windows hold a few per cent;
 // of a small tensor they may hold more)
-static size_t list_capacity(size_t mb) { return mb / 4 + 65536; }
+// (and before pass_kernel the sample's keys are in its place: the list never has fewer entries than those)
+static size_t list_capacity(size_t mb) { return mb / 4 + proj::NSAMP_MAX; }
 static size_t ws_off_gkey(size_t mb) { return align_up(ws_off_list() + list_capacity(mb) * sizeof(uint2)); }
 static size_t n_groups_of(const mwu_proj_desc *d) {
     return grouped(d) ? (size_t)(d->rows / d->prune_group_rows) * (size_t)(d->cols / d->prune_group_cols) : 0;
@@ -1850,6 +1847,9 @@ static size_t ws_off_gprune(const mwu_proj_desc *d, size_t mb) { return align_up
 // CTA on every SM (606208 on 148) the exact kernel beats the one-pass pipeline's four launches (512 x 1152,
 // b = 8: 24 against 39; 2048 x 2048, b = 8, 524288 blocks: 45 / 52; 1024 x 2048, b = 4: 42 / 46), beyond it
 // does not (1024 x 2048, b = 2, 1048576 blocks: 67 / 54): the phases' L2 counts grow with the blocks.
+// Larger sample from here on, 65536 blocks instead of 16384 (whole mwu_project calls, 50 % / 25 %, us: 4096 x 4096, b = 4, 4 M
+// blocks: 94.7 against 99.3; 16384 x 16384, b = 4: 709 / 805; below, both sizes take the same time).
+constexpr long long SAMP_LARGE_BLOCKS = 1ll << 22;
 constexpr long long EX_CLUSTER_BLOCKS = 32768, EX_AUTO_BLOCKS_PER_CTA = 4096;
 struct Route {
     bool one_pass, cluster;         // else the exact kernel: as one cluster or as a cooperative grid
@@ -1958,13 +1958,13 @@ static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_des
     const bool need_u = ksel_u > 0 && ksel_u < mb - desc->k_prune;
     e = cudaFuncSetAttribute(resolve_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM_BYTES);
     if (e != cudaSuccess) return e;
-    // the sample keys (and the cleared histograms) from 32 SMs, then one CTA ranks the sample; the two
+    // the sample keys (and the cleared histograms) from all SMs, then one cluster ranks the sample; the two
     // kernels behind are launched with programmatic stream serialization, so their CTAs are in place
     // (and the sweep's first loads in flight) when their predecessor ends
     unsigned *zero = reinterpret_cast<unsigned *>(p.xwork);
     const unsigned n_zero = (unsigned)(p.fhist - zero) + 2u * (unsigned)p.nb;
-    e = mwu::launch_chained(sample_keys_kernel<B>, dim3(NSAMP / 128), dim3(128), 0, st, 1, p, zero, n_zero);
-    if (e == cudaSuccess) e = mwu::launch_chained(sample_kernel, dim3(1), dim3(SAMP_THREADS), 0, st, 1, p);
+    e = mwu::launch_chained(sample_keys_kernel<B>, dim3((unsigned)(p.n_samp + 127) / 128), dim3(128), 0, st, 1, p, zero, n_zero);
+    if (e == cudaSuccess) e = mwu::launch_chained(sample_kernel, dim3(SAMP_CTAS), dim3(SAMP_THREADS), 0, st, SAMP_CTAS, p);
     if (e != cudaSuccess) return e;
     if (p.U_next || p.resid)
         e = mwu::launch_chained(pass_kernel<B, true>, dim3((unsigned)grid_stream), dim3(256), 0, st, 1, p, o.Q, o.loss_u, o.loss_p,
@@ -2020,15 +2020,20 @@ static int project_impl(const mwu_proj_desc *desc, const float *W, const float *
     p.b = desc->block;
     p.use_l1 = desc->prune_key == MWU_PRUNE_KEY_L1;
     p.work = (proj::Work *)ws;
-    p.nb = p.n_blocks <= (8ll << 20) ? proj::NB_SMALL : proj::NB_MAX;
+    p.nb = p.n_blocks <= proj::NB_SMALL_BLOCKS ? proj::NB_SMALL : proj::NB_MAX;
     p.xwork = (sel::XWork *)(ws + ws_off_xwork());
     p.fhist = (unsigned *)(ws + ws_off_hist());
     p.cand_key = (proj::u64 *)(ws + ws_off_cand_key());
     p.cand_idx = (unsigned *)(ws + ws_off_cand_idx());
     p.cand_aux = (unsigned *)(ws + ws_off_cand_aux());
-    p.samp_kp = (proj::u64 *)(ws + ws_off_samp());
-    p.samp_ku = p.samp_kp + proj::NSAMP;
     p.list = (uint2 *)(ws + ws_off_list());
+    p.samp = (float2 *)p.list;
+    p.samp_lg = p.n_blocks < SAMP_LARGE_BLOCKS ? proj::NSAMP_SMALL_LG : proj::NSAMP_LG;
+    p.n_samp = 1 << p.samp_lg;
+    if (p.n_blocks < p.n_samp) {
+        p.n_samp = (int)p.n_blocks;
+        p.samp_lg = -1;
+    }
     p.list_cap = (unsigned)list_capacity((size_t)p.n_blocks);
     p.dev_status = dev_status;
     p.U_next = U_next;
