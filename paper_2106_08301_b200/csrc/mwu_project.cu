@@ -61,8 +61,18 @@ struct Sel {
     u64 T_key, T_idx;           // selected  <=>  (key, index) <= (T_key, T_idx)
 };
 
+// Windows and provisional thresholds for pass_kernel's fp32 keys: a block whose keys lie outside [lo, hi) has its
+// final class.  The edges are moved outwards by what an fp32 key may differ from the exact one (make_filter).
+struct Filter {
+    float plo, phi, pt;         // prune key: window, threshold
+    float ulo, uhi, ut;         // L_u
+    float cap;                  // a survivor with a larger sum |v| is open whatever its L_u (the bound below does not hold)
+    float pad;
+};
+
 struct Work {
     Sel sel[2];                 // 0: prune, 1: unify
+    Filter filter;
     // one-pass pipeline
     unsigned fcand_count[2];    // threshold-bin candidates of the two halves of resolve_kernel
     unsigned fticket[2];
@@ -255,6 +265,32 @@ __device__ __forceinline__ void set_window(Sel *s, u64 lo, u64 hi, int nb) {
     s->lo0 = lo;
     s->hi0 = hi;
     s->shift0 = shift;
+}
+
+// Bounds of the fp32 keys of pass_kernel, with u = 2^-24, for a block of B <= 16 values a_i = |v_i| of sum S and mean q:
+//   sum of squares, sum        within B u (relative) of the exact one, as sums of positive terms;
+//   L_u = sum (a_i - q)^2      the computed mean is off by e <= 16 u q, which adds B e^2 exactly (the deviations from the
+//                              mean sum to zero); the rest is a sum of positive terms again: within (B + 3) u.
+// So with REL above 19 u plus a share of 1e-6 for B e^2: below REL * hi as long as S <= cap.  Results that
+// underflow are off by less than TINY more; one that overflows is infinite, and above any finite edge.
+__device__ __forceinline__ void make_filter(Filter *f, const Sel &sp, const Sel &su, u64 tp, u64 tu, int B) {
+    constexpr double REL = 4e-6, TINY = 0x1p-138;
+    const float inf = __int_as_float(0x7f800000), nan = __int_as_float(0x7fffffff);
+    auto lower = [](u64 k) { return __double2float_rd(fma(__longlong_as_double((long long)k), 1.0 - REL, -TINY)); };
+    auto upper = [&](u64 k) {
+        const float x = __double2float_ru(fma(__longlong_as_double((long long)k), 1.0 + REL, TINY));
+        return x < inf ? x : nan;                     // nothing is certainly above
+    };
+    auto point = [](u64 k) { return __double2float_rn(__longlong_as_double((long long)k)); };
+    // nothing open: no key is >= inf and below -1.  (mode 3, grouped pruning: pass_kernel sets pt by the group's bit.)
+    f->plo = sp.mode == 0u ? lower(sp.lo0) : inf;
+    f->phi = sp.mode == 0u ? upper(sp.hi0) : -1.f;
+    f->pt = sp.mode == 0u ? point(tp) : (sp.mode == 2u ? inf : -1.f);
+    f->ulo = su.mode == 0u ? lower(su.lo0) : inf;
+    f->uhi = su.mode == 0u ? upper(su.hi0) : -1.f;
+    f->ut = su.mode == 0u ? point(tu) : (su.mode == 2u ? inf : -1.f);
+    // B e^2 <= 256 u^2 S^2 / B <= 1e-6 hi
+    f->cap = su.mode == 0u ? __double2float_rd(sqrt(0.9e-6 * (double)B * __longlong_as_double((long long)su.hi0)) * (0x1p24 / 16.0)) : inf;
 }
 
 // inclusive prefix sum over the CTA's SAMP_THREADS values (one per thread)
@@ -502,6 +538,7 @@ __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
         su->mode = (ksel_u == 0) ? 1u : (ksel_u == elig ? 2u : 0u);
         su->k = (u64)ksel_u;
         p.work->That[1] = key64(That);
+        make_filter(&p.work->filter, *sp, *su, p.work->That[0], p.work->That[1], p.b);
     }
     sel::ClusterTeam::arrive();                       // nobody leaves while its counts are still read
     sel::ClusterTeam::wait();
@@ -1050,57 +1087,139 @@ __global__ void __launch_bounds__(WALK_THREADS) exact_walk_kernel(const __grid_c
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void one_pass_fail(const Params &p) { atomicExch(&p.work->failed, 1u); }
 
-// pass_kernel: keys, provisional classes and every output in one sweep over W (+U).
-// A block is a candidate when its final class is still open: its prune key lies inside the prune
-// window, or it certainly survives pruning and its L_u lies inside the unify window.  Candidates
-// are staged per warp with their two keys; when 32 have gathered, the whole warp turns them into
-// bin codes, window-histogram counts and list entries (every lane busy), so the sweep itself only
-// compares keys with the window edges.
-// ADMM: also the dual update V - Q and ||V - Q||_F^2 (mwu_admm_step); a separate instantiation so
-// that the plain projection keeps its register count.
-template <int B, bool ADMM>
-__global__ void __launch_bounds__(256) pass_kernel(Params p, float *Q, double *loss_u, double *loss_p,
-                                                   float *u_out, unsigned *pruned_bitmap,
-                                                   unsigned *unified_bitmap, unsigned *sign_bits) {
-    constexpr int NBT = 16 / B;
-    // Launched with programmatic stream serialization: the CTAs may start while sample_kernel still
-    // runs.  The first 64 bytes of W do not depend on it and are requested at once; everything
-    // sample_kernel writes (windows, cleared histograms) is read only behind the wait.
-    const long long n = p.n_floats;
-    const unsigned n_units = (unsigned)((n + 15) / 16);
-    unsigned unit = blockIdx.x * blockDim.x + threadIdx.x;
-    float nxt[16];
+// Values of warp step `step` (512 floats) that this lane handles; zero beyond the tensor.
+// B <= 4: the lane's four pieces of four floats lie a warp apart, so that every access of a warp is 512 contiguous
+// bytes and a block lies in one piece.  B >= 8: 64 contiguous bytes, so that a block lies in one lane.
+template <int B>
+__device__ __forceinline__ void load_step(const float *W, const float *U, unsigned step, int lane, long long n, float (&v)[16]) {
+    if constexpr (B <= 4) {
+        const long long f0 = (long long)step * 512 + lane * 4;
+        if ((long long)step * 512 + 512 <= n) {
 #pragma unroll
-    for (int l = 0; l < 16; ++l) nxt[l] = 0.f;
-    if (unit < n_units) load16(p.W, p.U, (long long)unit * 16, n, nxt);
+            for (int c = 0; c < 4; ++c) {
+                const float4 a = __ldg(reinterpret_cast<const float4 *>(W + f0) + c * 32);
+                v[4 * c] = a.x; v[4 * c + 1] = a.y; v[4 * c + 2] = a.z; v[4 * c + 3] = a.w;
+            }
+            if (U) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float4 d = __ldg(reinterpret_cast<const float4 *>(U + f0) + c * 32);
+                    v[4 * c] = __fadd_rn(v[4 * c], d.x); v[4 * c + 1] = __fadd_rn(v[4 * c + 1], d.y);
+                    v[4 * c + 2] = __fadd_rn(v[4 * c + 2], d.z); v[4 * c + 3] = __fadd_rn(v[4 * c + 3], d.w);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int l = 0; l < 16; ++l) {
+                const long long f = f0 + (l >> 2) * 128 + (l & 3);
+                v[l] = f < n ? load_v(W, U, f) : 0.f;
+            }
+        }
+    } else {
+        load16(W, U, (long long)step * 512 + lane * 16, n, v);
+    }
+}
+
+// 16 floats of a lane, laid out as by load_step, to step `step` of dst.  ws: 128 float4 of shared memory of the warp.
+template <int B>
+__device__ __forceinline__ void store_step(float *dst, unsigned step, int lane, long long n, const float (&q)[16], float4 *ws) {
+    const long long base = (long long)step * 512;
+    if (base + 512 > n) {
+#pragma unroll
+        for (int l = 0; l < 16; ++l) {
+            const long long f = base + (B <= 4 ? (l >> 2) * 128 + lane * 4 + (l & 3) : lane * 16 + l);
+            if (f < n) dst[f] = q[l];
+        }
+        return;
+    }
+    float4 *d4 = reinterpret_cast<float4 *>(dst + base);
+    if constexpr (B <= 4) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) d4[c * 32 + lane] = make_float4(q[4 * c], q[4 * c + 1], q[4 * c + 2], q[4 * c + 3]);
+    } else {
+        // 16-byte stores at a 64-byte stride reach L2 as four partial writes per 64 bytes, so the step goes through
+        // shared memory and leaves as four stores of 512 contiguous bytes.  Thread t keeps piece c at slot
+        // c ^ ((t >> 1) & 3), so neither side has bank conflicts.
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            ws[lane * 4 + (c ^ ((lane >> 1) & 3))] = make_float4(q[4 * c], q[4 * c + 1], q[4 * c + 2], q[4 * c + 3]);
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int t = 8 * k + (lane >> 2), c = lane & 3;
+            d4[k * 32 + lane] = ws[t * 4 + (c ^ ((t >> 1) & 3))];
+        }
+    }
+}
+
+// Bin codes (prune | L_u << 16) of the exact keys of block j, and the exact losses of step `step`: functions of their own,
+// so that the sweep's registers need not hold fp64 keys.
+template <int B>
+__device__ __noinline__ unsigned exact_codes(const Params &p, unsigned j) {
+    const Sel *sp = &p.work->sel[0], *su = &p.work->sel[1];
+    double S, Lu, Kp;
+    block_keys_at<B>(p.W, p.U, (long long)j, p.use_l1, &S, &Lu, &Kp);
+    return bin_of(key_bits(Kp), sp->lo0, sp->hi0, sp->shift0, (unsigned)p.nb) |
+           bin_of(key_bits(Lu), su->lo0, su->hi0, su->shift0, (unsigned)p.nb) << 16;
+}
+template <int B>
+__device__ __noinline__ void exact_losses(const Params &p, unsigned step, double *loss_u, double *loss_p) {
+#pragma unroll 1
+    for (int e = threadIdx.x & 31; e < 512 / B; e += 32) {
+        const unsigned j = step * (512 / B) + (unsigned)e;
+        if (j >= (unsigned)p.n_blocks) break;
+        double S, Lu, Kp;
+        block_keys_at<B>(p.W, p.U, (long long)j, p.use_l1, &S, &Lu, &Kp);
+        if (loss_u) loss_u[j] = Lu;
+        if (loss_p) loss_p[j] = Kp;
+    }
+}
+
+// pass_kernel: provisional classes and every output in one sweep over W (+U).
+// Classes come from fp32 keys: a block whose fp32 keys lie outside the windows by more than their error (Filter) has its
+// final class.  The others (a few per cent: those inside the windows, and a few in ten thousand near their edges) are
+// staged per warp; when 32 have gathered, the whole warp evaluates their exact fp64 keys and turns them into bin codes,
+// window-histogram counts and list entries.  In fp64 every block gets only its sum (u is its rounded mean).
+//
+// What bounds it: HBM for blocks of 4 and more (16384 x 16384, b = 4: 462 us for 2.45 GB, 5.3 TB/s; 16384 x 4096, b = 16: 105 us,
+// 5.3 TB/s), instruction issue for 2.  With fp64 keys of every block and 64-bit comparisons a block of 4 took 240
+// instructions, 16384 x 16384 with b = 4 650 us.
+// ADMM: also the dual update V - Q and ||V - Q||_F^2 (mwu_admm_step).
+constexpr int PASS_THREADS = 256, PASS_WARPS = PASS_THREADS / 32;
+// resident CTAs: blocks of 2 need the warps (16384 x 16384: 728 us a call with three, 804 with two), the others the registers
+// (b = 4: 537 / 511, b = 16: 477 / 435)
+constexpr int pass_ctas_per_sm(int b, bool admm) { return b == 2 && !admm ? 3 : 2; }
+template <int B, bool ADMM>
+__global__ void __launch_bounds__(PASS_THREADS, pass_ctas_per_sm(B, ADMM))
+pass_kernel(const __grid_constant__ Params p, float *Q, double *loss_u, double *loss_p, float *u_out, unsigned *pruned_bitmap,
+            unsigned *unified_bitmap, unsigned *sign_bits) {
+    constexpr int NBT = 16 / B;                          // blocks of a lane
+    constexpr int NBP = B <= 4 ? 4 / B : NBT;            // of them next to one another
+    const long long n = p.n_floats;
+    const unsigned n_steps = (unsigned)((n + 511) / 512), stride = gridDim.x * PASS_WARPS;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned step = blockIdx.x * PASS_WARPS + warp;
+    // Launched with programmatic stream serialization: the CTAs may start while sample_kernel still
+    // runs.  The first values do not depend on it and are requested at once; everything
+    // sample_kernel writes (windows, cleared histograms) is read only behind the wait.
+    float nxt[16];
+    if (step < n_steps) load_step<B>(p.W, p.U, step, lane, n, nxt);
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const Sel *sp = &p.work->sel[0];
-    const Sel *su = &p.work->sel[1];
-    const u64 plo = sp->lo0, phi = sp->hi0, ulo = su->lo0, uhi = su->hi0;
-    const unsigned psh = sp->shift0, ush = su->shift0;
-    const unsigned mode_p = sp->mode, mode_u = su->mode;
-    const u64 Tp = p.work->That[0], Tu = p.work->That[1];
+    const Filter F = p.work->filter;
+    const bool by_group = p.gprune != nullptr;
     const unsigned nb = (unsigned)p.nb, top = nb - 1u;
     unsigned *hist_p = p.fhist, *hist_u = p.fhist + p.nb;
-    __shared__ float4 s_q[8][128];                       // one warp step of Q per warp
-    // candidates waiting for a full 32-entry flush: block index and both keys
-    __shared__ unsigned s_cidx[8][STAGE_ENTRIES];
-    __shared__ u64 s_ckp[8][STAGE_ENTRIES], s_cku[8][STAGE_ENTRIES];
-    const int lane = threadIdx.x & 31;
-    float4 *wq = s_q[threadIdx.x >> 5];
-    unsigned *cidx = s_cidx[threadIdx.x >> 5];
-    u64 *ckp = s_ckp[threadIdx.x >> 5], *cku = s_cku[threadIdx.x >> 5];
-    const unsigned lt_mask = (1u << lane) - 1u;
+    __shared__ float4 s_q[B <= 4 ? 1 : PASS_WARPS][B <= 4 ? 1 : 128];       // one warp step of Q per warp
+    __shared__ unsigned s_cidx[PASS_WARPS][STAGE_ENTRIES];                   // blocks waiting for a full 32-entry flush
+    float4 *wq = s_q[B <= 4 ? 0 : warp];
+    unsigned *cidx = s_cidx[warp];
     unsigned fill = 0;                                   // warp-uniform
-    unsigned under_p = 0, over_p = 0, under_u = 0, over_u = 0, nonfinite = 0;
+    unsigned under_p = 0, under_u = 0, nonfinite = 0;
     double resid_acc = 0.0;
-    // fewer than 2^31 blocks of at least two values: units (16 values) and blocks count in 32 bits
-    const unsigned n_iter = (n_units + 31u) / 32u * 32u;  // whole warps take part in every step
-    const unsigned n_blocks = (unsigned)p.n_blocks;
-    const unsigned n_bm_words = (n_blocks + 31u) / 32u;
-    const unsigned ustride = gridDim.x * blockDim.x;
+    const unsigned n_blocks = (unsigned)p.n_blocks;      // fewer than 2^30
 
-    // staged candidates [from, from + cnt) -> bin codes, window histograms, list entries (whole warp)
+    // staged blocks [from, from + cnt) -> exact keys, bin codes, window histograms, list entries (whole warp)
     auto flush = [&](unsigned from, unsigned cnt) {
         unsigned base = 0;
         if (lane == 0) base = atomicAdd(&p.work->list_count, cnt);
@@ -1110,27 +1229,29 @@ __global__ void __launch_bounds__(256) pass_kernel(Params p, float *Q, double *l
             return;
         }
         if ((unsigned)lane < cnt) {
-            const u64 kp = ckp[from + lane], ku = cku[from + lane];
-            const unsigned bp = bin_of(kp, plo, phi, psh, nb), bu = bin_of(ku, ulo, uhi, ush, nb);
-            if (mode_p == 0u && bp != 0u && bp != top) atomicAdd(&hist_p[bp], 1u);       // open because of the prune window
-            else if (mode_u == 0u && bu != 0u && bu != top) atomicAdd(&hist_u[bu], 1u);  // a survivor inside the unify window
-            p.list[base + lane] = make_uint2(cidx[from + lane], bp | (bu << 16));
+            const unsigned ent = cidx[from + lane];
+            const unsigned codes = exact_codes<B>(p, ent & 0x3fffffffu), bp = codes & 0xffffu, bu = codes >> 16;
+            if (p.work->sel[0].mode == 0u && bp != top) {
+                if (bp == 0u) ++under_p;                                     // pruned
+                else atomicAdd(&hist_p[bp], 1u);                             // open because of the prune window
+            } else if (p.work->sel[1].mode == 0u) {                          // a survivor
+                if (bu == 0u) ++under_u;
+                else if (bu != top) atomicAdd(&hist_u[bu], 1u);
+            }
+            p.list[base + lane] = make_uint2(ent, codes);
         }
     };
 
-    for (; unit < n_iter; unit += ustride) {
+#pragma unroll 1
+    for (; step < n_steps; step += stride) {
         float v[16];
 #pragma unroll
         for (int l = 0; l < 16; ++l) v[l] = nxt[l];
-        // the next unit's 64 bytes travel while this one is evaluated
-        if (unit + ustride < n_units) load16(p.W, p.U, (long long)(unit + ustride) * 16, n, nxt);
-        else {
-#pragma unroll
-            for (int l = 0; l < 16; ++l) nxt[l] = 0.f;
-        }
-        const bool live = unit < n_units;
-        const bool warp_full = (long long)(unit - lane + 32u) * 16 <= n;      // all 512 floats of this warp step exist
-        const unsigned j0 = unit * NBT;
+        // the next step's values travel while this one is evaluated
+        if (step + stride < n_steps) load_step<B>(p.W, p.U, step + stride, lane, n, nxt);
+        const bool full = (long long)step * 512 + 512 <= n;
+        const unsigned j0 = step * (512 / B) + (B <= 4 ? lane * NBP : lane * NBT);   // this lane's first block
+        auto block_of = [&](int e) { return j0 + (unsigned)(e / NBP) * (128 / B) + (unsigned)(e % NBP); };
         // Sign plane: bit l = (v[l] < 0).  Without a zero among the warp's values that is the IEEE sign
         // bit, gathered with one funnel shift per value; a zero (it may be -0.0) takes the compare.
         float vmin = fabsf(v[0]);
@@ -1145,212 +1266,200 @@ __global__ void __launch_bounds__(256) pass_kernel(Params p, float *Q, double *l
 #pragma unroll
             for (int l = 0; l < 16; ++l) sb |= (v[l] < 0.f ? 1u : 0u) << l;
         }
-        if (live) {
-            unsigned short *halves = reinterpret_cast<unsigned short *>(sign_bits);
-            halves[unit] = (unsigned short)sb;
-            if (unit == n_units - 1 && (n_units & 1)) halves[unit + 1] = 0;
+        {
+            const unsigned n_halves = (unsigned)((n + 31) / 32) * 2u;
+            if constexpr (B <= 4) {
+                // the pieces' four bits each, spread to bytes; a pair of lanes completes the bytes
+                unsigned x = (sb | (sb << 8)) & 0x00ff00ffu;
+                x = ((x | (x << 4)) & 0x0f0f0f0fu) << (4 * (lane & 1));
+                x |= __shfl_xor_sync(0xffffffffu, x, 1);
+                if (lane & 1) x >>= 16;
+                unsigned char *dst = reinterpret_cast<unsigned char *>(sign_bits);
+                const unsigned at = step * 64u + (unsigned)((lane & 1) * 32 + (lane >> 1));
+                if (full || at < n_halves * 2u) dst[at] = (unsigned char)x;
+                if (full || at + 16u < n_halves * 2u) dst[at + 16u] = (unsigned char)(x >> 8);
+            } else {
+                const unsigned at = step * 32u + (unsigned)lane;
+                if (full || at < n_halves) reinterpret_cast<unsigned short *>(sign_bits)[at] = (unsigned short)sb;
+            }
         }
-        // grouped pruning: a unit's 16 values lie in one group (groups are at least 16 columns wide)
-        const bool grp = mode_p == 3u && j0 < n_blocks && group_pruned(p, j0);
-        unsigned cls_p = 0, cls_u = 0, cand = 0;             // bit e: block e of this thread
-        u64 kpb[NBT], kub[NBT];
-        float uo[NBT];
+        unsigned cls_p = 0, cls_u = 0, cand = 0;             // bit e: block e of this lane
+        float uo[NBT], pt = F.pt;
 #pragma unroll
         for (int e = 0; e < NBT; ++e) {
-            double S, Lu, Kp;
-            block_keys<B>(v + e * B, p.use_l1, &S, &Lu, &Kp);
-            const float qf = __double2float_rn(__dmul_rn(S, 1.0 / (double)B));
+            const float *x = v + e * B;
+            if (by_group && (e == 0 || (B <= 4 && e % NBP == 0))) {
+                // a lane's 64 bytes, or a piece of 16, lie in one group (groups are at least 16 columns wide)
+                pt = block_of(e) < n_blocks && group_pruned(p, block_of(e)) ? __int_as_float(0x7f800000) : -1.f;
+            }
+            // fp32 keys (any order of summation)
+            float s[B];
+#pragma unroll
+            for (int l = 0; l < B; ++l) s[l] = fabsf(x[l]);
+#pragma unroll
+            for (int w = 1; w < B; w <<= 1)
+#pragma unroll
+                for (int l = 0; l < B; l += 2 * w) s[l] += s[l + w];
+            const float S32 = s[0], q32 = S32 * (1.f / (float)B);
+            float kp = 0.f, ku = 0.f;
+#pragma unroll
+            for (int l = 0; l < B; ++l) {
+                const float d = fabsf(x[l]) - q32;
+                ku = fmaf(d, d, ku);
+                kp = fmaf(x[l], x[l], kp);
+            }
+            if (p.use_l1) kp = S32;
+            const bool there = full || block_of(e) < n_blocks;
+            const bool pr = kp <= pt && there, un = !pr && ku <= F.ut && there;
+            const bool open = ((kp >= F.plo && !(kp >= F.phi)) || (!pr && ((ku >= F.ulo && !(ku >= F.uhi)) || !(S32 <= F.cap)))) && there;
+            cls_p |= pr ? 1u << e : 0u;
+            cls_u |= un ? 1u << e : 0u;
+            cand |= open ? 1u << e : 0u;
+            // the mean as the exact keys have it
+            double a[B];
+#pragma unroll
+            for (int l = 0; l < B; ++l) a[l] = (double)fabsf(x[l]);
+            const double S = tree_sum<B>(a), qd = __dmul_rn(S, 1.0 / (double)B);
             // S = sum |v| is Inf or NaN exactly when some value of the block is
             nonfinite |= ((unsigned)__double2hiint(S) >= 0x7ff00000u) ? 1u : 0u;
-            kpb[e] = key_bits(Kp);
-            kub[e] = key_bits(Lu);
-            uo[e] = 0.f;
-            const unsigned j = j0 + e;
-            if (j < n_blocks) {
-                if (loss_u) loss_u[j] = Lu;
-                if (loss_p) loss_p[j] = Kp;
-                bool pr, survives, open = false;
-                if (mode_p == 0u) {
-                    const bool below = kpb[e] < plo, above = kpb[e] >= phi;
-                    pr = kpb[e] <= Tp;
-                    survives = above;
-                    under_p += below ? 1u : 0u;
-                    over_p += above ? 1u : 0u;
-                    open = !(below || above);
-                } else if (mode_p == 3u) {
-                    pr = grp;                              // grouped pruning: the class is the group's bit
-                    survives = !grp;
-                } else {
-                    pr = mode_p == 2u;
-                    survives = mode_p == 1u;
+            uo[e] = un ? __double2float_rn(qd) : 0.f;
+            if (ADMM && p.resid && (pr || un)) {
+                // squared distance of the block to its image: the loss of its (provisional) class
+                double t[B];
+#pragma unroll
+                for (int l = 0; l < B; ++l) {
+                    const double d = pr ? a[l] : __dsub_rn(a[l], qd);
+                    t[l] = __dmul_rn(d, d);
                 }
-                const bool un = !pr && (mode_u == 2u || (mode_u == 0u && kub[e] <= Tu));
-                if (survives && mode_u == 0u) {
-                    const bool below = kub[e] < ulo, above = kub[e] >= uhi;
-                    under_u += below ? 1u : 0u;
-                    over_u += above ? 1u : 0u;
-                    open = open || !(below || above);
-                }
-                cls_p |= (pr ? 1u : 0u) << e;
-                cls_u |= (un ? 1u : 0u) << e;
-                cand |= (open ? 1u : 0u) << e;
-                if (un) uo[e] = qf;
-                if (ADMM && p.resid) {
-                    // squared distance of the block to its image: the loss of its (provisional) class
-                    if (un) resid_acc += Lu;
-                    else if (pr) resid_acc += p.use_l1 ? block_sumsq<B>(v + e * B) : Kp;
-                }
+                resid_acc += tree_sum<B>(t);
             }
         }
-        if (live) {
-            if (j0 + NBT <= n_blocks) {
-                if (NBT == 1) u_out[j0] = uo[0];
-                else if (NBT == 2) *reinterpret_cast<float2 *>(u_out + j0) = make_float2(uo[0], uo[1 % NBT]);
-                else {
+        if (loss_u || loss_p) exact_losses<B>(p, step, loss_u, loss_p);
+        under_p += __popc(cls_p & ~cand);
+        under_u += __popc(cls_u & ~cand);
+        if (full) {
 #pragma unroll
-                    for (int e = 0; e < NBT; e += 4)
-                        *reinterpret_cast<float4 *>(u_out + j0 + e) =
-                            make_float4(uo[e % NBT], uo[(e + 1) % NBT], uo[(e + 2) % NBT], uo[(e + 3) % NBT]);
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < NBT; ++e)
-                    if (j0 + e < n_blocks) u_out[j0 + e] = uo[e];
+            for (int e = 0; e < NBT; e += NBP) {
+                if (NBP == 1) u_out[block_of(e)] = uo[e];
+                else *reinterpret_cast<float2 *>(u_out + block_of(e)) = make_float2(uo[e], uo[(e + 1) % NBT]);
             }
-            if (Q || (ADMM && p.U_next)) {
-                // q = v (kept), +-u (unified: magnitude u, sign of v), or +0
-                float q[16];
+        } else {
 #pragma unroll
-                for (int e = 0; e < NBT; ++e) {
-                    const bool pr = (cls_p >> e) & 1u, un = (cls_u >> e) & 1u;
-                    const unsigned mag = un ? __float_as_uint(uo[e]) : 0u;
-                    if (!has_zero) {
-                        // no zero in the warp: the sign of v is its IEEE sign bit
-                        const unsigned m1 = pr ? 0u : (un ? 0x80000000u : 0xffffffffu);
-#pragma unroll
-                        for (int l = 0; l < B; ++l) q[e * B + l] = __uint_as_float((__float_as_uint(v[e * B + l]) & m1) | mag);
-                    } else {
-                        const unsigned keep = (pr || un) ? 0u : 0xffffffffu;
-                        const unsigned sgn = un ? 0x80000000u : 0u;
-#pragma unroll
-                        for (int l = 0; l < B; ++l) {
-                            const int k = e * B + l;
-                            q[k] = __uint_as_float((__float_as_uint(v[k]) & keep) | mag | ((sb << (31 - k)) & sgn));
-                        }
-                    }
-                }
-                const long long f = (long long)unit * 16;
-                if (ADMM && p.U_next) {
-                    // dual update: one fp32 subtraction per entry (v for a pruned block, +0 for a kept one)
-                    if (f + 16 <= n) {
-                        float4 *dst = reinterpret_cast<float4 *>(p.U_next + f);
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            dst[c] = make_float4(__fsub_rn(v[4 * c], q[4 * c]), __fsub_rn(v[4 * c + 1], q[4 * c + 1]),
-                                                 __fsub_rn(v[4 * c + 2], q[4 * c + 2]), __fsub_rn(v[4 * c + 3], q[4 * c + 3]));
-                    } else {
-#pragma unroll
-                        for (int l = 0; l < 16; ++l)
-                            if (f + l < n) p.U_next[f + l] = __fsub_rn(v[l], q[l]);
-                    }
-                }
-                if (!Q) {
-                    // only the dual update was wanted
-                } else if (!warp_full) {
-                    if (f + 16 <= n) {
-                        float4 *dst = reinterpret_cast<float4 *>(Q + f);
-                        dst[0] = make_float4(q[0], q[1], q[2], q[3]);
-                        dst[1] = make_float4(q[4], q[5], q[6], q[7]);
-                        dst[2] = make_float4(q[8], q[9], q[10], q[11]);
-                        dst[3] = make_float4(q[12], q[13], q[14], q[15]);
-                    } else {
-#pragma unroll
-                        for (int l = 0; l < 16; ++l)
-                            if (f + l < n) Q[f + l] = q[l];
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        wq[lane * 4 + (c ^ ((lane >> 1) & 3))] = make_float4(q[4 * c], q[4 * c + 1], q[4 * c + 2], q[4 * c + 3]);
-                }
-            }
+            for (int e = 0; e < NBT; ++e)
+                if (block_of(e) < n_blocks) u_out[block_of(e)] = uo[e];
         }
-        // Q of a whole warp step (2 KB) leaves as four stores of 512 contiguous bytes: thread t keeps
-        // piece c at slot c ^ ((t >> 1) & 3), so neither side has bank conflicts.
-        if (Q && warp_full) {
-            __syncwarp();
-            float4 *dst = reinterpret_cast<float4 *>(Q + (long long)(unit - lane) * 16);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int t = 8 * k + (lane >> 2), c = lane & 3;
-                dst[k * 32 + lane] = wq[t * 4 + (c ^ ((t >> 1) & 3))];
-            }
-            __syncwarp();
-        }
-        // class bitmaps: the warp's 32 * NBT blocks make NBT words
-        {
-            const unsigned word0 = ((unit - lane) * NBT) >> 5;
-#pragma unroll
-            for (int w = 0; w < NBT; ++w) {
-                const int blk = w * 32 + lane;               // block of this warp step that lane reports
-                const unsigned xp = __shfl_sync(0xffffffffu, cls_p, blk / NBT);
-                const unsigned xu = __shfl_sync(0xffffffffu, cls_u, blk / NBT);
-                const unsigned wp = __ballot_sync(0xffffffffu, (xp >> (blk % NBT)) & 1u);
-                const unsigned wu = __ballot_sync(0xffffffffu, (xu >> (blk % NBT)) & 1u);
-                if (lane == 0 && word0 + w < n_bm_words) {
-                    pruned_bitmap[word0 + w] = wp;
-                    unified_bitmap[word0 + w] = wu;
-                }
-            }
-        }
-        // candidates gather in the warp's staging buffer and leave 32 at a time
-        if (__any_sync(0xffffffffu, cand != 0u)) {
+        if (Q || (ADMM && p.U_next)) {
+            // q = v (kept), +-u (unified: magnitude u, sign of v), or +0
+            float q[16];
 #pragma unroll
             for (int e = 0; e < NBT; ++e) {
-                const bool c = (cand >> e) & 1u;
-                const unsigned bal = __ballot_sync(0xffffffffu, c);
-                if (bal == 0u) continue;
-                if (c) {
-                    const unsigned pos = fill + __popc(bal & lt_mask);
-                    // block index with the provisional class in its top bits (fewer than 2^30 blocks)
-                    cidx[pos] = (j0 + e) | (((cls_p >> e) & 1u) << 31) | (((cls_u >> e) & 1u) << 30);
-                    ckp[pos] = kpb[e];
-                    cku[pos] = kub[e];
+                const bool pr = (cls_p >> e) & 1u, un = (cls_u >> e) & 1u;
+                const unsigned mag = __float_as_uint(uo[e]);               // 0 unless unified
+                if (!has_zero) {
+                    // no zero in the warp: the sign of v is its IEEE sign bit
+                    const unsigned m1 = pr ? 0u : (un ? 0x80000000u : 0xffffffffu);
+#pragma unroll
+                    for (int l = 0; l < B; ++l) q[e * B + l] = __uint_as_float((__float_as_uint(v[e * B + l]) & m1) | mag);
+                } else {
+                    const unsigned keep = (pr || un) ? 0u : 0xffffffffu;
+                    const unsigned sgn = un ? 0x80000000u : 0u;
+#pragma unroll
+                    for (int l = 0; l < B; ++l) {
+                        const int k = e * B + l;
+                        q[k] = __uint_as_float((__float_as_uint(v[k]) & keep) | mag | ((sb << (31 - k)) & sgn));
+                    }
                 }
-                fill += __popc(bal);
+            }
+            if (Q) store_step<B>(Q, step, lane, n, q, wq);
+            if (ADMM && p.U_next) {
+                // dual update: one fp32 subtraction per entry (v for a pruned block, +0 for a kept one)
+#pragma unroll
+                for (int l = 0; l < 16; ++l) q[l] = __fsub_rn(v[l], q[l]);
+                store_step<B>(p.U_next, step, lane, n, q, wq);
+            }
+        }
+        // class bitmaps: the step's 512 / B blocks make NBT words
+        {
+            const unsigned n_bm = (n_blocks + 31u) / 32u;
+            if constexpr (B == 2) {
+                // two bits of every piece, spread to bytes; four lanes complete the bytes, and each stores one piece's
+                auto bytes = [&](unsigned x) {
+                    x = (x | (x << 12)) & 0x000f000fu;
+                    x = ((x | (x << 6)) & 0x03030303u) << (2 * (lane & 3));
+                    x |= __shfl_xor_sync(0xffffffffu, x, 1);
+                    x |= __shfl_xor_sync(0xffffffffu, x, 2);
+                    return (unsigned char)(x >> (8 * (lane & 3)));
+                };
+                const unsigned char bp = bytes(cls_p), bu = bytes(cls_u);
+                const unsigned at = step * 32u + (unsigned)((lane & 3) * 8 + (lane >> 2));
+                if (full || at < n_bm * 4u) {
+                    reinterpret_cast<unsigned char *>(pruned_bitmap)[at] = bp;
+                    reinterpret_cast<unsigned char *>(unified_bitmap)[at] = bu;
+                }
+            } else if constexpr (B == 8) {
+                // two bits of each of 16 lanes make a word: bytes by four lanes, the first stores the pruned, the second the unified
+                unsigned x = (cls_p | (cls_u << 16)) << (2 * (lane & 3));
+                x |= __shfl_xor_sync(0xffffffffu, x, 1);
+                x |= __shfl_xor_sync(0xffffffffu, x, 2);
+                const unsigned at = step * 8u + (unsigned)(lane >> 2);
+                unsigned char *dst = reinterpret_cast<unsigned char *>((lane & 1) ? unified_bitmap : pruned_bitmap);
+                if ((lane & 3) < 2 && (full || at < n_bm * 4u)) dst[at] = (unsigned char)((lane & 1) ? x >> 16 : x);
+            } else {
+                unsigned wp[NBT], wu[NBT];
+#pragma unroll
+                for (int e = 0; e < NBT; ++e) {
+                    wp[e] = __ballot_sync(0xffffffffu, (cls_p >> e) & 1u);
+                    wu[e] = __ballot_sync(0xffffffffu, (cls_u >> e) & 1u);
+                }
+                // lane e stores a word of the pruned, lane NBT + e of the unified
+                unsigned word = wp[0];
+#pragma unroll
+                for (int e = 0; e < NBT; ++e) {
+                    if (lane == e) word = wp[e];
+                    if (lane == NBT + e) word = wu[e];
+                }
+                const unsigned at = step * NBT + (unsigned)(lane % NBT);
+                if (lane < 2 * NBT && (full || at < n_bm)) (lane < NBT ? pruned_bitmap : unified_bitmap)[at] = word;
+            }
+        }
+        // open blocks gather in the warp's staging buffer and leave 32 at a time
+#pragma unroll 1
+        for (;;) {
+            const unsigned bal = __ballot_sync(0xffffffffu, cand != 0u);
+            if (bal == 0u) break;
+            if (cand) {
+                const int e = __ffs((int)cand) - 1;
+                cand &= cand - 1u;
+                // block index with the provisional class in its top bits
+                cidx[fill + __popc(bal & ((1u << lane) - 1u))] = block_of(e) | (((cls_p >> e) & 1u) << 31) | (((cls_u >> e) & 1u) << 30);
+            }
+            fill += __popc(bal);
+            __syncwarp();
+            if (fill >= 32u) {
+                fill -= 32u;
+                flush(fill, 32u);
                 __syncwarp();
-                if (fill >= 32u) {
-                    fill -= 32u;
-                    flush(fill, 32u);
-                    __syncwarp();
-                }
             }
         }
     }
     if (fill > 0u) flush(0u, fill);
-    // block-level totals of the catch-all bins
-    __shared__ unsigned s_tot[4];
-    if (threadIdx.x < 4) s_tot[threadIdx.x] = 0;
+    // block-level totals of the lowest bins
+    __shared__ unsigned s_tot[2];
+    if (threadIdx.x < 2) s_tot[threadIdx.x] = 0;
     __syncthreads();
-    for (int m = 16; m > 0; m >>= 1) {
-        under_p += __shfl_xor_sync(0xffffffffu, under_p, m);
-        over_p += __shfl_xor_sync(0xffffffffu, over_p, m);
-        under_u += __shfl_xor_sync(0xffffffffu, under_u, m);
-        over_u += __shfl_xor_sync(0xffffffffu, over_u, m);
-    }
+    under_p = __reduce_add_sync(0xffffffffu, under_p);
+    under_u = __reduce_add_sync(0xffffffffu, under_u);
     if (lane == 0) {
         if (under_p) atomicAdd(&s_tot[0], under_p);
-        if (over_p) atomicAdd(&s_tot[1], over_p);
-        if (under_u) atomicAdd(&s_tot[2], under_u);
-        if (over_u) atomicAdd(&s_tot[3], over_u);
+        if (under_u) atomicAdd(&s_tot[1], under_u);
     }
     if (nonfinite) atomicOr(p.dev_status, (unsigned)MWU_DEV_NONFINITE);
     __syncthreads();
     if (threadIdx.x == 0) {
         if (s_tot[0]) atomicAdd(&hist_p[0], s_tot[0]);
-        if (s_tot[1]) atomicAdd(&hist_p[top], s_tot[1]);
-        if (s_tot[2]) atomicAdd(&hist_u[0], s_tot[2]);
-        if (s_tot[3]) atomicAdd(&hist_u[top], s_tot[3]);
+        if (s_tot[1]) atomicAdd(&hist_u[0], s_tot[1]);
+        // the highest bins: nobody counts what lies above a window, only that it is enough
+        if (blockIdx.x == 0) { hist_p[top] = n_blocks; hist_u[top] = n_blocks; }
     }
     if (ADMM && p.resid) block_add_double(resid_acc, p.resid);
 }
@@ -1488,7 +1597,7 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
             alive = false;
         }
         if (alive) {
-            unsigned under = 0, over = 0;
+            unsigned under = 0;
             const u128 lo0 = from_halves(s_sel.lo_hi, s_sel.lo_lo);
             const u128 hi0 = from_halves(s_sel.hi_hi, s_sel.hi_lo);
             // a thread's entries are requested together (each iteration would otherwise wait for its own load)
@@ -1524,18 +1633,11 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
                 }
                 if (mode_u != 0u) continue;
                 if (bu == 0u) ++under;
-                else if (bu == top) ++over;
-                else atomicAdd(&hist_u[bu], 1u);
+                else if (bu != top) atomicAdd(&hist_u[bu], 1u);
               }
             }
-            for (int m = 16; m > 0; m >>= 1) {
-                under += __shfl_xor_sync(0xffffffffu, under, m);
-                over += __shfl_xor_sync(0xffffffffu, over, m);
-            }
-            if ((threadIdx.x & 31) == 0) {
-                if (under) atomicAdd(&hist_u[0], under);
-                if (over) atomicAdd(&hist_u[top], over);
-            }
+            under = __reduce_add_sync(0xffffffffu, under);
+            if ((threadIdx.x & 31) == 0 && under) atomicAdd(&hist_u[0], under);
         }
         if (!grid_sync(&p.work->bar, ++k)) {              // bounded; every CTA runs into the same limit
             if (threadIdx.x == 0) atomicOr(p.dev_status, (unsigned)MWU_DEV_TIMEOUT);
@@ -1949,9 +2051,9 @@ static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_des
                                   sm_count, st, p, o,
                                   mwu::sel::problem_of(p.n_blocks, p.k_prune, p.k_unify, p.gprune != nullptr, WALK_THREADS));
     }
-    const long long want = (n_units + 255) / 256;
-    const long long cap_blocks = (long long)sm_count * 8;
-    const int grid_stream = (int)(want < cap_blocks ? (want > 0 ? want : 1) : cap_blocks);
+    const bool admm = p.U_next || p.resid;
+    const long long want = (n_units + PASS_THREADS - 1) / PASS_THREADS, resident = (long long)sm_count * pass_ctas_per_sm(B, admm);
+    const int grid_stream = (int)(want < resident ? want : resident);
     const long long mb = p.n_blocks;
     const bool need_p = !p.gprune && desc->k_prune > 0 && desc->k_prune < mb;
     const long long ksel_u = desc->k_unify - desc->k_prune;
@@ -1966,11 +2068,11 @@ static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_des
     e = mwu::launch_chained(sample_keys_kernel<B>, dim3((unsigned)(p.n_samp + 127) / 128), dim3(128), 0, st, 1, p, zero, n_zero);
     if (e == cudaSuccess) e = mwu::launch_chained(sample_kernel, dim3(SAMP_CTAS), dim3(SAMP_THREADS), 0, st, SAMP_CTAS, p);
     if (e != cudaSuccess) return e;
-    if (p.U_next || p.resid)
-        e = mwu::launch_chained(pass_kernel<B, true>, dim3((unsigned)grid_stream), dim3(256), 0, st, 1, p, o.Q, o.loss_u, o.loss_p,
+    if (admm)
+        e = mwu::launch_chained(pass_kernel<B, true>, dim3((unsigned)grid_stream), dim3(PASS_THREADS), 0, st, 1, p, o.Q, o.loss_u, o.loss_p,
                                 o.u, o.pruned_bitmap, o.unified_bitmap, o.sign_bits);
     else
-        e = mwu::launch_chained(pass_kernel<B, false>, dim3((unsigned)grid_stream), dim3(256), 0, st, 1, p, o.Q, o.loss_u, o.loss_p,
+        e = mwu::launch_chained(pass_kernel<B, false>, dim3((unsigned)grid_stream), dim3(PASS_THREADS), 0, st, 1, p, o.Q, o.loss_u, o.loss_p,
                                 o.u, o.pruned_bitmap, o.unified_bitmap, o.sign_bits);
     if (e != cudaSuccess) return e;
     mwu::count_launch(3);

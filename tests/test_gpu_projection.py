@@ -326,3 +326,22 @@ def test_projection_exact_kernel_ties_beyond_the_candidate_list(rows, k_prune, k
     W = blk.repeat(rows * 128).reshape(rows, 1024).contiguous()
     W[:, 512:516] += 0.01
     check_against_oracle(W, 8, k_unify, k_prune, algos=(B.MWU_ALGO_AUTO,))
+
+
+@pytest.mark.parametrize("b", [2, 4, 8, 16])
+@pytest.mark.parametrize("kind", ["ragged", "tiny", "subnormal_keys", "huge", "overflowing_keys", "near_equal", "mixed_scales"])
+def test_projection_one_pass_fp32_classes_are_exact(b, kind):
+    """The sweep decides most classes from fp32 keys: ranges where those keys lose their digits, and a last
+    warp step that the tensor does not fill (512 values).  Classes, losses and Q must match bit for bit."""
+    rows, cols = (37, 512 + b) if kind == "ragged" else (96, 1024)
+    W = inputs.normal_weights(rows, cols, 0.02, 7000 + b)
+    scale = {"tiny": 1e-12, "subnormal_keys": 1e-20, "huge": 1e16, "overflowing_keys": 1e21}
+    if kind in scale:
+        W = W * scale[kind]
+    elif kind == "near_equal":                       # L_u far below the rounding of the fp32 mean
+        g = torch.Generator().manual_seed(b)
+        W = torch.where(W < 0, -1.0, 1.0) * (1.0 + torch.randint(0, 4, W.shape, generator=g) * 2.0 ** -23)
+    elif kind == "mixed_scales":                     # a few blocks of a far larger mean
+        W[::7, : cols // 2] *= 1e9
+    Mb = rows * cols // b
+    check_against_oracle(W.contiguous(), b, Mb * 5 // 10, Mb * 25 // 100, algos=(B.MWU_ALGO_ONE_PASS,))
