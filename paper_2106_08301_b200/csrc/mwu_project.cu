@@ -39,10 +39,12 @@ constexpr int CAP = 2048;       // candidates sorted by the last step
 // sample blocks ranked by sample_kernel: at most NSAMP_MAX, SAMP_PER to a thread
 constexpr int SAMP_CTAS = 8, SAMP_THREADS = 1024, SAMP_PER = 8;
 constexpr int NSAMP_MAX = SAMP_CTAS * SAMP_THREADS * SAMP_PER;
+constexpr int SAMP_A = 128;       // of the samples, ranked first
 constexpr int NSAMP_SMALL_LG = 14, NSAMP_LG = 16;
 static_assert(NSAMP_MAX == 1 << NSAMP_LG, "the larger sample fills the cluster");
 constexpr int STAGE_ENTRIES = 64;  // per-warp staging of candidate-list entries in pass_kernel
-constexpr int FIN_THREADS = 1024;   // block size of the kernels whose last CTA finalises
+constexpr int FIN_THREADS = 1024;   // block size of the kernels that scan the histograms
+constexpr int PASS_GROUPS = 8;      // groups of CTAs of pass_kernel that share out its last steps
 static_assert(NB_MAX / FIN_THREADS <= 64, "scan_hist searches one thread's bins with one warp, two per lane");
 
 typedef unsigned long long u64;
@@ -75,13 +77,12 @@ struct Work {
     Filter filter;
     // one-pass pipeline
     unsigned fcand_count[2];    // threshold-bin candidates of the two halves of resolve_kernel
-    unsigned fticket[2];
     unsigned list_count;        // entries appended to the candidate list
     unsigned failed;            // != 0: the one-pass result is void, the exact phases run
     u64 That[2];                // provisional thresholds (key bit patterns)
-    unsigned release;           // resolve_kernel: the prune threshold and the unify bin are published
     unsigned bar;               // resolve_kernel: arrivals at its grid barriers (only ever grows)
     unsigned pad1[2];
+    struct __align__(128) { unsigned ticket; } group[PASS_GROUPS];      // pass_kernel: steps of its last part given out to a group of CTAs
 };
 
 struct Params {
@@ -260,7 +261,8 @@ __device__ __forceinline__ void load16(const float *W, const float *U, long long
 __device__ __forceinline__ void set_window(Sel *s, u64 lo, u64 hi, int nb) {
     if (hi < lo) hi = lo;
     const int width = 64 - __clzll((long long)(hi - lo));
-    unsigned shift = width > 16 ? (unsigned)(width - 16) : 0u;         // nb - 2 < 2^16: start just below
+    const int nb_bits = 31 - __clz(nb);
+    unsigned shift = width > nb_bits ? (unsigned)(width - nb_bits) : 0u;      // one more when the last bins would be missed
     while (((hi - lo) >> shift) >= (u64)(nb - 2)) ++shift;
     s->lo0 = lo;
     s->hi0 = hi;
@@ -320,61 +322,56 @@ __device__ __forceinline__ void window_ranks_f(int n, float frac, int *il, int *
 }
 
 // Level-B counts of one selection; the cluster adds its eight up
-struct SampCounts {
+struct __align__(16) SampCounts {
     unsigned bins[SAMP_THREADS];
     unsigned under, n_valid;
 };
+constexpr unsigned NO_SAMPLE = 0xffffffffu;           // key of a sample that takes no part: above every window
 
-// One selection of sample_kernel, by all CTAs of the cluster alike.  key[t] / valid[t]: this thread's
-// sample keys (bits of non-negative floats); a_key / a_valid: the level-A key that this thread and its
-// three neighbours rank.  `frac` of the valid ones are to be selected.  Level A ranks 256 of the sample
-// keys to get a coarse window; level B counts all valid ones in SAMP_THREADS bins across that window and
+// One selection of sample_kernel, by all CTAs of the cluster alike.  key[t]: this thread's sample keys (bits of non-negative floats, or NO_SAMPLE);
+// a_key: the level-A key that this thread and its seven neighbours rank.  `frac` of the keys are to be selected.  Level A
+// ranks 128 of the sample keys to get a coarse window; level B counts all in SAMP_THREADS bins across that window and
 // reads the final window [lo, hi) and the provisional threshold from the bin edges.  c: cleared before a
-// cluster barrier.
-__device__ void sample_select(const unsigned (&key)[SAMP_PER], const unsigned (&valid)[SAMP_PER], unsigned a_key, bool a_valid,
-                              float frac, SampCounts *c, unsigned *lo_out, unsigned *hi_out, unsigned *t_out) {
-    constexpr int NA = SAMP_THREADS / 4;
-    // level-A keys, shortened to the top 24 bits below the (clear) sign bit, with the key's index in
-    // the low byte: distinct words, one 32-bit compare per pair; invalid keys rank last
-    __shared__ __align__(16) unsigned s_a[NA];
+// cluster barrier.  all: room for the cluster's counts.
+__device__ __forceinline__ uint3 sample_select(const unsigned (&key)[SAMP_PER], unsigned a_key, float frac, SampCounts *c, uint4 *all) {
+    constexpr int A_PARTS = SAMP_THREADS / SAMP_A;
+    // level-A keys, shortened to the top 25 bits below the (clear) sign bit, with the key's index in
+    // the low seven: distinct words, one 32-bit compare per pair; invalid keys rank last
+    __shared__ __align__(16) unsigned s_a[SAMP_A];
     __shared__ unsigned s_edge[2];                    // shortened keys at the coarse window's ranks
     __shared__ unsigned s_warp[32];
     __shared__ unsigned s_res[3];
-    static_assert(NA == 256, "the index of a level-A key fills the low byte of its shortened form");
-    const int tid = threadIdx.x, lane = tid & 31;
-    const bool is_a = (tid % 4) == 0;
-    const int a = tid / 4;
-    a_valid = a_valid && is_a;
+    static_assert(SAMP_A == 128 && A_PARTS == 8, "the index of a level-A key fills the low seven bits of its shortened form");
+    const int tid = threadIdx.x, lane = tid & 31, a = tid / A_PARTS, part = tid % A_PARTS;
+    const bool a_valid = part == 0 && a_key != NO_SAMPLE;
     __syncthreads();                                  // an earlier call's shared words are no longer read
-    if (is_a) s_a[a] = a_valid ? ((a_key >> 7) << 8) | (unsigned)a : 0xffffffffu;
+    if (part == 0) s_a[a] = a_valid ? (((a_key << 1) >> 7) << 7) | (unsigned)a : 0xffffffffu;
     const int na_raw = __syncthreads_count(a_valid);  // also orders the stores above
     const int na = na_raw > 0 ? na_raw : 1;
     int il, ih, ipos;
     window_ranks_f(na, frac, &il, &ih, &ipos);
     {
-        // four threads rank one level-A key, each against a quarter of the keys (every fourth
-        // group of four: the four threads read 64 contiguous bytes, no bank conflict)
-        const int part = tid % 4;
+        // eight threads rank one level-A key, each against an eighth of the keys (neighbours read neighbouring
+        // 16 bytes, no bank conflict)
         const unsigned k = s_a[a];
         int r = 0;
         const uint4 *q = reinterpret_cast<const uint4 *>(s_a) + part;
-#pragma unroll 4
-        for (int t = 0; t < NA / 16; ++t) {
-            const uint4 x = q[4 * t];
+#pragma unroll
+        for (int t = 0; t < SAMP_A / 4 / A_PARTS; ++t) {
+            const uint4 x = q[A_PARTS * t];
             r += (x.x < k ? 1 : 0) + (x.y < k ? 1 : 0) + (x.z < k ? 1 : 0) + (x.w < k ? 1 : 0);
         }
-        r += __shfl_xor_sync(0xffffffffu, r, 1);
-        r += __shfl_xor_sync(0xffffffffu, r, 2);
-        if (is_a) {
+#pragma unroll
+        for (int m = 1; m < A_PARTS; m <<= 1) r += __shfl_xor_sync(0xffffffffu, r, m);
+        if (part == 0) {
             if (r == il) s_edge[0] = k;
             if (r == ih) s_edge[1] = k;
         }
     }
     __syncthreads();
-    // back to full keys: the low 7 bits of the edges are zero (any window is a valid window)
-    unsigned clo = (s_edge[0] >> 8) << 7, chi = (s_edge[1] >> 8) << 7;
-    if (s_edge[0] == 0xffffffffu) clo = 0x7fffffffu;
-    if (s_edge[1] == 0xffffffffu) chi = 0x7fffffffu;
+    // back to full keys: the low 6 bits of the edges are zero (any window is a valid window)
+    const unsigned clo = s_edge[0] == 0xffffffffu ? 0x7fffffffu : (s_edge[0] >> 7) << 6;
+    unsigned chi = s_edge[1] == 0xffffffffu ? 0x7fffffffu : (s_edge[1] >> 7) << 6;
     if (chi < clo) chi = clo;
     // smallest shift with ((chi - clo) >> shift) < SAMP_THREADS (a power of two)
     const int width = 32 - __clz((int)(chi - clo));                    // bits of chi - clo
@@ -384,11 +381,10 @@ __device__ void sample_select(const unsigned (&key)[SAMP_PER], const unsigned (&
     unsigned n_under = 0, n_valid = 0;
 #pragma unroll
     for (int t = 0; t < SAMP_PER; ++t) {
-        if (!valid[t]) continue;
-        ++n_valid;
-        const unsigned k = key[t];
-        if (k < clo) ++n_under;
-        else if (k < chi) atomicAdd(&c->bins[(k - clo) >> shift], 1u);
+        const unsigned d = key[t] - clo;
+        if (d < chi - clo) atomicAdd(&c->bins[d >> shift], 1u);
+        n_under += key[t] < clo ? 1u : 0u;
+        n_valid += key[t] != NO_SAMPLE ? 1u : 0u;
     }
     n_under = __reduce_add_sync(0xffffffffu, n_under);
     n_valid = __reduce_add_sync(0xffffffffu, n_valid);
@@ -398,17 +394,29 @@ __device__ void sample_select(const unsigned (&key)[SAMP_PER], const unsigned (&
     }
     sel::ClusterTeam::arrive();
     sel::ClusterTeam::wait();
-    unsigned mine = 0, under = 0, total = 0;
+    // The bins of all CTAs come here as 16-byte words, two to a thread, and are added up out of shared memory (eight 4-byte
+    // loads by every thread took 1.7 us); the two totals are read by one lane each (32 lanes that read one word of
+    // another CTA are served one by one).
+    unsigned under = 0, total = 0;
+    constexpr int WORDS = SAMP_THREADS / 4;           // of 16 bytes
 #pragma unroll
-    for (unsigned r = 0; r < SAMP_CTAS; ++r) {
-        unsigned x, y, z;
-        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x) : "r"(sel::ClusterTeam::in_cta(sel::ClusterTeam::addr(&c->bins[tid]), r)) : "memory");
-        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(y) : "r"(sel::ClusterTeam::in_cta(sel::ClusterTeam::addr(&c->under), r)) : "memory");
-        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(z) : "r"(sel::ClusterTeam::in_cta(sel::ClusterTeam::addr(&c->n_valid), r)) : "memory");
-        mine += x;
-        under += y;
-        total += z;
+    for (int h = 0; h < SAMP_CTAS * WORDS / SAMP_THREADS; ++h) {
+        const int w = h * SAMP_THREADS + tid;
+        uint4 x;
+        asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w)
+                     : "r"(sel::ClusterTeam::in_cta(sel::ClusterTeam::addr(&c->bins[(w % WORDS) * 4]), (unsigned)(w / WORDS))) : "memory");
+        all[w] = x;
     }
+    if (lane < SAMP_CTAS)
+        asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];"
+                     : "=r"(under), "=r"(total) : "r"(sel::ClusterTeam::in_cta(sel::ClusterTeam::addr(&c->under), (unsigned)lane)) : "memory");
+    under = __reduce_add_sync(0xffffffffu, under);
+    total = __reduce_add_sync(0xffffffffu, total);
+    __syncthreads();
+    unsigned mine = 0;
+#pragma unroll
+    for (int r = 0; r < SAMP_CTAS; ++r) mine += reinterpret_cast<const unsigned *>(all)[r * SAMP_THREADS + tid];
     const unsigned incl = block_scan_incl(mine, s_warp) + under;
     const unsigned excl = incl - mine;
     window_ranks_f(total > 0u ? (int)total : 1, frac, &il, &ih, &ipos);
@@ -432,9 +440,7 @@ __device__ void sample_select(const unsigned (&key)[SAMP_PER], const unsigned (&
     unsigned That = s_res[2];
     if (That < lo) That = lo;
     if (hi > lo && That >= hi) That = hi - 1;         // the provisional threshold lies inside [lo, hi)
-    *lo_out = lo;
-    *hi_out = hi;
-    *t_out = That;
+    return make_uint3(lo, hi, That);
 }
 
 // block of the i-th of the evenly spaced samples, without a division (their number is a power of
@@ -473,6 +479,7 @@ __global__ void __launch_bounds__(128) sample_keys_kernel(Params p, unsigned *ze
 // blocks of a 50 % / 25 % projection were listed, with 65536 it is 3 %.
 __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
     __shared__ SampCounts s_counts[2];
+    __shared__ uint4 s_all[SAMP_CTAS * SAMP_THREADS / 4];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (blockIdx.x == 0) {
         unsigned *w = reinterpret_cast<unsigned *>(p.work);
@@ -487,24 +494,23 @@ __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
     const bool by_group = p.gprune != nullptr;
     const int ns = p.n_samp;
     constexpr unsigned SIGN = 0x80000000u;
-    unsigned kp[SAMP_PER], ku[SAMP_PER], valid[SAMP_PER];
-#pragma unroll
-    for (int t = 0; t < SAMP_PER; ++t) {
-        const int i = (t * SAMP_CTAS + (int)blockIdx.x) * SAMP_THREADS + (int)threadIdx.x;
+    unsigned kp[SAMP_PER], ku[SAMP_PER];
+    auto take = [&](int i, unsigned *k0, unsigned *k1) {
         const float2 x = i < ns ? __ldg(&p.samp[i]) : make_float2(0.f, 0.f);
-        kp[t] = __float_as_uint(x.x);
-        ku[t] = __float_as_uint(x.y) & ~SIGN;
-        valid[t] = i < ns && !(by_group && (__float_as_uint(x.y) & SIGN)) ? 1u : 0u;
-    }
-    const int a = (int)threadIdx.x / 4;
-    const int ia = p.samp_lg >= 8 ? a << (p.samp_lg - 8) : a;      // 256 of the samples, evenly spaced
-    const float2 xa = ia < ns ? __ldg(&p.samp[ia]) : make_float2(0.f, 0.f);
-    bool a_valid = ia < ns && !(by_group && (__float_as_uint(xa.y) & SIGN));
+        const bool valid = i < ns && !(by_group && (__float_as_uint(x.y) & SIGN));
+        *k0 = valid ? __float_as_uint(x.x) : NO_SAMPLE;
+        *k1 = valid ? __float_as_uint(x.y) & ~SIGN : NO_SAMPLE;
+    };
+#pragma unroll
+    for (int t = 0; t < SAMP_PER; ++t) take((t * SAMP_CTAS + (int)blockIdx.x) * SAMP_THREADS + (int)threadIdx.x, &kp[t], &ku[t]);
+    const int a = (int)threadIdx.x / (SAMP_THREADS / SAMP_A);
+    unsigned kp_a, ku_a;
+    take(p.samp_lg >= 7 ? a << (p.samp_lg - 7) : a, &kp_a, &ku_a);      // SAMP_A of the samples, evenly spaced
+    static_assert(SAMP_A == 1 << 7, "");
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     Sel *sp = &p.work->sel[0];
     Sel *su = &p.work->sel[1];
     const long long ksel_u = k_unify - k_prune;
-    unsigned lo, hi, That = 0;
     auto key64 = [](unsigned x) { return key_bits((double)__uint_as_float(x < 0x7f800000u ? x : 0x7f800000u)); };
     if (lead && p.resid) *p.resid = 0.0;              // the kernels that follow add to it
     sel::ClusterTeam::arrive();                       // every CTA's counts are cleared
@@ -518,26 +524,27 @@ __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
             p.work->That[0] = 0;
         }
     } else {
-        sample_select(kp, valid, __float_as_uint(xa.x), a_valid, (float)((double)k_prune / (double)mb), &s_counts[0], &lo, &hi, &That);
+        const uint3 wp = sample_select(kp, kp_a, (float)((double)k_prune / (double)mb), &s_counts[0], s_all);
         if (lead) {
-            set_window(sp, key64(lo), key64(hi), p.nb);
+            set_window(sp, key64(wp.x), key64(wp.y), p.nb);
             sp->mode = (k_prune == 0) ? 1u : (k_prune == mb ? 2u : 0u);
             sp->k = (u64)k_prune;
-            p.work->That[0] = key64(That);
+            p.work->That[0] = key64(wp.z);
         }
         // the sample blocks that survive the (estimated) prune threshold
+        if (k_prune != 0) {
 #pragma unroll
-        for (int t = 0; t < SAMP_PER; ++t) valid[t] = valid[t] && (k_prune == 0 || kp[t] > That) ? 1u : 0u;
-        a_valid = a_valid && (k_prune == 0 || __float_as_uint(xa.x) > That);
+            for (int t = 0; t < SAMP_PER; ++t) ku[t] = kp[t] > wp.z ? ku[t] : NO_SAMPLE;
+            ku_a = kp_a > wp.z ? ku_a : NO_SAMPLE;
+        }
     }
     const long long elig = mb - k_prune;
-    sample_select(ku, valid, __float_as_uint(xa.y) & ~SIGN, a_valid, elig > 0 ? (float)((double)ksel_u / (double)elig) : 0.f,
-                  &s_counts[1], &lo, &hi, &That);
+    const uint3 wu = sample_select(ku, ku_a, elig > 0 ? (float)((double)ksel_u / (double)elig) : 0.f, &s_counts[1], s_all);
     if (lead) {
-        set_window(su, key64(lo), key64(hi), p.nb);
+        set_window(su, key64(wu.x), key64(wu.y), p.nb);
         su->mode = (ksel_u == 0) ? 1u : (ksel_u == elig ? 2u : 0u);
         su->k = (u64)ksel_u;
-        p.work->That[1] = key64(That);
+        p.work->That[1] = key64(wu.z);
         make_filter(&p.work->filter, *sp, *su, p.work->That[0], p.work->That[1], p.b);
     }
     sel::ClusterTeam::arrive();                       // nobody leaves while its counts are still read
@@ -545,23 +552,8 @@ __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// finalisation helpers, run by the last CTA of a kernel (FIN_THREADS threads)
+// finalisation helpers, run by whole CTAs of FIN_THREADS threads
 // ---------------------------------------------------------------------------------------------
-// true in exactly one CTA: the one whose threads arrive last.  Everything the other CTAs wrote
-// before is visible to it afterwards.
-__device__ __forceinline__ bool last_block_done(unsigned *ticket) {
-    __shared__ bool s_last;
-    __syncthreads();                       // every write of this CTA happens before thread 0's fence
-    if (threadIdx.x == 0) {
-        __threadfence();                   // cumulative: publishes what the barrier made visible to thread 0
-        const unsigned t = atomicAdd(ticket, 1u);
-        s_last = (t == gridDim.x - 1);
-        if (s_last) __threadfence();
-    }
-    __syncthreads();
-    return s_last;
-}
-
 // find the bin holding the r-th element; hist has nb entries
 // `extra` (shared memory, n_extra bin numbers, may be null): one more element in each of these bins,
 // counted on top of what the histogram holds (the CTA's own corrections, not yet in global memory).
@@ -1198,8 +1190,14 @@ pass_kernel(const __grid_constant__ Params p, float *Q, double *loss_u, double *
     constexpr int NBP = B <= 4 ? 4 / B : NBT;            // of them next to one another
     const long long n = p.n_floats;
     const unsigned n_steps = (unsigned)((n + 511) / 512), stride = gridDim.x * PASS_WARPS;
+    // The last eighth of the steps goes to whichever warp is free: SMs differ by several per cent in how fast they stream
+    // (16384 x 16384, b = 4: with equal shares the last CTA ended 35 us after the first).  Every eighth of those steps belongs
+    // to one group of CTAs; one counter for all is asked more often than L2 answers.
+    const unsigned n_fixed = max((n_steps - n_steps / 8u) / stride, 1u) * stride;
+    unsigned *ticket = &p.work->group[blockIdx.x % PASS_GROUPS].ticket;
+    auto last_step = [&]() { return n_fixed + atomicAdd(ticket, 1u) * PASS_GROUPS + blockIdx.x % PASS_GROUPS; };
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned step = blockIdx.x * PASS_WARPS + warp;
+    unsigned step = blockIdx.x * PASS_WARPS + warp, next = step + stride;
     // Launched with programmatic stream serialization: the CTAs may start while sample_kernel still
     // runs.  The first values do not depend on it and are requested at once; everything
     // sample_kernel writes (windows, cleared histograms) is read only behind the wait.
@@ -1242,13 +1240,19 @@ pass_kernel(const __grid_constant__ Params p, float *Q, double *loss_u, double *
         }
     };
 
+    if (next >= n_fixed) {
+        if (lane == 0) next = last_step();
+        next = __shfl_sync(0xffffffffu, next, 0);
+    }
 #pragma unroll 1
-    for (; step < n_steps; step += stride) {
+    while (step < n_steps) {
         float v[16];
 #pragma unroll
         for (int l = 0; l < 16; ++l) v[l] = nxt[l];
         // the next step's values travel while this one is evaluated
-        if (step + stride < n_steps) load_step<B>(p.W, p.U, step + stride, lane, n, nxt);
+        if (next < n_steps) load_step<B>(p.W, p.U, next, lane, n, nxt);
+        unsigned after = next + stride;                      // the step behind the next: asked for a step ahead
+        if (after >= n_fixed && lane == 0 && next < n_steps) after = last_step();
         const bool full = (long long)step * 512 + 512 <= n;
         const unsigned j0 = step * (512 / B) + (B <= 4 ? lane * NBP : lane * NBT);   // this lane's first block
         auto block_of = [&](int e) { return j0 + (unsigned)(e / NBP) * (128 / B) + (unsigned)(e % NBP); };
@@ -1441,6 +1445,8 @@ pass_kernel(const __grid_constant__ Params p, float *Q, double *loss_u, double *
                 __syncwarp();
             }
         }
+        step = next;
+        next = __shfl_sync(0xffffffffu, after, 0);
     }
     if (fill > 0u) flush(0u, fill);
     // block-level totals of the lowest bins
@@ -1468,6 +1474,19 @@ constexpr unsigned IDX_MASK = 0x3fffffffu;           // list entry: block index;
 
 // Block idx gets final class (pr, un) where pass_kernel had written (pr0, un0): bitmaps, u, Q (and
 // the dual update) are rewritten.  Returns the change of ||V - Q||^2.
+// the B values of block j, with stores as wide as load_block's loads; nothing when dst is null
+template <int B>
+__device__ __forceinline__ void store_block(float *dst, long long j, const float (&q)[B]) {
+    if (!dst) return;
+    if constexpr (B == 2) {
+        *reinterpret_cast<float2 *>(dst + j * 2) = make_float2(q[0], q[1]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < B / 4; ++c)
+            *(reinterpret_cast<float4 *>(dst) + j * (B / 4) + c) = make_float4(q[4 * c], q[4 * c + 1], q[4 * c + 2], q[4 * c + 3]);
+    }
+}
+
 template <int B>
 __device__ __forceinline__ double apply_class(const Params &p, float *Q, float *u_out, unsigned *pruned_bitmap,
                                               unsigned *unified_bitmap, unsigned idx, bool pr, bool un, bool pr0,
@@ -1476,18 +1495,27 @@ __device__ __forceinline__ double apply_class(const Params &p, float *Q, float *
     unsigned *wp = pruned_bitmap + (idx >> 5), *wu = unified_bitmap + (idx >> 5);
     if (pr != pr0) { if (pr) atomicOr(wp, bit); else atomicAnd(wp, ~bit); }
     if (un != un0) { if (un) atomicOr(wu, bit); else atomicAnd(wu, ~bit); }
+    // each of these is a trip to DRAM: only what the change needs
     const long long j = (long long)idx;
     float v[B];
-    load_block<B>(p.W, p.U, j, v);
-    double S, Lu, Kp;
-    block_keys<B>(v, p.use_l1, &S, &Lu, &Kp);
-    const float qf = __double2float_rn(__dmul_rn(S, 1.0 / (double)B));
-    u_out[j] = un ? qf : 0.f;
+    double S = 0.0, Lu = 0.0, Kp = 0.0;
+    if (!pr || p.U_next || p.resid) {
+        load_block<B>(p.W, p.U, j, v);
+        block_keys<B>(v, p.use_l1, &S, &Lu, &Kp);
+    } else {
 #pragma unroll
-    for (int l = 0; l < B; ++l) {
-        const float q = pr ? 0.f : (un ? (v[l] < 0.f ? -qf : qf) : v[l]);
-        if (Q) Q[j * B + l] = q;
-        if (p.U_next) p.U_next[j * B + l] = __fsub_rn(v[l], q);
+        for (int l = 0; l < B; ++l) v[l] = 0.f;
+    }
+    const float qf = __double2float_rn(__dmul_rn(S, 1.0 / (double)B));
+    if (un || un0) u_out[j] = un ? qf : 0.f;
+    float q[B];
+#pragma unroll
+    for (int l = 0; l < B; ++l) q[l] = pr ? 0.f : (un ? (v[l] < 0.f ? -qf : qf) : v[l]);
+    store_block<B>(Q, j, q);
+    if (p.U_next) {
+#pragma unroll
+        for (int l = 0; l < B; ++l) q[l] = __fsub_rn(v[l], q[l]);
+        store_block<B>(p.U_next, j, q);
     }
     // change of ||V - Q||^2: the loss of the new class minus that of the provisional one
     if (!p.resid) return 0.0;
@@ -1495,10 +1523,10 @@ __device__ __forceinline__ double apply_class(const Params &p, float *Q, float *
     return (pr ? sq : (un ? Lu : 0.0)) - (pr0 ? sq : (un0 ? Lu : 0.0));
 }
 
-constexpr int RES_SMEM_BYTES = (int)sizeof(ExactSmem<FIN_THREADS>);
-constexpr int CHG_PER_THREAD = 3;                    // list entries a thread classifies before the changed ones are applied
-static_assert(RES_SMEM_BYTES >= CAP * 20 + CHG_PER_THREAD * FIN_THREADS * 8,
-              "candidate buffers, corrections and the compaction buffer share the staging memory");
+constexpr int CHG_PER_THREAD = 4;                    // list entries a thread classifies before the changed ones are applied
+// candidate buffers, corrections and the compaction buffer; the fallback's staging memory
+constexpr int RES_SMEM_USED = CAP * 20 + CHG_PER_THREAD * FIN_THREADS * 8;
+constexpr int RES_SMEM_BYTES = RES_SMEM_USED > (int)sizeof(ExactSmem<FIN_THREADS>) ? RES_SMEM_USED : (int)sizeof(ExactSmem<FIN_THREADS>);
 
 // rank the m candidates in shared memory (c_key, c_idx) by (key, index); m <= CAP
 // c_aux (when the candidates fit one per thread: the return value) receives g_aux in the same order
@@ -1551,10 +1579,10 @@ __device__ bool rank_candidates(const Params &p, const u64 *g_key, const unsigne
 //      histogram, and finds the unify threshold bin.
 //   3  every CTA gives the blocks of its list slice their final class: the class pass_kernel wrote
 //      travels in the entry, so nothing is read for the nine in ten whose class stands; the others
-//      are gathered 32 to a warp and rewritten.  Blocks of the unify threshold bin are ranked by
-//      the CTA that finishes last, which fixes the threshold element and their classes.
+//      are gathered 32 to a warp and rewritten.  Blocks of the unify threshold bin become candidates.
 //      -- grid barrier --
-//   4  if any step gave the one-pass result up (a threshold outside its window, a threshold bin or
+//   4  one CTA ranks those, which fixes the threshold element and their classes.
+//   5  if any step gave the one-pass result up (a threshold outside its window, a threshold bin or
 //      tie group too large to rank, a full list), the exact phases redo the projection here.
 template <int B>
 __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_constant__ Params p,
@@ -1571,6 +1599,15 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
     unsigned *s_extra = reinterpret_cast<unsigned *>(mp_smem + CAP * 16);               // bins of surviving candidates
     unsigned *s_chg = reinterpret_cast<unsigned *>(mp_smem + CAP * 20);                 // entries whose class changes
     unsigned k = 0;                                    // grid barriers passed
+    // a thread's first list entries travel while the selection state is read (whatever lies there beyond the list's end: looked
+    // at once its length is known), and serve both passes over the list
+    const unsigned gstride = gridDim.x * blockDim.x, i_first = blockIdx.x * blockDim.x + threadIdx.x;
+    uint2 ent0[CHG_PER_THREAD];
+#pragma unroll
+    for (int t = 0; t < CHG_PER_THREAD; ++t) {
+        const unsigned i = i_first + (unsigned)t * gstride;
+        ent0[t] = i < p.list_cap ? __ldg(&p.list[i]) : make_uint2(0u, 0u);
+    }
     load_work(p.work, &w);
     Sel *sp = &p.work->sel[0];
     Sel *su = &p.work->sel[1];
@@ -1601,16 +1638,17 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
             const u128 lo0 = from_halves(s_sel.lo_hi, s_sel.lo_lo);
             const u128 hi0 = from_halves(s_sel.hi_hi, s_sel.hi_lo);
             // a thread's entries are requested together (each iteration would otherwise wait for its own load)
-            const unsigned gstride = gridDim.x * blockDim.x;
-            for (unsigned i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < n_list; i0 += 4u * gstride) {
-              uint2 ent[4];
+#pragma unroll 1
+            for (unsigned i0 = i_first; i0 < n_list; i0 += CHG_PER_THREAD * gstride) {
+              uint2 ent[CHG_PER_THREAD];
 #pragma unroll
-              for (int t4 = 0; t4 < 4; ++t4) {
+              for (int t4 = 0; t4 < CHG_PER_THREAD; ++t4) {
                   const unsigned i = i0 + (unsigned)t4 * gstride;
-                  ent[t4] = i < n_list ? __ldg(&p.list[i]) : make_uint2(0u, 0u);      // code 0: skipped below
+                  if (i0 == i_first) ent[t4] = i < n_list ? ent0[t4] : make_uint2(0u, 0u);
+                  else ent[t4] = i < n_list ? __ldg(&p.list[i]) : make_uint2(0u, 0u);      // code 0: skipped below
               }
 #pragma unroll
-              for (int t4 = 0; t4 < 4; ++t4) {
+              for (int t4 = 0; t4 < CHG_PER_THREAD; ++t4) {
                 const uint2 e = ent[t4];
                 const unsigned idx = e.x & IDX_MASK;
                 const unsigned bp = e.y & 0xffffu, bu = e.y >> 16;
@@ -1685,6 +1723,7 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
         double resid_delta = 0.0;
         const unsigned per_round = CHG_PER_THREAD * gridDim.x * blockDim.x;
         const unsigned rounds = (n_list + per_round - 1u) / per_round;
+#pragma unroll 1
         for (unsigned rd = 0; rd < rounds; ++rd) {
             if (threadIdx.x == 0) s_n_chg = 0;
             __syncthreads();
@@ -1694,7 +1733,8 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
             for (int t3 = 0; t3 < CHG_PER_THREAD; ++t3) {
                 const unsigned i = ((rd * CHG_PER_THREAD + t3) * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
                 have[t3] = i < n_list;
-                ent[t3] = have[t3] ? __ldg(&p.list[i]) : make_uint2(0u, 0u);
+                if (rd == 0u) ent[t3] = ent0[t3];
+                else ent[t3] = have[t3] ? __ldg(&p.list[i]) : make_uint2(0u, 0u);
             }
 #pragma unroll
             for (int t3 = 0; t3 < CHG_PER_THREAD; ++t3) {
@@ -1708,7 +1748,7 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
                 if (!pr) {
                     if (mode_u == 2u) un = true;
                     else if (mode_u == 0u) {
-                        if (bu == Bu) {                            // ranked by the last CTA
+                        if (bu == Bu) {                            // ranked after the barrier
                             const u64 key = exact_key<B>(p, (long long)idx, 1);
                             const u128 c = make_c(key, (u64)idx);
                             if (c >= lo && c < hi) {
@@ -1742,37 +1782,36 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
             __syncthreads();
         }
         if (p.resid) block_add_double(resid_delta, p.resid);
-        if (mode_u == 0u && last_block_done(&p.work->fticket[1])) {
-            // ---- the CTA that finishes last: the blocks of the unify threshold bin ----
-            const unsigned m = ld_vol(&p.work->fcand_count[1]);
-            if (m > (unsigned)CAP || r_u < 1 || r_u > (u64)m) {
-                if (threadIdx.x == 0) one_pass_fail(p);
-            } else {
-                const bool have_aux = rank_candidates(p, p.cand_key + CAP, p.cand_idx + CAP, p.cand_aux + CAP, m, c_key,
-                                                      c_idx, c_aux);
-                if (threadIdx.x == 0) { su->T_key = c_key[r_u - 1]; su->T_idx = (u64)c_idx[r_u - 1]; }
-                const unsigned r = (unsigned)r_u;
-                double tail_delta = 0.0;
-                for (unsigned i = threadIdx.x; i < m; i += blockDim.x) {
-                    // the class pass_kernel wrote for this block: carried with the candidate, else read back
-                    const unsigned idx = c_idx[i], bit = 1u << (idx & 31u);
-                    const bool pr0 = have_aux ? ((c_aux[i] >> 1) & 1u) != 0u : (ld_vol(pruned_bitmap + (idx >> 5)) & bit) != 0u;
-                    const bool un0 = have_aux ? (c_aux[i] & 1u) != 0u : (ld_vol(unified_bitmap + (idx >> 5)) & bit) != 0u;
-                    const bool un = i < r;
-                    if (pr0 || un != un0)
-                        tail_delta += apply_class<B>(p, Q, u_out, pruned_bitmap, unified_bitmap, idx, false, un, pr0, un0);
-                }
-                if (p.resid) block_add_double(tail_delta, p.resid);
-            }
-        }
     }
-    // ---------------- 4: the fallback, if the one-pass result was given up anywhere ----------------
     if (!grid_sync(&p.work->bar, ++k)) {
         if (threadIdx.x == 0) atomicOr(p.dev_status, (unsigned)MWU_DEV_TIMEOUT);
         return;
     }
-    load_work(p.work, &w);
-    if (w.failed == 0u) return;
+    // ---------------- 4: the blocks of the unify threshold bin ----------------
+    const unsigned m = ld_vol(&p.work->fcand_count[1]);
+    bool failed = ld_vol(&p.work->failed) != 0u;          // both settled: the same in all CTAs
+    if (alive && !failed && mode_u == 0u) {
+        if (m > (unsigned)CAP || r_u < 1 || r_u > (u64)m) failed = true;
+        else if (blockIdx.x == 0) {
+            const bool have_aux = rank_candidates(p, p.cand_key + CAP, p.cand_idx + CAP, p.cand_aux + CAP, m, c_key,
+                                                  c_idx, c_aux);
+            if (threadIdx.x == 0) { su->T_key = c_key[r_u - 1]; su->T_idx = (u64)c_idx[r_u - 1]; }
+            const unsigned r = (unsigned)r_u;
+            double tail_delta = 0.0;
+            for (unsigned i = threadIdx.x; i < m; i += blockDim.x) {
+                // the class pass_kernel wrote for this block: carried with the candidate, else read back
+                const unsigned idx = c_idx[i], bit = 1u << (idx & 31u);
+                const bool pr0 = have_aux ? ((c_aux[i] >> 1) & 1u) != 0u : (ld_vol(pruned_bitmap + (idx >> 5)) & bit) != 0u;
+                const bool un0 = have_aux ? (c_aux[i] & 1u) != 0u : (ld_vol(unified_bitmap + (idx >> 5)) & bit) != 0u;
+                const bool un = i < r;
+                if (pr0 || un != un0)
+                    tail_delta += apply_class<B>(p, Q, u_out, pruned_bitmap, unified_bitmap, idx, false, un, pr0, un0);
+            }
+            if (p.resid) block_add_double(tail_delta, p.resid);
+        }
+    }
+    // ---------------- 5: the fallback, if the one-pass result was given up anywhere ----------------
+    if (!failed) return;
     ExactSmem<FIN_THREADS> &sm = *reinterpret_cast<ExactSmem<FIN_THREADS> *>(mp_smem);
     sel::GridTeam team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u};
     const Outs o = {Q, loss_u, loss_p, u_out, pruned_bitmap, unified_bitmap, sign_bits};
