@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 #include <stddef.h>
+#include <atomic>
 
 #include "mwu.h"
 
@@ -137,6 +138,36 @@ inline cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block,
     cfg.attrs = attr;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// Can this device run clusters of `ctas` CTAs, one to an SM?  Sixteen is more than every device has to offer.  A fact of
+// the device: asked once for each, with any kernel that uses such clusters.
+template <typename... KArgs>
+inline bool cluster_runs(void (*kern)(KArgs...), int ctas, int threads) {
+    constexpr int DEVICES = 64;
+    static std::atomic<signed char> known[DEVICES];         // 0: not asked yet, 1: yes, -1: no
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= DEVICES) return false;
+    signed char k = known[dev].load(std::memory_order_relaxed);
+    if (k == 0) {
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)ctas;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)ctas);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        const bool yes = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                         cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0;
+        if (!yes) cudaGetLastError();
+        k = yes ? 1 : -1;
+        known[dev].store(k, std::memory_order_relaxed);
+    }
+    return k > 0;
 }
 
 // adds n to the process-wide count of kernels launched (mwu_kernel_launches)

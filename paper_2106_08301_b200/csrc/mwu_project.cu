@@ -996,7 +996,7 @@ constexpr int GR_THREADS = 512;                          // grid form
 constexpr int EX_SLOTS = 8192;                           // most blocks a CTA holds: 16 bytes of keys each
 
 // The whole projection in one launch, keys held in shared memory: `units` units of 64 bytes a thread.
-// CLUSTER: one cluster of eight CTAs; otherwise a cooperative grid over a counter that the host has
+// CLUSTER: one cluster of sixteen CTAs; otherwise a cooperative grid over a counter that the host has
 // cleared.
 template <int B, bool CLUSTER>
 __global__ void __launch_bounds__(CLUSTER ? CL_THREADS : GR_THREADS) exact_kernel(Params p, Outs o, sel::Problem pb, unsigned units) {
@@ -1018,7 +1018,8 @@ __global__ void __launch_bounds__(CLUSTER ? CL_THREADS : GR_THREADS) exact_kerne
         team.k = 0;
     }
     float v[16];
-    const unsigned first = blockIdx.x * NT + threadIdx.x;
+    // warps are dealt out over the CTAs, so that a tensor with less than a unit a thread keeps all SMs busy
+    const unsigned first = (threadIdx.x >> 5) * gridDim.x * 32u + blockIdx.x * 32u + (threadIdx.x & 31u);
     load16(p.W, p.U, (long long)first * 16, p.n_floats, v);              // in flight beside the sample's loads
     float sp, su;
     const bool samp_ok = sample_of<B, NT>(p, pb, &sp, &su);
@@ -1982,16 +1983,17 @@ static size_t ws_off_gprune(const mwu_proj_desc *d, size_t mb) { return align_up
 
 // Which pipeline, and how many units of 64 bytes a thread of the exact kernel holds.
 //
-// Both lines were measured on whole mwu_project calls (50 % / 25 %, us).  Up to 32768 blocks a cluster
-// beats the grid (256 x 256, b = 4: 18.7 against 27.2; 256 x 1024, b = 16: 23.1 / 27.1; at the line, b = 8:
-// 29.0 / 28.1): its barriers cost half, but its eight SMs also have all the arithmetic.  Up to 4096 blocks a
+// All lines were measured on whole mwu_project calls (50 % / 25 %, us).  One cluster of sixteen CTAs against the grid, whose
+// launch and barriers cost 10 us more but which has all SMs: 256 x 256, b = 4: 15.5 / 25.7; 256 x 512, b = 2 (a unit a thread):
+// 24.8 / 29.9, with 256 x 576 36.2 / 29.9; b = 4, 256 x 768, 49152 blocks: 23.0 / 26.1, 256 x 1024: 26.9 / 25.7; b = 8, 256 x 1152,
+// 18432 units: 24.0 / 25.7; b = 16, 256 x 1152: 19.0 / 23.7, 512 x 1024, 32768 units: 24.4 / 23.8.  Up to 4096 blocks a
 // CTA on every SM (606208 on 148) the exact kernel beats the one-pass pipeline's four launches (512 x 1152,
 // b = 8: 24 against 39; 2048 x 2048, b = 8, 524288 blocks: 45 / 52; 1024 x 2048, b = 4: 42 / 46), beyond it
 // does not (1024 x 2048, b = 2, 1048576 blocks: 67 / 54): the phases' L2 counts grow with the blocks.
 // Larger sample from here on, 65536 blocks instead of 16384 (whole mwu_project calls, 50 % / 25 %, us: 4096 x 4096, b = 4, 4 M
 // blocks: 94.7 against 99.3; 16384 x 16384, b = 4: 709 / 805; below, both sizes take the same time).
 constexpr long long SAMP_LARGE_BLOCKS = 1ll << 22;
-constexpr long long EX_CLUSTER_BLOCKS = 32768, EX_AUTO_BLOCKS_PER_CTA = 4096;
+constexpr long long EX_CLUSTER_BLOCKS = 49152, EX_CLUSTER_UNITS = 20480, EX_AUTO_BLOCKS_PER_CTA = 4096;
 struct Route {
     bool one_pass, cluster;         // else the exact kernel: as one cluster or as a cooperative grid
     int grid, held;                 // its CTAs and units per thread (0: keys evaluated in every phase)
@@ -2007,11 +2009,12 @@ static Route route_of(const mwu_proj_desc *desc, int sm_count) {
         r.one_pass = true;
         return r;
     }
-    r.cluster = mb <= EX_CLUSTER_BLOCKS;
+    r.cluster = ((mb <= EX_CLUSTER_BLOCKS && units <= EX_CLUSTER_UNITS) || units <= sel::CLUSTER_CTAS * proj::CL_THREADS) &&
+                cluster_runs(proj::exact_kernel<16, true>, sel::CLUSTER_CTAS, proj::CL_THREADS);
     const long long threads = r.cluster ? proj::CL_THREADS : proj::GR_THREADS;
-    const long long ctas = (units + threads - 1) / threads;          // with one unit a thread
+    const long long ctas = (units + 127) / 128;                      // four warps with a unit a lane
     r.grid = r.cluster ? sel::CLUSTER_CTAS : (int)(ctas < sm_count ? ctas : sm_count);
-    const long long held = (ctas + r.grid - 1) / r.grid;
+    const long long held = (units + r.grid * threads - 1) / (r.grid * threads);
     if (held * threads * (16 / desc->block) <= proj::EX_SLOTS) r.held = (int)held;
     else {
         r.cluster = false;
@@ -2055,6 +2058,7 @@ static cudaError_t launch_exact_held(const mwu::proj::Params &p, const mwu::proj
     auto kern = route.cluster ? exact_kernel<B, true> : exact_kernel<B, false>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, EX_SLOTS * 16);
     if (e != cudaSuccess) return e;
+    if (route.cluster && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return cudaErrorUnknown;
     if (!route.cluster)
         return launch_cooperative(kern, route.grid, threads, (size_t)smem, sm_count, st, p, o, pb, (unsigned)route.held);
     mwu::count_launch();

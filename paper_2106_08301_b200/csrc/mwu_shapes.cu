@@ -243,6 +243,8 @@ __global__ void __launch_bounds__(256) lower_kernel(long long n_runs, long long 
     }
 }
 
+constexpr int SH_CLUSTER_PER = 2;                        // most blocks of a thread in the cluster form
+
 static int grid_for(long long items, int sm_count) {
     const long long want = (items + 255) / 256, cap = (long long)sm_count * 16;
     return (int)(want < cap ? (want > 0 ? want : 1) : cap);
@@ -255,14 +257,16 @@ template <int N>
 static cudaError_t launch(const SParams &p, const mwu_proj_desc *desc, int sm_count, cudaStream_t st) {
     const long long mb = p.mb, ctas = (mb + SH_THREADS - 1) / SH_THREADS;
     const sel::Problem pb = sel::problem_of(mb, desc->k_prune, desc->k_unify, false, SH_THREADS);
-    // One cluster up to 8192 blocks (two a thread): gathering is most of the work, and a grid has more SMs for
-    // it than the cluster's barriers save (20480 blocks: 34 us as a cluster, 25 as a grid; 5120: 18).  Keys
-    // held while a CTA's fit.
-    if (mb <= 2ll * sel::CLUSTER_CTAS * SH_THREADS) {
+    // One cluster up to 16384 blocks (two a thread): gathering is most of the work, and a grid has more SMs for
+    // it than the cluster's barriers save (9216 blocks: 19.4 us as a cluster, 25.8 as a grid; 18432: 25.5 / 25.8; 27648:
+    // 30.6 / 26.0).  Keys held while a CTA's fit.
+    if (mb <= (long long)SH_CLUSTER_PER * sel::CLUSTER_CTAS * SH_THREADS &&
+        cluster_runs(shape_kernel<2, CLUSTER>, sel::CLUSTER_CTAS, SH_THREADS)) {
         const unsigned per = (unsigned)((ctas + sel::CLUSTER_CTAS - 1) / sel::CLUSTER_CTAS);
         const size_t smem = (size_t)per * SH_THREADS * 16;
-        const cudaError_t e = cudaFuncSetAttribute(shape_kernel<N, CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * SH_THREADS * 16);
+        const cudaError_t e = cudaFuncSetAttribute(shape_kernel<N, CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, SH_CLUSTER_PER * SH_THREADS * 16);
         if (e != cudaSuccess) return e;
+        if (cudaFuncSetAttribute(shape_kernel<N, CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return cudaErrorUnknown;
         count_launch();
         return launch_chained(shape_kernel<N, CLUSTER>, dim3(sel::CLUSTER_CTAS), dim3(SH_THREADS), smem, st, sel::CLUSTER_CTAS, p, pb, per);
     }

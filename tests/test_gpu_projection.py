@@ -345,3 +345,13 @@ def test_projection_one_pass_fp32_classes_are_exact(b, kind):
         W[::7, : cols // 2] *= 1e9
     Mb = rows * cols // b
     check_against_oracle(W.contiguous(), b, Mb * 5 // 10, Mb * 25 // 100, algos=(B.MWU_ALGO_ONE_PASS,))
+
+
+@pytest.mark.parametrize("b,rows,cols", [(2, 256, 512), (2, 256, 514),                  # one unit a thread of the cluster, one more
+                                         (4, 256, 768), (4, 257, 768),                  # the most blocks of the cluster form
+                                         (16, 320, 1024), (16, 321, 1024),              # the most units
+                                         (2, 1, 34), (8, 33, 24)])
+def test_projection_exact_kernel_cluster_edges(b, rows, cols):
+    W = inputs.normal_weights(rows, cols, 0.02, 6100 + b)
+    Mb = rows * cols // b
+    check_against_oracle(W, b, Mb // 2, Mb // 4, algos=(B.MWU_ALGO_AUTO,))
