@@ -12,7 +12,8 @@
 //                 place in the round-robin order of its class list; the places go to shared memory.
 //                 Then the lists leave in list order, consecutive threads writing consecutive
 //                 entries; a dense block's values are read by the lanes that share its 64-byte run.
-// The three are chained with programmatic stream serialization.
+// The three are chained with programmatic stream serialization.  Weights of up to 655360 blocks need fill_kernel alone: its
+// CTAs count what comes before their records themselves.
 #include "mwu_common.cuh"
 
 namespace mwu {
@@ -157,6 +158,43 @@ __device__ __forceinline__ void scan_cluster_sync() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// header and gaps, by the first six warps of a CTA
+__device__ __forceinline__ void write_header(const Params &p) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // the padding between the sections must read as zero (each gap is shorter than the alignment)
+    {
+        const int g = wid - 1;                              // a warp to a gap; the first warp writes the header
+        if (g >= 0 && g < 5)
+            for (unsigned long long a = p.gap[g][0] + lane; a < p.gap[g][1]; a += 32) p.packed[a] = 0;
+    }
+    if (threadIdx.x < 32) {
+        unsigned long long *h = reinterpret_cast<unsigned long long *>(p.packed);
+        unsigned long long v = 0;
+        switch (threadIdx.x) {
+            case 0: v = kMagic; break;
+            case 1: v = 4; break;
+            case 2: v = (unsigned long long)p.rows; break;
+            case 3: v = (unsigned long long)p.cols; break;
+            case 4: v = (unsigned long long)p.b; break;
+            case 5: v = (unsigned long long)p.L.n_pad; break;
+            case 6: v = (unsigned long long)p.L.n_tiles; break;
+            case 7: v = (unsigned long long)p.L.n_stages; break;
+            case 8: v = (unsigned long long)p.L.n_pruned; break;
+            case 9: v = (unsigned long long)p.L.n_unified; break;
+            case 10: v = (unsigned long long)p.L.n_dense; break;
+            case 11: v = (unsigned long long)p.L.n_plist; break;
+            case 12: v = (unsigned long long)p.L.off_rec; break;
+            case 13: v = (unsigned long long)p.L.off_ulist; break;
+            case 14: v = (unsigned long long)p.L.off_dpos; break;
+            case 15: v = (unsigned long long)p.L.off_dpay; break;
+            case 16: v = (unsigned long long)p.L.off_ppos; break;
+            case 17: v = (unsigned long long)p.L.total; break;
+            default: v = 0;
+        }
+        h[threadIdx.x] = v;
+    }
+}
+
 // Bound by latency: a handful of dependent L2 round trips and cluster barriers (8192 records on one CTA, in
 // two rounds, took 13 us).  Counts the records itself when count_kernel has not (`counted` == 0).
 __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(Params p, int counted) {
@@ -268,39 +306,14 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(Params p, int counte
             atomicOr(p.dev_status, (unsigned)MWU_DEV_BOUNDS);
         recs[n_rec] = make_uint4((unsigned)au, (unsigned)ad, (unsigned)ap, 0u);
     }
-    // the padding between the sections must read as zero (each gap is shorter than the alignment)
-    {
-        const int g = wid - 1;                              // a warp to a gap; the first warp writes the header
-        if (g >= 0 && g < 5)
-            for (unsigned long long a = p.gap[g][0] + lane; a < p.gap[g][1]; a += 32) p.packed[a] = 0;
-    }
-    if (threadIdx.x < 32) {
-        unsigned long long *h = reinterpret_cast<unsigned long long *>(p.packed);
-        unsigned long long v = 0;
-        switch (threadIdx.x) {
-            case 0: v = kMagic; break;
-            case 1: v = 4; break;
-            case 2: v = (unsigned long long)p.rows; break;
-            case 3: v = (unsigned long long)p.cols; break;
-            case 4: v = (unsigned long long)p.b; break;
-            case 5: v = (unsigned long long)p.L.n_pad; break;
-            case 6: v = (unsigned long long)p.L.n_tiles; break;
-            case 7: v = (unsigned long long)p.L.n_stages; break;
-            case 8: v = (unsigned long long)p.L.n_pruned; break;
-            case 9: v = (unsigned long long)p.L.n_unified; break;
-            case 10: v = (unsigned long long)p.L.n_dense; break;
-            case 11: v = (unsigned long long)p.L.n_plist; break;
-            case 12: v = (unsigned long long)p.L.off_rec; break;
-            case 13: v = (unsigned long long)p.L.off_ulist; break;
-            case 14: v = (unsigned long long)p.L.off_dpos; break;
-            case 15: v = (unsigned long long)p.L.off_dpay; break;
-            case 16: v = (unsigned long long)p.L.off_ppos; break;
-            case 17: v = (unsigned long long)p.L.total; break;
-            default: v = 0;
-        }
-        h[threadIdx.x] = v;
-    }
+    write_header(p);
 }
+
+constexpr unsigned OWN_THREADS = 512;
+// Most blocks (padding rows included) of the form without a scan: every CTA reads on average half of the bitmaps.  Whole
+// mwu_pack calls, us, with it and without: 256 x 256, b = 4: 8.5 / 13.0; 1000 x 1216, b = 2: 13.7 / 17.0; 2048 x 2048, b = 8,
+// 524288 blocks: 12.5 / 15.1; 3072 x 2048, b = 8, 786432: 19.0 / 19.7; 1024 x 2048, b = 2, 1048576: 26.0 / 17.7.
+constexpr long long OWN_BLOCKS = 655360;
 
 // row and block of a tile offset (the inverse of tile_offset)
 __device__ __forceinline__ void row_block_of(unsigned off, int b, unsigned *r, unsigned *i) {
@@ -310,13 +323,18 @@ __device__ __forceinline__ void row_block_of(unsigned off, int b, unsigned *r, u
     *i = (c * 16u + (off & 15u)) / (2u * (unsigned)b);
 }
 
-template <int B>
-__global__ void __launch_bounds__(128) fill_kernel(Params p) {
+// Bounded by latency where records are few (a chain of some dozen L2 round trips, out of a cold instruction cache).
+// OWN: the base of the record's lists is counted here too, from the bitmaps of everything before it: no record table, no
+// kernel before this one; the lists are then written by four times the threads.
+template <int B, bool OWN>
+__global__ void __launch_bounds__(OWN ? OWN_THREADS : 128) fill_kernel(Params p) {
+    constexpr unsigned NT = OWN ? OWN_THREADS : 128;
     constexpr int NBK = kStageK / B;
     constexpr unsigned MASK = (NBK >= 32) ? 0xffffffffu : ((1u << NBK) - 1u);
     constexpr int STORE = (B >= 8) ? 16 : 2 * B;            // bytes of one shared-memory store
     constexpr int G = 128 / STORE;                          // store slots of a 128-byte row
     constexpr int LPB = (B >= 4) ? B / 4 : 1;               // lanes that share a dense block's run of W
+    if (OWN) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned rec = blockIdx.x;
     const unsigned tile_u = rec / p.n_stages;
@@ -334,10 +352,45 @@ __global__ void __launch_bounds__(128) fill_kernel(Params p) {
     __shared__ unsigned short s_full[3][kTileRows + 1];     // per class and q: list entries of rounds 0 .. q-1
     __shared__ unsigned s_more[3][kTileRows + 1];           // per class and q: slots that have a round q
     __shared__ unsigned short s_off[3][kTileRows * NBK];    // tile offsets of each class list, in list order
-    unsigned P, U;
-    unsigned long long sgn;
-    row_masks(p, NBK, tile, stage, r, &P, &U, &sgn);
-    const unsigned D = ~P & ~U & MASK;
+    const bool has_row = !OWN || r < kTileRows;             // a thread to a row; the others join at the lists
+    unsigned P = 0, U = 0, D = 0;
+    if (has_row) {
+        unsigned long long sgn;
+        row_masks(p, NBK, tile, stage, r, &P, &U, &sgn);
+        D = ~P & ~U & MASK;
+    }
+    __shared__ unsigned s_own[3];                           // unified and pruned blocks before the record; its live slices
+    if (OWN) {
+        if (r < 3) s_own[r] = 0u;
+        // whole tiles before this one, then this tile's columns before this record
+        unsigned cu = 0, cp = 0;
+        const long long words = tile * kTileRows * p.bpr / 32;
+        for (long long w = r; w < words; w += NT) {
+            const unsigned x = __ldg(p.pruned_bitmap + w), y = __ldg(p.unified_bitmap + w);
+            cp += __popc(x);
+            cu += __popc(y & ~x);
+        }
+        const long long n = tile * kTileRows + (r & (kTileRows - 1)), j0 = n * p.bpr, j1 = j0 + stage * NBK;
+        if (n < p.rows) {
+            for (long long w = (j0 >> 5) + r / kTileRows; w * 32 < j1; w += NT / kTileRows) {
+                unsigned m = 0xffffffffu;
+                if (w * 32 < j0) m <<= j0 & 31;
+                if (w * 32 + 32 > j1) m &= 0xffffffffu >> (32 - (j1 & 31));
+                const unsigned x = __ldg(p.pruned_bitmap + w) & m, y = __ldg(p.unified_bitmap + w) & m;
+                cp += __popc(x);
+                cu += __popc(y & ~x);
+            }
+        } else if (r < kTileRows) cp += (unsigned)(stage * NBK);             // padding rows are all-pruned
+        const unsigned live = __reduce_or_sync(0xffffffffu, has_row ? live_of(P, B) : 0u);
+        cu = __reduce_add_sync(0xffffffffu, cu);
+        cp = __reduce_add_sync(0xffffffffu, cp);
+        __syncthreads();
+        if (lane == 0) {
+            if (cu) atomicAdd(&s_own[0], cu);
+            if (cp) atomicAdd(&s_own[1], cp);
+            if (live) atomicOr(&s_own[2], live);
+        }
+    }
     // class of block i: 0 pruned, 1 dense, 2 unified.  occ[class]: the store slots this row fills with it
     // (a row never has two blocks in one slot)
     unsigned occ[3] = {0u, 0u, 0u};
@@ -349,18 +402,20 @@ __global__ void __launch_bounds__(128) fill_kernel(Params p) {
         occ[1] |= ((D >> i) & 1u) ? bit : 0u;
         occ[2] |= ((U >> i) & 1u) ? bit : 0u;
     }
+    if (has_row) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+      for (int c = 0; c < 3; ++c) {
 #pragma unroll
         for (int sl = 0; sl < G; ++sl) {
             const unsigned bal = __ballot_sync(0xffffffffu, (occ[c] >> sl) & 1u);
             if (lane == ((c * G + sl) & 31)) s_bal[warp][c * G + sl] = bal;
         }
+      }
     }
     __syncthreads();
     // blocks per (class, slot) in the record, and in the warps before each warp (population counts
     // are few to a clock, so each is taken once per CTA, not once per thread)
-    for (int t = r; t < 4 * 3 * G; t += kTileRows) {
+    for (int t = r; t < 4 * 3 * G; t += (int)NT) {
         const int ww = t / (3 * G), f = t % (3 * G);
         unsigned before = 0;
         for (int w2 = 0; w2 < ww; ++w2) before += __popc(s_bal[w2][f]);
@@ -370,7 +425,7 @@ __global__ void __launch_bounds__(128) fill_kernel(Params p) {
     __syncthreads();
     // round-robin order of a class list: round q takes the q-th block of every slot that has one.
     // Thread q (and thread 0 for q = 128) tabulates what comes before round q.
-    for (int q = r; q <= kTileRows; q += kTileRows) {
+    for (int q = r; q <= kTileRows; q += (int)NT) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             // four slots at a time: bytewise minimum summed with a dot product, bytewise compare
@@ -392,6 +447,7 @@ __global__ void __launch_bounds__(128) fill_kernel(Params p) {
 
     // every block's place in its class list
     const unsigned below = (1u << lane) - 1u;
+    if (has_row)
 #pragma unroll 4
     for (int i = 0; i < NBK; ++i) {
         const unsigned off = tile_offset((unsigned)r, (unsigned)i, B);
@@ -404,9 +460,26 @@ __global__ void __launch_bounds__(128) fill_kernel(Params p) {
         const unsigned idx = s_full[cls][q] + __popc(s_more[cls][q] & ((1u << slot) - 1u));
         s_off[cls][idx] = (unsigned short)off;
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");      // the record table holds the bases
-    const uint4 me = recs[rec], nx = recs[rec + 1];         // (ubase, dbase, pbase, live); the table ends with the totals
-    __syncthreads();
+    uint4 me, nx;                                           // (ubase, dbase, pbase, live); the table ends with the totals
+    if (OWN) {
+        __syncthreads();
+        me = make_uint4(s_own[0], rec * (unsigned)(kTileRows * NBK) - s_own[0] - s_own[1], s_own[1], s_own[2]);
+        nx = make_uint4(me.x + s_full[2][kTileRows], me.y + s_full[1][kTileRows], me.z + s_full[0][kTileRows], 0u);
+        uint4 *table = reinterpret_cast<uint4 *>(p.packed + p.L.off_rec);
+        if (r == 0) table[rec] = me;
+        if (rec == gridDim.x - 1u && r == 0) {
+            table[rec + 1] = nx;
+            if (nx.x != (unsigned long long)p.L.n_unified || nx.y != (unsigned long long)p.L.n_dense ||
+                nx.z != (unsigned long long)p.L.n_plist)
+                atomicOr(p.dev_status, (unsigned)MWU_DEV_BOUNDS);
+        }
+        if (rec == 0u) write_header(p);
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");  // the record table holds the bases
+        me = recs[rec];
+        nx = recs[rec + 1];
+        __syncthreads();
+    }
 
     bool bad = false;
     constexpr unsigned BMASK = (B >= 32) ? 0xffffffffu : ((1u << B) - 1u);
@@ -422,11 +495,11 @@ __global__ void __launch_bounds__(128) fill_kernel(Params p) {
         const long long f_base = row_base * p.cols + stage * kStageK;          // first weight of the record
         // pruned blocks: positions only
         unsigned short *pp = ppos + me.z;
-        for (unsigned t = (unsigned)r; t < len_p; t += 128u) pp[t] = s_off[0][t];
+        for (unsigned t = (unsigned)r; t < len_p; t += NT) pp[t] = s_off[0][t];
         // unified blocks: sign bits, position, magnitude
         uint2 *ul = ulist + me.x;
         const long long j_base = row_base * p.bpr + stage * NBK;
-        for (unsigned t = (unsigned)r; t < len_u; t += 128u) {
+        for (unsigned t = (unsigned)r; t < len_u; t += NT) {
             const unsigned off = s_off[2][t];
             unsigned rr, i;
             row_block_of(off, B, &rr, &i);
@@ -437,9 +510,9 @@ __global__ void __launch_bounds__(128) fill_kernel(Params p) {
         }
         // dense blocks: position, then the values, LPB lanes to a block
         unsigned short *dp = dpos + me.y;
-        for (unsigned t = (unsigned)r; t < len_d; t += 128u) dp[t] = s_off[1][t];
+        for (unsigned t = (unsigned)r; t < len_d; t += NT) dp[t] = s_off[1][t];
         unsigned char *pay = dpay + (unsigned long long)me.y * (2 * B);
-        for (unsigned q = (unsigned)r; q < len_d * (unsigned)LPB; q += 128u) {
+        for (unsigned q = (unsigned)r; q < len_d * (unsigned)LPB; q += NT) {
             const unsigned t = q / (unsigned)LPB, part = q % (unsigned)LPB;
             unsigned rr, i;
             row_block_of(s_off[1][t], B, &rr, &i);
@@ -526,18 +599,30 @@ extern "C" int mwu_pack(const mwu_proj_desc *desc, const float *W, const float *
     // memory themselves.  Up to two units for every team of the scan cluster it counts them itself, in two
     // rounds of loads at most; beyond that a grid of CTAs is faster.
     const long long units = p.L.n_tiles * ((p.L.n_stages + 31) / 32);
+    const bool own = (long long)n_rec * (kTileRows * kStageK / desc->block) <= pack::OWN_BLOCKS;
     const int counted = units > 2 * pack::SCAN_CTAS * (pack::SCAN_THREADS / (32 * pack::COUNT_WARPS)) ? 1 : 0;
     cudaError_t e = cudaSuccess;
+    const dim3 grid((unsigned)n_rec), block(own ? pack::OWN_THREADS : 128u);
+    if (own) {
+        switch (desc->block) {
+            case 2: e = launch_chained(pack::fill_kernel<2, true>, grid, block, 0, st, 1, p); break;
+            case 4: e = launch_chained(pack::fill_kernel<4, true>, grid, block, 0, st, 1, p); break;
+            case 8: e = launch_chained(pack::fill_kernel<8, true>, grid, block, 0, st, 1, p); break;
+            default: e = launch_chained(pack::fill_kernel<16, true>, grid, block, 0, st, 1, p); break;
+        }
+        if (e != cudaSuccess) return MWU_ERR_CUDA;
+        count_launch(1);
+        return cudaGetLastError() == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
+    }
     if (counted) e = launch_chained(pack::count_kernel, dim3((unsigned)units), dim3(32 * pack::COUNT_WARPS), 0, st, 1, p);
     if (e == cudaSuccess)
         e = launch_chained(pack::scan_kernel, dim3(pack::SCAN_CTAS), dim3(pack::SCAN_THREADS), 0, st, pack::SCAN_CTAS, p, counted);
     if (e == cudaSuccess) {
-        const dim3 grid((unsigned)n_rec), block(128);
         switch (desc->block) {
-            case 2: e = launch_chained(pack::fill_kernel<2>, grid, block, 0, st, 1, p); break;
-            case 4: e = launch_chained(pack::fill_kernel<4>, grid, block, 0, st, 1, p); break;
-            case 8: e = launch_chained(pack::fill_kernel<8>, grid, block, 0, st, 1, p); break;
-            default: e = launch_chained(pack::fill_kernel<16>, grid, block, 0, st, 1, p); break;
+            case 2: e = launch_chained(pack::fill_kernel<2, false>, grid, block, 0, st, 1, p); break;
+            case 4: e = launch_chained(pack::fill_kernel<4, false>, grid, block, 0, st, 1, p); break;
+            case 8: e = launch_chained(pack::fill_kernel<8, false>, grid, block, 0, st, 1, p); break;
+            default: e = launch_chained(pack::fill_kernel<16, false>, grid, block, 0, st, 1, p); break;
         }
     }
     if (e != cudaSuccess) return MWU_ERR_CUDA;

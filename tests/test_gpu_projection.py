@@ -355,3 +355,14 @@ def test_projection_exact_kernel_cluster_edges(b, rows, cols):
     W = inputs.normal_weights(rows, cols, 0.02, 6100 + b)
     Mb = rows * cols // b
     check_against_oracle(W, b, Mb // 2, Mb // 4, algos=(B.MWU_ALGO_AUTO,))
+
+
+@pytest.mark.parametrize("b,rows,cols", [(2, 1280, 1024), (2, 1281, 1024),      # the most blocks packed by one kernel, more
+                                         (4, 1, 64), (8, 130, 192), (16, 257, 1088)])
+def test_pack_one_kernel_edges(b, rows, cols):
+    W = inputs.normal_weights(rows, cols, 0.02, 6200 + b)
+    Mb = rows * cols // b
+    desc, bufs, Wd, _, p = check_against_oracle(W, b, Mb * 6 // 10, Mb * 3 // 10, algos=(B.MWU_ALGO_AUTO,))
+    packed = bufs.pack(Wd)
+    torch.cuda.synchronize()
+    check_pack(desc, bufs, packed, p, b)
