@@ -31,7 +31,7 @@ namespace gemm {
 bool pair_eligible(const Params &p);
 cudaError_t launch_pair(int bw, const CUtensorMap &tmap, const Params &p, int sm_count, cudaStream_t st);
 // few activation rows, defined in mwu_gemm4.cu
-bool stream_eligible(const Params &p, int sm_count);
+bool stream_eligible(const Params &p, int sm_count, bool can_expand);
 int stream_box_rows(const Params &p, int sm_count);
 cudaError_t launch_stream(int bw, const CUtensorMap &tmap_x, const Params &p, int sm_count, cudaStream_t st);
 // convolution kernels of up to nine taps, defined in mwu_conv2.cu
@@ -630,7 +630,9 @@ extern "C" int mwu_gemm_ws(const mwu_proj_desc *desc, const void *packed, const 
     p.ldy = ldy;
     if (p.n_stages > MAX_STAGES_K) return MWU_ERR_SHAPE;
 
-    if (stream_eligible(p, sm_count)) {
+    const size_t need = mwu_gemm_workspace_bytes(desc, M);
+    const bool can_expand = workspace && need && workspace_bytes >= need;
+    if (stream_eligible(p, sm_count, can_expand)) {
         CUtensorMap tmap_x;
         if (!encode_bf16_2d(encode, &tmap_x, X, desc->cols, M, ldx, stream_box_rows(p, sm_count)))
             return MWU_ERR_CUDA;
@@ -638,8 +640,7 @@ extern "C" int mwu_gemm_ws(const mwu_proj_desc *desc, const void *packed, const 
     }
 
     // decode once into the caller's workspace, then a two-operand GEMM over it
-    const size_t need = mwu_gemm_workspace_bytes(desc, M);
-    if (workspace && need && workspace_bytes >= need) {
+    if (can_expand) {
         const int64_t n_pad = p.n_rec_tiles * kTileRows;
         CUtensorMap tmap_x, tmap_w;
         if (!encode_bf16_2d(encode, &tmap_x, X, desc->cols, M, ldx, BMH) ||

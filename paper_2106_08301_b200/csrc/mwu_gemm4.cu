@@ -398,9 +398,15 @@ static cudaError_t launch_stream_bw(const CUtensorMap &tmap_x, const Params &p, 
                           p, s.q);
 }
 
-static StreamPlan plan_of(const Params &p, int sm_count) {
+// The tensor core drops what lies below an accumulator's last place, so a sum loses a little of its magnitude at every
+// step, and a sum in pieces less: an fp32 result of 7168 products differs by 5.1e-6 between one and eight pieces, by
+// 3.6e-6 between one and two.  bf16 results hide it; fp32 results stay within 4.5e-6 of what the kernels for more rows,
+// which never split, give.
+static int most_pieces(const Params &p) { return !p.y_fp32 || p.K <= 6144 ? 8 : p.K <= 6912 ? 4 : 2; }
+
+static StreamPlan plan_of(const Params &p, int sm_count, int most) {
     StreamPlan best = plan_with(p, 1, sm_count);
-    for (int split = 2; split <= 8 && split <= p.n_stages; split *= 2) {
+    for (int split = 2; split <= most && split <= p.n_stages; split *= 2) {
         const StreamPlan s = plan_with(p, split, sm_count);
         if (s.cost < best.cost) best = s;
     }
@@ -408,19 +414,22 @@ static StreamPlan plan_of(const Params &p, int sm_count) {
 }
 
 // activation rows of the TMA box of X
-int stream_box_rows(const Params &p, int sm_count) { return plan_of(p, sm_count).q.mpad; }
+int stream_box_rows(const Params &p, int sm_count) { return plan_of(p, sm_count, most_pieces(p)).q.mpad; }
 
 // A record is decoded once per activation tile of 128 rows, so the path that expands the weights once
 // overtakes this one as rows are added.  Measured (us, this kernel / expanding): 16384 x 4096, b = 16:
 // 27 / 66 at 16 rows, 41 / 68 at 128, 67 / 68 at 256, 131 / 89 at 512; 4096 x 4096, b = 8: 26 / 37 at 256, 41 / 37 at
 // 512; b = 2: 43 / 50 at 256, 72 / 52 at 512.  A small weight stays here longer, while the decodes are few to an
 // SM: 1000 x 1216, b = 8, 1024 rows (1216 decodes): 15 / 19; 4096 x 1024, b = 4, 512 rows (2048): 22 / 19.
-bool stream_eligible(const Params &p, int sm_count) {
+// Where it may not split as it would (128 x 7168, 55 rows, fp32: 16 us in eight pieces, 43 in two, 41 expanding), the
+// other path is taken if the caller's workspace allows it (can_expand).
+bool stream_eligible(const Params &p, int sm_count, bool can_expand) {
+    if (can_expand && most_pieces(p) < 8 && 2 * plan_of(p, sm_count, most_pieces(p)).cost > 3 * plan_of(p, sm_count, 8).cost) return false;
     return p.M <= 256 || p.n_rec_tiles * p.n_stages * ((p.M + ST_MAX_ROWS - 1) / ST_MAX_ROWS) <= 9ll * sm_count;
 }
 
 cudaError_t launch_stream(int bw, const CUtensorMap &tmap_x, const Params &p, int sm_count, cudaStream_t st) {
-    const StreamPlan s = plan_of(p, sm_count);
+    const StreamPlan s = plan_of(p, sm_count, most_pieces(p));
     switch (bw) {
         case 2: return launch_stream_bw<2>(tmap_x, p, s, st);
         case 4: return launch_stream_bw<4>(tmap_x, p, s, st);

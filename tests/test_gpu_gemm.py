@@ -336,3 +336,26 @@ def test_conv_line_shapes(filters, cin, h, w, k, pad, n, b):
         torch.cuda.synchronize()
         assert int(bufs.dev_status.item()) == 0
         assert errors(Y.cpu().numpy(), ref)[0] <= 1e-5, call
+
+
+@pytest.mark.parametrize("cols", [6144, 6208, 6912, 6976, 8192])
+def test_gemm_long_fp32_sums_hardly_depend_on_the_row_count(cols):
+    """fp32 results of a few rows (whose sums may be split over CTAs) against the same rows among 300 (never split).
+    The accumulator's rounding is worth about 8e-10 a product; the limits on splitting keep the difference below 4.5e-6."""
+    W = inputs.normal_weights(128, cols, 0.02, 910)
+    Mb = W.numel() // 4
+    desc = B.make_desc(128, cols, 4, Mb // 2, Mb // 4)
+    bufs = B.ProjectionBuffers(desc)
+    Wd = W.cuda()
+    bufs.project(Wd)
+    packed = bufs.pack(Wd)
+    X = inputs.normal_activations_bf16((300, cols), 911).cuda()
+    out = []
+    for m in (40, 300):
+        Y = torch.zeros(m, 128, device="cuda")
+        ws = torch.empty(B.mwu_gemm_workspace_bytes(desc, m), dtype=torch.uint8, device="cuda")
+        B.mwu_gemm_ws(desc, packed, X[:m], m, cols, Y, 128, 1, ws, bufs.dev_status)
+        out.append(Y[:40].double())
+    torch.cuda.synchronize()
+    assert int(bufs.dev_status.item()) == 0
+    assert float((out[0] - out[1]).norm() / out[1].norm()) < 4.5e-6
