@@ -310,6 +310,10 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(Params p, int counte
 }
 
 constexpr unsigned OWN_THREADS = 512;
+// CTAs to an SM that the registers are cut to: enough warps to hide the gathers of W and u, few enough that their lines stay in
+// L1 until the neighbouring blocks' turn (16384 x 4096, 50 % / 25 %, b = 2: 175 us with 12, 181 with 8, 317 with 16; b = 4: 109,
+// 112, 114; b = 8: 84 with 16, 88 with 8).
+__host__ __device__ constexpr int fill_ctas(int b, bool own) { return own ? 0 : b <= 4 ? 12 : 16; }
 // Most blocks (padding rows included) of the form without a scan: every CTA reads on average half of the bitmaps.  Whole
 // mwu_pack calls, us, with it and without: 256 x 256, b = 4: 8.5 / 13.0; 1000 x 1216, b = 2: 13.7 / 17.0; 2048 x 2048, b = 8,
 // 524288 blocks: 12.5 / 15.1; 3072 x 2048, b = 8, 786432: 19.0 / 19.7; 1024 x 2048, b = 2, 1048576: 26.0 / 17.7.
@@ -327,7 +331,7 @@ __device__ __forceinline__ void row_block_of(unsigned off, int b, unsigned *r, u
 // OWN: the base of the record's lists is counted here too, from the bitmaps of everything before it: no record table, no
 // kernel before this one; the lists are then written by four times the threads.
 template <int B, bool OWN>
-__global__ void __launch_bounds__(OWN ? OWN_THREADS : 128) fill_kernel(Params p) {
+__global__ void __launch_bounds__(OWN ? OWN_THREADS : 128, fill_ctas(B, OWN)) fill_kernel(Params p) {
     constexpr unsigned NT = OWN ? OWN_THREADS : 128;
     constexpr int NBK = kStageK / B;
     constexpr unsigned MASK = (NBK >= 32) ? 0xffffffffu : ((1u << NBK) - 1u);
@@ -351,7 +355,9 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128) fill_kernel(Params p)
     __shared__ __align__(4) unsigned char s_len[3 * G];     // ... and in all (at most 128 each: a byte)
     __shared__ unsigned short s_full[3][kTileRows + 1];     // per class and q: list entries of rounds 0 .. q-1
     __shared__ unsigned s_more[3][kTileRows + 1];           // per class and q: slots that have a round q
-    __shared__ unsigned short s_off[3][kTileRows * NBK];    // tile offsets of each class list, in list order
+    // Tile offsets of the pruned, the dense and the unified list.  Without a gap between them where CTAs crowd on an SM (the
+    // shared memory of three full lists took b = 4 from 109 to 231 us); with their beginnings fixed in the form of few CTAs.
+    __shared__ unsigned short s_off[(OWN ? 3 : 1) * kTileRows * NBK];
     const bool has_row = !OWN || r < kTileRows;             // a thread to a row; the others join at the lists
     unsigned P = 0, U = 0, D = 0;
     if (has_row) {
@@ -446,6 +452,8 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128) fill_kernel(Params p)
     __syncthreads();
 
     // every block's place in its class list
+    const unsigned first_d = OWN ? kTileRows * NBK : s_full[0][kTileRows];
+    const unsigned first_u = OWN ? 2 * kTileRows * NBK : first_d + s_full[1][kTileRows];
     const unsigned below = (1u << lane) - 1u;
     if (has_row)
 #pragma unroll 4
@@ -458,7 +466,7 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128) fill_kernel(Params p)
         const unsigned q = s_before[warp][f] + __popc(s_bal[warp][f] & below);
         // q full rounds before it, then the lower slots of its own round
         const unsigned idx = s_full[cls][q] + __popc(s_more[cls][q] & ((1u << slot) - 1u));
-        s_off[cls][idx] = (unsigned short)off;
+        s_off[(cls == 0u ? 0u : cls == 1u ? first_d : first_u) + idx] = (unsigned short)off;
     }
     uint4 me, nx;                                           // (ubase, dbase, pbase, live); the table ends with the totals
     if (OWN) {
@@ -495,12 +503,12 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128) fill_kernel(Params p)
         const long long f_base = row_base * p.cols + stage * kStageK;          // first weight of the record
         // pruned blocks: positions only
         unsigned short *pp = ppos + me.z;
-        for (unsigned t = (unsigned)r; t < len_p; t += NT) pp[t] = s_off[0][t];
+        for (unsigned t = (unsigned)r; t < len_p; t += NT) pp[t] = s_off[t];
         // unified blocks: sign bits, position, magnitude
         uint2 *ul = ulist + me.x;
         const long long j_base = row_base * p.bpr + stage * NBK;
         for (unsigned t = (unsigned)r; t < len_u; t += NT) {
-            const unsigned off = s_off[2][t];
+            const unsigned off = s_off[first_u + t];
             unsigned rr, i;
             row_block_of(off, B, &rr, &i);
             const long long f = f_base + (long long)rr * p.cols + i * B;
@@ -510,12 +518,12 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128) fill_kernel(Params p)
         }
         // dense blocks: position, then the values, LPB lanes to a block
         unsigned short *dp = dpos + me.y;
-        for (unsigned t = (unsigned)r; t < len_d; t += NT) dp[t] = s_off[1][t];
+        for (unsigned t = (unsigned)r; t < len_d; t += NT) dp[t] = s_off[first_d + t];
         unsigned char *pay = dpay + (unsigned long long)me.y * (2 * B);
         for (unsigned q = (unsigned)r; q < len_d * (unsigned)LPB; q += NT) {
             const unsigned t = q / (unsigned)LPB, part = q % (unsigned)LPB;
             unsigned rr, i;
-            row_block_of(s_off[1][t], B, &rr, &i);
+            row_block_of(s_off[first_d + t], B, &rr, &i);
             const long long f = f_base + (long long)rr * p.cols + i * B + part * 4;
             unsigned char *dst = pay + q * 8u;               // = t * 2B + part * 8 when a block takes LPB lanes
             if (B >= 4) {
