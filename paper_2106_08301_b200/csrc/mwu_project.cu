@@ -1827,8 +1827,14 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
 // over the group's columns with shuffles (the pairing of the block keys continued across blocks);
 // the rows of a group are then summed as a pairwise tree in shared memory.  Everything is fp64 with
 // one rounding per operation, in a fixed order: the keys do not depend on the launch shape.
+// Four rows at a time and eight CTAs an SM: the loads in flight are what counts (a grouped projection of 16384 x 4096, b = 16,
+// 256 x 64: 213 us; six CTAs 221, eight rows and four CTAs 237, all sixteen rows and three CTAs 270; all lanes at every level of
+// the column tree 223).
+constexpr int GS_ROWS = 4, GS_CTAS = 8;
 template <int GC>                                      // columns of a group: 16, 32 or 64
-__global__ void __launch_bounds__(256) group_stats_kernel(Params p, double *gkey, long long rows, long long cols) {
+__global__ void __launch_bounds__(256, GS_CTAS) group_stats_kernel(Params p, double *gkey, long long rows, long long cols) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ double s_row[256][4];
     constexpr unsigned gc = GC;
     const unsigned gr = p.group_rows;
@@ -1839,26 +1845,50 @@ __global__ void __launch_bounds__(256) group_stats_kernel(Params p, double *gkey
     const long long col = col0 + (lane & 15) * 4;
     const long long first = (row0 + warp * 32 + (lane >> 4)) * cols + col;      // this thread's rows: every second one from here
     const bool l1 = p.use_l1 != 0;
-#pragma unroll 4
-    for (int it = 0; it < 16; ++it) {
-        const int r = warp * 32 + it * 2 + (lane >> 4);
-        const long long row = row0 + r;
-        const long long at = first + (long long)it * 2 * cols;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (row < rows && col < cols) {
-            v = __ldg(reinterpret_cast<const float4 *>(p.W + at));
-            if (p.U) {
-                const float4 d = __ldg(reinterpret_cast<const float4 *>(p.U + at));
-                v.x = __fadd_rn(v.x, d.x); v.y = __fadd_rn(v.y, d.y); v.z = __fadd_rn(v.z, d.z); v.w = __fadd_rn(v.w, d.w);
+    // ROWS rows at a time.  Up the tree over the columns a lane keeps one of two rows at each level and gives its partner the
+    // other, so a level takes half of the shuffles of the one before; after it the row's low bits are lane bits.
+    constexpr int ROWS = GS_ROWS, LEVELS = (int)lanes_per_slice < ROWS ? (int)lanes_per_slice : ROWS;      // lanes that share rows out
+    constexpr int KEPT = ROWS / LEVELS;                 // rows a lane ends up with
+#pragma unroll 1
+    for (int it0 = 0; it0 < 16; it0 += ROWS) {
+        double t[ROWS];                                 // sums of this thread's four columns, row by row
+#pragma unroll
+        for (int k = 0; k < ROWS; ++k) {
+            const int it = it0 + k, r = warp * 32 + it * 2 + (lane >> 4);
+            const long long row = row0 + r;
+            const long long at = first + (long long)it * 2 * cols;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row < rows && col < cols) {
+                v = __ldg(reinterpret_cast<const float4 *>(p.W + at));
+                if (p.U) {
+                    const float4 d = __ldg(reinterpret_cast<const float4 *>(p.U + at));
+                    v.x = __fadd_rn(v.x, d.x); v.y = __fadd_rn(v.y, d.y); v.z = __fadd_rn(v.z, d.z); v.w = __fadd_rn(v.w, d.w);
+                }
+            }
+            const double a0 = (double)fabsf(v.x), a1 = (double)fabsf(v.y), a2 = (double)fabsf(v.z), a3 = (double)fabsf(v.w);
+            if (l1) t[k] = __dadd_rn(__dadd_rn(a0, a1), __dadd_rn(a2, a3));
+            else t[k] = __dadd_rn(__fma_rn(a0, a0, __dmul_rn(a1, a1)), __fma_rn(a2, a2, __dmul_rn(a3, a3)));   // squares are exact
+        }
+#pragma unroll
+        for (int m = 1, n = ROWS; m < LEVELS; m <<= 1, n >>= 1) {
+            const bool odd = (lane & m) != 0;
+#pragma unroll
+            for (int i = 0; i < n / 2; ++i) {
+                const double keep = odd ? t[2 * i + 1] : t[2 * i], give = odd ? t[2 * i] : t[2 * i + 1];
+                t[i] = __dadd_rn(keep, __shfl_xor_sync(0xffffffffu, give, m));
             }
         }
-        const double a0 = (double)fabsf(v.x), a1 = (double)fabsf(v.y), a2 = (double)fabsf(v.z), a3 = (double)fabsf(v.w);
-        double t;
-        if (l1) t = __dadd_rn(__dadd_rn(a0, a1), __dadd_rn(a2, a3));
-        else t = __dadd_rn(__fma_rn(a0, a0, __dmul_rn(a1, a1)), __fma_rn(a2, a2, __dmul_rn(a3, a3)));   // squares are exact
 #pragma unroll
-        for (unsigned m = 1; m < lanes_per_slice; m <<= 1) t = __dadd_rn(t, __shfl_xor_sync(0xffffffffu, t, m));
-        if (((unsigned)lane & (lanes_per_slice - 1u)) == 0u) s_row[r][((unsigned)lane & 15u) / lanes_per_slice] = t;
+        for (int m = LEVELS; m < (int)lanes_per_slice; m <<= 1)
+#pragma unroll
+            for (int k = 0; k < KEPT; ++k) t[k] = __dadd_rn(t[k], __shfl_xor_sync(0xffffffffu, t[k], m));
+        if (((lane & 15) % (int)lanes_per_slice) / LEVELS == 0) {
+#pragma unroll
+            for (int k = 0; k < KEPT; ++k) {
+                const int it = it0 + k * LEVELS + (lane & (LEVELS - 1));
+                s_row[warp * 32 + it * 2 + (lane >> 4)][((unsigned)lane & 15u) / lanes_per_slice] = t[k];
+            }
+        }
     }
     __syncthreads();
     // rows of a group: r with r ^ 1, then r ^ 2, ...
@@ -1883,8 +1913,10 @@ __global__ void __launch_bounds__(256) group_stats_kernel(Params p, double *gkey
 __global__ void __launch_bounds__(FIN_THREADS) group_select_kernel(const double *gkey, unsigned n_groups, unsigned kg,
                                                                    unsigned *gprune) {
     __shared__ unsigned s_hist[256];
-    __shared__ u64 s_prefix;
-    __shared__ unsigned s_r;
+    __shared__ u64 s_prefix, s_diff;
+    __shared__ unsigned s_r, s_left;             // rank of the wanted key among those with the prefix; their number
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ unsigned s_warp[32];
     const u64 *keys = reinterpret_cast<const u64 *>(gkey);
     const unsigned n_words = (n_groups + 31u) / 32u;
@@ -1896,9 +1928,32 @@ __global__ void __launch_bounds__(FIN_THREADS) group_select_kernel(const double 
         }
         return;
     }
-    if (threadIdx.x == 0) { s_prefix = 0; s_r = kg; }
-    u64 mask = 0;
-    for (int shift = 56; shift >= 0; shift -= 8) {
+    // the bits that all keys share need no round (keys are sums of like size: their exponents and first digits agree)
+    u64 all = ~0ull, any = 0ull;
+    for (unsigned i = threadIdx.x; i < n_groups; i += blockDim.x) {
+        const u64 k = __ldg(keys + i);
+        all &= k;
+        any |= k;
+    }
+    if (threadIdx.x == 0) { s_prefix = 0; s_r = kg; s_diff = 0; s_left = n_groups; }
+    __syncthreads();
+    {
+        // a bit differs when some key has it and some has not
+        const u64 first = __ldg(keys);
+        const u64 diff = any & ~all;                    // within this thread's keys ...
+        const u64 d = n_groups > threadIdx.x ? (diff | (all ^ first)) : 0ull;        // ... or against the first key
+        const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)d), hi = __reduce_or_sync(0xffffffffu, (unsigned)(d >> 32));
+        if ((threadIdx.x & 31u) == 0u) atomicOr(&s_diff, (u64)hi << 32 | lo);
+    }
+    __syncthreads();
+    const u64 diff = s_diff;
+    const int top = diff ? 63 - __clzll((long long)diff) : -1;
+    u64 mask = top >= 63 ? 0ull : ~0ull << (top + 1);
+    if (threadIdx.x == 0) s_prefix = __ldg(keys) & mask;
+    __syncthreads();
+    // Rounds of eight bits, until one key is left (its low bits are then read from it) or the bits run out.
+    for (int shift = top - 7; top >= 0 && s_left > 1u; shift -= 8) {
+        if (shift < 0) shift = 0;
         for (unsigned i = threadIdx.x; i < 256u; i += blockDim.x) s_hist[i] = 0;
         __syncthreads();
         const u64 prefix = s_prefix;
@@ -1926,10 +1981,21 @@ __global__ void __launch_bounds__(FIN_THREADS) group_select_kernel(const double 
                 unsigned left = r - (incl - sum), d = 0;
                 while (d < 7u && mine[d] < left) { left -= mine[d]; ++d; }
                 s_r = left;
-                s_prefix = prefix | ((u64)(lane * 8u + d) << shift);
+                s_left = mine[d];
+                s_prefix = (prefix & ~((u64)255 << shift)) | ((u64)(lane * 8u + d) << shift);
             }
         }
         mask |= (u64)255 << shift;
+        __syncthreads();
+        if (shift == 0) break;
+    }
+    if (~mask != 0ull && s_left == 1u) {                // the only key with this prefix
+        const u64 prefix = s_prefix;
+        __syncthreads();
+        for (unsigned i = threadIdx.x; i < n_groups; i += blockDim.x) {
+            const u64 k = __ldg(keys + i);
+            if ((k & mask) == prefix) s_prefix = k;
+        }
         __syncthreads();
     }
     const u64 T = s_prefix;
@@ -2074,14 +2140,14 @@ static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_des
     if (p.gprune) {
         // grouped pruning: the groups' keys, then the groups to zero (a bit per group)
         const dim3 grid((unsigned)((desc->cols + 63) / 64), (unsigned)((desc->rows + 255) / 256));
-        switch (desc->prune_group_cols) {
-            case 16: group_stats_kernel<16><<<grid, 256, 0, st>>>(p, gkey, desc->rows, desc->cols); break;
-            case 32: group_stats_kernel<32><<<grid, 256, 0, st>>>(p, gkey, desc->rows, desc->cols); break;
-            default: group_stats_kernel<64><<<grid, 256, 0, st>>>(p, gkey, desc->rows, desc->cols); break;
-        }
         const unsigned n_groups = (unsigned)mwu::n_groups_of(desc);
         const unsigned per_group = (unsigned)(desc->prune_group_rows * desc->prune_group_cols / desc->block);
-        group_select_kernel<<<1, FIN_THREADS, 0, st>>>(gkey, n_groups, (unsigned)(desc->k_prune / per_group), gprune);
+        auto stats = desc->prune_group_cols == 16 ? group_stats_kernel<16> : desc->prune_group_cols == 32 ? group_stats_kernel<32> : group_stats_kernel<64>;
+        e = mwu::launch_chained(stats, grid, dim3(256), 0, st, 1, p, gkey, (long long)desc->rows, (long long)desc->cols);
+        if (e == cudaSuccess)
+            e = mwu::launch_chained(group_select_kernel, dim3(1), dim3(FIN_THREADS), 0, st, 1, (const double *)gkey, n_groups,
+                                    (unsigned)(desc->k_prune / per_group), gprune);
+        if (e != cudaSuccess) return e;
         mwu::count_launch(2);
     }
     const long long n_units = (p.n_floats + 15) / 16;
