@@ -10,7 +10,7 @@
 //
 // One-pass pipeline (MWU_ALGO_ONE_PASS; the default for larger tensors):
 //   sample_keys_kernel, sample_kernel
-//                   rank the keys of <= 65536 evenly spaced blocks; for each selection (prune key, L_u
+//                   rank the keys of <= 262144 evenly spaced blocks; for each selection (prune key, L_u
 //                   of the survivors) the sample quantile is a provisional threshold and the sample
 //                   keys 4 sigma of rank to either side a window.
 //   pass_kernel     streams W (+U) once, evaluates the fp64 keys of every block and writes every
@@ -36,12 +36,12 @@ constexpr int NB_MAX = 65536;   // level-0 bins (codes fit 16 bits): bin 0 = bel
 constexpr int NB_SMALL = 8192;  // used up to NB_SMALL_BLOCKS blocks: fewer bins to clear and scan
 constexpr long long NB_SMALL_BLOCKS = 1ll << 27;    // about 1.4 % of them in a window: at most 450 to a bin
 constexpr int CAP = 2048;       // candidates sorted by the last step
-// sample blocks ranked by sample_kernel: at most NSAMP_MAX, SAMP_PER to a thread
+// sample blocks ranked by sample_kernel: SAMP_PER to a thread at a time
 constexpr int SAMP_CTAS = 8, SAMP_THREADS = 1024, SAMP_PER = 8;
-constexpr int NSAMP_MAX = SAMP_CTAS * SAMP_THREADS * SAMP_PER;
+constexpr int SAMP_ROUND = SAMP_CTAS * SAMP_THREADS * SAMP_PER;
 constexpr int SAMP_A = 128;       // of the samples, ranked first
-constexpr int NSAMP_SMALL_LG = 14, NSAMP_LG = 16;
-static_assert(NSAMP_MAX == 1 << NSAMP_LG, "the larger sample fills the cluster");
+constexpr int NSAMP_SMALL_LG = 14, NSAMP_LG = 16, NSAMP_LARGE_LG = 18;
+static_assert(SAMP_ROUND == 1 << NSAMP_LG, "the middle sample fills the cluster");
 constexpr int STAGE_ENTRIES = 64;  // per-warp staging of candidate-list entries in pass_kernel
 constexpr int FIN_THREADS = 1024;   // block size of the kernels that scan the histograms
 constexpr int PASS_GROUPS = 8;      // groups of CTAs of pass_kernel that share out its last steps
@@ -332,8 +332,10 @@ constexpr unsigned NO_SAMPLE = 0xffffffffu;           // key of a sample that ta
 // a_key: the level-A key that this thread and its seven neighbours rank.  `frac` of the keys are to be selected.  Level A
 // ranks 128 of the sample keys to get a coarse window; level B counts all in SAMP_THREADS bins across that window and
 // reads the final window [lo, hi) and the provisional threshold from the bin edges.  c: cleared before a
-// cluster barrier.  all: room for the cluster's counts.
-__device__ __forceinline__ uint3 sample_select(const unsigned (&key)[SAMP_PER], unsigned a_key, float frac, SampCounts *c, uint4 *all) {
+// cluster barrier.  all: room for the cluster's counts.  more(f): f(key) for this thread's sample keys beyond those.
+template <class More>
+__device__ __forceinline__ uint3 sample_select(const unsigned (&key)[SAMP_PER], unsigned a_key, float frac, SampCounts *c, uint4 *all,
+                                               More more) {
     constexpr int A_PARTS = SAMP_THREADS / SAMP_A;
     // level-A keys, shortened to the top 25 bits below the (clear) sign bit, with the key's index in
     // the low seven: distinct words, one 32-bit compare per pair; invalid keys rank last
@@ -379,13 +381,15 @@ __device__ __forceinline__ uint3 sample_select(const unsigned (&key)[SAMP_PER], 
     static_assert(SAMP_THREADS == 1024, "ten bits of bin index");
     // level B
     unsigned n_under = 0, n_valid = 0;
-#pragma unroll
-    for (int t = 0; t < SAMP_PER; ++t) {
-        const unsigned d = key[t] - clo;
+    auto count = [&](unsigned k) {
+        const unsigned d = k - clo;
         if (d < chi - clo) atomicAdd(&c->bins[d >> shift], 1u);
-        n_under += key[t] < clo ? 1u : 0u;
-        n_valid += key[t] != NO_SAMPLE ? 1u : 0u;
-    }
+        n_under += k < clo ? 1u : 0u;
+        n_valid += k != NO_SAMPLE ? 1u : 0u;
+    };
+#pragma unroll
+    for (int t = 0; t < SAMP_PER; ++t) count(key[t]);
+    more(count);
     n_under = __reduce_add_sync(0xffffffffu, n_under);
     n_valid = __reduce_add_sync(0xffffffffu, n_valid);
     if (lane == 0) {
@@ -444,7 +448,7 @@ __device__ __forceinline__ uint3 sample_select(const unsigned (&key)[SAMP_PER], 
 }
 
 // block of the i-th of the evenly spaced samples, without a division (their number is a power of
-// two, or that of all blocks); i < 2^16 and n_blocks < 2^31, so the product fits 64 bits
+// two, or that of all blocks); i < 2^18 and n_blocks < 2^31, so the product fits 64 bits
 __device__ __forceinline__ long long sample_block(const Params &p, int i) {
     return p.samp_lg >= 0 ? (long long)(((u64)i * (u64)p.n_blocks) >> p.samp_lg) : (long long)i;
 }
@@ -476,7 +480,7 @@ __global__ void __launch_bounds__(128) sample_keys_kernel(Params p, unsigned *ze
 //
 // Why a cluster: a window is +-4 sigma of rank, so the share of blocks that pass_kernel has to list, and
 // resolve_kernel to go through, falls with the root of the sample's size.  With 4096 samples (one CTA) 11 % of the
-// blocks of a 50 % / 25 % projection were listed, with 65536 it is 3 %.
+// blocks of a 50 % / 25 % projection were listed, with 65536 it is 3 %, with 262144 1.4 %.
 __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
     __shared__ SampCounts s_counts[2];
     __shared__ uint4 s_all[SAMP_CTAS * SAMP_THREADS / 4];
@@ -501,8 +505,20 @@ __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
         *k0 = valid ? __float_as_uint(x.x) : NO_SAMPLE;
         *k1 = valid ? __float_as_uint(x.y) & ~SIGN : NO_SAMPLE;
     };
+    auto index = [](int t) { return (t * SAMP_CTAS + (int)blockIdx.x) * SAMP_THREADS + (int)threadIdx.x; };
 #pragma unroll
-    for (int t = 0; t < SAMP_PER; ++t) take((t * SAMP_CTAS + (int)blockIdx.x) * SAMP_THREADS + (int)threadIdx.x, &kp[t], &ku[t]);
+    for (int t = 0; t < SAMP_PER; ++t) take(index(t), &kp[t], &ku[t]);
+    // what a larger sample has beyond that is read again for each selection
+    auto later = [&](auto f) {
+#pragma unroll 1
+        for (int t0 = SAMP_PER; t0 < ns / (SAMP_CTAS * SAMP_THREADS); t0 += SAMP_PER) {
+            unsigned k0[SAMP_PER], k1[SAMP_PER];
+#pragma unroll
+            for (int t = 0; t < SAMP_PER; ++t) take(index(t0 + t), &k0[t], &k1[t]);
+#pragma unroll
+            for (int t = 0; t < SAMP_PER; ++t) f(k0[t], k1[t]);
+        }
+    };
     const int a = (int)threadIdx.x / (SAMP_THREADS / SAMP_A);
     unsigned kp_a, ku_a;
     take(p.samp_lg >= 7 ? a << (p.samp_lg - 7) : a, &kp_a, &ku_a);      // SAMP_A of the samples, evenly spaced
@@ -512,6 +528,8 @@ __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
     Sel *su = &p.work->sel[1];
     const long long ksel_u = k_unify - k_prune;
     auto key64 = [](unsigned x) { return key_bits((double)__uint_as_float(x < 0x7f800000u ? x : 0x7f800000u)); };
+    unsigned floor_p = 0;                             // estimated prune threshold
+    bool any_pruned = false;
     if (lead && p.resid) *p.resid = 0.0;              // the kernels that follow add to it
     sel::ClusterTeam::arrive();                       // every CTA's counts are cleared
     sel::ClusterTeam::wait();
@@ -524,7 +542,8 @@ __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
             p.work->That[0] = 0;
         }
     } else {
-        const uint3 wp = sample_select(kp, kp_a, (float)((double)k_prune / (double)mb), &s_counts[0], s_all);
+        const uint3 wp = sample_select(kp, kp_a, (float)((double)k_prune / (double)mb), &s_counts[0], s_all,
+                                       [&](auto count) { later([&](unsigned k0, unsigned) { count(k0); }); });
         if (lead) {
             set_window(sp, key64(wp.x), key64(wp.y), p.nb);
             sp->mode = (k_prune == 0) ? 1u : (k_prune == mb ? 2u : 0u);
@@ -533,13 +552,17 @@ __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
         }
         // the sample blocks that survive the (estimated) prune threshold
         if (k_prune != 0) {
+            floor_p = wp.z;
+            any_pruned = true;
 #pragma unroll
             for (int t = 0; t < SAMP_PER; ++t) ku[t] = kp[t] > wp.z ? ku[t] : NO_SAMPLE;
             ku_a = kp_a > wp.z ? ku_a : NO_SAMPLE;
         }
     }
     const long long elig = mb - k_prune;
-    const uint3 wu = sample_select(ku, ku_a, elig > 0 ? (float)((double)ksel_u / (double)elig) : 0.f, &s_counts[1], s_all);
+    const uint3 wu = sample_select(ku, ku_a, elig > 0 ? (float)((double)ksel_u / (double)elig) : 0.f, &s_counts[1], s_all, [&](auto count) {
+        later([&](unsigned k0, unsigned k1) { count(any_pruned && k0 <= floor_p ? NO_SAMPLE : k1); });
+    });
     if (lead) {
         set_window(su, key64(wu.x), key64(wu.y), p.nb);
         su->mode = (ksel_u == 0) ? 1u : (ksel_u == elig ? 2u : 0u);
@@ -2040,7 +2063,7 @@ static size_t ws_off_list() { return align_up(ws_off_cand_aux() + 2 * proj::CAP 
 // candidate list of the one-pass pipeline: a quarter of the blocks (the windows hold a few per cent;
 // of a small tensor they may hold more)
 // (and before pass_kernel the sample's keys are in its place: the list never has fewer entries than those)
-static size_t list_capacity(size_t mb) { return mb / 4 + proj::NSAMP_MAX; }
+static size_t list_capacity(size_t mb) { return mb / 4 + (1 << proj::NSAMP_LG); }
 static size_t ws_off_gkey(size_t mb) { return align_up(ws_off_list() + list_capacity(mb) * sizeof(uint2)); }
 static size_t n_groups_of(const mwu_proj_desc *d) {
     return grouped(d) ? (size_t)(d->rows / d->prune_group_rows) * (size_t)(d->cols / d->prune_group_cols) : 0;
@@ -2056,9 +2079,11 @@ static size_t ws_off_gprune(const mwu_proj_desc *d, size_t mb) { return align_up
 // CTA on every SM (606208 on 148) the exact kernel beats the one-pass pipeline's four launches (512 x 1152,
 // b = 8: 24 against 39; 2048 x 2048, b = 8, 524288 blocks: 45 / 52; 1024 x 2048, b = 4: 42 / 46), beyond it
 // does not (1024 x 2048, b = 2, 1048576 blocks: 67 / 54): the phases' L2 counts grow with the blocks.
-// Larger sample from here on, 65536 blocks instead of 16384 (whole mwu_project calls, 50 % / 25 %, us: 4096 x 4096, b = 4, 4 M
-// blocks: 94.7 against 99.3; 16384 x 16384, b = 4: 709 / 805; below, both sizes take the same time).
-constexpr long long SAMP_LARGE_BLOCKS = 1ll << 22;
+// Larger samples from here on, 65536 blocks instead of 16384, then 262144 (whole mwu_project calls, 50 % / 25 %, us: 4096 x 4096,
+// b = 4, 4 M blocks: 94.7 against 99.3; 16384 x 8192, b = 4, 33 M: 277 / 285; 16384 x 16384, b = 4: 496 / 518 / 610, b = 2: 645 / 695;
+// below each line both sizes take the same time).
+constexpr long long SAMP_LARGE_BLOCKS = 1ll << 22, SAMP_HUGE_BLOCKS = 1ll << 25;
+static_assert((SAMP_HUGE_BLOCKS >> 2) >= 1ll << proj::NSAMP_LARGE_LG, "the largest sample fits the list");
 constexpr long long EX_CLUSTER_BLOCKS = 49152, EX_CLUSTER_UNITS = 20480, EX_AUTO_BLOCKS_PER_CTA = 4096;
 struct Route {
     bool one_pass, cluster;         // else the exact kernel: as one cluster or as a cooperative grid
@@ -2239,7 +2264,7 @@ static int project_impl(const mwu_proj_desc *desc, const float *W, const float *
     p.cand_aux = (unsigned *)(ws + ws_off_cand_aux());
     p.list = (uint2 *)(ws + ws_off_list());
     p.samp = (float2 *)p.list;
-    p.samp_lg = p.n_blocks < SAMP_LARGE_BLOCKS ? proj::NSAMP_SMALL_LG : proj::NSAMP_LG;
+    p.samp_lg = p.n_blocks < SAMP_LARGE_BLOCKS ? proj::NSAMP_SMALL_LG : p.n_blocks < SAMP_HUGE_BLOCKS ? proj::NSAMP_LG : proj::NSAMP_LARGE_LG;
     p.n_samp = 1 << p.samp_lg;
     if (p.n_blocks < p.n_samp) {
         p.n_samp = (int)p.n_blocks;
