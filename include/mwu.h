@@ -279,6 +279,8 @@ int mwu_decode(const mwu_proj_desc *desc, const void *packed, void *Wd, int64_t 
  * tensor-core GEMM reads them, still skipping the column slices that are pruned in every row
  * of a weight tile.  The result is the same contraction with the same rounding of operands
  * (bf16 x bf16, fp32 accumulation); only the summation order inside the tensor cores may differ.
+ * Few rows (up to 256, or more where the weights are few) are multiplied without expanding anything
+ * and mostly leave the workspace alone.
  * mwu_gemm_workspace_bytes returns 0 when M is too small for this to pay (or desc is invalid);
  * with workspace == NULL, or fewer bytes than that, the call behaves exactly like mwu_gemm.
  * The workspace holds nothing between calls and may be shared by calls on the same stream.
@@ -303,9 +305,9 @@ int mwu_conv_implicit(const mwu_proj_desc *desc, const void *packed, const void 
 /*
  * mwu_conv_implicit_ws -- mwu_conv_implicit with a caller-owned scratch buffer, the counterpart
  * of mwu_gemm_ws: given `workspace` of at least mwu_conv_workspace_bytes(...) bytes (device
- * memory, 256-byte aligned) the weights are expanded once per call as by mwu_decode and the
- * tensor-core kernel reads them beside the gathered activation tiles, instead of decoding every
- * weight record again for every activation tile.  Same contraction, same rounding of operands.
+ * memory, 256-byte aligned) the weights are expanded and the image is laid out pixel by pixel once
+ * per call, and the tensor-core kernel reads both, instead of decoding every weight record again
+ * for every activation tile.  Same contraction, same rounding of operands.
  * mwu_conv_workspace_bytes returns 0 when the shape is not served by this path (or desc is
  * invalid); with workspace == NULL, or fewer bytes than that, the call behaves exactly like
  * mwu_conv_implicit.  The workspace holds nothing between calls.
