@@ -1198,8 +1198,8 @@ __device__ __noinline__ void exact_losses(const Params &p, unsigned step, double
 // staged per warp; when 32 have gathered, the whole warp evaluates their exact fp64 keys and turns them into bin codes,
 // window-histogram counts and list entries.  In fp64 every block gets only its sum (u is its rounded mean).
 //
-// What bounds it: HBM for blocks of 4 and more (16384 x 16384, b = 4: 462 us for 2.45 GB, 5.3 TB/s; 16384 x 4096, b = 16: 105 us,
-// 5.3 TB/s), instruction issue for 2.  With fp64 keys of every block and 64-bit comparisons a block of 4 took 240
+// What bounds it: HBM for blocks of 4 and more (16384 x 16384, b = 4: 435 us for 2.45 GB, 5.6 TB/s; 16384 x 4096, b = 16: 95 us,
+// 5.9 TB/s), instruction issue for 2.  With fp64 keys of every block and 64-bit comparisons a block of 4 took 240
 // instructions, 16384 x 16384 with b = 4 650 us.
 // ADMM: also the dual update V - Q and ||V - Q||_F^2 (mwu_admm_step).
 constexpr int PASS_THREADS = 256, PASS_WARPS = PASS_THREADS / 32;
