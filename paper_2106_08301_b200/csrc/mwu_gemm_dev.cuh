@@ -62,6 +62,8 @@ struct Params {
 // The packed buffer's header against what the host derived from the descriptor.  Every thread of
 // every CTA evaluates it at kernel entry (the same few cached words), so the whole grid takes the
 // same decision; on a mismatch the caller raises MWU_DEV_BOUNDS and returns before touching anything.
+// (A kernel that looks before its griddepcontrol.wait waits here: one that ended earlier would let the kernel behind it
+// start beside the one before it, which may still be writing the workspace.)
 __device__ __forceinline__ bool header_matches(const Params &p) {
     const unsigned long long *h = reinterpret_cast<const unsigned long long *>(p.packed);
     return __ldg(h) == kMagic && __ldg(h + 2) == (unsigned long long)p.N && __ldg(h + 3) == (unsigned long long)p.K &&
@@ -71,6 +73,7 @@ __device__ __forceinline__ bool header_matches(const Params &p) {
 #define MWU_CHECK_HEADER(p)                                                        \
     do {                                                                           \
         if (!header_matches(p)) {                                                  \
+            asm volatile("griddepcontrol.wait;" ::: "memory");                     \
             if (threadIdx.x == 0) atomicOr((p).dev_status, (unsigned)MWU_DEV_BOUNDS); \
             return;                                                                \
         }                                                                          \

@@ -1,0 +1,51 @@
+"""Rules that every kernel launched with programmatic stream serialization has to follow, checked in the sources."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2106_08301_b200", "csrc")
+WAIT = "griddepcontrol.wait"
+
+
+def _strip_comments(text):
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def _kernels():
+    """(name, body) of every __global__ function."""
+    out = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        text = _strip_comments(open(path).read())
+        for m in re.finditer(r"__global__", text):
+            start = text.index("{", text.index(")", text.index("(", re.compile(r"\w+_kernel\s*\(").search(text, m.end()).start())))
+            name = re.compile(r"(\w+_kernel)\s*\(").search(text, m.end()).group(1)
+            depth, end = 0, start
+            for end in range(start, len(text)):
+                depth += {"{": 1, "}": -1}.get(text[end], 0)
+                if depth == 0:
+                    break
+            out.append((name, text[start:end + 1]))
+    return out
+
+
+CHAINED = [(n, b) for n, b in _kernels() if WAIT in b]
+
+
+def _header_check():
+    text = open(os.path.join(CSRC, "mwu_gemm_dev.cuh")).read()
+    return text[text.index("#define MWU_CHECK_HEADER"):].split("while (0)")[0]
+
+
+def test_the_kernels_were_found():
+    assert len(CHAINED) >= 15
+
+
+@pytest.mark.parametrize("name,body", CHAINED, ids=[n for n, _ in CHAINED])
+def test_no_chained_kernel_ends_before_it_has_waited(name, body):
+    before = body[:body.index(WAIT)]
+    assert not re.search(r"\breturn\s*;", before)
+    if "MWU_CHECK_HEADER" in before:
+        check = _header_check()
+        assert WAIT in check and check.index(WAIT) < check.index("return;")
