@@ -317,7 +317,6 @@ __device__ __forceinline__ void gather_rows(const HaloParams &p, unsigned char *
 template <int BW>
 __global__ void __launch_bounds__(CV_THREADS, 1) mwu_conv_halo_kernel(const __grid_constant__ HaloParams p) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     MWU_CHECK_HEADER(p.g);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = smem_raw + smem_pad_1024(smem_raw);
@@ -352,7 +351,11 @@ __global__ void __launch_bounds__(CV_THREADS, 1) mwu_conv_halo_kernel(const __gr
         sm->group2[lane] = make_int4(t.base, t.dy, t.dx, 0);
     }
     __syncwarp();
-    if (warp == CV_MMA_WARP) tmem_alloc(smem_u32(&sm->tmem_base), p.tmem_cols);
+    if (warp == CV_MMA_WARP) {
+        tmem_alloc(smem_u32(&sm->tmem_base), p.tmem_cols);
+        // by this warp, and only now: the kernel behind may take all of an SM's tensor memory before it waits for this one
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

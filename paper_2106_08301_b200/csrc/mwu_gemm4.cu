@@ -90,7 +90,6 @@ __global__ void __launch_bounds__(ST_MAX_THREADS)
 mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ Params p,
                        const __grid_constant__ StreamParams q) {
     asm volatile("griddepcontrol.wait;" ::: "memory");      // launched while the kernel before may still run
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     MWU_CHECK_HEADER(p);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *base = smem_raw + smem_pad_1024(smem_raw);
@@ -123,7 +122,12 @@ mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
-    if (warp == mma_warp) tmem_alloc(smem_u32(&sm->tmem_base), q.tmem_cols);
+    if (warp == mma_warp) {
+        tmem_alloc(smem_u32(&sm->tmem_base), q.tmem_cols);
+        // By this warp, and only now (one thread's trigger is the CTA's): the kernel behind may take all of an SM's tensor
+        // memory before it waits for this one, and must not get there first.
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
     // the record table of this CTA's stages
     if (n_st > 0) {
         const uint4 *recs = reinterpret_cast<const uint4 *>(p.packed + p.off_rec) + rt * p.n_stages + k0;

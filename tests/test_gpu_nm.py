@@ -75,3 +75,25 @@ def test_keep_2_of_4_then_dense_gemm(N, K, M):
         assert int(st.item()) == 0
         fro, mx = errors(Y.float().cpu().numpy(), ref)
         assert fro <= tol and mx <= 1e-2, (y_dtype, fro, mx)
+
+
+def test_products_back_to_back_share_tensor_memory():
+    """The streaming product lets its successor start early, and the plain product takes all of tensor memory at its start."""
+    torch.manual_seed(5)
+    rows, cols, m = 1024, 512, 16
+    W = torch.randn(rows, cols, device="cuda") * 0.02
+    desc = B.make_desc(rows, cols, 8, rows * cols // 16, rows * cols // 32)
+    bufs = B.ProjectionBuffers(desc)
+    bufs.project(W)
+    packed = bufs.pack(W)
+    Wd = torch.empty(rows, cols, dtype=torch.bfloat16, device="cuda")
+    B.mwu_decode(desc, packed, Wd, cols, bufs.dev_status)
+    X = torch.randn(m, cols, device="cuda").bfloat16()
+    Y, Z = torch.empty(m, rows, device="cuda"), torch.empty(m, rows, device="cuda")
+    for _ in range(50):
+        B.mwu_gemm(desc, packed, X, m, cols, Y, rows, 1, bufs.dev_status)
+        B.mwu_gemm_dense(rows, cols, Wd, cols, X, m, cols, Z, rows, 1, bufs.dev_status)
+    torch.cuda.synchronize()
+    assert int(bufs.dev_status.item()) == 0
+    ref = X.double() @ Wd.double().t()
+    assert float((Y.double() - ref).norm() / ref.norm()) <= 1e-5 and float((Z.double() - ref).norm() / ref.norm()) <= 1e-5

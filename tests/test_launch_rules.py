@@ -49,3 +49,12 @@ def test_no_chained_kernel_ends_before_it_has_waited(name, body):
     if "MWU_CHECK_HEADER" in before:
         check = _header_check()
         assert WAIT in check and check.index(WAIT) < check.index("return;")
+
+
+@pytest.mark.parametrize("name,body", [k for k in CHAINED if "tmem_alloc" in k[1] and "launch_dependents" in k[1]],
+                         ids=lambda x: x if x.endswith("_kernel") else "")
+def test_dependents_start_only_once_tensor_memory_is_held(name, body):
+    # A dependent may take all 512 columns of an SM before its own wait, which lasts until this kernel has ended.  One
+    # thread's trigger counts for its CTA, so it is the warp that holds the allocation which triggers.
+    assert re.search(r"\{\s*tmem_alloc\([^;]*;\s*asm volatile\(\"griddepcontrol.launch_dependents;\"[^;]*\);\s*\}", body)
+    assert body.count("griddepcontrol.launch_dependents") == 1
