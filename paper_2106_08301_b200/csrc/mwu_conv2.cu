@@ -592,7 +592,12 @@ static void halo_geometry(HaloParams &p, int sm_count) {
     p.tmem_cols = mine > 2 ? 512u : (mine > 1 ? 256u : 128u);
 }
 
-bool halo_eligible(int kh, int kw) { return (long long)kh * kw <= CV_TAPS; }
+// Shapes this kernel serves: up to nine taps, and an image whose padded rows and columns can be counted in 32 bits (the
+// paddings of an image of a few pixels may reach 32767).  The rest take the kernel for any number of taps.
+bool halo_eligible(int h, int w, int kh, int kw, int stride, int pad) {
+    const long long hp = (h + 2ll * pad + stride - 1) / stride, wp = (w + 2ll * pad + stride - 1) / stride;
+    return (long long)kh * kw <= CV_TAPS && hp * wp < (1ll << 31);
+}
 
 // `g` carries the packed weights and the output; the image is X [n][c][h][w]
 int run_conv_halo(const Params &g, const void *X, int n, int c, int h, int w, int kh, int kw, int stride, int pad, int sm_count,

@@ -35,7 +35,7 @@ bool stream_eligible(const Params &p, int sm_count, bool can_expand);
 int stream_box_rows(const Params &p, int sm_count);
 cudaError_t launch_stream(int bw, const CUtensorMap &tmap_x, const Params &p, int sm_count, cudaStream_t st);
 // convolution kernels of up to nine taps, defined in mwu_conv2.cu
-bool halo_eligible(int kh, int kw);
+bool halo_eligible(int h, int w, int kh, int kw, int stride, int pad);
 int run_conv_halo(const Params &g, const void *X, int n, int c, int h, int w, int kh, int kw, int stride, int pad, int sm_count,
                   cudaStream_t st);
 // decode-once path, defined in mwu_gemm3.cu
@@ -711,7 +711,7 @@ extern "C" int mwu_conv_implicit(const mwu_proj_desc *desc, const void *packed, 
     Params p = {};
     fill_common(p, desc, packed, Y_nchw, y_dtype, dev_status);
     if (p.n_stages > MAX_STAGES_K) return MWU_ERR_SHAPE;
-    if (halo_eligible(kh, kw))
+    if (halo_eligible(h, w, kh, kw, stride, pad))
         return run_conv_halo(p, X_nchw, n, c, h, w, kh, kw, stride, pad, sm_count, (cudaStream_t)cuda_stream);
     p.X = (const __nv_bfloat16 *)X_nchw;
     p.C = c; p.H = h; p.W = w; p.KH = kh; p.KW = kw; p.stride = stride; p.pad = pad;

@@ -359,3 +359,19 @@ def test_gemm_long_fp32_sums_hardly_depend_on_the_row_count(cols):
     torch.cuda.synchronize()
     assert int(bufs.dev_status.item()) == 0
     assert float((out[0] - out[1]).norm() / out[1].norm()) < 4.5e-6
+
+
+def test_conv_padding_of_two_to_the_32_pixels():
+    """Paddings may be 32767 wide: 2 x 2 pixels become 65536 x 65536, whose number does not fit 32 bits."""
+    W = inputs.normal_weights(8, 64, 0.05, 797)
+    desc, bufs, packed, p = project_and_pack(W[:1].contiguous(), 4, 8, 4)
+    x = inputs.normal_activations_bf16((1, 64, 2, 2), 798)
+    Y = torch.full((1, 1, 65536, 65536), float("nan"), dtype=torch.bfloat16, device="cuda")
+    B.mwu_conv_implicit(desc, packed, x.cuda(), 1, 64, 2, 2, 1, 1, 1, 32767, Y, 0, bufs.dev_status)
+    torch.cuda.synchronize()
+    assert int(bufs.dev_status.item()) == 0
+    ref = np.einsum("ok,nkhw->nohw", O.decoded_weights(p), x.to(torch.float64).numpy())
+    inner = Y[:, :, 32767:32769, 32767:32769]
+    assert errors(inner.float().cpu().numpy(), ref)[1] <= 1e-2
+    inner.zero_()
+    assert all(int(torch.count_nonzero(Y[0, 0, r:r + 8192])) == 0 for r in range(0, 65536, 8192))
