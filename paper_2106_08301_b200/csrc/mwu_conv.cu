@@ -35,7 +35,7 @@ struct ConvParams {
     long long M;                        // its pixels: NIMG * Hp * Wp
     unsigned img_magic, row_magic;
     int tm;                             // pixels of a tile: 128 or 256
-    int rows_apart;                     // 1: a fetch serves one kernel row, not all taps
+    int fetches;                        // fetches of a tile and 64 channels: one for all taps, one per kernel row, or one per tap
     int a_rows, a_bufs, box_rows;       // rows of a fetch, buffers, rows of a TMA box
     int b_stages;
     int n_ntiles;                       // 128-filter tiles
@@ -198,7 +198,7 @@ mwu_conv_line_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_co
     volatile int *abort = &sm->abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int chunks = p.C / BK;                            // of 64 channels
-    const int fetches = p.rows_apart ? p.KH : 1, taps_per = p.KH * p.KW / fetches;
+    const int fetches = p.fetches, taps_per = p.KH * p.KW / fetches;
     const int m_tiles = (int)((p.M + p.tm - 1) / p.tm);
     const long long total_tiles = (long long)m_tiles * p.n_ntiles;
     const long long limit = p.wait_limit;
@@ -242,13 +242,14 @@ mwu_conv_line_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_co
             for (long long t = blockIdx.x; ok && t < total_tiles; t += gridDim.x) {
                 const int p0 = (int)(t / p.n_ntiles) * p.tm;
                 for (int f = 0; f < chunks * fetches; ++f) {
-                    const int chunk = f / fetches, di = f - chunk * fetches;
+                    const int chunk = f / fetches, part = f - chunk * fetches;
                     ok = mbar_wait_lim<true>(smem_u32(&sm->a_empty[buf]), phase ^ 1u, abort, limit);
                     if (!ok) break;
                     const unsigned bar = smem_u32(&sm->a_full[buf]);
                     mbar_expect_tx(bar, a_bytes);
                     // a box may start before the first pixel or end after the last: zeros there
-                    const int row = p0 - p.shift * (p.Wp + 1) + (p.rows_apart ? di * p.Wp : 0);
+                    const int first = fetches > p.KH ? part / p.KW * p.Wp + part % p.KW : part * p.Wp;      // its first tap's shift
+                    const int row = p0 - p.shift * (p.Wp + 1) + first;
                     for (int b = 0; b * p.box_rows < p.a_rows; ++b)
                         tma_load_2d(smem_u32(sA + buf * a_bytes + (unsigned)(b * p.box_rows) * 128u), &tmap_x, bar, chunk * BK,
                                     row + b * p.box_rows);
@@ -457,11 +458,13 @@ static int run_line(ConvParams &p, int bw, const void *Wd, long long ldw, const 
     p.wait_limit = g_wait_limit;
     p.withhold = g_withhold;
     // Tiles of 256 pixels share a weight box between two accumulators; of 128 where those would leave SMs idle.
-    // All taps from one fetch where two buffers of it fit beside four weight boxes, else a fetch per kernel row.
+    // All taps from one fetch where two buffers of it fit beside four weight boxes, else a fetch per kernel row, and for
+    // kernels too wide for that (some 1300 columns) one per tap.
     const long long room = L_SMEM - 2048;
     p.tm = (p.M + 255) / 256 * p.n_ntiles * 10 >= 6ll * sm_count ? 256 : 128;
-    for (p.rows_apart = 0;; p.rows_apart = 1) {
-        const long long rows = p.tm + (p.rows_apart ? 0 : (long long)(kh - 1) * p.Wp) + kw - 1;
+    for (const int fetches : {1, kh, kh * kw}) {
+        const long long rows = p.tm + (fetches > 1 ? 0 : (long long)(kh - 1) * p.Wp) + (fetches > kh ? 0 : kw - 1);
+        p.fetches = fetches;
         const long long boxes = (rows + 255) / 256;
         p.box_rows = (int)(((rows + boxes - 1) / boxes + 7) / 8 * 8);
         const long long a_rows = boxes * p.box_rows;
@@ -470,7 +473,6 @@ static int run_line(ConvParams &p, int bw, const void *Wd, long long ldw, const 
         p.a_rows = (int)a_rows;
         p.b_stages = left / REC_BYTES > L_MAX_STAGES ? L_MAX_STAGES : (int)(left / REC_BYTES);
         if (left >= 2 * REC_BYTES) break;
-        if (p.rows_apart) return MWU_ERR_SHAPE;
     }
     unsigned short *xt = (unsigned short *)workspace;
     unsigned short *wt = (unsigned short *)((char *)workspace + line_bytes(n, c, h, w, kh, kw, pad));

@@ -375,3 +375,37 @@ def test_conv_padding_of_two_to_the_32_pixels():
     assert errors(inner.float().cpu().numpy(), ref)[1] <= 1e-2
     inner.zero_()
     assert all(int(torch.count_nonzero(Y[0, 0, r:r + 8192])) == 0 for r in range(0, 65536, 8192))
+
+
+@pytest.mark.parametrize("kh,kw,h,w,n", [(1, 1400, 3, 1450, 1),      # the widest kernel row that one fetch holds
+                                         (1, 1450, 3, 1500, 1),      # a fetch per tap
+                                         (2, 1450, 4, 1500, 1),
+                                         (1, 1450, 64, 1500, 2)])    # the same with tiles of 256 pixels
+def test_conv_wide_kernels_with_workspace(kh, kw, h, w, n):
+    torch.manual_seed(800 + kh + kw + h)
+    rows, cin, cols = 16, 64, 64 * kh * kw
+    W = torch.randn(rows, cols, device="cuda") * 0.02
+    x = torch.randn(n, cin, h, w, device="cuda").bfloat16()
+    desc = B.make_desc(rows, cols, 16, rows * cols // 32, rows * cols // 64)
+    bufs = B.ProjectionBuffers(desc)
+    bufs.project(W)
+    packed = bufs.pack(W)
+    Wd = torch.empty(128, cols, dtype=torch.bfloat16, device="cuda")
+    B.mwu_decode(desc, packed, Wd, cols, bufs.dev_status)
+    # im2col is all it takes: the kernel spans almost the whole row
+    A = x.double().unfold(2, kh, 1).unfold(3, kw, 1).permute(0, 2, 3, 1, 4, 5)
+    ref = torch.stack([A[i].reshape(A.shape[1], A.shape[2], cols) @ Wd[:rows].double().t() for i in range(n)]).permute(0, 3, 1, 2)
+    args = (x, n, cin, h, w, kh, kw, 1, 0)
+    ws = torch.empty(max(B.mwu_conv_workspace_bytes(desc, *args[1:]), B.mwu_conv_dense_workspace_bytes(rows, *args[1:])),
+                     dtype=torch.uint8, device="cuda")
+    for call in ("dense", "packed"):
+        Y = torch.full(ref.shape, float("nan"), device="cuda")
+        if call == "dense":
+            B.mwu_conv_dense(rows, Wd, cols, *args, Y, 1, ws, bufs.dev_status)
+        else:
+            B.mwu_conv_implicit_ws(desc, packed, *args, Y, 1, ws, bufs.dev_status)
+        torch.cuda.synchronize()
+        assert int(bufs.dev_status.item()) == 0
+        # an MMA adds 16 products and may cut its accumulator off at 2^-23 of itself; the partial sums of independent
+        # products are no larger, in the mean, than the whole
+        assert float((Y.double() - ref).norm() / ref.norm()) <= 2.0 ** -23 * cols / 16, call
