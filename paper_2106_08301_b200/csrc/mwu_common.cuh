@@ -140,10 +140,11 @@ inline cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block,
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// Can this device run clusters of `ctas` CTAs, one to an SM?  Sixteen is more than every device has to offer.  A fact of
-// the device: asked once for each, with any kernel that uses such clusters.
-template <typename... KArgs>
-inline bool cluster_runs(void (*kern)(KArgs...), int ctas, int threads) {
+// Can this device run clusters of CTAS CTAs of THREADS threads of this kernel, with SMEM bytes of dynamic shared memory each (the
+// most that its launches take)?  Sixteen is more than every device, or part of one, has to offer.  A fact of the device and the
+// kernel: asked once for each.
+template <auto KERN, int CTAS, int THREADS, int SMEM>
+inline bool cluster_runs() {
     constexpr int DEVICES = 64;
     static std::atomic<signed char> known[DEVICES];         // 0: not asked yet, 1: yes, -1: no
     int dev = 0;
@@ -152,17 +153,19 @@ inline bool cluster_runs(void (*kern)(KArgs...), int ctas, int threads) {
     if (k == 0) {
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)ctas;
+        attr[0].val.clusterDim.x = CTAS;
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)ctas);
-        cfg.blockDim = dim3((unsigned)threads);
+        cfg.gridDim = dim3(CTAS);
+        cfg.blockDim = dim3(THREADS);
+        cfg.dynamicSmemBytes = SMEM;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        const bool yes = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                         cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0;
+        const bool yes = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) == cudaSuccess &&
+                         cudaFuncSetAttribute(KERN, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                         cudaOccupancyMaxActiveClusters(&n, KERN, &cfg) == cudaSuccess && n > 0;
         if (!yes) cudaGetLastError();
         k = yes ? 1 : -1;
         known[dev].store(k, std::memory_order_relaxed);

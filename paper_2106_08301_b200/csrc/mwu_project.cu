@@ -2101,7 +2101,7 @@ static Route route_of(const mwu_proj_desc *desc, int sm_count) {
         return r;
     }
     r.cluster = ((mb <= EX_CLUSTER_BLOCKS && units <= EX_CLUSTER_UNITS) || units <= sel::CLUSTER_CTAS * proj::CL_THREADS) &&
-                cluster_runs(proj::exact_kernel<16, true>, sel::CLUSTER_CTAS, proj::CL_THREADS);
+                cluster_runs<proj::exact_kernel<16, true>, sel::CLUSTER_CTAS, proj::CL_THREADS, proj::EX_SLOTS * 16>();
     const long long threads = r.cluster ? proj::CL_THREADS : proj::GR_THREADS;
     const long long ctas = (units + 127) / 128;                      // four warps with a unit a lane
     r.grid = r.cluster ? sel::CLUSTER_CTAS : (int)(ctas < sm_count ? ctas : sm_count);

@@ -261,7 +261,7 @@ static cudaError_t launch(const SParams &p, const mwu_proj_desc *desc, int sm_co
     // it than the cluster's barriers save (9216 blocks: 19.4 us as a cluster, 25.8 as a grid; 18432: 25.5 / 25.8; 27648:
     // 30.6 / 26.0).  Keys held while a CTA's fit.
     if (mb <= (long long)SH_CLUSTER_PER * sel::CLUSTER_CTAS * SH_THREADS &&
-        cluster_runs(shape_kernel<2, CLUSTER>, sel::CLUSTER_CTAS, SH_THREADS)) {
+        cluster_runs<shape_kernel<N, CLUSTER>, sel::CLUSTER_CTAS, SH_THREADS, SH_CLUSTER_PER * SH_THREADS * 16>()) {
         const unsigned per = (unsigned)((ctas + sel::CLUSTER_CTAS - 1) / sel::CLUSTER_CTAS);
         const size_t smem = (size_t)per * SH_THREADS * 16;
         const cudaError_t e = cudaFuncSetAttribute(shape_kernel<N, CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, SH_CLUSTER_PER * SH_THREADS * 16);

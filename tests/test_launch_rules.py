@@ -58,3 +58,12 @@ def test_dependents_start_only_once_tensor_memory_is_held(name, body):
     # thread's trigger counts for its CTA, so it is the warp that holds the allocation which triggers.
     assert re.search(r"\{\s*tmem_alloc\([^;]*;\s*asm volatile\(\"griddepcontrol.launch_dependents;\"[^;]*\);\s*\}", body)
     assert body.count("griddepcontrol.launch_dependents") == 1
+
+
+def test_the_question_for_clusters_names_their_shared_memory():
+    # without it several CTAs seem to fit an SM, and a part of a device that cannot place the cluster would answer yes
+    text = _strip_comments(open(os.path.join(CSRC, "mwu_common.cuh")).read())
+    body = text[text.index("inline bool cluster_runs"):]
+    body = body[:body.index("\n}\n")]
+    ask = body.index("cudaOccupancyMaxActiveClusters")
+    assert "dynamicSmemBytes" in body[:ask] and "cudaFuncAttributeMaxDynamicSharedMemorySize" in body[:ask]
