@@ -68,8 +68,6 @@ struct Sel {
 struct Filter {
     float plo, phi, pt;         // prune key: window, threshold
     float ulo, uhi, ut;         // L_u
-    float cap;                  // a survivor with a larger sum |v| is open whatever its L_u (the bound below does not hold)
-    float pad;
 };
 
 struct Work {
@@ -269,30 +267,53 @@ __device__ __forceinline__ void set_window(Sel *s, u64 lo, u64 hi, int nb) {
     s->shift0 = shift;
 }
 
-// Bounds of the fp32 keys of pass_kernel, with u = 2^-24, for a block of B <= 16 values a_i = |v_i| of sum S and mean q:
-//   sum of squares, sum        within B u (relative) of the exact one, as sums of positive terms;
-//   L_u = sum (a_i - q)^2      the computed mean is off by e <= 16 u q, which adds B e^2 exactly (the deviations from the
-//                              mean sum to zero); the rest is a sum of positive terms again: within (B + 3) u.
-// So with REL above 19 u plus a share of 1e-6 for B e^2: below REL * hi as long as S <= cap.  Results that
-// underflow are off by less than TINY more; one that overflows is infinite, and above any finite edge.
+// L_u = sum (a_i - q)^2 and *S = sum a_i of a block in fp32, a_i = |v_i| and q their mean, from the differences d_i = a_i - a_0 and not
+// from q, which fp32 rounds by more than the spread of an almost uniform block: L_u = sum d_i^2 - (sum d_i)^2 / B.  With u = 2^-24 every
+// d_i is within u of itself, sum d_i^2 within (B + 1) u, (sum d_i)^2 / B within 2 B u of sum d_i^2, and that is L_u + B (a_0 - q)^2 <= B L_u.
+// So L_u is within B (3 B + 1) u of itself, however small it is beside the block's mean; S within B^2 u.  L_u is NaN where sum d_i
+// overflows.
+template <int B>
+__device__ __forceinline__ float loss_u32(const float *x, float *S) {
+    const float a0 = fabsf(x[0]);
+    float sum = fabsf(x[1]) - a0;
+    if constexpr (B == 2) {
+        *S = a0 + fabsf(x[1]);
+        return 0.5f * sum * sum;
+    } else {
+        float sq = sum * sum;
+#pragma unroll
+        for (int l = 2; l < B; ++l) {
+            const float d = fabsf(x[l]) - a0;
+            sum += d;
+            sq = fmaf(d, d, sq);
+        }
+        *S = fmaf((float)B, a0, sum);
+        return fmaf(sum * (-1.f / (float)B), sum, sq);
+    }
+}
+
+// Edges of the windows for pass_kernel's fp32 keys.  The edges hold for any tensor: with a limit on how small L_u may be beside the
+// mean (which keys from an fp32 mean need) almost uniform blocks, or a threshold that few blocks reach, overflowed the candidate list
+// (16384 x 4096, b = 4, blocks uniform to 1e-4: 1380 us a call, so 165).  A sum of squares, all positive, is within (B + 1) u of the exact one, the others
+// within the bounds of loss_u32.  Results that underflow are off by less than TINY more.  Sums that overflow are infinite, and
+// the exact key may be a B-th of the largest fp32 number then: an edge not far below that has nothing certainly above it.
 __device__ __forceinline__ void make_filter(Filter *f, const Sel &sp, const Sel &su, u64 tp, u64 tu, int B) {
-    constexpr double REL = 4e-6, TINY = 0x1p-138;
+    constexpr double U = 0x1p-24, TINY = 0x1p-138;
     const float inf = __int_as_float(0x7f800000), nan = __int_as_float(0x7fffffff);
-    auto lower = [](u64 k) { return __double2float_rd(fma(__longlong_as_double((long long)k), 1.0 - REL, -TINY)); };
-    auto upper = [&](u64 k) {
-        const float x = __double2float_ru(fma(__longlong_as_double((long long)k), 1.0 + REL, TINY));
-        return x < inf ? x : nan;                     // nothing is certainly above
+    const double rel_p = (double)(B * B + 32) * U, rel_u = (double)(B * (3 * B + 4)) * U;
+    auto lower = [](u64 k, double rel) { return __double2float_rd(fma(__longlong_as_double((long long)k), 1.0 - rel, -TINY)); };
+    auto upper = [&](u64 k, double rel) {
+        const float x = __double2float_ru(fma(__longlong_as_double((long long)k), 1.0 + rel, TINY));
+        return x < 0x1p122f ? x : nan;
     };
     auto point = [](u64 k) { return __double2float_rn(__longlong_as_double((long long)k)); };
     // nothing open: no key is >= inf and below -1.  (mode 3, grouped pruning: pass_kernel sets pt by the group's bit.)
-    f->plo = sp.mode == 0u ? lower(sp.lo0) : inf;
-    f->phi = sp.mode == 0u ? upper(sp.hi0) : -1.f;
+    f->plo = sp.mode == 0u ? lower(sp.lo0, rel_p) : inf;
+    f->phi = sp.mode == 0u ? upper(sp.hi0, rel_p) : -1.f;
     f->pt = sp.mode == 0u ? point(tp) : (sp.mode == 2u ? inf : -1.f);
-    f->ulo = su.mode == 0u ? lower(su.lo0) : inf;
-    f->uhi = su.mode == 0u ? upper(su.hi0) : -1.f;
+    f->ulo = su.mode == 0u ? lower(su.lo0, rel_u) : inf;
+    f->uhi = su.mode == 0u ? upper(su.hi0, rel_u) : -1.f;
     f->ut = su.mode == 0u ? point(tu) : (su.mode == 2u ? inf : -1.f);
-    // B e^2 <= 256 u^2 S^2 / B <= 1e-6 hi
-    f->cap = su.mode == 0u ? __double2float_rd(sqrt(0.9e-6 * (double)B * __longlong_as_double((long long)su.hi0)) * (0x1p24 / 16.0)) : inf;
 }
 
 // inclusive prefix sum over the CTA's SAMP_THREADS values (one per thread)
@@ -1229,6 +1250,7 @@ pass_kernel(const __grid_constant__ Params p, float *Q, double *loss_u, double *
     if (step < n_steps) load_step<B>(p.W, p.U, step, lane, n, nxt);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const Filter F = p.work->filter;
+    const bool some_u = F.ut >= 0.f;
     const bool by_group = p.gprune != nullptr;
     const unsigned nb = (unsigned)p.nb, top = nb - 1u;
     unsigned *hist_p = p.fhist, *hist_u = p.fhist + p.nb;
@@ -1320,26 +1342,17 @@ pass_kernel(const __grid_constant__ Params p, float *Q, double *loss_u, double *
                 // a lane's 64 bytes, or a piece of 16, lie in one group (groups are at least 16 columns wide)
                 pt = block_of(e) < n_blocks && group_pruned(p, block_of(e)) ? __int_as_float(0x7f800000) : -1.f;
             }
-            // fp32 keys (any order of summation)
-            float s[B];
+            // fp32 keys (see make_filter)
+            float S32;
+            const float ku = loss_u32<B>(x, &S32);
+            float kp = x[0] * x[0];
 #pragma unroll
-            for (int l = 0; l < B; ++l) s[l] = fabsf(x[l]);
-#pragma unroll
-            for (int w = 1; w < B; w <<= 1)
-#pragma unroll
-                for (int l = 0; l < B; l += 2 * w) s[l] += s[l + w];
-            const float S32 = s[0], q32 = S32 * (1.f / (float)B);
-            float kp = 0.f, ku = 0.f;
-#pragma unroll
-            for (int l = 0; l < B; ++l) {
-                const float d = fabsf(x[l]) - q32;
-                ku = fmaf(d, d, ku);
-                kp = fmaf(x[l], x[l], kp);
-            }
+            for (int l = 1; l < B; ++l) kp = fmaf(x[l], x[l], kp);
             if (p.use_l1) kp = S32;
             const bool there = full || block_of(e) < n_blocks;
-            const bool pr = kp <= pt && there, un = !pr && ku <= F.ut && there;
-            const bool open = ((kp >= F.plo && !(kp >= F.phi)) || (!pr && ((ku >= F.ulo && !(ku >= F.uhi)) || !(S32 <= F.cap)))) && there;
+            // (a NaN is open, and unified where everything is)
+            const bool pr = kp <= pt && there, un = !pr && !(ku > F.ut) && some_u && there;
+            const bool open = ((kp >= F.plo && !(kp >= F.phi)) || (!pr && !(ku < F.ulo) && !(ku >= F.uhi))) && there;
             cls_p |= pr ? 1u << e : 0u;
             cls_u |= un ? 1u << e : 0u;
             cand |= open ? 1u << e : 0u;

@@ -366,3 +366,47 @@ def test_pack_one_kernel_edges(b, rows, cols):
     packed = bufs.pack(Wd)
     torch.cuda.synchronize()
     check_pack(desc, bufs, packed, p, b)
+
+
+@pytest.mark.parametrize("b,kind", [(2, "1e-3"), (4, "1e-3"), (4, "1e-5"), (16, "1e-4"), (16, "1e-6")])
+def test_one_pass_is_not_given_up_where_unified_blocks_are_few_or_blocks_almost_uniform(b, kind):
+    """L_u at the threshold is then a small part of the blocks' means.  Were their fp32 keys too coarse for that, most
+    blocks would be listed as open, the list would overflow and the exact phases take three to six times as long."""
+    rows = cols = 4096
+    g = torch.Generator(device="cuda").manual_seed(40 + b)
+    plain = torch.randn(rows, cols, generator=g, device="cuda") * 0.02
+    W, share, prune = plain, 0.0005, 0.0
+    if kind != "few unified":
+        m = plain.view(rows, -1, b).abs().mean(-1, keepdim=True) * (1 + float(kind) * torch.randn(rows, cols // b, b, generator=g, device="cuda"))
+        W, share, prune = (torch.sign(plain).view(rows, -1, b) * m).view(rows, cols).contiguous(), 0.5, 0.25
+    Mb = rows * cols // b
+
+    def project(W, ku, kp, algo):
+        bufs = B.ProjectionBuffers(B.make_desc(rows, cols, b, ku, kp, algo=algo))
+        times = []
+        for _ in range(8):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            bufs.project(W)
+            end.record()
+            torch.cuda.synchronize()
+            times.append(start.elapsed_time(end))
+        assert int(bufs.dev_status.item()) == 0
+        return bufs, min(times)
+
+    got, t = project(W, int(Mb * share), int(Mb * prune), B.MWU_ALGO_ONE_PASS)
+    ref, _ = project(W, int(Mb * share), int(Mb * prune), B.MWU_ALGO_MULTI_PASS)
+    _, t_plain = project(plain, Mb // 2, Mb // 4, B.MWU_ALGO_ONE_PASS)
+    for name in ("Q", "u", "pruned_bitmap", "unified_bitmap", "sign_bits"):
+        assert torch.equal(getattr(got, name), getattr(ref, name)), name
+    assert t <= 2 * t_plain, (t, t_plain)
+
+
+@pytest.mark.parametrize("b", [2, 4, 16])
+@pytest.mark.parametrize("share,prune", [(5, 2), (10, 0), (10, 4), (4, 4)])       # tenths: both thresholds, one of them, none
+def test_one_pass_where_differences_overflow(b, share, prune):
+    W = inputs.normal_weights(64, 1024, 0.02, 7100 + b)
+    W = W / W.abs().max() * 3.3e38
+    W[:, 512:] *= 1e-3                                # and some whose sums do not
+    Mb = W.numel() // b
+    check_against_oracle(W.contiguous(), b, Mb * share // 10, Mb * prune // 10, algos=(B.MWU_ALGO_ONE_PASS,))
