@@ -287,7 +287,7 @@ __device__ __forceinline__ float loss_u32(const float *x, float *S) {
             sum += d;
             sq = fmaf(d, d, sq);
         }
-        *S = fmaf((float)B, a0, sum);
+        *S = fabsf(fmaf((float)B, a0, sum));            // infinite, not -inf, where sum d_i overflows
         return fmaf(sum * (-1.f / (float)B), sum, sq);
     }
 }

@@ -404,9 +404,10 @@ def test_one_pass_is_not_given_up_where_unified_blocks_are_few_or_blocks_almost_
 
 @pytest.mark.parametrize("b", [2, 4, 16])
 @pytest.mark.parametrize("share,prune", [(5, 2), (10, 0), (10, 4), (4, 4)])       # tenths: both thresholds, one of them, none
-def test_one_pass_where_differences_overflow(b, share, prune):
+@pytest.mark.parametrize("prune_key", [B.MWU_PRUNE_KEY_L2SQ, B.MWU_PRUNE_KEY_L1])
+def test_one_pass_where_differences_overflow(b, share, prune, prune_key):
     W = inputs.normal_weights(64, 1024, 0.02, 7100 + b)
     W = W / W.abs().max() * 3.3e38
     W[:, 512:] *= 1e-3                                # and some whose sums do not
     Mb = W.numel() // b
-    check_against_oracle(W.contiguous(), b, Mb * share // 10, Mb * prune // 10, algos=(B.MWU_ALGO_ONE_PASS,))
+    check_against_oracle(W.contiguous(), b, Mb * share // 10, Mb * prune // 10, prune_key=prune_key, algos=(B.MWU_ALGO_ONE_PASS,))
