@@ -368,15 +368,19 @@ def test_pack_one_kernel_edges(b, rows, cols):
     check_pack(desc, bufs, packed, p, b)
 
 
-@pytest.mark.parametrize("b,kind", [(2, "1e-3"), (4, "1e-3"), (4, "1e-5"), (16, "1e-4"), (16, "1e-6")])
+@pytest.mark.parametrize("b,kind", [(2, "1e-3"), (4, "1e-3"), (4, "1e-5"), (16, "1e-4"), (16, "1e-6"),
+                                    (2, "few unified"), (4, "few unified"), (16, "few unified"), (4, "few pruned"), (4, "few kept")])
 def test_one_pass_is_not_given_up_where_unified_blocks_are_few_or_blocks_almost_uniform(b, kind):
-    """L_u at the threshold is then a small part of the blocks' means.  Were their fp32 keys too coarse for that, most
-    blocks would be listed as open, the list would overflow and the exact phases take three to six times as long."""
+    """L_u at the threshold is then a small part of the blocks' means, and the threshold near an end of the sample.  Were the
+    fp32 keys too coarse most blocks would be listed as open and the list overflow; were the sample's window to miss the
+    threshold the result would be void.  Either way the exact phases then take three to six times as long."""
     rows = cols = 4096
     g = torch.Generator(device="cuda").manual_seed(40 + b)
     plain = torch.randn(rows, cols, generator=g, device="cuda") * 0.02
-    W, share, prune = plain, 0.0005, 0.0
-    if kind != "few unified":
+    W = plain
+    if kind.startswith("few"):
+        share, prune = {"few unified": (0.0005, 0.0), "few pruned": (0.5, 0.0005), "few kept": (0.9995, 0.9)}[kind]
+    else:
         m = plain.view(rows, -1, b).abs().mean(-1, keepdim=True) * (1 + float(kind) * torch.randn(rows, cols // b, b, generator=g, device="cuda"))
         W, share, prune = (torch.sign(plain).view(rows, -1, b) * m).view(rows, cols).contiguous(), 0.5, 0.25
     Mb = rows * cols // b
