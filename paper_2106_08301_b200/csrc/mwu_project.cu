@@ -984,9 +984,14 @@ struct WalkedKeys {
         const unsigned n_units = (unsigned)((p.n_floats + 15) / 16);
         const Outs none = {};
         unsigned bad = 0;
+        float nxt[16];
+        if (first < n_units) load16(p.W, p.U, (long long)first * 16, p.n_floats, nxt);
+#pragma unroll 1
         for (unsigned unit = first; unit < n_units; unit += stride) {
             float v[16];
-            load16(p.W, p.U, (long long)unit * 16, p.n_floats, v);
+#pragma unroll
+            for (int l = 0; l < 16; ++l) v[l] = nxt[l];
+            if (unit + stride < n_units) load16(p.W, p.U, (long long)(unit + stride) * 16, p.n_floats, nxt);      // travels meanwhile
 #pragma unroll
             for (int e = 0; e < NBT; ++e) {
                 u64 kp, ku;
@@ -1021,6 +1026,8 @@ template <int B, int NT>
 __device__ __noinline__ void exact_walk(const Params &p, const Outs &o, const sel::Problem &pb, sel::GridTeam &team, ExactSmem<NT> &sm) {
     constexpr int NBT = 16 / B;
     const WalkedKeys<B> src = {p, team.cta * NT + threadIdx.x, team.n_cta * NT};
+    __syncthreads();                                     // a caller's shared memory is no longer read
+    for (int i = threadIdx.x; i < sel::GRID_BINS; i += NT) team.local[i] = 0u;
     if (p.resid && team.cta == 0 && threadIdx.x == 0) *p.resid = 0.0;
     sel::Thresholds T;
     float sp, su;
@@ -1033,10 +1040,15 @@ __device__ __noinline__ void exact_walk(const Params &p, const Outs &o, const se
     const unsigned n_units = (unsigned)((p.n_floats + 15) / 16);
     double resid = 0.0;
     unsigned bad = 0;
+    float nxt[16];
+    load16(p.W, p.U, (long long)src.first * 16, p.n_floats, nxt);
+#pragma unroll 1
     for (unsigned unit = src.first; unit < (n_units + 31u) / 32u * 32u; unit += src.stride) {
         float v[16];
         unsigned cp = 0, cu = 0;
-        load16(p.W, p.U, (long long)unit * 16, p.n_floats, v);
+#pragma unroll
+        for (int l = 0; l < 16; ++l) v[l] = nxt[l];
+        if (unit + src.stride < n_units) load16(p.W, p.U, (long long)(unit + src.stride) * 16, p.n_floats, nxt);
 #pragma unroll
         for (int e = 0; e < NBT; ++e) {
             u64 kp, ku;
@@ -1074,6 +1086,7 @@ __global__ void __launch_bounds__(CLUSTER ? CL_THREADS : GR_THREADS) exact_kerne
         team.n_cta = gridDim.x;
         team.x = p.xwork;
         team.k = 0;
+        team.local = nullptr;
     }
     float v[16];
     // warps are dealt out over the CTAs, so that a tensor with less than a unit a thread keeps all SMs busy
@@ -1125,11 +1138,13 @@ __global__ void __launch_bounds__(CLUSTER ? CL_THREADS : GR_THREADS) exact_kerne
 
 // MWU_ALGO_MULTI_PASS on tensors whose keys do not fit
 constexpr int WALK_THREADS = 512;
+constexpr int WALK_SMEM = (int)sizeof(ExactSmem<WALK_THREADS>) + sel::GRID_BINS * 4;
 template <int B>
 __global__ void __launch_bounds__(WALK_THREADS) exact_walk_kernel(const __grid_constant__ Params p, const __grid_constant__ Outs o,
                                                                   const __grid_constant__ sel::Problem pb) {
-    __shared__ ExactSmem<WALK_THREADS> sm;
-    sel::GridTeam team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u};
+    extern __shared__ __align__(16) unsigned char mp_smem[];
+    ExactSmem<WALK_THREADS> &sm = *reinterpret_cast<ExactSmem<WALK_THREADS> *>(mp_smem);
+    sel::GridTeam team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u, reinterpret_cast<unsigned *>(mp_smem + sizeof(sm))};
     exact_walk<B, WALK_THREADS>(p, o, pb, team, sm);
 }
 
@@ -1577,7 +1592,8 @@ __device__ __forceinline__ double apply_class(const Params &p, float *Q, float *
 constexpr int CHG_PER_THREAD = 4;                    // list entries a thread classifies before the changed ones are applied
 // candidate buffers, corrections and the compaction buffer; the fallback's staging memory
 constexpr int RES_SMEM_USED = CAP * 20 + CHG_PER_THREAD * FIN_THREADS * 8;
-constexpr int RES_SMEM_BYTES = RES_SMEM_USED > (int)sizeof(ExactSmem<FIN_THREADS>) ? RES_SMEM_USED : (int)sizeof(ExactSmem<FIN_THREADS>);
+constexpr int RES_SMEM_EXACT = (int)sizeof(ExactSmem<FIN_THREADS>) + sel::GRID_BINS * 4;
+constexpr int RES_SMEM_BYTES = RES_SMEM_USED > RES_SMEM_EXACT ? RES_SMEM_USED : RES_SMEM_EXACT;
 
 // rank the m candidates in shared memory (c_key, c_idx) by (key, index); m <= CAP
 // c_aux (when the candidates fit one per thread: the return value) receives g_aux in the same order
@@ -1864,7 +1880,7 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
     // ---------------- 5: the fallback, if the one-pass result was given up anywhere ----------------
     if (!failed) return;
     ExactSmem<FIN_THREADS> &sm = *reinterpret_cast<ExactSmem<FIN_THREADS> *>(mp_smem);
-    sel::GridTeam team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u};
+    sel::GridTeam team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u, reinterpret_cast<unsigned *>(mp_smem + sizeof(sm))};
     const Outs o = {Q, loss_u, loss_p, u_out, pruned_bitmap, unified_bitmap, sign_bits};
     exact_walk<B, FIN_THREADS>(p, o, pb, team, sm);
 }
@@ -2208,7 +2224,9 @@ static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_des
         if (!route.cluster && cudaMemsetAsync(p.xwork, 0, mwu::sel::XWORK_ZERO_BYTES, st) != cudaSuccess) return cudaErrorUnknown;
         if (route.held) return launch_exact_held<B>(p, o, route, sm_count, st);
         const long long want = (n_units + WALK_THREADS - 1) / WALK_THREADS;
-        return launch_cooperative(exact_walk_kernel<B>, (int)(want < 2ll * sm_count ? want : 2ll * sm_count), WALK_THREADS, 0,
+        e = cudaFuncSetAttribute(exact_walk_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, WALK_SMEM);
+        if (e != cudaSuccess) return e;
+        return launch_cooperative(exact_walk_kernel<B>, (int)(want < 2ll * sm_count ? want : 2ll * sm_count), WALK_THREADS, (size_t)WALK_SMEM,
                                   sm_count, st, p, o,
                                   mwu::sel::problem_of(p.n_blocks, p.k_prune, p.k_unify, p.gprune != nullptr, WALK_THREADS));
     }

@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(SH_THREADS) shape_kernel(const __grid_constant
         team.n_cta = gridDim.x;
         team.x = p.xwork;
         team.k = 0;
+        team.local = nullptr;
     }
     const unsigned first = blockIdx.x * SH_THREADS + threadIdx.x, stride = gridDim.x * SH_THREADS;
     const int lane = threadIdx.x & 31;

@@ -415,3 +415,30 @@ def test_one_pass_where_differences_overflow(b, share, prune, prune_key):
     W[:, 512:] *= 1e-3                                # and some whose sums do not
     Mb = W.numel() // b
     check_against_oracle(W.contiguous(), b, Mb * share // 10, Mb * prune // 10, prune_key=prune_key, algos=(B.MWU_ALGO_ONE_PASS,))
+
+
+@pytest.mark.parametrize("kind", ["zeros", "quantised"])
+def test_one_pass_given_up_over_ties_does_not_crowd_one_counter(kind):
+    """Millions of equal keys fall into one bin of the exact phases: counted CTA by CTA in shared memory, a round costs what it
+    does for other inputs, counted in L2 it took some five times the whole call."""
+    rows = cols = 4096
+    b = 4
+    g = torch.Generator(device="cuda").manual_seed(60)
+    W = torch.randn(rows, cols, generator=g, device="cuda") * 0.02
+    W = torch.zeros_like(W) if kind == "zeros" else (W * 64).round() / 64
+    Mb = rows * cols // b
+    bufs = B.ProjectionBuffers(B.make_desc(rows, cols, b, Mb // 2, Mb // 4))
+    times = []
+    for _ in range(6):
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        bufs.project(W)
+        end.record()
+        torch.cuda.synchronize()
+        times.append(start.elapsed_time(end))
+    assert int(bufs.dev_status.item()) == 0
+    p = O.project(W.cpu().numpy(), b, Mb // 2, Mb // 4)
+    assert np.array_equal(bufs.pruned_bitmap.cpu().numpy().view(np.uint32), O.bitmap_words(p.pruned))
+    assert np.array_equal(bufs.unified_bitmap.cpu().numpy().view(np.uint32), O.bitmap_words(p.unified))
+    assert np.array_equal(bufs.Q.cpu().numpy().view(np.uint32), p.Q.reshape(-1).view(np.uint32))
+    assert min(times) < 2.5, times
