@@ -1023,7 +1023,7 @@ union ExactSmem {
 // The projection with keys evaluated in every phase, by all CTAs of a cooperative launch.  `team` has
 // its counters cleared.
 template <int B, int NT>
-__device__ __noinline__ void exact_walk(const Params &p, const Outs &o, const sel::Problem &pb, sel::GridTeam &team, ExactSmem<NT> &sm) {
+__device__ __noinline__ void exact_walk(const Params &p, const Outs &o, const sel::Problem &pb, sel::GridTeam<true> &team, ExactSmem<NT> &sm) {
     constexpr int NBT = 16 / B;
     const WalkedKeys<B> src = {p, team.cta * NT + threadIdx.x, team.n_cta * NT};
     __syncthreads();                                     // a caller's shared memory is no longer read
@@ -1073,7 +1073,7 @@ __global__ void __launch_bounds__(CLUSTER ? CL_THREADS : GR_THREADS) exact_kerne
     constexpr int NBT = 16 / B, NT = CLUSTER ? CL_THREADS : GR_THREADS;
     extern __shared__ __align__(16) unsigned char mp_smem[];
     __shared__ ExactSmem<NT> sm;
-    typename std::conditional<CLUSTER, sel::ClusterTeam, sel::GridTeam>::type team;
+    typename std::conditional<CLUSTER, sel::ClusterTeam, sel::GridTeam<false>>::type team;
     team.cta = blockIdx.x;
     team.s = &sm.sel;
     if constexpr (CLUSTER) {
@@ -1144,7 +1144,7 @@ __global__ void __launch_bounds__(WALK_THREADS) exact_walk_kernel(const __grid_c
                                                                   const __grid_constant__ sel::Problem pb) {
     extern __shared__ __align__(16) unsigned char mp_smem[];
     ExactSmem<WALK_THREADS> &sm = *reinterpret_cast<ExactSmem<WALK_THREADS> *>(mp_smem);
-    sel::GridTeam team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u, reinterpret_cast<unsigned *>(mp_smem + sizeof(sm))};
+    sel::GridTeam<true> team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u, reinterpret_cast<unsigned *>(mp_smem + sizeof(sm))};
     exact_walk<B, WALK_THREADS>(p, o, pb, team, sm);
 }
 
@@ -1880,7 +1880,7 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
     // ---------------- 5: the fallback, if the one-pass result was given up anywhere ----------------
     if (!failed) return;
     ExactSmem<FIN_THREADS> &sm = *reinterpret_cast<ExactSmem<FIN_THREADS> *>(mp_smem);
-    sel::GridTeam team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u, reinterpret_cast<unsigned *>(mp_smem + sizeof(sm))};
+    sel::GridTeam<true> team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u, reinterpret_cast<unsigned *>(mp_smem + sizeof(sm))};
     const Outs o = {Q, loss_u, loss_p, u_out, pruned_bitmap, unified_bitmap, sign_bits};
     exact_walk<B, FIN_THREADS>(p, o, pb, team, sm);
 }

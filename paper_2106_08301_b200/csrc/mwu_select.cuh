@@ -8,7 +8,7 @@
 //   round    keys inside the window are counted in equal bins, keys below it in one counter;
 //            after a team barrier every CTA finds the bin of the k-th element and that bin becomes
 //            the next window.  One round is the rule; a window that missed, or a bin that holds
-//            more than XCAP keys, takes another one.  A bin of one single key value that many
+//            more than XLIST keys, takes another one.  A bin of one single key value that many
 //            blocks share is divided further by block index, so ties of any number are exact;
 //   gather   the blocks of the final bin are listed; after a team barrier every CTA ranks them
 //            (a few dozen, by counting) and knows the threshold element.
@@ -31,7 +31,9 @@ namespace sel {
 
 typedef unsigned long long u64;
 
-constexpr int XCAP = 1024;          // most candidates a gather phase lists
+// Candidates that a gather phase may list, and how many it does: every CTA ranks them all, so more of them take longer than another
+// round (64 x 64 zeros in 2x2 blocks, 1024 equal keys: 166 us when they were all listed, so 39).
+constexpr int XCAP = 896, XLIST = 256;
 constexpr int XSAMP_MAX = 128;      // most sample blocks
 constexpr int ABOVE = 0x7fffffff;
 constexpr int XROUNDS_MAX = 64;     // 63 key bits and 31 index bits at 10 or 11 a round, plus windows that missed
@@ -241,8 +243,9 @@ struct XWork {
 constexpr size_t XWORK_ZERO_BYTES = offsetof(XWork, cand);
 static_assert(XWORK_ZERO_BYTES % 16 == 0 && offsetof(XWork, hist) % 16 == 0 && XCOPIES == 4, "16-byte accesses");
 
-// `local` (GRID_BINS words of shared memory, cleared, or null): a CTA of many blocks counts there first.  (Projections given up by
+// LOCAL: a CTA counts in shared memory first (`local`: GRID_BINS words, cleared).  (Projections given up by
 // the one pass, 4096 x 4096, b = 4: zeros 7650 us counted in L2, 620 so; 16384 x 4096, b = 4, projected once more 35900, 3660.)
+template <bool LOCAL>
 struct GridTeam {
     static constexpr int BIN_BITS = GRID_BIN_BITS;
     unsigned cta, n_cta;
@@ -274,12 +277,12 @@ struct GridTeam {
         return s_ok != 0;
     }
     __device__ __forceinline__ void count(unsigned buf, int bin) const {
-        if (local) atomicAdd(&local[bin], 1u);
+        if (LOCAL) atomicAdd(&local[bin], 1u);
         else atomicAdd(&x->hist[buf][bin * XCOPIES + (cta & 3u)], 1u);
     }
     // the counts of this CTA, before the barrier that ends their round
     __device__ __forceinline__ void flush(unsigned buf) const {
-        if (!local) return;
+        if (!LOCAL) return;
         __syncthreads();
         for (unsigned i = threadIdx.x; i < (unsigned)GRID_BINS; i += blockDim.x) {
             const unsigned n = local[i];
@@ -379,7 +382,7 @@ __device__ __forceinline__ bool narrow(Window &w, const Found &f, unsigned n_blo
         const u64 end = base + (1ull << w.shift);
         w.lo = base;
         if (end < w.hi) w.hi = end;
-        if (!w.by_index && f.cnt > (unsigned)XCAP && w.hi - w.lo == 1) {
+        if (!w.by_index && f.cnt > (unsigned)XLIST && w.hi - w.lo == 1) {
             w.by_index = true;              // one key value shared by many blocks: go on by index
             w.key = w.lo;
             w.lo = 0;
@@ -538,7 +541,7 @@ __device__ bool select_exact(const Src &src, TeamT &team, SelSmem &s, const Prob
             r = f.r;
             cnt = f.cnt;
             if (!narrow(wp, f, pb.n_blocks, TeamT::BIN_BITS) || rnd > (unsigned)XROUNDS_MAX) { fine = false; break; }
-            if (f.where == 0 && f.cnt <= (unsigned)XCAP) break;
+            if (f.where == 0 && f.cnt <= (unsigned)XLIST) break;
         }
         if (fine) {
             // candidates of the threshold bin; the survivors' first L_u round
@@ -594,7 +597,7 @@ __device__ bool select_exact(const Src &src, TeamT &team, SelSmem &s, const Prob
             r = f.r;
             cnt = f.cnt;
             if (!narrow(wu, f, pb.n_blocks, TeamT::BIN_BITS) || rnd > 2u * (unsigned)XROUNDS_MAX) { fine = false; break; }
-            if (f.where == 0 && f.cnt <= (unsigned)XCAP) break;
+            if (f.where == 0 && f.cnt <= (unsigned)XLIST) break;
         }
         if (fine) {
             src.for_blocks([&](unsigned j, u64 kp, u64 ku) {

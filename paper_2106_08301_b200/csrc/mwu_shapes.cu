@@ -103,7 +103,8 @@ __device__ __forceinline__ double emit_n(const SParams &p, unsigned j, long long
 constexpr u64 NO_KEY = ~0ull;
 constexpr int SH_THREADS = 512;
 constexpr int SH_SLOTS = 8192;                           // most blocks a CTA holds: 16 bytes of keys each
-enum Form { CLUSTER, GRID, WALK };                       // WALK: a grid that gathers the keys again in every phase
+// LARGE: a grid whose CTAs count in shared memory first; WALK: one that also gathers the keys again in every phase
+enum Form { CLUSTER, GRID, LARGE, WALK };
 
 // what select_exact sees: block first + t * stride in slot t of this thread's column ...
 struct Held {
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(SH_THREADS) shape_kernel(const __grid_constant
                                                            const __grid_constant__ sel::Problem pb, unsigned per) {
     extern __shared__ __align__(16) unsigned char key_smem[];
     __shared__ sel::SelSmem sm;
-    typename std::conditional<FORM == CLUSTER, sel::ClusterTeam, sel::GridTeam>::type team;
+    typename std::conditional<FORM == CLUSTER, sel::ClusterTeam, sel::GridTeam<FORM != GRID>>::type team;
     team.cta = blockIdx.x;
     team.s = &sm;
     if constexpr (FORM == CLUSTER) {
@@ -151,7 +152,12 @@ __global__ void __launch_bounds__(SH_THREADS) shape_kernel(const __grid_constant
         team.n_cta = gridDim.x;
         team.x = p.xwork;
         team.k = 0;
-        team.local = nullptr;
+        if constexpr (FORM == GRID) team.local = nullptr;
+        else {
+            __shared__ unsigned s_bins[sel::GRID_BINS];
+            for (int i = threadIdx.x; i < sel::GRID_BINS; i += SH_THREADS) s_bins[i] = 0u;      // (a barrier comes before any use)
+            team.local = s_bins;
+        }
     }
     const unsigned first = blockIdx.x * SH_THREADS + threadIdx.x, stride = gridDim.x * SH_THREADS;
     const int lane = threadIdx.x & 31;
@@ -246,6 +252,10 @@ __global__ void __launch_bounds__(256) lower_kernel(long long n_runs, long long 
 
 constexpr int SH_CLUSTER_PER = 2;                        // most blocks of a thread in the cluster form
 
+// Counting in shared memory costs a microsecond (20480 blocks: 24.8 us without, 26.2 with), and makes up for it above (262144 blocks:
+// 35.2 / 35.0; all keys equal: 1930 / 91).
+constexpr long long SH_GRID_BLOCKS = 65536;
+
 static int grid_for(long long items, int sm_count) {
     const long long want = (items + 255) / 256, cap = (long long)sm_count * 16;
     return (int)(want < cap ? (want > 0 ? want : 1) : cap);
@@ -275,7 +285,7 @@ static cudaError_t launch(const SParams &p, const mwu_proj_desc *desc, int sm_co
     const int grid = (int)(ctas < sm_count ? ctas : sm_count);
     unsigned per = (unsigned)((ctas + grid - 1) / grid);
     const bool held = (long long)per * SH_THREADS <= SH_SLOTS;
-    auto kern = held ? shape_kernel<N, GRID> : shape_kernel<N, WALK>;
+    auto kern = !held ? shape_kernel<N, WALK> : mb <= SH_GRID_BLOCKS ? shape_kernel<N, GRID> : shape_kernel<N, LARGE>;
     if (held) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SH_SLOTS * 16);
         if (e != cudaSuccess) return e;

@@ -168,3 +168,30 @@ def test_block_shape_projection_size_edges(shape, rows, cols):
     W = inputs.normal_weights(rows, cols, 0.02, 1900 + rows + cols)
     W[:: max(rows // 16, 1)] = 0.0                       # equal keys across many blocks
     check_shape(W, shape, 600, 300)
+
+
+@pytest.mark.parametrize("rows,cin,taps,dt", [(64, 64, 1, 1), (1024, 1024, 1, 1)])       # one cluster, a grid
+def test_shapes_of_equal_keys_take_no_multiple_of_the_time(rows, cin, taps, dt):
+    """All keys equal: they must be neither all ranked against one another nor all counted at one place in L2."""
+    times = {}
+    for kind in ("normal", "zeros"):
+        W = inputs.normal_weights(rows, cin * taps, 0.02, 50).cuda()
+        if kind == "zeros":
+            W.zero_()
+        mb = B.make_desc(rows, cin * taps, 2, 0, 0, block_rows=2, block_taps=dt, taps=taps).n_blocks
+        desc = B.make_desc(rows, cin * taps, 2, mb // 2, mb // 4, block_rows=2, block_taps=dt, taps=taps)
+        bufs = B.ProjectionBuffers(desc)
+        runs = []
+        for _ in range(10):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            bufs.project(W)
+            end.record()
+            torch.cuda.synchronize()
+            runs.append(start.elapsed_time(end))
+        assert int(bufs.dev_status.item()) == 0
+        times[kind] = min(runs)
+    # ten rounds more, and the lower block indices win
+    words = bufs.pruned_bitmap.cpu().numpy().view(np.uint32)
+    assert np.array_equal(np.unpackbits(words.view(np.uint8), bitorder="little")[:mb], np.arange(mb) < mb // 4)
+    assert times["zeros"] < 12 * times["normal"], times
