@@ -361,7 +361,8 @@ mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
 // host
 // ------------------------------------------------------------------------------------------
 // Shape of a launch: rows per CTA, CTAs per cluster, decode groups.  `cost` estimates the call in record times of
-// one CTA: waves of resident CTAs, each its stages plus a fixed part.
+// one CTA: waves of resident CTAs, each its stages plus a fixed part; a cluster's barriers and sums count two records and more
+// (256 x 256, b = 4, 8192 rows, 128 tiles of four records: 10.2 us unsplit, 13.9 in pieces of two).
 struct StreamPlan {
     StreamParams q;
     size_t smem;
@@ -388,7 +389,7 @@ static StreamPlan plan_with(const Params &p, int split, int sm_count) {
     const long long units = p.n_rec_tiles * s.q.m_tiles;
     s.grid = units * split;
     const long long waves = (s.grid + (long long)resident * sm_count - 1) / ((long long)resident * sm_count);
-    s.cost = waves * (s.q.stages_per + 4 + split / 2);
+    s.cost = waves * (s.q.stages_per + 4 + (split > 1 ? 1 + split / 2 : 0));
     return s;
 }
 
@@ -425,11 +426,24 @@ int stream_box_rows(const Params &p, int sm_count) { return plan_of(p, sm_count,
 // 27 / 66 at 16 rows, 41 / 68 at 128, 67 / 68 at 256, 131 / 89 at 512; 4096 x 4096, b = 8: 26 / 37 at 256, 41 / 37 at
 // 512; b = 2: 43 / 50 at 256, 72 / 52 at 512.  A small weight stays here longer, while the decodes are few to an
 // SM: 1000 x 1216, b = 8, 1024 rows (1216 decodes): 15 / 19; 4096 x 1024, b = 4, 512 rows (2048): 22 / 19.
+// bf16 results of more than 256 rows stay only while the tiles of 128 x 128 outputs are one to an SM, or two where the other path has
+// much to expand for its rows, or nothing expanded to work on (us, this kernel / the other: 1024 x 64, b = 4, 8192 rows, 512 tiles: 19.5 / 12.1;
+// 256 x 256, 16384 rows, 256 tiles: 14.2 / 11.1; 128 x 192, b = 16, 32768 rows, 256 tiles: 11.5 / 12.7; 4096 x 256, 777 rows, 224 tiles: 11.5 / 12.0;
+// without a workspace 512 x 256, 8192 rows, 256 tiles: 14.1 / 18.8, 128 x 192, 256 tiles: 11.0 / 10.6).  Nor where a reduction of less
+// than 1024 has to be split to two CTAs an SM (512 x 512, b = 4, 4096 rows: 15.9 / 12.0; 2048 x 512, 300 rows: 12.1 / 13.4).
+// fp32 results, which the other paths store in pieces of a row, stay (1024 x 64, 8192 rows: 19.2 / 20.3; 512 x 512, 2048 rows: 13.1 / 15.4).
 // Where it may not split as it would (128 x 7168, 55 rows, fp32: 16 us in eight pieces, 43 in two, 41 expanding), the
 // other path is taken if the caller's workspace allows it (can_expand).
 bool stream_eligible(const Params &p, int sm_count, bool can_expand) {
-    if (can_expand && most_pieces(p) < 8 && 2 * plan_of(p, sm_count, most_pieces(p)).cost > 3 * plan_of(p, sm_count, 8).cost) return false;
-    return p.M <= 256 || p.n_rec_tiles * p.n_stages * ((p.M + ST_MAX_ROWS - 1) / ST_MAX_ROWS) <= 9ll * sm_count;
+    const StreamPlan s = plan_of(p, sm_count, most_pieces(p));
+    if (can_expand && most_pieces(p) < 8 && 2 * s.cost > 3 * plan_of(p, sm_count, 8).cost) return false;
+    if (p.M <= 256) return true;
+    const long long tiles = p.n_rec_tiles * s.q.m_tiles;
+    if (tiles * p.n_stages > 9ll * sm_count) return false;
+    if (p.y_fp32) return true;
+    if (can_expand && p.n_stages < 16 && s.q.split > 1 && s.grid > sm_count && p.M > 512) return false;
+    const bool two = can_expand ? p.n_rec_tiles == 1 || s.q.m_tiles <= 8 : p.n_rec_tiles > 1 || p.n_stages > 1;
+    return tiles <= (two ? 2ll : 1ll) * sm_count;
 }
 
 cudaError_t launch_stream(int bw, const CUtensorMap &tmap_x, const Params &p, int sm_count, cudaStream_t st) {

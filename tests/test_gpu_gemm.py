@@ -361,22 +361,6 @@ def test_gemm_long_fp32_sums_hardly_depend_on_the_row_count(cols):
     assert float((out[0] - out[1]).norm() / out[1].norm()) < 4.5e-6
 
 
-def test_conv_padding_of_two_to_the_32_pixels():
-    """Paddings may be 32767 wide: 2 x 2 pixels become 65536 x 65536, whose number does not fit 32 bits."""
-    W = inputs.normal_weights(8, 64, 0.05, 797)
-    desc, bufs, packed, p = project_and_pack(W[:1].contiguous(), 4, 8, 4)
-    x = inputs.normal_activations_bf16((1, 64, 2, 2), 798)
-    Y = torch.full((1, 1, 65536, 65536), float("nan"), dtype=torch.bfloat16, device="cuda")
-    B.mwu_conv_implicit(desc, packed, x.cuda(), 1, 64, 2, 2, 1, 1, 1, 32767, Y, 0, bufs.dev_status)
-    torch.cuda.synchronize()
-    assert int(bufs.dev_status.item()) == 0
-    ref = np.einsum("ok,nkhw->nohw", O.decoded_weights(p), x.to(torch.float64).numpy())
-    inner = Y[:, :, 32767:32769, 32767:32769]
-    assert errors(inner.float().cpu().numpy(), ref)[1] <= 1e-2
-    inner.zero_()
-    assert all(int(torch.count_nonzero(Y[0, 0, r:r + 8192])) == 0 for r in range(0, 65536, 8192))
-
-
 @pytest.mark.parametrize("kh,kw,h,w,n", [(1, 1400, 3, 1450, 1),      # the widest kernel row that one fetch holds
                                          (1, 1450, 3, 1500, 1),      # a fetch per tap
                                          (2, 1450, 4, 1500, 1),
@@ -409,3 +393,30 @@ def test_conv_wide_kernels_with_workspace(kh, kw, h, w, n):
         # an MMA adds 16 products and may cut its accumulator off at 2^-23 of itself; the partial sums of independent
         # products are no larger, in the mean, than the whole
         assert float((Y.double() - ref).norm() / ref.norm()) <= 2.0 ** -23 * cols / 16, call
+
+
+@pytest.mark.parametrize("rows,cols,m,launches", [(1024, 64, 4096, 2), (1024, 64, 1024, 1),       # two tiles an SM; one
+                                                  (256, 256, 8192, 1), (256, 256, 16384, 2),
+                                                  (512, 512, 2048, 2), (512, 512, 512, 1)])       # split to two CTAs an SM
+def test_gemm_many_rows_of_a_small_weight(rows, cols, m, launches):
+    """Where the streaming kernel (one launch) gives way to expanding the weights (two): results on both sides of the line."""
+    torch.manual_seed(920)
+    W = torch.randn(rows, cols, device="cuda") * 0.02
+    Mb = rows * cols // 4
+    desc = B.make_desc(rows, cols, 4, Mb * 6 // 10, Mb * 4 // 10)
+    bufs = B.ProjectionBuffers(desc)
+    bufs.project(W)
+    packed = bufs.pack(W)
+    Wd = torch.empty(rows, cols, dtype=torch.bfloat16, device="cuda")
+    B.mwu_decode(desc, packed, Wd, cols, bufs.dev_status)
+    X = torch.randn(m, cols, device="cuda").bfloat16()
+    Y = torch.full((m, rows), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(B.mwu_gemm_workspace_bytes(desc, m), dtype=torch.uint8, device="cuda")
+    before = B.mwu_kernel_launches()
+    B.mwu_gemm_ws(desc, packed, X, m, cols, Y, rows, 0, ws, bufs.dev_status)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert B.mwu_kernel_launches() - before == launches
+    torch.cuda.synchronize()
+    assert int(bufs.dev_status.item()) == 0
+    ref = X.double() @ Wd.double().t()
+    assert float((Y.double() - ref).norm() / ref.norm()) <= 2e-3
