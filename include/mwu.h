@@ -278,7 +278,9 @@ int mwu_decode(const mwu_proj_desc *desc, const void *packed, void *Wd, int64_t 
  * aligned) the weights are expanded once per call as by mwu_decode and a two-operand
  * tensor-core GEMM reads them, still skipping the column slices that are pruned in every row
  * of a weight tile.  The result is the same contraction with the same rounding of operands
- * (bf16 x bf16, fp32 accumulation); only the summation order inside the tensor cores may differ.
+ * (bf16 x bf16, fp32 accumulation).  Which kernel runs, and in how many pieces it adds up the reduction, depends on M, on
+ * the sizes, on whether a workspace is given and on the device, and with it the last bits of an fp32 result (sums of K
+ * products of independent values: about 1e-9 K of their size in one piece, less in several).
  * Few rows (up to 256, or more where the weights are few) are multiplied without expanding anything
  * and mostly leave the workspace alone.
  * mwu_gemm_workspace_bytes returns 0 when M is too small for this to pay (or desc is invalid);

@@ -404,9 +404,10 @@ static cudaError_t launch_stream_bw(const CUtensorMap &tmap_x, const Params &p, 
 }
 
 // The tensor core drops what lies below an accumulator's last place, so a sum loses a little of its magnitude at every
-// step, and a sum in pieces less: an fp32 result of 7168 products differs by 5.1e-6 between one and eight pieces, by
-// 3.6e-6 between one and two.  bf16 results hide it; fp32 results stay within 4.5e-6 of what the kernels for more rows,
-// which never split, give.
+// step, and a sum in pieces less.  fp32 results of 128 x K, b = 4, 40 rows, against fp64: K = 6144 5.7e-7 in eight pieces (5.9e-6 in
+// one), 6912 1.4e-6 in four (6.7e-6), 16384 8.0e-6 in two (1.7e-5).  bf16 results hide it.  Results of few rows and of many, which the other
+// kernels never split, therefore differ by up to 5.6e-6 where this kernel takes over at K <= 6912; the limits keep it from
+// growing in proportion to K above (two pieces without a workspace: 5.1e-6 at 8192, 1.05e-5 at 16384).
 static int most_pieces(const Params &p) { return !p.y_fp32 || p.K <= 6144 ? 8 : p.K <= 6912 ? 4 : 2; }
 
 static StreamPlan plan_of(const Params &p, int sm_count, int most) {

@@ -338,27 +338,46 @@ def test_conv_line_shapes(filters, cin, h, w, k, pad, n, b):
         assert errors(Y.cpu().numpy(), ref)[0] <= 1e-5, call
 
 
-@pytest.mark.parametrize("cols", [6144, 6208, 6912, 6976, 8192])
-def test_gemm_long_fp32_sums_hardly_depend_on_the_row_count(cols):
-    """fp32 results of a few rows (whose sums may be split over CTAs) against the same rows among 300 (never split).
-    The accumulator's rounding is worth about 8e-10 a product; the limits on splitting keep the difference below 4.5e-6."""
-    W = inputs.normal_weights(128, cols, 0.02, 910)
+@pytest.mark.parametrize("cols", [6144, 6208, 6912, 6976, 8192, 16384])
+@pytest.mark.parametrize("workspace", [True, False])
+def test_gemm_long_fp32_sums_of_few_rows_are_as_exact_as_whole_ones(cols, workspace):
+    """40 rows, whose sums may be taken in pieces, and the same rows by the kernel that never splits, both against fp64."""
+    W = inputs.normal_weights(128, cols, 0.02, 910).cuda()
     Mb = W.numel() // 4
     desc = B.make_desc(128, cols, 4, Mb // 2, Mb // 4)
     bufs = B.ProjectionBuffers(desc)
-    Wd = W.cuda()
-    bufs.project(Wd)
-    packed = bufs.pack(Wd)
-    X = inputs.normal_activations_bf16((300, cols), 911).cuda()
-    out = []
-    for m in (40, 300):
-        Y = torch.zeros(m, 128, device="cuda")
-        ws = torch.empty(B.mwu_gemm_workspace_bytes(desc, m), dtype=torch.uint8, device="cuda")
-        B.mwu_gemm_ws(desc, packed, X[:m], m, cols, Y, 128, 1, ws, bufs.dev_status)
-        out.append(Y[:40].double())
+    bufs.project(W)
+    packed = bufs.pack(W)
+    Wd = torch.empty(128, cols, dtype=torch.bfloat16, device="cuda")
+    B.mwu_decode(desc, packed, Wd, cols, bufs.dev_status)
+    X = inputs.normal_activations_bf16((40, cols), 911).cuda()
+    Y, Z = torch.zeros(40, 128, device="cuda"), torch.zeros(40, 128, device="cuda")
+    ws = torch.empty(B.mwu_gemm_workspace_bytes(desc, 40), dtype=torch.uint8, device="cuda") if workspace else None
+    B.mwu_gemm_ws(desc, packed, X, 40, cols, Y, 128, 1, ws, bufs.dev_status)
+    B.mwu_gemm_dense(128, cols, Wd, cols, X, 40, cols, Z, 128, 1, bufs.dev_status)
     torch.cuda.synchronize()
     assert int(bufs.dev_status.item()) == 0
-    assert float((out[0] - out[1]).norm() / out[1].norm()) < 4.5e-6
+    ref = X.double() @ Wd.double().t()
+    few, whole = (float((y.double() - ref).norm() / ref.norm()) for y in (Y, Z))
+    # a sum in pieces meets a smaller accumulator at every step; the margin is for sums that were not split at all
+    assert few <= 1.02 * whole and whole <= 2.0 ** -23 * cols / 16
+
+
+
+def test_conv_padding_of_two_to_the_32_pixels():
+    """Paddings may be 32767 wide: 2 x 2 pixels become 65536 x 65536, whose number does not fit 32 bits."""
+    W = inputs.normal_weights(8, 64, 0.05, 797)
+    desc, bufs, packed, p = project_and_pack(W[:1].contiguous(), 4, 8, 4)
+    x = inputs.normal_activations_bf16((1, 64, 2, 2), 798)
+    Y = torch.full((1, 1, 65536, 65536), float("nan"), dtype=torch.bfloat16, device="cuda")
+    B.mwu_conv_implicit(desc, packed, x.cuda(), 1, 64, 2, 2, 1, 1, 1, 32767, Y, 0, bufs.dev_status)
+    torch.cuda.synchronize()
+    assert int(bufs.dev_status.item()) == 0
+    ref = np.einsum("ok,nkhw->nohw", O.decoded_weights(p), x.to(torch.float64).numpy())
+    inner = Y[:, :, 32767:32769, 32767:32769]
+    assert errors(inner.float().cpu().numpy(), ref)[1] <= 1e-2
+    inner.zero_()
+    assert all(int(torch.count_nonzero(Y[0, 0, r:r + 8192])) == 0 for r in range(0, 65536, 8192))
 
 
 @pytest.mark.parametrize("kh,kw,h,w,n", [(1, 1400, 3, 1450, 1),      # the widest kernel row that one fetch holds
