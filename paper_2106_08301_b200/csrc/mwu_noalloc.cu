@@ -14,8 +14,8 @@
 namespace {
 
 // Enough for MWU_STATIC_MAX_BLOCKS 1-dim blocks: 8 bytes per entry of the candidate list (a quarter of
-// the blocks) and the fixed selection state of mwu_project, which is under 1 MiB.  2- and 3-dim block
-// shapes take 16 bytes per block for their keys, which the rest of the array leaves room for.
+// the blocks and 65536 more) and the fixed selection state of mwu_project, which is under 1 MiB.  2- and
+// 3-dim block shapes need the selection state alone.
 constexpr size_t kScratchBytes = (size_t)1536 * 1024 + 4 * ((size_t)MWU_STATIC_MAX_BLOCKS + 8) +
                                  8 * ((size_t)MWU_STATIC_MAX_BLOCKS / 4 + 4096) + 1024;
 

@@ -33,7 +33,7 @@ struct Params {
     long long bpr;                  // blocks per row: cols / b
     unsigned n_stages;              // L.n_stages, for 32-bit record arithmetic (records < 2^31)
     PackedLayout L;
-    unsigned long long gap[5][2];   // byte ranges between the sections (alignment padding), zeroed by scan_kernel
+    unsigned long long gap[5][2];   // byte ranges between the sections (alignment padding), zeroed with the header
 };
 
 // class masks of row r of a record; padding rows are all-pruned
@@ -593,8 +593,8 @@ extern "C" int mwu_pack(const mwu_proj_desc *desc, const float *W, const float *
     p.bpr = desc->cols / desc->block;
     p.n_stages = (unsigned)p.L.n_stages;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // header and the gaps between sections must read as zero: scan_kernel writes all 32 header
-    // words and clears the gaps
+    // header and the gaps between sections must read as zero: scan_kernel, or fill_kernel where it runs
+    // alone, writes all 32 header words and clears the gaps
     const size_t n_rec = (size_t)p.L.n_tiles * p.L.n_stages;
     const size_t gaps[5][2] = {
         {p.L.off_rec + 16 * (n_rec + 1), p.L.off_ulist},

@@ -13,7 +13,8 @@
 //                   rank the keys of <= 262144 evenly spaced blocks; for each selection (prune key, L_u
 //                   of the survivors) the sample quantile is a provisional threshold and the sample
 //                   keys 4 sigma of rank to either side a window.
-//   pass_kernel     streams W (+U) once, evaluates the fp64 keys of every block and writes every
+//   pass_kernel     streams W (+U) once, evaluates fp32 keys of bounded error for every block (fp64 keys for
+//                   those near a window's edge or inside it) and writes every
 //                   output -- Q, u, sign plane, bitmaps -- with the class the provisional
 //                   thresholds give.  A block whose key lies outside the window has its final class
 //                   (as long as the exact threshold lies inside, which the counts prove afterwards);
@@ -197,8 +198,7 @@ __device__ __forceinline__ void load_block(const float *W, const float *U, long 
 }
 
 // Approximate keys of block j in fp32, for the sample only: the sample steers the windows (any
-// window gives the same result), so its keys need no more than a few good digits, and sample_kernel,
-// a single CTA, has one SM's fp64 units.
+// window gives the same result), so its keys need no more than a few good digits.
 template <int B>
 __device__ __forceinline__ void block_keys_sample(const float *W, const float *U, long long j, int use_l1, float *kp,
                                                   float *ku) {
@@ -1974,7 +1974,7 @@ __global__ void __launch_bounds__(256, GS_CTAS) group_stats_kernel(Params p, dou
 }
 
 // One CTA: the kg groups with the smallest (key, index) get their bit in gprune.  Radix selection on
-// the keys' bit patterns (eight passes of eight bits) gives the threshold key and how many groups
+// the keys' bit patterns (eight bits a round, none for those that all keys share) gives the threshold key and how many groups
 // holding exactly that key are taken; those are the ones with the lowest indices.
 __global__ void __launch_bounds__(FIN_THREADS) group_select_kernel(const double *gkey, unsigned n_groups, unsigned kg,
                                                                    unsigned *gprune) {
