@@ -10,23 +10,31 @@
 // that share a tile's stages form a cluster (`split` of them) and add up their partial sums through
 // distributed shared memory, in rank order.  Roles:
 //   decode     groups of two warps, each with a weight tile and a box of X of its own, take the records in
-//              turn.  A record is a chain of short waits (list entries from L2, the tile's last MMA, zeroing,
+//              turn.  A record is a chain of short waits (list entries from L2, the tile's last MMA, clearing,
 //              scattering, the proxy fence, the next MMA), about 2000 cycles however many threads share
-//              it, so 6 to 12 groups an SM work on as many records at a time: two groups of eight warps an SM
-//              took 38 us for the call above.  The lists of a group's next record are brought to L2 one turn
-//              ahead.  The tile is zeroed first, so pruned blocks need neither their list nor a store.
+//              it, so up to ten groups an SM work on as many records at a time.  The lists of a group's next
+//              record are brought to L2 one turn ahead.  The tile is cleared first, so pruned blocks need neither
+//              their list nor a store.
 //   MMA        one warp: tensor memory, the MMAs in record order, a commit per record frees its group.
 // Two CTAs to an SM.
+//
+// What bounds it: 16384 x 4096, b = 16, 16 rows: 19.3 us, about 7 of them before the first record and after the last; the records
+// are then at four fifths of what shared memory passes (144 cycles a record for the operands, 104 to clear and write, lists).
+// Before, the MMA warp's instructions a record, between those of twelve decode groups' warps, were the limit (26.6 us; with a
+// sixth group a CTA 21.8 instead of 19.3, with three groups 20.3).
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises MWU_DEV_TIMEOUT, waits for
 // its copies in flight, frees tensor memory and returns.  Tensor memory is given back before the cluster
 // barrier, so holding it never depends on another CTA.
+#include <cstddef>
+
 #include "mwu_gemm_dev.cuh"
 
 namespace mwu {
 namespace gemm {
 
 constexpr int ST_GROUP = 64;                        // threads of a decode group
-constexpr int ST_MAX_GROUPS = 6;
+constexpr unsigned ST_BATCH = 4;                    // list entries a thread reads before it stores any
+constexpr int ST_MAX_GROUPS = 5;
 constexpr int ST_MAX_THREADS = ST_MAX_GROUPS * ST_GROUP + 32;
 constexpr int ST_MAX_ROWS = 128;                    // activation rows of a CTA
 constexpr int ST_SMEM_CTA = 227 * 512 - 1024;       // two CTAs an SM; each costs 1 KB besides
@@ -41,13 +49,13 @@ struct StreamParams {
 };
 
 struct StreamSmem {
-    unsigned long long x_full[ST_MAX_GROUPS], tile_full[ST_MAX_GROUPS], tile_empty[ST_MAX_GROUPS], tfull;
+    unsigned long long tile_full[ST_MAX_GROUPS], tile_empty[ST_MAX_GROUPS], tfull;
     unsigned tmem_base;
     int abort;
     int drain_abort;
+    int n_live;
 };
 
-__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void tmem_ld16(unsigned taddr, unsigned (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
@@ -62,31 +70,50 @@ __device__ __forceinline__ float4 ld_cluster_f4(unsigned addr) {
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
     return v;
 }
-// barrier over the 64 threads of one decode group; true when `pred` held in any of them
-__device__ __forceinline__ bool group_any(int group, bool pred) {
-    unsigned r;
-    __syncwarp();
-    asm volatile(
-        "{\n\t.reg .pred a, b;\n\t"
-        "setp.ne.u32 a, %1, 0;\n\t"
-        "bar.red.or.pred b, %2, %3, a;\n\t"
-        "selp.u32 %0, 1, 0, b;\n\t}"
-        : "=r"(r) : "r"(pred ? 1u : 0u), "r"(1 + group), "n"(ST_GROUP) : "memory");
-    return r != 0u;
+// a whole warp waits, polling for long; the same answer in all lanes
+__device__ __forceinline__ bool warp_wait_spin(unsigned bar, unsigned parity, volatile int *abort) {
+#pragma unroll 1
+    for (int i = 0; i < 4096; ++i)
+        if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
 }
 
+// barrier over the threads of one decode group
 __device__ __forceinline__ void group_sync(int group) {
     __syncwarp();
     asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(ST_GROUP) : "memory");
 }
 
-// the lines of `bytes` bytes from p on, spread over a decode group
+// the values of a block, WORDS pairs of them: from the packed list, and to its place in a swizzled tile
+template <int WORDS>
+__device__ __forceinline__ void ld_words(const unsigned char *p, unsigned (&v)[WORDS]) {
+    if constexpr (WORDS == 8)
+        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p));
+    else if constexpr (WORDS == 4) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p));
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else if constexpr (WORDS == 2) {
+        const uint2 x = __ldg(reinterpret_cast<const uint2 *>(p));
+        v[0] = x.x; v[1] = x.y;
+    } else v[0] = __ldg(reinterpret_cast<const unsigned *>(p));
+}
+template <int WORDS>
+__device__ __forceinline__ void st_words(unsigned char *tile, unsigned at, const unsigned (&v)[WORDS]) {
+    if constexpr (WORDS >= 4) *reinterpret_cast<uint4 *>(tile + at) = make_uint4(v[0], v[1], v[2], v[3]);
+    if constexpr (WORDS == 8) *reinterpret_cast<uint4 *>(tile + (at ^ 16u)) = make_uint4(v[4], v[5], v[6], v[7]);
+    if constexpr (WORDS == 2) *reinterpret_cast<uint2 *>(tile + at) = make_uint2(v[0], v[1]);
+    if constexpr (WORDS == 1) *reinterpret_cast<unsigned *>(tile + at) = v[0];
+}
+
+// the lines of `bytes` bytes from p on to L2, spread over a decode group
 __device__ __forceinline__ void prefetch_span(const unsigned char *p, unsigned bytes, unsigned t0) {
-    for (unsigned l = t0 * 128u; l < bytes; l += ST_GROUP * 128u) prefetch_l2(p + l);
+#pragma unroll 1
+    for (unsigned l = t0 * 128u; l < bytes; l += ST_GROUP * 128u) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + l) : "memory");
 }
 
 template <int BW>
-__global__ void __launch_bounds__(ST_MAX_THREADS)
+__global__ void __launch_bounds__(ST_MAX_THREADS, 2)
 mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ Params p,
                        const __grid_constant__ StreamParams q) {
     asm volatile("griddepcontrol.wait;" ::: "memory");      // launched while the kernel before may still run
@@ -112,8 +139,7 @@ mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
 
     if (tid == 0) {
         for (int g = 0; g < ST_MAX_GROUPS; ++g) {
-            mbar_init(smem_u32(&sm->x_full[g]), 1);
-            mbar_init(smem_u32(&sm->tile_full[g]), ST_GROUP / 32);
+            mbar_init(smem_u32(&sm->tile_full[g]), ST_GROUP / 32 + 1);      // the warps, and the box of X
             mbar_init(smem_u32(&sm->tile_empty[g]), 1);
         }
         mbar_init(smem_u32(&sm->tfull), 1);
@@ -137,50 +163,67 @@ mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     __syncthreads();
     tc_fence_after();
     const unsigned tmem_base = *reinterpret_cast<volatile unsigned *>(&sm->tmem_base);
-    // a record whose ranges do not lie inside the sections is not touched
-    for (int i = tid; i < n_st; i += n_threads) {
-        const uint4 a = srec[i], b = srec[i + 1];
-        if (a.x > b.x || b.x > p.n_unified || a.y > b.y || b.y > p.n_dense ||
-            (b.x - a.x) + (b.y - a.y) > (unsigned)(kTileRows * BK / BW)) {
-            atomicOr(p.dev_status, (unsigned)MWU_DEV_BOUNDS);
-            srec[i].w = 0u;
+    if (warp == 0) {
+        // The live stages, in order (z and w of entry j: the j-th one's number and live slices).  A record whose ranges do not lie inside the sections is not touched.
+        int n = 0;
+        for (int i0 = 0; i0 < n_st; i0 += 32) {
+            const int i = i0 + lane;
+            bool take = false;
+            unsigned live = 0u;
+            if (i < n_st) {
+                const uint4 a = srec[i], b = srec[i + 1];
+                const bool bad = a.x > b.x || b.x > p.n_unified || a.y > b.y || b.y > p.n_dense ||
+                                 (b.x - a.x) + (b.y - a.y) > (unsigned)(kTileRows * BK / BW);
+                if (bad) atomicOr(p.dev_status, (unsigned)MWU_DEV_BOUNDS);
+                live = a.w & 0xFu;
+                take = !bad && live != 0u;
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, take);       // (and entries i0 to i0 + 31 are read before they are written)
+            if (take) *reinterpret_cast<uint2 *>(&srec[n + __popc(bal & ((1u << lane) - 1u))].z) = make_uint2((unsigned)i, live);
+            n += __popc(bal);
         }
+        if (lane == 0) sm->n_live = n;
     }
     __syncthreads();
-    bool any = false;
-    for (int i = 0; i < n_st; ++i) any = any || (srec[i].w & 0xFu) != 0u;
+    const int n_live = sm->n_live;
 
     if (warp == mma_warp) {
         // ---------------- MMA issuer ----------------
+        // Every record of the CTA passes through this warp in turn, between decode warps that compete for its issue slots, so
+        // what counts is its instructions a record.
         const unsigned idesc = make_idesc(q.mpad);
-        unsigned n = 0, g = 0, phase = 0;
-        bool ok = true;
-        for (int i = 0; i < n_st; ++i) {
-            const unsigned live = srec[i].w & 0xFu;
-            if (!live) continue;
-            if (!mbar_wait_spin(smem_u32(&sm->tile_full[g]), phase, abort) ||
-                !mbar_wait_spin(smem_u32(&sm->x_full[g]), phase, abort)) ok = false;
-            if (!__all_sync(0xffffffffu, ok)) break;
+        const unsigned long long adesc0 = make_desc(smem_u32(tiles)), bdesc0 = make_desc(smem_u32(xbuf));
+        const unsigned a_step = REC_BYTES / 16, b_step = x_bytes / 16, bar0 = smem_u32(&sm->tile_full[0]);
+        constexpr unsigned EMPTY = (unsigned)(offsetof(StreamSmem, tile_empty) - offsetof(StreamSmem, tile_full));
+        unsigned g = 0, phase = 0, live = n_live ? srec[0].w : 0u;
+#pragma unroll 1
+        for (int j = 0; j < n_live; ++j) {
+            const unsigned bar = bar0 + g * 8u, next = j + 1 < n_live ? srec[j + 1].w : 0u;
+            if (!warp_wait_spin(bar, phase, abort)) break;
             tc_fence_after();
-            const unsigned long long adesc = make_desc(smem_u32(tiles + g * REC_BYTES));
-            const unsigned long long bdesc = make_desc(smem_u32(xbuf + g * x_bytes));
+            const unsigned long long adesc = adesc0 + g * a_step, bdesc = bdesc0 + g * b_step;
             if (elect_one()) {
-                bool first = n == 0;
+                unsigned acc = j != 0 ? 1u : 0u;
+                if (live == 0xFu) {
 #pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4) {
-                    if ((live >> k4) & 1u) {
-                        umma_bf16(tmem_base, adesc + (unsigned long long)(k4 * 2), bdesc + (unsigned long long)(k4 * 2), idesc,
-                                  first ? 0u : 1u);
-                        first = false;
+                    for (int k4 = 0; k4 < 4; ++k4)
+                        umma_bf16(tmem_base, adesc + (unsigned long long)(k4 * 2), bdesc + (unsigned long long)(k4 * 2), idesc, k4 ? 1u : acc);
+                } else {
+#pragma unroll
+                    for (int k4 = 0; k4 < 4; ++k4) {
+                        if ((live >> k4) & 1u) {
+                            umma_bf16(tmem_base, adesc + (unsigned long long)(k4 * 2), bdesc + (unsigned long long)(k4 * 2), idesc, acc);
+                            acc = 1u;
+                        }
                     }
                 }
-                umma_commit(smem_u32(&sm->tile_empty[g]));
+                umma_commit(bar + EMPTY);
             }
             __syncwarp();
-            ++n;
+            live = next;
             if (++g == (unsigned)q.groups) { g = 0; phase ^= 1u; }
         }
-        if (n) {
+        if (n_live) {
             if (elect_one()) umma_commit(smem_u32(&sm->tfull));
             __syncwarp();
             // nothing this warp issued may be running when tensor memory is freed
@@ -191,112 +234,135 @@ mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
         // ---------------- decode: this group takes every q.groups-th live record ----------------
         constexpr unsigned OFF_MASK = DecodeCfg<BW, ST_GROUP>::OFF_MASK;
         constexpr int WORDS = BW / 2;
-        constexpr unsigned BATCH = 4;                       // entries a thread reads before it stores any
-        constexpr unsigned PIECES = BW == 16 ? 2 : 1;       // 16-byte pieces of a dense block (or the block, if smaller)
-        constexpr unsigned PIECE_BYTES = BW >= 8 ? 16 : 2 * BW;
+        constexpr unsigned BATCH = ST_BATCH;
+        // Dense blocks: a lane to a block, whose halves then reach different banks in both stores (two lanes to a block of 16 met
+        // in one bank every other time).
+        constexpr unsigned DBATCH = BW == 16 ? BATCH / 2 : BATCH;
+        // Blocks of 16: the tile is cleared where the group's last record wrote, as long as a batch held all of it (clearing
+        // the whole tile takes 128 cycles of the SM's shared memory: 16384 x 4096, 16 rows 20.8 us, so 19.3; blocks of 8 gain nothing).
+        constexpr bool UNDO = BW == 16;
         const int group = warp / (ST_GROUP / 32);
         const unsigned t0 = (unsigned)tid & (ST_GROUP - 1u);
         unsigned char *tile = tiles + group * REC_BYTES;
-        const unsigned char *ulist = p.packed + p.off_ulist, *dposl = p.packed + p.off_dpos, *dpayl = p.packed + p.off_dpay;
-        int turn = group;                                   // live records until this group's next one
-        unsigned mine = 0;
-        bool ok = true;
-        for (int i = 0; i < n_st; ++i) {
-            const uint4 a = srec[i];
-            if (!(a.w & 0xFu)) continue;
-            if (turn == 0) {
-                turn = q.groups;
-                const uint4 b = srec[i + 1];
-                const unsigned n_u = b.x - a.x, n_p = (b.y - a.y) * PIECES;
-                const uint2 *ul = reinterpret_cast<const uint2 *>(ulist) + a.x;
-                const unsigned short *dpos = reinterpret_cast<const unsigned short *>(dposl) + a.y;
-                const unsigned char *pay = dpayl + (unsigned long long)a.y * (2 * BW);
-                // the first entries travel while the tile is waited for and zeroed
-                uint2 ent[BATCH];                           // x: spread signs, y: off | bf16(u) << 16
-                unsigned off[BATCH];
-                uint4 v[BATCH];
-                auto read_u = [&](unsigned e0) {
+        const uint2 *ulist = reinterpret_cast<const uint2 *>(p.packed + p.off_ulist) + t0;
+        const unsigned short *dposl = reinterpret_cast<const unsigned short *>(p.packed + p.off_dpos) + t0;
+        const unsigned char *dpayl = p.packed + p.off_dpay + t0 * (2u * BW);
+        unsigned mine = 0, old_u = 0, old_d = 0;            // entries of the group's last record
+        bool ok = true, cleared = false;                    // nothing but those entries is in the tile
+        unsigned at_u[BATCH], at_d[DBATCH];                 // where this thread wrote them
 #pragma unroll
-                    for (unsigned k = 0; k < BATCH; ++k)
-                        if (e0 + k * ST_GROUP < n_u) ent[k] = __ldg(ul + e0 + k * ST_GROUP);
-                };
-                auto read_d = [&](unsigned e0) {
+        for (unsigned k = 0; k < BATCH; ++k) at_u[k] = at_d[k % DBATCH] = 0u;
+        // A thread that ran out of time goes through the rest of the loop without touching anything, so that the group's
+        // barriers stay matched.
+#pragma unroll 1
+        for (int j = group; j < n_live; j += q.groups) {
+            const unsigned i = srec[j].z;
+            const uint2 a = *reinterpret_cast<const uint2 *>(&srec[i]), b = *reinterpret_cast<const uint2 *>(&srec[i + 1]);
+            const unsigned n_u = b.x - a.x, n_d = b.y - a.y;
+            const uint2 *ul = ulist + a.x;
+            const unsigned short *dpos = dposl + a.y;
+            const unsigned char *pay = dpayl + (unsigned long long)a.y * (2 * BW);
+            // the first entries travel while the tile is waited for and zeroed
+            uint2 ent[BATCH];                               // x: spread signs, y: off | bf16(u) << 16
+            unsigned off[DBATCH];
+            unsigned v[DBATCH][WORDS];
+            auto read_u = [&](unsigned e0) {                // entries e0 + t0, and every ST_GROUP-th from there
 #pragma unroll
-                    for (unsigned k = 0; k < BATCH; ++k) {
-                        const unsigned e = e0 + k * ST_GROUP;
-                        if (e >= n_p) continue;
-                        off[k] = (__ldg(dpos + e / PIECES) & OFF_MASK) ^ (PIECES == 2 ? (e & 1u) << 4 : 0u);
-                        if (BW >= 8) v[k] = __ldg(reinterpret_cast<const uint4 *>(pay + (size_t)e * PIECE_BYTES));
-                        if (BW == 4) { const uint2 h = __ldg(reinterpret_cast<const uint2 *>(pay + (size_t)e * PIECE_BYTES)); v[k].x = h.x; v[k].y = h.y; }
-                        if (BW == 2) v[k].x = __ldg(reinterpret_cast<const unsigned *>(pay + (size_t)e * PIECE_BYTES));
-                    }
-                };
-                auto write_u = [&](unsigned e0) {
+                for (unsigned k = 0; k < BATCH; ++k)
+                    if (e0 + t0 + k * ST_GROUP < n_u) ent[k] = __ldg(ul + e0 + k * ST_GROUP);
+            };
+            auto read_d = [&](unsigned e0) {
 #pragma unroll
-                    for (unsigned k = 0; k < BATCH; ++k) {
-                        if (e0 + k * ST_GROUP >= n_u) break;
-                        const unsigned at = ent[k].y & OFF_MASK, u2 = __byte_perm(ent[k].y, 0u, 0x3232);
-                        unsigned w[8];
-#pragma unroll
-                        for (int t = 0; t < 8; ++t)         // weights 2t, 2t+1: sign bits t and 16+t
-                            w[t] = (t < WORDS) ? (((ent[k].x << (15 - t)) & 0x80008000u) ^ u2) : 0u;
-                        if (BW >= 8) *reinterpret_cast<uint4 *>(tile + at) = make_uint4(w[0], w[1], w[2], w[3]);
-                        if (BW == 16) *reinterpret_cast<uint4 *>(tile + (at ^ 16u)) = make_uint4(w[4], w[5], w[6], w[7]);
-                        if (BW == 4) *reinterpret_cast<uint2 *>(tile + at) = make_uint2(w[0], w[1]);
-                        if (BW == 2) *reinterpret_cast<unsigned *>(tile + at) = w[0];
-                    }
-                };
-                auto write_d = [&](unsigned e0) {
-#pragma unroll
-                    for (unsigned k = 0; k < BATCH; ++k) {
-                        if (e0 + k * ST_GROUP >= n_p) break;
-                        if (BW >= 8) *reinterpret_cast<uint4 *>(tile + off[k]) = v[k];
-                        if (BW == 4) *reinterpret_cast<uint2 *>(tile + off[k]) = make_uint2(v[k].x, v[k].y);
-                        if (BW == 2) *reinterpret_cast<unsigned *>(tile + off[k]) = v[k].x;
-                    }
-                };
-                read_u(t0);
-                read_d(t0);
-                // lists of this group's next record (its stage if none between is dead)
-                if (i + q.groups < n_st) {
-                    const uint4 na = srec[i + q.groups], nb = srec[i + q.groups + 1];
-                    if (na.w & 0xFu) {
-                        prefetch_span(ulist + (size_t)na.x * 8u, (nb.x - na.x) * 8u, t0);
-                        prefetch_span(dpayl + (size_t)na.y * (2u * BW), (nb.y - na.y) * (2u * BW), t0);
-                        prefetch_span(dposl + (size_t)na.y * 2u, (nb.y - na.y) * 2u, t0);
-                    }
+                for (unsigned k = 0; k < DBATCH; ++k) {
+                    if (e0 + t0 + k * ST_GROUP >= n_d) continue;
+                    off[k] = __ldg(dpos + e0 + k * ST_GROUP);
+                    ld_words<WORDS>(pay + (e0 + k * ST_GROUP) * (2u * BW), v[k]);
                 }
-                // tile and box are free once the group's last record is multiplied
-                if (mine && !mbar_wait(smem_u32(&sm->tile_empty[group]), (mine - 1u) & 1u, abort)) ok = false;
-                if (group_any(group, !ok)) { ok = false; break; }          // the same decision in every thread of the group
+            };
+            auto write_u = [&](unsigned e0) {
+#pragma unroll
+                for (unsigned k = 0; k < BATCH; ++k) {
+                    if (e0 + t0 + k * ST_GROUP >= n_u) break;
+                    const unsigned at = ent[k].y & OFF_MASK, u2 = __byte_perm(ent[k].y, 0u, 0x3232);
+                    unsigned w[WORDS];
+#pragma unroll
+                    for (int t = 0; t < WORDS; ++t)         // weights 2t, 2t+1: sign bits t and 16+t
+                        w[t] = ((ent[k].x << (15 - t)) & 0x80008000u) ^ u2;
+                    st_words<WORDS>(tile, at, w);
+                    if (UNDO) at_u[k] = at;
+                }
+            };
+            auto write_d = [&](unsigned e0) {
+#pragma unroll
+                for (unsigned k = 0; k < DBATCH; ++k) {
+                    if (e0 + t0 + k * ST_GROUP >= n_d) break;
+                    const unsigned at = off[k] & OFF_MASK;
+                    st_words<WORDS>(tile, at, v[k]);
+                    if (UNDO) at_d[k] = at;
+                }
+            };
+            read_u(0u);
+            read_d(0u);
+            // lists of the group's next record
+            if (j + q.groups < n_live) {
+                const unsigned ni = srec[j + q.groups].z;
+                const uint2 na = *reinterpret_cast<const uint2 *>(&srec[ni]), nb = *reinterpret_cast<const uint2 *>(&srec[ni + 1]);
+                prefetch_span(p.packed + p.off_ulist + (size_t)na.x * 8u, (nb.x - na.x) * 8u, t0);
+                prefetch_span(p.packed + p.off_dpay + (size_t)na.y * (2u * BW), (nb.y - na.y) * (2u * BW), t0);
+                prefetch_span(p.packed + p.off_dpos + (size_t)na.y * 2u, (nb.y - na.y) * 2u, t0);
+            }
+            // tile and box are free once the group's last record is multiplied
+            if (ok && mine && !mbar_wait(smem_u32(&sm->tile_empty[group]), (mine - 1u) & 1u, abort)) ok = false;
+            __syncwarp();
+            if (ok) {
                 if (t0 == 0) {
-                    mbar_expect_tx(smem_u32(&sm->x_full[group]), x_bytes);
-                    tma_load_2d(smem_u32(xbuf + group * x_bytes), &tmap_x, smem_u32(&sm->x_full[group]), (k0 + i) * BK, (int)mt * q.mpad);
+                    mbar_expect_tx(smem_u32(&sm->tile_full[group]), x_bytes);
+                    tma_load_2d(smem_u32(xbuf + group * x_bytes), &tmap_x, smem_u32(&sm->tile_full[group]), (k0 + (int)i) * BK, (int)mt * q.mpad);
                 }
-                uint4 *z = reinterpret_cast<uint4 *>(tile) + t0;
+                if (UNDO && cleared) {
+                    const unsigned zero[WORDS] = {};
 #pragma unroll
-                for (int t = 0; t < REC_BYTES / 16 / ST_GROUP; ++t) z[t * ST_GROUP] = make_uint4(0, 0, 0, 0);
-                group_sync(group);
-                write_u(t0);
-                write_d(t0);
-                for (unsigned e0 = t0 + BATCH * ST_GROUP; e0 < n_u; e0 += BATCH * ST_GROUP) { read_u(e0); write_u(e0); }
-                for (unsigned e0 = t0 + BATCH * ST_GROUP; e0 < n_p; e0 += BATCH * ST_GROUP) { read_d(e0); write_d(e0); }
+                    for (unsigned k = 0; k < BATCH; ++k) {
+                        if (t0 + k * ST_GROUP >= old_u) break;
+                        st_words<WORDS>(tile, at_u[k], zero);
+                    }
+#pragma unroll
+                    for (unsigned k = 0; k < DBATCH; ++k) {
+                        if (t0 + k * ST_GROUP >= old_d) break;
+                        st_words<WORDS>(tile, at_d[k], zero);
+                    }
+                } else {
+                    uint4 *z = reinterpret_cast<uint4 *>(tile) + t0;
+#pragma unroll
+                    for (int t = 0; t < REC_BYTES / 16 / ST_GROUP; ++t) z[t * ST_GROUP] = make_uint4(0, 0, 0, 0);
+                }
+            }
+            group_sync(group);
+            if (ok) {
+                write_u(0u);
+                write_d(0u);
+                for (unsigned e0 = BATCH * ST_GROUP; e0 < n_u; e0 += BATCH * ST_GROUP) { read_u(e0); write_u(e0); }
+                for (unsigned e0 = DBATCH * ST_GROUP; e0 < n_d; e0 += DBATCH * ST_GROUP) { read_d(e0); write_d(e0); }
+                if (UNDO) {
+                    old_u = n_u;
+                    old_d = n_d;
+                    cleared = n_u <= BATCH * ST_GROUP && n_d <= DBATCH * ST_GROUP;
+                }
                 fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&sm->tile_full[group]));
                 ++mine;
             }
-            --turn;
+            __syncwarp();
+            if (ok && lane == 0) mbar_arrive(smem_u32(&sm->tile_full[group]));
         }
         // a box of X that is still on its way must land before this CTA's shared memory goes away
-        if (t0 == 0 && mine) mbar_wait(smem_u32(&sm->x_full[group]), (mine - 1u) & 1u, &sm->drain_abort);
+        if (t0 == 0 && mine) mbar_wait(smem_u32(&sm->tile_full[group]), (mine - 1u) & 1u, &sm->drain_abort);
         __syncwarp();
-        if (any && ok) mbar_wait(smem_u32(&sm->tfull), 0, abort);
+        if (n_live && ok) mbar_wait(smem_u32(&sm->tfull), 0, abort);
         __syncwarp();
     }
     __syncthreads();
     // ---------------- epilogue: partial sums to shared memory, tensor memory given back ----------------
-    const bool sums = any && *abort == 0;
+    const bool sums = n_live && *abort == 0;
     const int readers = mma_warp >= 8 ? 2 : 1;              // warps to a quarter of the lanes
     if (warp < 4 * readers) {
         tc_fence_after();
@@ -377,7 +443,7 @@ static StreamPlan plan_with(const Params &p, int split, int sm_count) {
     s.q.split = split;
     s.q.stages_per = (int)((p.n_stages + split - 1) / split);
     s.q.tmem_cols = s.q.mpad <= 32 ? 32u : (s.q.mpad <= 64 ? 64u : 128u);
-    // as many groups as tiles and boxes of X fit: six up to 16 rows, three at 128
+    // as many groups as tiles and boxes of X fit: five up to 32 rows, three at 128
     const size_t x = (size_t)s.q.mpad * BK * 2;
     const size_t fixed = 1024 + sizeof(StreamSmem) + 16 + (size_t)(s.q.stages_per + 1) * 16;
     size_t groups = ((size_t)ST_SMEM_CTA - fixed) / (REC_BYTES + x);
@@ -424,9 +490,13 @@ int stream_box_rows(const Params &p, int sm_count) { return plan_of(p, sm_count,
 
 // A record is decoded once per activation tile of 128 rows, so the path that expands the weights once
 // overtakes this one as rows are added.  Measured (us, this kernel / expanding): 16384 x 4096, b = 16:
-// 27 / 66 at 16 rows, 41 / 68 at 128, 67 / 68 at 256, 131 / 89 at 512; 4096 x 4096, b = 8: 26 / 37 at 256, 41 / 37 at
-// 512; b = 2: 43 / 50 at 256, 72 / 52 at 512.  A small weight stays here longer, while the decodes are few to an
+// 19 / 66 at 16 rows, 29 / 68 at 128, 45 / 68 at 256, 85 / 87 at 512; 4096 x 4096, b = 8: 22 / 37 at 256, 35 / 35 at
+// 512; b = 2: 35 / 50 at 256, 58 / 56 at 512.  A small weight stays here longer, while the decodes are few to an
 // SM: 1000 x 1216, b = 8, 1024 rows (1216 decodes): 15 / 19; 4096 x 1024, b = 4, 512 rows (2048): 22 / 19.
+// So do up to 640 rows of a long reduction where the other path's tiles are few, which work through it alone (bf16, 512 rows:
+// 2048 x 8192, b = 16, 16 tiles: 28 / 53; b = 8: 37 / 53; 1024 x 4096, b = 16: 17 / 30; 2048 x 2048, b = 2: 22.5 / 24.8, but
+// 2048 x 4096, b = 2, 4096 decodes: 41 / 40; 4096 x 2048, b = 4, 32 tiles: 27.4 / 24.7).  Without a workspace the other path decodes
+// once per 512 rows (4096 x 4096, b = 4: 43 / 87, b = 2: 58 / 179; 8192 x 8192, b = 4, 32 tiles: 148 / 281; 16384 x 4096, b = 16, 64 tiles: 85 / 74).
 // bf16 results of more than 256 rows stay only while the tiles of 128 x 128 outputs are one to an SM, or two where the other path has
 // much to expand for its rows, or nothing expanded to work on (us, this kernel / the other: 1024 x 64, b = 4, 8192 rows, 512 tiles: 19.5 / 12.1;
 // 256 x 256, 16384 rows, 256 tiles: 14.2 / 11.1; 128 x 192, b = 16, 32768 rows, 256 tiles: 11.5 / 12.7; 4096 x 256, 777 rows, 224 tiles: 11.5 / 12.0;
@@ -440,6 +510,11 @@ bool stream_eligible(const Params &p, int sm_count, bool can_expand) {
     if (can_expand && most_pieces(p) < 8 && 2 * s.cost > 3 * plan_of(p, sm_count, 8).cost) return false;
     if (p.M <= 256) return true;
     const long long tiles = p.n_rec_tiles * s.q.m_tiles;
+    if (!p.y_fp32 && p.M <= 640 && p.n_stages >= 32) {
+        const long long wide = (p.n_rec_tiles + 1) / 2, pairs = sm_count / 2;          // tiles of a CTA pair along the weight rows
+        if (can_expand ? 4 * wide * ((p.M + 255) / 256) <= pairs && (p.bw > 2 || tiles * p.n_stages <= 2048)
+                       : 2 * wide * ((p.M + 511) / 512) <= pairs) return true;
+    }
     if (tiles * p.n_stages > 9ll * sm_count) return false;
     if (p.y_fp32) return true;
     if (can_expand && p.n_stages < 16 && s.q.split > 1 && s.grid > sm_count && p.M > 512) return false;

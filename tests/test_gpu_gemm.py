@@ -294,6 +294,19 @@ def test_gemm_few_rows(b, rows, cols, M, ku, kp):
     check_gemm(W, b, Mb * ku // 10, Mb * kp // 10, M, seed=40 + b)
 
 
+@pytest.mark.parametrize("b,M,pr,un", [(16, 20, 4, 7), (16, 3, 1, 2), (16, 100, 6, 9), (8, 20, 4, 7), (4, 5, 3, 6), (2, 17, 3, 6)])
+def test_gemm_few_rows_uneven_records(b, M, pr, un):
+    """A run of more than 32 stages whose records differ: dead ones, nearly empty ones, all-dense and all-unified ones that
+    need several batches, so that every way of clearing a tile follows every other (pr, un in tenths)."""
+    rows, cols = 296, 64 * 70
+    gen = torch.Generator().manual_seed(b * 100 + M)
+    W = torch.randn(rows, cols, generator=gen) * 0.02
+    scale = torch.tensor([0.0001, 1.0, 30.0, 0.01])[torch.randint(0, 4, (cols // 64,), generator=gen)]
+    W = W * scale.repeat_interleave(64)[None, :]
+    Mb = W.numel() // b
+    check_gemm(W, b, Mb * un // 10, Mb * pr // 10, M)
+
+
 @pytest.mark.parametrize("filters,cin,h,w,k,stride,pad,n,b", [(128, 64, 13, 11, 3, 2, 1, 2, 4),    # four planes, odd sizes
                                                               (136, 128, 9, 9, 3, 1, 1, 1, 8),     # two chunks over a cluster, ragged filters
                                                               (256, 64, 30, 29, 3, 1, 1, 24, 16),  # several tiles to a CTA, two filter tiles
