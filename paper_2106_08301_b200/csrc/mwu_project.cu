@@ -1647,8 +1647,8 @@ __device__ bool rank_candidates(const Params &p, const u64 *g_key, const unsigne
 //   3  every CTA gives the blocks of its list slice their final class: the class pass_kernel wrote
 //      travels in the entry, so nothing is read for the nine in ten whose class stands; the others
 //      are gathered 32 to a warp and rewritten.  Blocks of the unify threshold bin become candidates.
-//      -- grid barrier --
-//   4  one CTA ranks those, which fixes the threshold element and their classes.
+//   4  the CTA that is through with that last ranks those, which fixes the threshold element and their classes; the
+//      others do not wait for it.
 //   5  if any step gave the one-pass result up (a threshold outside its window, a threshold bin or
 //      tie group too large to rank, a full list), the exact phases redo the projection here.
 template <int B>
@@ -1684,8 +1684,10 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
     const u64 ulo = w.sel[1].lo0, uhi = w.sel[1].hi0;
     const unsigned ush = w.sel[1].shift0;
     const unsigned n_list = min(w.list_count, p.list_cap);
-    // every condition up to the second barrier is the same in all CTAs: they all take the same path
-    bool alive = w.failed == 0u && !(mode_p != 0u && mode_u != 0u);
+    // Every condition that gives the one-pass result up comes from the same words in all CTAs, none of which changes while it may
+    // still be read: they all take the same path.
+    bool alive = w.failed == 0u;
+    if (alive && mode_p != 0u && mode_u != 0u) return;         // no threshold: every class is final
     if (threadIdx.x == 0) { s_sel.B = 0; s_sel.r = 0; s_sel.cnt = 0; s_sel.lo_hi = s_sel.lo_lo = s_sel.hi_hi = s_sel.hi_lo = 0; s_n_extra = 0; }
     __syncthreads();
 
@@ -1696,10 +1698,7 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
         const unsigned Bp = s_sel.B;
         const u64 r_p = s_sel.r;
         // the threshold bin must be a real bin of the window and small enough to rank
-        if (!(Bp >= 1u && Bp <= nb - 2u && s_sel.cnt <= (u64)CAP)) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) one_pass_fail(p);
-            alive = false;
-        }
+        if (!(Bp >= 1u && Bp <= nb - 2u && s_sel.cnt <= (u64)CAP)) alive = false;
         if (alive) {
             unsigned under = 0;
             const u128 lo0 = from_halves(s_sel.lo_hi, s_sel.lo_lo);
@@ -1751,10 +1750,8 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
         if (alive) {
             // ---------------- 2: exact prune threshold, corrections, unify threshold bin ----------------
             const unsigned m = ld_vol(&p.work->fcand_count[0]);
-            if (m > (unsigned)CAP || r_p < 1 || r_p > (u64)m) {
-                if (blockIdx.x == 0 && threadIdx.x == 0) one_pass_fail(p);
-                alive = false;
-            } else {
+            if (m > (unsigned)CAP || r_p < 1 || r_p > (u64)m) alive = false;
+            else {
                 const bool have_aux = rank_candidates(p, p.cand_key, p.cand_idx, p.cand_aux, m, c_key, c_idx, c_aux);
                 vp.B = Bp;
                 vp.T_key = c_key[r_p - 1];
@@ -1780,10 +1777,7 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
         r_u = s_sel.r;
         lo = from_halves(s_sel.lo_hi, s_sel.lo_lo);
         hi = from_halves(s_sel.hi_hi, s_sel.hi_lo);
-        if (!(Bu >= 1u && Bu <= nb - 2u && s_sel.cnt <= (u64)CAP)) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) one_pass_fail(p);
-            alive = false;
-        }
+        if (!(Bu >= 1u && Bu <= nb - 2u && s_sel.cnt <= (u64)CAP)) alive = false;
     }
     if (alive) {
         // ---------------- 3: final classes of the listed blocks ----------------
@@ -1850,35 +1844,40 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
         }
         if (p.resid) block_add_double(resid_delta, p.resid);
     }
-    if (!grid_sync(&p.work->bar, ++k)) {
-        if (threadIdx.x == 0) atomicOr(p.dev_status, (unsigned)MWU_DEV_TIMEOUT);
+    if (alive) {
+        // ---------------- 4: the blocks of the unify threshold bin, by the CTA that gets here last ----------------
+        if (mode_u != 0u) return;
+        __shared__ unsigned s_last;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_last = atomicAdd(&p.work->bar, 1u) == (k + 1u) * gridDim.x - 1u ? 1u : 0u;
+            __threadfence();
+        }
+        __syncthreads();
+        if (!s_last) return;
+        const unsigned m = ld_vol(&p.work->fcand_count[1]);
+        if (m > (unsigned)CAP || r_u < 1 || r_u > (u64)m) {      // (never: they are the blocks that the bin's count had, at most CAP)
+            if (threadIdx.x == 0) atomicOr(p.dev_status, (unsigned)MWU_DEV_SELECT);
+            return;
+        }
+        const bool have_aux = rank_candidates(p, p.cand_key + CAP, p.cand_idx + CAP, p.cand_aux + CAP, m, c_key, c_idx, c_aux);
+        if (threadIdx.x == 0) { su->T_key = c_key[r_u - 1]; su->T_idx = (u64)c_idx[r_u - 1]; }
+        const unsigned r = (unsigned)r_u;
+        double tail_delta = 0.0;
+        for (unsigned i = threadIdx.x; i < m; i += blockDim.x) {
+            // the class pass_kernel wrote for this block: carried with the candidate, else read back
+            const unsigned idx = c_idx[i], bit = 1u << (idx & 31u);
+            const bool pr0 = have_aux ? ((c_aux[i] >> 1) & 1u) != 0u : (ld_vol(pruned_bitmap + (idx >> 5)) & bit) != 0u;
+            const bool un0 = have_aux ? (c_aux[i] & 1u) != 0u : (ld_vol(unified_bitmap + (idx >> 5)) & bit) != 0u;
+            const bool un = i < r;
+            if (pr0 || un != un0)
+                tail_delta += apply_class<B>(p, Q, u_out, pruned_bitmap, unified_bitmap, idx, false, un, pr0, un0);
+        }
+        if (p.resid) block_add_double(tail_delta, p.resid);
         return;
     }
-    // ---------------- 4: the blocks of the unify threshold bin ----------------
-    const unsigned m = ld_vol(&p.work->fcand_count[1]);
-    bool failed = ld_vol(&p.work->failed) != 0u;          // both settled: the same in all CTAs
-    if (alive && !failed && mode_u == 0u) {
-        if (m > (unsigned)CAP || r_u < 1 || r_u > (u64)m) failed = true;
-        else if (blockIdx.x == 0) {
-            const bool have_aux = rank_candidates(p, p.cand_key + CAP, p.cand_idx + CAP, p.cand_aux + CAP, m, c_key,
-                                                  c_idx, c_aux);
-            if (threadIdx.x == 0) { su->T_key = c_key[r_u - 1]; su->T_idx = (u64)c_idx[r_u - 1]; }
-            const unsigned r = (unsigned)r_u;
-            double tail_delta = 0.0;
-            for (unsigned i = threadIdx.x; i < m; i += blockDim.x) {
-                // the class pass_kernel wrote for this block: carried with the candidate, else read back
-                const unsigned idx = c_idx[i], bit = 1u << (idx & 31u);
-                const bool pr0 = have_aux ? ((c_aux[i] >> 1) & 1u) != 0u : (ld_vol(pruned_bitmap + (idx >> 5)) & bit) != 0u;
-                const bool un0 = have_aux ? (c_aux[i] & 1u) != 0u : (ld_vol(unified_bitmap + (idx >> 5)) & bit) != 0u;
-                const bool un = i < r;
-                if (pr0 || un != un0)
-                    tail_delta += apply_class<B>(p, Q, u_out, pruned_bitmap, unified_bitmap, idx, false, un, pr0, un0);
-            }
-            if (p.resid) block_add_double(tail_delta, p.resid);
-        }
-    }
-    // ---------------- 5: the fallback, if the one-pass result was given up anywhere ----------------
-    if (!failed) return;
+    // ---------------- 5: the fallback, once the one-pass result was given up ----------------
     ExactSmem<FIN_THREADS> &sm = *reinterpret_cast<ExactSmem<FIN_THREADS> *>(mp_smem);
     sel::GridTeam<true> team = {blockIdx.x, gridDim.x, p.xwork, &sm.sel, 0u, reinterpret_cast<unsigned *>(mp_smem + sizeof(sm))};
     const Outs o = {Q, loss_u, loss_p, u_out, pruned_bitmap, unified_bitmap, sign_bits};
