@@ -8,6 +8,20 @@ namespace mwu {
 static std::atomic<unsigned long long> g_launches{0};
 void count_launch(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
 
+// One 16-byte word a thread.  (Before a cooperative launch: a memset starts 2 us after the kernel before it has ended, this
+// kernel is in place by then.  mwu_project of 1000 x 1216, b = 8: 29.0 us, so 27.2; 2x2x2 blocks of 128 x 1152: 25.5, so 22.9.)
+__global__ void __launch_bounds__(256) clear_kernel(uint4 *p, unsigned n) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const unsigned i = blockIdx.x * 256u + threadIdx.x;
+    if (i < n) p[i] = make_uint4(0, 0, 0, 0);
+}
+
+cudaError_t launch_clear(void *p, size_t bytes, cudaStream_t st) {
+    const unsigned n = (unsigned)(bytes / 16);
+    count_launch();
+    return launch_chained(clear_kernel, dim3((n + 255) / 256), dim3(256), 0, st, 1, (uint4 *)p, n);
+}
+
 int check_device(int *sm_count) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return MWU_ERR_CUDA;

@@ -173,6 +173,9 @@ inline bool cluster_runs() {
     return k > 0;
 }
 
+// clears `bytes` (a multiple of 16) of 16-byte aligned memory, as a kernel launched by launch_chained
+cudaError_t launch_clear(void *p, size_t bytes, cudaStream_t st);
+
 // adds n to the process-wide count of kernels launched (mwu_kernel_launches)
 void count_launch(int n = 1);
 

@@ -2220,7 +2220,7 @@ static cudaError_t launch_project(const mwu::proj::Params &p, const mwu_proj_des
     const long long n_units = (p.n_floats + 15) / 16;
     if (!route.one_pass) {
         // the grid form's barrier counter and counts start at zero; a cluster clears them itself
-        if (!route.cluster && cudaMemsetAsync(p.xwork, 0, mwu::sel::XWORK_ZERO_BYTES, st) != cudaSuccess) return cudaErrorUnknown;
+        if (!route.cluster && mwu::launch_clear(p.xwork, mwu::sel::XWORK_ZERO_BYTES, st) != cudaSuccess) return cudaErrorUnknown;
         if (route.held) return launch_exact_held<B>(p, o, route, sm_count, st);
         const long long want = (n_units + WALK_THREADS - 1) / WALK_THREADS;
         e = cudaFuncSetAttribute(exact_walk_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, WALK_SMEM);

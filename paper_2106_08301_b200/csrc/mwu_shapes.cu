@@ -281,7 +281,7 @@ static cudaError_t launch(const SParams &p, const mwu_proj_desc *desc, int sm_co
         count_launch();
         return launch_chained(shape_kernel<N, CLUSTER>, dim3(sel::CLUSTER_CTAS), dim3(SH_THREADS), smem, st, sel::CLUSTER_CTAS, p, pb, per);
     }
-    if (cudaMemsetAsync(p.xwork, 0, sel::XWORK_ZERO_BYTES, st) != cudaSuccess) return cudaErrorUnknown;
+    if (launch_clear(p.xwork, sel::XWORK_ZERO_BYTES, st) != cudaSuccess) return cudaErrorUnknown;
     const int grid = (int)(ctas < sm_count ? ctas : sm_count);
     unsigned per = (unsigned)((ctas + grid - 1) / grid);
     const bool held = (long long)per * SH_THREADS <= SH_SLOTS;
