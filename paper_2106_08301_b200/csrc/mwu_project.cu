@@ -46,7 +46,6 @@ static_assert(SAMP_ROUND == 1 << NSAMP_LG, "the middle sample fills the cluster"
 constexpr int STAGE_ENTRIES = 64;  // per-warp staging of candidate-list entries in pass_kernel
 constexpr int FIN_THREADS = 1024;   // block size of the kernels that scan the histograms
 constexpr int PASS_GROUPS = 8;      // groups of CTAs of pass_kernel that share out its last steps
-static_assert(NB_MAX / FIN_THREADS <= 64, "scan_hist searches one thread's bins with one warp, two per lane");
 
 typedef unsigned long long u64;
 typedef unsigned __int128 u128;
@@ -612,140 +611,73 @@ __global__ void __launch_bounds__(SAMP_THREADS) sample_kernel(Params p) {
 // ---------------------------------------------------------------------------------------------
 // finalisation helpers, run by whole CTAs of FIN_THREADS threads
 // ---------------------------------------------------------------------------------------------
-// find the bin holding the r-th element; hist has nb entries
-// `extra` (shared memory, n_extra bin numbers, may be null): one more element in each of these bins,
-// counted on top of what the histogram holds (the CTA's own corrections, not yet in global memory).
-__device__ void scan_hist(const unsigned *hist, int nb, u64 r, unsigned *bin_out, u64 *r_in_bin, u64 *cnt_out,
-                          unsigned *err, const unsigned *extra = nullptr, unsigned n_extra = 0) {
-    __shared__ u64 s_part[32];
-    const int PER = nb / FIN_THREADS;
-    u64 sum = 0;
-    unsigned mine8[8];                                       // this thread's bins when there are eight of them
-    if (PER == 8) {
-        // two 16-byte loads that bypass L1 (the histogram may have been updated by other CTAs of this kernel)
-        const uint4 h0 = __ldcg(reinterpret_cast<const uint4 *>(hist) + threadIdx.x * 2);
-        const uint4 h1 = __ldcg(reinterpret_cast<const uint4 *>(hist) + threadIdx.x * 2 + 1);
-        mine8[0] = h0.x; mine8[1] = h0.y; mine8[2] = h0.z; mine8[3] = h0.w;
-        mine8[4] = h1.x; mine8[5] = h1.y; mine8[6] = h1.z; mine8[7] = h1.w;
+// A thread's eight bins of a histogram of NB_SMALL, with loads that bypass L1 (other CTAs of the kernel may have updated them)
+struct Bins8 {
+    unsigned c[8];
+};
+static_assert(NB_SMALL / FIN_THREADS == 8, "eight bins to a thread");
+__device__ __forceinline__ Bins8 load_bins8(const unsigned *hist) {
+    const uint4 h0 = __ldcg(reinterpret_cast<const uint4 *>(hist) + threadIdx.x * 2);
+    const uint4 h1 = __ldcg(reinterpret_cast<const uint4 *>(hist) + threadIdx.x * 2 + 1);
+    return {{h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w}};
+}
+
+// What select_bin found, kept in shared memory for the CTA that ran it
+struct BinSel {
+    unsigned B;
+    u64 r, cnt;                 // rank of the k-th element in its bin, and the bin's count
+    u64 lo_hi, lo_lo, hi_hi, hi_lo;     // composite range of the bin
+};
+
+// Level 0, by the whole CTA: the bin of the k-th element (k >= 1) and its composite range -> *out; bin 0 and MWU_DEV_SELECT when
+// the counts are fewer.  Two barriers, the second behind the results; counts add up to less than 2^31.
+// first: this thread's bins when there are NB_SMALL.  extra (shared memory, n_extra bin numbers): one more element in each of
+// these bins, on top of what the histogram holds (the CTA's own corrections, not in global memory).
+// sr: the CTA's copy of the selection (count and window); s: the global one, written when `publish`.
+// (With 64-bit sums, five barriers and the bins loaded on entry it took 3 us.)
+__device__ void select_bin(const Params &p, const Sel *sr, Sel *s, const unsigned *hist, const Bins8 &first, BinSel *out, bool publish,
+                           const unsigned *extra = nullptr, unsigned n_extra = 0) {
+    __shared__ unsigned s_part[32];
+    const int nb = p.nb, per = nb / FIN_THREADS, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    Bins8 mine = first;
+    unsigned sum = 0;
+    if (per == 8) {
         for (unsigned x = 0; x < n_extra; ++x) {
             const unsigned bx = extra[x];
             if ((bx >> 3) == threadIdx.x) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) mine8[i] += ((bx & 7u) == (unsigned)i) ? 1u : 0u;
+                for (int i = 0; i < 8; ++i) mine.c[i] += ((bx & 7u) == (unsigned)i) ? 1u : 0u;
             }
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) sum += mine8[i];
-    } else if (PER == 64) {
+        for (int i = 0; i < 8; ++i) sum += mine.c[i];
+    } else {
         // A thread's 64 bins are 256 bytes: read by the thread itself, every load of a warp would
         // touch 32 cache lines (the L1 tag stage then takes 65 000 cycles per CTA for 65536 bins).
-        // The warp sums them together instead: two coalesced loads and a shuffle tree per thread.
-        const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+        // The warp sums them together instead: two coalesced loads and a sum per thread.
 #pragma unroll 4
         for (int e = 0; e < 32; ++e) {
-            const int base = (w * 32 + e) * 64;
-            unsigned a = ld_vol(&hist[base + l]) + ld_vol(&hist[base + 32 + l]);
-            for (int m = 16; m > 0; m >>= 1) a += __shfl_xor_sync(0xffffffffu, a, m);
-            if (l == e) sum = a;
+            const int base = (wid * 32 + e) * 64;
+            const unsigned a = __reduce_add_sync(0xffffffffu, ld_vol(&hist[base + lane]) + ld_vol(&hist[base + 32 + lane]));
+            if (lane == e) sum = a;
         }
         for (unsigned x = 0; x < n_extra; ++x) sum += ((extra[x] >> 6) == threadIdx.x) ? 1u : 0u;
-    } else {
-#pragma unroll 8
-        for (int i = 0; i < PER; ++i) sum += ld_vol(&hist[threadIdx.x * PER + i]);
-        for (unsigned x = 0; x < n_extra; ++x) sum += (extra[x] / (unsigned)PER == threadIdx.x) ? 1u : 0u;
     }
-    // inclusive scan of the per-thread sums: shuffles inside a warp, then over the 32 warp totals
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    u64 incl = sum;
+    static_assert(NB_MAX / FIN_THREADS == 64, "64 bins to a thread, or eight");
+    unsigned incl = sum;
+#pragma unroll
     for (int m = 1; m < 32; m <<= 1) {
-        const u64 y = __shfl_up_sync(0xffffffffu, incl, m);
+        const unsigned y = __shfl_up_sync(0xffffffffu, incl, m);
         if (lane >= m) incl += y;
     }
-    __syncthreads();                                         // s_part may still be read by an earlier call
     if (lane == 31) s_part[wid] = incl;
     __syncthreads();
-    if (wid == 0) {
-        u64 t = s_part[lane];
-        for (int m = 1; m < 32; m <<= 1) {
-            const u64 y = __shfl_up_sync(0xffffffffu, t, m);
-            if (lane >= m) t += y;
-        }
-        s_part[lane] = t;
-    }
-    __syncthreads();
-    if (wid) incl += s_part[wid - 1];
-    const u64 run = incl - sum;
-    if (threadIdx.x == FIN_THREADS - 1 && incl < r) *err = 1;
-    if (PER == 8) {
-        // the thread whose range holds the r-th element finds the bin among its eight counts
-        if (run < r && r <= incl) {
-            u64 before = run;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const u64 c = mine8[i];
-                if (before < r && r <= before + c) { *bin_out = threadIdx.x * 8 + i; *r_in_bin = r - before; *cnt_out = c; }
-                before += c;
-            }
-        }
-        __syncthreads();
-        return;
-    }
-    __shared__ int s_owner;
-    __shared__ u64 s_run;
-    if (threadIdx.x == 0) s_owner = -1;
-    __syncthreads();
-    if (run < r && r <= incl) { s_owner = threadIdx.x; s_run = run; }     // the bin is in this thread's range
-    __syncthreads();
-    // warp 0 scans the owner's PER (<= 64) bins together
-    if (wid == 0 && s_owner >= 0) {
-        const int base = s_owner * PER;
-        u64 c0 = lane < PER ? (u64)ld_vol(&hist[base + lane]) : 0ull;
-        u64 c1 = lane + 32 < PER ? (u64)ld_vol(&hist[base + lane + 32]) : 0ull;
-        for (unsigned x = 0; x < n_extra; ++x) {
-            c0 += (extra[x] == (unsigned)(base + lane)) ? 1u : 0u;
-            c1 += (extra[x] == (unsigned)(base + lane + 32)) ? 1u : 0u;
-        }
-        u64 i0 = c0;                                   // inclusive scan over bins 0..31, then 32..63
-        for (int m = 1; m < 32; m <<= 1) {
-            const u64 y = __shfl_up_sync(0xffffffffu, i0, m);
-            if (lane >= m) i0 += y;
-        }
-        const u64 tot0 = __shfl_sync(0xffffffffu, i0, 31);
-        u64 i1 = c1;
-        for (int m = 1; m < 32; m <<= 1) {
-            const u64 y = __shfl_up_sync(0xffffffffu, i1, m);
-            if (lane >= m) i1 += y;
-        }
-        i1 += tot0;
-        const u64 before0 = s_run + i0 - c0, before1 = s_run + i1 - c1;
-        if (c0 && before0 < r && r <= before0 + c0) { *bin_out = base + lane; *r_in_bin = r - before0; *cnt_out = c0; }
-        if (c1 && before1 < r && r <= before1 + c1) { *bin_out = base + lane + 32; *r_in_bin = r - before1; *cnt_out = c1; }
-    }
-    __syncthreads();
-}
-
-// what select_bin found, kept in shared memory for the CTA that ran it
-struct BinSel {
-    unsigned B;
-    u64 r, cnt;
-    u64 lo_hi, lo_lo, hi_hi, hi_lo;
-};
-
-// level 0: which bin holds the k-th element; writes the bin and its composite range
-// sr: the CTA's copy of the selection (count and window); s: the global one, written when `publish`
-__device__ void select_bin(const Params &p, const Sel *sr, Sel *s, const unsigned *hist, BinSel *out, bool publish,
-                           const unsigned *extra = nullptr, unsigned n_extra = 0) {
-    __shared__ unsigned s_bin, s_err;
-    __shared__ u64 s_r, s_cnt;
-    if (threadIdx.x == 0) { s_err = 0; s_bin = 0; s_r = 0; s_cnt = 0; }
-    __syncthreads();
-    scan_hist(hist, p.nb, sr->k, &s_bin, &s_r, &s_cnt, &s_err, extra, n_extra);
-    if (threadIdx.x == 0) {
-        if (s_err) atomicOr(p.dev_status, (unsigned)MWU_DEV_SELECT);
-        const unsigned B = s_bin;
+    incl += __reduce_add_sync(0xffffffffu, lane < wid ? s_part[lane] : 0u);
+    const unsigned k = (unsigned)sr->k, run = incl - sum;
+    auto found = [&](unsigned B, unsigned r, unsigned cnt) {
         u64 klo, khi;
         if (B == 0) { klo = 0; khi = sr->lo0; }
-        else if (B == (unsigned)p.nb - 1u) { klo = sr->hi0; khi = ~0ull >> 1; }     // keys are < 2^63
+        else if (B == (unsigned)nb - 1u) { klo = sr->hi0; khi = ~0ull >> 1; }     // keys are < 2^63
         else {
             klo = sr->lo0 + ((u64)(B - 1) << sr->shift0);
             khi = sr->lo0 + ((u64)B << sr->shift0);
@@ -754,14 +686,52 @@ __device__ void select_bin(const Params &p, const Sel *sr, Sel *s, const unsigne
         const u128 lo = make_c(klo, 0), hi = make_c(khi, 0);
         if (publish) {                                   // for the phases that follow
             s->B = B;
-            s->r = s_r;
-            s->cnt = s_cnt;
+            s->r = r;
+            s->cnt = cnt;
             s->lo_hi = (u64)(lo >> 64); s->lo_lo = (u64)lo;
             s->hi_hi = (u64)(hi >> 64); s->hi_lo = (u64)hi;
         }
-        out->B = B; out->r = s_r; out->cnt = s_cnt;
+        out->B = B; out->r = r; out->cnt = cnt;
         out->lo_hi = (u64)(lo >> 64); out->lo_lo = (u64)lo;
         out->hi_hi = (u64)(hi >> 64); out->hi_lo = (u64)hi;
+    };
+    if (threadIdx.x == FIN_THREADS - 1 && incl < k) {
+        atomicOr(p.dev_status, (unsigned)MWU_DEV_SELECT);
+        found(0u, 0u, 0u);
+    }
+    // the k-th element is among this thread's bins
+    const bool owner = run < k && k <= incl;
+    if (per == 8) {
+        if (owner) {
+            unsigned before = run, B = 0, cnt = 0, at = 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (before < k && k <= before + mine.c[i]) { B = threadIdx.x * 8 + i; at = before; cnt = mine.c[i]; }
+                before += mine.c[i];
+            }
+            found(B, k - at, cnt);
+        }
+    } else {
+        // its warp scans the owner's 64 bins together
+        const unsigned who = __ballot_sync(0xffffffffu, owner);
+        if (who) {
+            const int o = __ffs((int)who) - 1, base = (wid * 32 + o) * 64;
+            const unsigned start = __shfl_sync(0xffffffffu, run, o);
+            unsigned c0 = ld_vol(&hist[base + 2 * lane]), c1 = ld_vol(&hist[base + 2 * lane + 1]);
+            for (unsigned x = 0; x < n_extra; ++x) {
+                c0 += (extra[x] == (unsigned)(base + 2 * lane)) ? 1u : 0u;
+                c1 += (extra[x] == (unsigned)(base + 2 * lane + 1)) ? 1u : 0u;
+            }
+            unsigned i1 = c0 + c1;
+#pragma unroll
+            for (int m = 1; m < 32; m <<= 1) {
+                const unsigned y = __shfl_up_sync(0xffffffffu, i1, m);
+                if (lane >= m) i1 += y;
+            }
+            const unsigned b1 = start + i1 - c1, b0 = b1 - c0;
+            if (b0 < k && k <= b1) found((unsigned)(base + 2 * lane), k - b0, c0);
+            else if (b1 < k && k <= b1 + c1) found((unsigned)(base + 2 * lane + 1), k - b1, c1);
+        }
     }
     __syncthreads();
 }
@@ -1675,12 +1645,16 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
         const unsigned i = i_first + (unsigned)t * gstride;
         ent0[t] = i < p.list_cap ? __ldg(&p.list[i]) : make_uint2(0u, 0u);
     }
+    // (so do its bins of the histogram that is scanned first)
+    unsigned *hist_u = p.fhist + p.nb;
+    const bool by_key = !p.gprune && p.k_prune != 0 && p.k_prune != p.n_blocks;        // mode_p == 0
+    Bins8 bins = {};
+    if (p.nb == NB_SMALL) bins = load_bins8(by_key ? p.fhist : hist_u);
     load_work(p.work, &w);
     Sel *sp = &p.work->sel[0];
     Sel *su = &p.work->sel[1];
     const unsigned mode_p = w.sel[0].mode, mode_u = w.sel[1].mode;
     const unsigned nb = (unsigned)p.nb, top = nb - 1u;
-    unsigned *hist_u = p.fhist + p.nb;
     const u64 ulo = w.sel[1].lo0, uhi = w.sel[1].hi0;
     const unsigned ush = w.sel[1].shift0;
     const unsigned n_list = min(w.list_count, p.list_cap);
@@ -1694,7 +1668,7 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
     SelView vp = view_of(&w.sel[0]);
     if (alive && mode_p == 0u) {
         // ---------------- 1: the prune threshold bin, its candidates, the survivors' L_u counts ----------------
-        select_bin(p, &w.sel[0], sp, p.fhist, &s_sel, blockIdx.x == 0);
+        select_bin(p, &w.sel[0], sp, p.fhist, bins, &s_sel, blockIdx.x == 0);
         const unsigned Bp = s_sel.B;
         const u64 r_p = s_sel.r;
         // the threshold bin must be a real bin of the window and small enough to rank
@@ -1772,7 +1746,8 @@ __global__ void __launch_bounds__(FIN_THREADS) resolve_kernel(const __grid_const
     u64 r_u = 0;
     u128 lo = 0, hi = 0;
     if (alive && mode_u == 0u) {
-        select_bin(p, &w.sel[1], su, hist_u, &s_sel, blockIdx.x == 0, s_extra, s_n_extra);
+        if (mode_p == 0u && p.nb == NB_SMALL) bins = load_bins8(hist_u);                // complete only now
+        select_bin(p, &w.sel[1], su, hist_u, bins, &s_sel, blockIdx.x == 0, s_extra, s_n_extra);
         Bu = s_sel.B;
         r_u = s_sel.r;
         lo = from_halves(s_sel.lo_hi, s_sel.lo_lo);
