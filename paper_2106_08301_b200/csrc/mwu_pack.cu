@@ -62,20 +62,16 @@ __device__ __forceinline__ unsigned tile_offset(unsigned r, unsigned i, int b) {
     return (r >> 3) * 1024u + (r & 7u) * 128u + ((c ^ (r & 7u)) << 4) + within;
 }
 
-// sign bits of one block (bit l = weight l) -> bit l/2 + 16 * (l % 2): the even bits closed up in the
+// sign bits of one block (bit l = weight l, at most 16 of them) -> bit l/2 + 16 * (l % 2): the even bits closed up in the
 // low half, the odd bits in the high half
-__device__ __forceinline__ unsigned close_up_even_bits(unsigned x) {
-    x &= 0x55555555u;
-    x = (x | (x >> 1)) & 0x33333333u;
-    x = (x | (x >> 2)) & 0x0f0f0f0fu;
-    x = (x | (x >> 4)) & 0x00ff00ffu;
-    x = (x | (x >> 8)) & 0x0000ffffu;
-    return x;
-}
-__device__ __forceinline__ unsigned spread_signs(unsigned sb, int b) {
-    const unsigned m = (b >= 32) ? 0xffffffffu : ((1u << b) - 1u);
-    sb &= m;
-    return close_up_even_bits(sb) | (close_up_even_bits(sb >> 1) << 16);
+__device__ __forceinline__ unsigned spread_signs(unsigned x) {
+    unsigned t = (x ^ (x >> 1)) & 0x2222u;
+    x ^= t ^ (t << 1);
+    t = (x ^ (x >> 2)) & 0x0c0cu;
+    x ^= t ^ (t << 2);
+    t = (x ^ (x >> 4)) & 0x00f0u;
+    x ^= t ^ (t << 4);
+    return __byte_perm(x, 0u, 0x4140);
 }
 
 __device__ __forceinline__ unsigned live_of(unsigned P, int b) {
@@ -311,9 +307,9 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(Params p, int counte
 
 constexpr unsigned OWN_THREADS = 512;
 // CTAs to an SM that the registers are cut to: enough warps to hide the gathers of W and u, few enough that their lines stay in
-// L1 until the neighbouring blocks' turn (16384 x 4096, 50 % / 25 %, b = 2: 175 us with 12, 181 with 8, 317 with 16; b = 4: 109,
-// 112, 114; b = 8: 84 with 16, 88 with 8).
-__host__ __device__ constexpr int fill_ctas(int b, bool own) { return own ? 0 : b <= 4 ? 12 : 16; }
+// L1 until the neighbouring blocks' turn (16384 x 4096, 50 % / 25 %, b = 2: 160 us with 12; 181 with 8 and 317 with 16 where 12 took 175;
+// b = 4: 107; b = 8: 83 with 16, 88 with 8).  Without a scan: all 512 CTAs of 2048 x 2048 at once (three to an SM: 13.5 us instead of 12.9).
+__host__ __device__ constexpr int fill_ctas(int b, bool own) { return own ? (b == 2 ? 3 : 4) : b <= 4 ? 12 : 16; }
 // Most blocks (padding rows included) of the form without a scan: every CTA reads on average half of the bitmaps.  Whole
 // mwu_pack calls, us, with it and without: 256 x 256, b = 4: 8.5 / 13.0; 1000 x 1216, b = 2: 13.7 / 17.0; 2048 x 2048, b = 8,
 // 524288 blocks: 12.5 / 15.1; 3072 x 2048, b = 8, 786432: 19.0 / 19.7; 1024 x 2048, b = 2, 1048576: 26.0 / 17.7.
@@ -327,6 +323,31 @@ __device__ __forceinline__ void row_block_of(unsigned off, int b, unsigned *r, u
     *i = (c * 16u + (off & 15u)) / (2u * (unsigned)b);
 }
 
+// words of a bit matrix over the lanes of a warp: bit b of lane l becomes bit l of lane b
+__device__ __forceinline__ unsigned warp_transpose(unsigned w, int lane) {
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) {
+        const unsigned m = k == 16 ? 0x0000ffffu : k == 8 ? 0x00ff00ffu : k == 4 ? 0x0f0f0f0fu : k == 2 ? 0x33333333u : 0x55555555u;
+        const unsigned y = __shfl_xor_sync(0xffffffffu, w, k);
+        w = (lane & k) ? ((w & ~m) | ((y >> k) & m)) : ((w & m) | ((y & m) << k));
+    }
+    return w;
+}
+
+// Bits of a row's blocks moved to their store slots: slot = (number of the block's first one) ^ (r % 8 chunks of STEP slots).
+template <int STEP>
+__device__ __forceinline__ unsigned to_slots(unsigned w, unsigned r) {
+#pragma unroll
+    for (int k = 1; k <= 4; k <<= 1) {
+        const int d = k * STEP;
+        const unsigned m = d == 16 ? 0x0000ffffu : d == 8 ? 0x00ff00ffu : d == 4 ? 0x0f0f0f0fu : d == 2 ? 0x33333333u : 0x55555555u;
+        if (r & (unsigned)k) w = ((w & m) << d) | ((w >> d) & m);
+    }
+    return w;
+}
+
+// Bounded by instruction issue and latency (16384 x 4096, b = 16, 80 % / 60 %: 51 us the whole call with a ballot for each
+// (class, slot) and 64-bit addresses, 47 so; b = 2 175 / 160; 256 x 256, b = 4: 7.7 / 6.8).
 // Bounded by latency where records are few (a chain of some dozen L2 round trips, out of a cold instruction cache).
 // OWN: the base of the record's lists is counted here too, from the bitmaps of everything before it: no record table, no
 // kernel before this one; the lists are then written by four times the threads.
@@ -350,11 +371,17 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128, fill_ctas(B, OWN)) fi
     unsigned char *dpay = p.packed + p.L.off_dpay;
     unsigned short *ppos = reinterpret_cast<unsigned short *>(p.packed + p.L.off_ppos);
 
+    // Rows that can have a block in a given slot: every second one where a block takes two.
+    constexpr int QMAX = B == 16 ? kTileRows / 2 : kTileRows;
     __shared__ unsigned s_bal[4][3 * G];                    // per warp and (class, slot): the rows that have such a block
     __shared__ unsigned char s_before[4][3 * G];            // ... how many in the warps before
-    __shared__ __align__(4) unsigned char s_len[3 * G];     // ... and in all (at most 128 each: a byte)
-    __shared__ unsigned short s_full[3][kTileRows + 1];     // per class and q: list entries of rounds 0 .. q-1
-    __shared__ unsigned s_more[3][kTileRows + 1];           // per class and q: slots that have a round q
+    // ... and in all; slots w and w + G/2 in word w
+    __shared__ __align__(4) unsigned short s_len[3][G];
+    // per class and q: list entries of rounds 0 .. q-1, and the slots that have a round q (above bit 16 where they fit there)
+    constexpr bool ONE_WORD = G <= 16;
+    __shared__ unsigned s_round[3][QMAX + 1];
+    __shared__ unsigned short s_full[ONE_WORD ? 1 : 3][ONE_WORD ? 1 : QMAX + 1];
+    auto full_before = [&](int c, unsigned q) -> unsigned { return ONE_WORD ? s_round[c][q] & 0xffffu : s_full[ONE_WORD ? 0 : c][ONE_WORD ? 0 : q]; };
     // Tile offsets of the pruned, the dense and the unified list.  Without a gap between them where CTAs crowd on an SM (the
     // shared memory of three full lists took b = 4 from 109 to 231 us); with their beginnings fixed in the form of few CTAs.
     __shared__ unsigned short s_off[(OWN ? 3 : 1) * kTileRows * NBK];
@@ -397,26 +424,31 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128, fill_ctas(B, OWN)) fi
             if (live) atomicOr(&s_own[2], live);
         }
     }
-    // class of block i: 0 pruned, 1 dense, 2 unified.  occ[class]: the store slots this row fills with it
-    // (a row never has two blocks in one slot)
-    unsigned occ[3] = {0u, 0u, 0u};
-#pragma unroll
-    for (int i = 0; i < NBK; ++i) {
-        const unsigned slot = (tile_offset((unsigned)r, (unsigned)i, B) & 127u) / STORE;
-        const unsigned bit = 1u << slot;
-        occ[0] |= ((P >> i) & 1u) ? bit : 0u;
-        occ[1] |= ((D >> i) & 1u) ? bit : 0u;
-        occ[2] |= ((U >> i) & 1u) ? bit : 0u;
-    }
+    // Class 0 pruned, 1 dense, 2 unified.  The row's dense and unified blocks as bits of their store slots (a row never has two
+    // blocks in one), and the bits of 32 rows turned into a word per (class, slot) with five shuffles (a ballot for each takes
+    // three to four times the instructions).
     if (has_row) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-#pragma unroll
-        for (int sl = 0; sl < G; ++sl) {
-            const unsigned bal = __ballot_sync(0xffffffffu, (occ[c] >> sl) & 1u);
-            if (lane == ((c * G + sl) & 31)) s_bal[warp][c * G + sl] = bal;
+        constexpr int STEP = 16 / STORE;                        // slots of a 16-byte chunk
+        if constexpr (G <= 16) {
+            unsigned w = D | (U << 16);
+            if (B == 16) {                                      // block i: the slots from 2 i on
+                w = (w | (w << 2)) & 0x00330033u;
+                w = (w | (w << 1)) & 0x00550055u;
+            }
+            w = warp_transpose(to_slots<STEP>(w, (unsigned)r), lane);      // lane f: dense slot f; lane 16 + f: unified slot f
+            const unsigned other = __shfl_xor_sync(0xffffffffu, w, 16);
+            const unsigned there = B == 16 ? 0x55555555u << (lane & 1) : 0xffffffffu;
+            const int f = lane & 15;
+            if (f < G) {
+                s_bal[warp][(lane < 16 ? G : 2 * G) + f] = w;
+                if (lane < 16) s_bal[warp][f] = there & ~(w | other);
+            }
+        } else {
+            const unsigned d = warp_transpose(to_slots<STEP>(D, (unsigned)r), lane), u = warp_transpose(to_slots<STEP>(U, (unsigned)r), lane);
+            s_bal[warp][lane] = ~(d | u);
+            s_bal[warp][G + lane] = d;
+            s_bal[warp][2 * G + lane] = u;
         }
-      }
     }
     __syncthreads();
     // blocks per (class, slot) in the record, and in the warps before each warp (population counts
@@ -426,34 +458,38 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128, fill_ctas(B, OWN)) fi
         unsigned before = 0;
         for (int w2 = 0; w2 < ww; ++w2) before += __popc(s_bal[w2][f]);
         s_before[ww][f] = (unsigned char)before;
-        if (ww == 3) s_len[f] = (unsigned char)(before + __popc(s_bal[3][f]));
+        if (ww == 3) {
+            const int c = f / G, sl = f % G;
+            s_len[c][(sl % (G / 2)) * 2 + sl / (G / 2)] = (unsigned short)(before + __popc(s_bal[3][f]));
+        }
     }
     __syncthreads();
     // round-robin order of a class list: round q takes the q-th block of every slot that has one.
-    // Thread q (and thread 0 for q = 128) tabulates what comes before round q.
-    for (int q = r; q <= kTileRows; q += (int)NT) {
+    for (int t = r; t < 3 * (QMAX + 1); t += (int)NT) {
+        const int c = t / (QMAX + 1), q = t - c * (QMAX + 1);
+        // two slots at a time, in halves of a word
+        unsigned full = 0, more = 0;
+        const unsigned q2 = (unsigned)q * 0x00010001u;
+        const unsigned *len2 = reinterpret_cast<const unsigned *>(s_len[c]);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            // four slots at a time: bytewise minimum summed with a dot product, bytewise compare
-            // gathered into a bit per slot
-            unsigned full = 0, more = 0;
-            const unsigned q4 = (unsigned)q * 0x01010101u;
-            const unsigned *len4 = reinterpret_cast<const unsigned *>(s_len + c * G);
-#pragma unroll
-            for (int w = 0; w < G / 4; ++w) {
-                const unsigned l4 = len4[w];
-                full = __dp4a(__vminu4(l4, q4), 0x01010101u, full);
-                more |= (((__vcmpgtu4(l4, q4) & 0x80808080u) * 0x00204081u) >> 28) << (4 * w);
-            }
-            s_full[c][q] = (unsigned short)full;
-            s_more[c][q] = more;
+        for (int w = 0; w < G / 2; ++w) {
+            const unsigned l2 = len2[w];
+            full += __vminu2(l2, q2);
+            more |= (~((q2 | 0x80008000u) - l2) & 0x80008000u) >> (15 - w);      // the top bit of a half stays where q >= length
+        }
+        full = (full & 0xffffu) + (full >> 16);
+        more = (more & 0xffffu) | ((more >> 16) << (G / 2));
+        if (ONE_WORD) s_round[c][q] = full | (more << 16);
+        else {
+            s_round[c][q] = more;
+            s_full[ONE_WORD ? 0 : c][ONE_WORD ? 0 : q] = (unsigned short)full;
         }
     }
     __syncthreads();
 
     // every block's place in its class list
-    const unsigned first_d = OWN ? kTileRows * NBK : s_full[0][kTileRows];
-    const unsigned first_u = OWN ? 2 * kTileRows * NBK : first_d + s_full[1][kTileRows];
+    const unsigned first_d = OWN ? kTileRows * NBK : full_before(0, QMAX);
+    const unsigned first_u = OWN ? 2 * kTileRows * NBK : first_d + full_before(1, QMAX);
     const unsigned below = (1u << lane) - 1u;
     if (has_row)
 #pragma unroll 4
@@ -465,14 +501,16 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128, fill_ctas(B, OWN)) fi
         // earlier rows with the same class and slot
         const unsigned q = s_before[warp][f] + __popc(s_bal[warp][f] & below);
         // q full rounds before it, then the lower slots of its own round
-        const unsigned idx = s_full[cls][q] + __popc(s_more[cls][q] & ((1u << slot) - 1u));
+        const unsigned round = s_round[cls][q];
+        const unsigned idx = ONE_WORD ? (round & 0xffffu) + __popc((round >> 16) & ((1u << slot) - 1u))
+                                      : full_before((int)cls, q) + __popc(round & ((1u << slot) - 1u));
         s_off[(cls == 0u ? 0u : cls == 1u ? first_d : first_u) + idx] = (unsigned short)off;
     }
     uint4 me, nx;                                           // (ubase, dbase, pbase, live); the table ends with the totals
     if (OWN) {
         __syncthreads();
         me = make_uint4(s_own[0], rec * (unsigned)(kTileRows * NBK) - s_own[0] - s_own[1], s_own[1], s_own[2]);
-        nx = make_uint4(me.x + s_full[2][kTileRows], me.y + s_full[1][kTileRows], me.z + s_full[0][kTileRows], 0u);
+        nx = make_uint4(me.x + full_before(2, QMAX), me.y + full_before(1, QMAX), me.z + full_before(0, QMAX), 0u);
         uint4 *table = reinterpret_cast<uint4 *>(p.packed + p.L.off_rec);
         if (r == 0) table[rec] = me;
         if (rec == gridDim.x - 1u && r == 0) {
@@ -490,7 +528,7 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128, fill_ctas(B, OWN)) fi
     }
 
     bool bad = false;
-    constexpr unsigned BMASK = (B >= 32) ? 0xffffffffu : ((1u << B) - 1u);
+    constexpr unsigned BMASK = (1u << B) - 1u;
     const unsigned len_u = nx.x - me.x, len_d = nx.y - me.y, len_p = nx.z - me.z;
     // the record's three list ranges must lie inside the sections (checked once, not per entry)
     if (len_u + len_d + len_p != (unsigned)(kTileRows * NBK) ||
@@ -500,21 +538,28 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128, fill_ctas(B, OWN)) fi
         bad = true;                                          // the table does not describe this record
     else {
         const long long row_base = tile * kTileRows;
-        const long long f_base = row_base * p.cols + stage * kStageK;          // first weight of the record
+        // the record's first block; block i of its row rr is number rr * bpr + i from there on (blocks are fewer than 2^31)
+        const long long j_base = row_base * p.bpr + stage * NBK;
+        const unsigned bpr = (unsigned)p.bpr;
+        const float *Wb = p.W + j_base * B, *Ub = p.U ? p.U + j_base * B : nullptr;
         // pruned blocks: positions only
         unsigned short *pp = ppos + me.z;
         for (unsigned t = (unsigned)r; t < len_p; t += NT) pp[t] = s_off[t];
         // unified blocks: sign bits, position, magnitude
         uint2 *ul = ulist + me.x;
-        const long long j_base = row_base * p.bpr + stage * NBK;
+        const float *ub = p.u + j_base;
+        const unsigned *sgn = p.sign_bits + j_base * B / 32;    // (a record begins at a multiple of 64 weights)
         for (unsigned t = (unsigned)r; t < len_u; t += NT) {
             const unsigned off = s_off[first_u + t];
             unsigned rr, i;
             row_block_of(off, B, &rr, &i);
-            const long long f = f_base + (long long)rr * p.cols + i * B;
-            const unsigned sb = (__ldg(p.sign_bits + (f >> 5)) >> (f & 31)) & BMASK;
-            const unsigned ub = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(__ldg(p.u + j_base + (long long)rr * p.bpr + i)));
-            ul[t] = make_uint2(spread_signs(sb, B), off | (ub << 16));
+            const unsigned j = rr * bpr + i;
+            unsigned sb;
+            if (B == 16) sb = __ldg(reinterpret_cast<const unsigned short *>(sgn) + j);
+            else if (B == 8) sb = __ldg(reinterpret_cast<const unsigned char *>(sgn) + j);
+            else sb = (__ldg(sgn + j / (32 / B)) >> (j % (32 / B) * B)) & BMASK;
+            const unsigned mag = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(__ldg(ub + j)));
+            ul[t] = make_uint2(spread_signs(sb), off | (mag << 16));
         }
         // dense blocks: position, then the values, LPB lanes to a block
         unsigned short *dp = dpos + me.y;
@@ -524,21 +569,21 @@ __global__ void __launch_bounds__(OWN ? OWN_THREADS : 128, fill_ctas(B, OWN)) fi
             const unsigned t = q / (unsigned)LPB, part = q % (unsigned)LPB;
             unsigned rr, i;
             row_block_of(s_off[first_d + t], B, &rr, &i);
-            const long long f = f_base + (long long)rr * p.cols + i * B + part * 4;
+            const size_t f = (size_t)(rr * bpr + i) * B + part * 4;
             unsigned char *dst = pay + q * 8u;               // = t * 2B + part * 8 when a block takes LPB lanes
             if (B >= 4) {
-                float4 a = __ldg(reinterpret_cast<const float4 *>(p.W + f));
-                if (p.U) {
-                    const float4 d = __ldg(reinterpret_cast<const float4 *>(p.U + f));
+                float4 a = __ldg(reinterpret_cast<const float4 *>(Wb + f));
+                if (Ub) {
+                    const float4 d = __ldg(reinterpret_cast<const float4 *>(Ub + f));
                     a.x = __fadd_rn(a.x, d.x); a.y = __fadd_rn(a.y, d.y); a.z = __fadd_rn(a.z, d.z); a.w = __fadd_rn(a.w, d.w);
                 }
                 const __nv_bfloat162 h0 = __floats2bfloat162_rn(a.x, a.y), h1 = __floats2bfloat162_rn(a.z, a.w);
                 *reinterpret_cast<uint2 *>(dst) = make_uint2(*reinterpret_cast<const unsigned *>(&h0),
                                                              *reinterpret_cast<const unsigned *>(&h1));
             } else {
-                float2 a = __ldg(reinterpret_cast<const float2 *>(p.W + f));
-                if (p.U) {
-                    const float2 d = __ldg(reinterpret_cast<const float2 *>(p.U + f));
+                float2 a = __ldg(reinterpret_cast<const float2 *>(Wb + f));
+                if (Ub) {
+                    const float2 d = __ldg(reinterpret_cast<const float2 *>(Ub + f));
                     a.x = __fadd_rn(a.x, d.x); a.y = __fadd_rn(a.y, d.y);
                 }
                 const __nv_bfloat162 h0 = __floats2bfloat162_rn(a.x, a.y);
