@@ -39,6 +39,8 @@ bool halo_eligible(int h, int w, int kh, int kw, int stride, int pad);
 int run_conv_halo(const Params &g, const void *X, int n, int c, int h, int w, int kh, int kw, int stride, int pad, int sm_count,
                   cudaStream_t st);
 // decode-once path, defined in mwu_gemm3.cu
+bool resident_eligible(const Params &p, int sm_count);
+cudaError_t launch_resident(int bw, const CUtensorMap &tmap_x, const CUtensorMap &tmap_y, const Params &p, int sm_count, cudaStream_t st);
 cudaError_t launch_decode(int bw, const Params &p, __nv_bfloat16 *Wd, long long ldw, cudaStream_t st);
 cudaError_t launch_dense(const CUtensorMap &tmap_x, const CUtensorMap &tmap_w, const CUtensorMap &tmap_y,
                          const Params &p, int sm_count,
@@ -566,15 +568,20 @@ static void fill_common(Params &p, const mwu_proj_desc *desc, const void *packed
 // every 512-row activation tile.
 static const int64_t kDecodeOnceMinRows = 1;
 
+// boxes of 128 bytes x box_rows: 64 columns of bf16, 32 of fp32
+static bool encode_2d(mwu::gemm::EncodeTiledFn encode, CUtensorMap *tmap, bool fp32, const void *ptr, int64_t inner, int64_t outer,
+                      int64_t ld, int box_rows) {
+    const cuuint64_t gdim[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
+    const cuuint64_t gstride[1] = {(cuuint64_t)ld * (fp32 ? 4 : 2)};
+    const cuuint32_t box[2] = {(cuuint32_t)(fp32 ? 32 : mwu::gemm::BK), (cuuint32_t)box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    return encode(tmap, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), gdim,
+                  gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 static bool encode_bf16_2d(mwu::gemm::EncodeTiledFn encode, CUtensorMap *tmap, const void *ptr, int64_t inner,
                            int64_t outer, int64_t ld, int box_rows) {
-    const cuuint64_t gdim[2] = {(cuuint64_t)inner, (cuuint64_t)outer};
-    const cuuint64_t gstride[1] = {(cuuint64_t)ld * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)mwu::gemm::BK, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return encode(tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), gdim, gstride, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_2d(encode, tmap, false, ptr, inner, outer, ld, box_rows);
 }
 
 extern "C" size_t mwu_gemm_workspace_bytes(const mwu_proj_desc *desc, int64_t M) {
@@ -637,6 +644,14 @@ extern "C" int mwu_gemm_ws(const mwu_proj_desc *desc, const void *packed, const 
         if (!encode_bf16_2d(encode, &tmap_x, X, desc->cols, M, ldx, stream_box_rows(p, sm_count)))
             return MWU_ERR_CUDA;
         return launch_stream(desc->block, tmap_x, p, sm_count, st) == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
+    }
+
+    // a short reduction: the weights stay in shared memory
+    if (resident_eligible(p, sm_count)) {
+        CUtensorMap tmap_x, tmap_y;
+        if (!encode_bf16_2d(encode, &tmap_x, X, desc->cols, M, ldx, BMH) ||
+            !encode_2d(encode, &tmap_y, y_dtype != 0, Y, desc->rows, M, ldy, 32)) return MWU_ERR_CUDA;
+        return launch_resident(desc->block, tmap_x, tmap_y, p, sm_count, st) == cudaSuccess ? MWU_OK : MWU_ERR_CUDA;
     }
 
     // decode once into the caller's workspace, then a two-operand GEMM over it

@@ -1,4 +1,4 @@
-// Decode-once path of mwu_gemm for many activation rows.
+// Decode-once path of mwu_gemm for many activation rows (short reductions: mwu_gemm5.cu).
 //
 // The fused kernels decode a weight record again for every activation tile that meets it.  When
 // the caller lends a workspace, the packed weights are instead expanded once per call into a
@@ -380,22 +380,10 @@ mwu_dense_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
                     // the last store out of this buffer has read it
                     if (lane == 0) { if (D_EPI_BUFS == 2) bulk_wait_read_1(); else bulk_wait_read(); }
                     __syncwarp();
-                    // row `lane`: eight 16-byte pieces, piece j at position j ^ (lane % 8) (128-byte swizzle)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const unsigned *src = (j < 4) ? (v[2 * h] + 8 * j) : (v[2 * h + 1] + 8 * (j - 4));
-                        uint4 o;
-                        __nv_bfloat162 h2;
-                        h2 = __floats2bfloat162_rn(__uint_as_float(src[0]), __uint_as_float(src[1]));
-                        o.x = *reinterpret_cast<unsigned *>(&h2);
-                        h2 = __floats2bfloat162_rn(__uint_as_float(src[2]), __uint_as_float(src[3]));
-                        o.y = *reinterpret_cast<unsigned *>(&h2);
-                        h2 = __floats2bfloat162_rn(__uint_as_float(src[4]), __uint_as_float(src[5]));
-                        o.z = *reinterpret_cast<unsigned *>(&h2);
-                        h2 = __floats2bfloat162_rn(__uint_as_float(src[6]), __uint_as_float(src[7]));
-                        o.w = *reinterpret_cast<unsigned *>(&h2);
-                        *reinterpret_cast<uint4 *>(sbuf + lane * 128 + ((j ^ (lane & 7)) << 4)) = o;
-                    }
+                    unsigned w[32];
+                    pack_bf16(v[2 * h], w);
+                    pack_bf16(v[2 * h + 1], w + 16);
+                    stage_row64(w, sbuf, lane);
                     fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) {

@@ -70,42 +70,6 @@ __device__ __forceinline__ float4 ld_cluster_f4(unsigned addr) {
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
     return v;
 }
-// a whole warp waits, polling for long; the same answer in all lanes
-__device__ __forceinline__ bool warp_wait_spin(unsigned bar, unsigned parity, volatile int *abort) {
-#pragma unroll 1
-    for (int i = 0; i < 4096; ++i)
-        if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
-}
-
-// barrier over the threads of one decode group
-__device__ __forceinline__ void group_sync(int group) {
-    __syncwarp();
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(ST_GROUP) : "memory");
-}
-
-// the values of a block, WORDS pairs of them: from the packed list, and to its place in a swizzled tile
-template <int WORDS>
-__device__ __forceinline__ void ld_words(const unsigned char *p, unsigned (&v)[WORDS]) {
-    if constexpr (WORDS == 8)
-        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p));
-    else if constexpr (WORDS == 4) {
-        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p));
-        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-    } else if constexpr (WORDS == 2) {
-        const uint2 x = __ldg(reinterpret_cast<const uint2 *>(p));
-        v[0] = x.x; v[1] = x.y;
-    } else v[0] = __ldg(reinterpret_cast<const unsigned *>(p));
-}
-template <int WORDS>
-__device__ __forceinline__ void st_words(unsigned char *tile, unsigned at, const unsigned (&v)[WORDS]) {
-    if constexpr (WORDS >= 4) *reinterpret_cast<uint4 *>(tile + at) = make_uint4(v[0], v[1], v[2], v[3]);
-    if constexpr (WORDS == 8) *reinterpret_cast<uint4 *>(tile + (at ^ 16u)) = make_uint4(v[4], v[5], v[6], v[7]);
-    if constexpr (WORDS == 2) *reinterpret_cast<uint2 *>(tile + at) = make_uint2(v[0], v[1]);
-    if constexpr (WORDS == 1) *reinterpret_cast<unsigned *>(tile + at) = v[0];
-}
-
 // the lines of `bytes` bytes from p on to L2, spread over a decode group
 __device__ __forceinline__ void prefetch_span(const unsigned char *p, unsigned bytes, unsigned t0) {
 #pragma unroll 1
@@ -283,11 +247,9 @@ mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
 #pragma unroll
                 for (unsigned k = 0; k < BATCH; ++k) {
                     if (e0 + t0 + k * ST_GROUP >= n_u) break;
-                    const unsigned at = ent[k].y & OFF_MASK, u2 = __byte_perm(ent[k].y, 0u, 0x3232);
+                    const unsigned at = ent[k].y & OFF_MASK;
                     unsigned w[WORDS];
-#pragma unroll
-                    for (int t = 0; t < WORDS; ++t)         // weights 2t, 2t+1: sign bits t and 16+t
-                        w[t] = ((ent[k].x << (15 - t)) & 0x80008000u) ^ u2;
+                    unified_words<WORDS>(ent[k], w);
                     st_words<WORDS>(tile, at, w);
                     if (UNDO) at_u[k] = at;
                 }
@@ -337,7 +299,7 @@ mwu_gemm_stream_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
                     for (int t = 0; t < REC_BYTES / 16 / ST_GROUP; ++t) z[t * ST_GROUP] = make_uint4(0, 0, 0, 0);
                 }
             }
-            group_sync(group);
+            group_barrier<ST_GROUP>(1 + group);
             if (ok) {
                 write_u(0u);
                 write_d(0u);

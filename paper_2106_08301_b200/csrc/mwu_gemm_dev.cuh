@@ -139,6 +139,19 @@ __device__ __forceinline__ bool mbar_wait_spin(unsigned bar, unsigned parity, vo
         if (mbar_test(bar, parity)) return true;
     return mbar_wait(bar, parity, abort);
 }
+// a whole warp waits, polling for long; the same answer in all lanes
+__device__ __forceinline__ bool warp_wait_spin(unsigned bar, unsigned parity, volatile int *abort) {
+#pragma unroll 1
+    for (int i = 0; i < 4096; ++i)
+        if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+}
+// barrier over the THREADS threads (whole warps) that name barrier `id`
+template <int THREADS>
+__device__ __forceinline__ void group_barrier(int id) {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(THREADS) : "memory");
+}
 template <int BYTES>
 __device__ __forceinline__ void cp_async_if(unsigned dst, const void *src, unsigned pred) {
     asm volatile(
@@ -163,6 +176,10 @@ __device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap *map
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y) : "memory");
+}
+// a box of the tensor to L2
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *map, int x, int y) {
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
 __device__ __forceinline__ void tmem_alloc(unsigned dst_smem, unsigned ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols) : "memory");
@@ -354,6 +371,22 @@ __device__ __forceinline__ void store_chunk_staged(const Params &p, long long mr
     }
 }
 
+// 32 accumulators of a row as 16 pairs of bf16
+__device__ __forceinline__ void pack_bf16(const unsigned (&v)[32], unsigned *w) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+        w[j] = *reinterpret_cast<const unsigned *>(&h);
+    }
+}
+// 32 words (64 bf16 columns) to row `lane` of a 4 KB box: eight 16-byte pieces, piece j at position j ^ (lane % 8) (128-byte
+// swizzle)
+__device__ __forceinline__ void stage_row64(const unsigned (&w)[32], unsigned char *box, int lane) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        *reinterpret_cast<uint4 *>(box + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+}
+
 // K-major operand, 128-byte swizzle: rows of 128 bytes, 8-row groups 1024 bytes apart
 __device__ __forceinline__ unsigned long long make_desc(unsigned smem_addr) {
     unsigned long long d = 0;
@@ -393,6 +426,35 @@ struct DecodeCfg {
     static constexpr int WORDS = BW / 2;                    // 32-bit words per block
     static constexpr unsigned OFF_MASK = (unsigned)(REC_BYTES - 1) & ~(unsigned)((BW >= 8 ? 16 : 2 * BW) - 1);
 };
+
+// the values of a block, WORDS pairs of them: from the packed list, and to its place in a swizzled tile
+template <int WORDS>
+__device__ __forceinline__ void ld_words(const unsigned char *p, unsigned (&v)[WORDS]) {
+    if constexpr (WORDS == 8)
+        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p));
+    else if constexpr (WORDS == 4) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p));
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else if constexpr (WORDS == 2) {
+        const uint2 x = __ldg(reinterpret_cast<const uint2 *>(p));
+        v[0] = x.x; v[1] = x.y;
+    } else v[0] = __ldg(reinterpret_cast<const unsigned *>(p));
+}
+template <int WORDS>
+__device__ __forceinline__ void st_words(unsigned char *tile, unsigned at, const unsigned (&v)[WORDS]) {
+    if constexpr (WORDS >= 4) *reinterpret_cast<uint4 *>(tile + at) = make_uint4(v[0], v[1], v[2], v[3]);
+    if constexpr (WORDS == 8) *reinterpret_cast<uint4 *>(tile + (at ^ 16u)) = make_uint4(v[4], v[5], v[6], v[7]);
+    if constexpr (WORDS == 2) *reinterpret_cast<uint2 *>(tile + at) = make_uint2(v[0], v[1]);
+    if constexpr (WORDS == 1) *reinterpret_cast<unsigned *>(tile + at) = v[0];
+}
+// ... and of a unified block from its list entry (x: spread signs, y: off | bf16(u) << 16)
+template <int WORDS>
+__device__ __forceinline__ void unified_words(const uint2 ent, unsigned (&w)[WORDS]) {
+    const unsigned u2 = __byte_perm(ent.y, 0u, 0x3232);     // bf16(u) in both halves
+#pragma unroll
+    for (int t = 0; t < WORDS; ++t) w[t] = ((ent.x << (15 - t)) & 0x80008000u) ^ u2;    // weights 2t, 2t+1: sign bits t and 16+t
+}
 
 template <int BW, int NDEC_THREADS>
 __device__ __forceinline__ void fetch_entries(const PackedRec r0, const PackedRec r1, const Params &p, int tid,

@@ -307,6 +307,31 @@ def test_gemm_few_rows_uneven_records(b, M, pr, un):
     check_gemm(W, b, Mb * un // 10, Mb * pr // 10, M)
 
 
+@pytest.mark.parametrize("rows,cols,b,M", [(96, 128, 8, 37900),          # one record tile: half a tile of outputs (fp32: the streaming kernel)
+                                           (640, 192, 4, 12801),         # five record tiles, a ragged last row, two boxes a warp
+                                           (1000, 256, 2, 9604),         # ragged weight rows; one box a warp
+                                           (16384, 64, 16, 620),         # 64 weight tiles: CTAs change weights on the way
+                                           (264, 256, 16, 20000)])
+def test_gemm_short_reduction(rows, cols, b, M):
+    """Weights kept in shared memory: at least two tiles of 128 x 256 outputs an SM, with dead stages and slices where there is room."""
+    W = inputs.normal_weights(rows, cols, 0.02, 500 + b)
+    if cols > 128:
+        W[:, 64:144] = 0.0                       # a dead stage and a dead slice
+    Mb = W.numel() // b
+    assert -(-rows // 256) * -(-M // 128) >= 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    desc, bufs, packed, p = check_gemm(W, b, Mb * 7 // 10, Mb // 2, M, seed=60 + b)
+    # gaps behind the rows of X and Y; what lies in them is neither read nor written
+    X = inputs.normal_activations_bf16((M, cols + 8), 4243)
+    X[:, cols:] = float("nan")
+    ref = O.gemm(X[:, :cols].to(torch.float64).numpy(), O.decoded_weights(p, b))
+    for dtype, tol in ((torch.bfloat16, 2e-3), (torch.float32, 1e-5)):
+        Y = torch.full((M, rows + 8), float("nan"), dtype=dtype, device="cuda")
+        B.mwu_gemm(desc, packed, X.cuda(), M, cols + 8, Y, rows + 8, int(dtype == torch.float32), bufs.dev_status)
+        assert int(bufs.dev_status.item()) == 0
+        assert bool(torch.isnan(Y[:, rows:]).all())
+        assert errors(Y[:, :rows].float().cpu().numpy(), ref)[0] <= tol
+
+
 @pytest.mark.parametrize("filters,cin,h,w,k,stride,pad,n,b", [(128, 64, 13, 11, 3, 2, 1, 2, 4),    # four planes, odd sizes
                                                               (136, 128, 9, 9, 3, 1, 1, 1, 8),     # two chunks over a cluster, ragged filters
                                                               (256, 64, 30, 29, 3, 1, 1, 24, 16),  # several tiles to a CTA, two filter tiles
