@@ -281,8 +281,8 @@ int mwu_decode(const mwu_proj_desc *desc, const void *packed, void *Wd, int64_t 
  * (bf16 x bf16, fp32 accumulation).  Which kernel runs, and in how many pieces it adds up the reduction, depends on M, on
  * the sizes, on whether a workspace is given and on the device, and with it the last bits of an fp32 result (sums of K
  * products of independent values: about 1e-9 K of their size in one piece, less in several).
- * Few rows (up to 256, or more where the weights are few) are multiplied without expanding anything
- * and mostly leave the workspace alone.
+ * Few rows (up to 256, or more where the weights or the outputs are few) and short reductions of many rows (up to 256
+ * columns) are multiplied without expanding anything and mostly leave the workspace alone.
  * mwu_gemm_workspace_bytes returns 0 when M is too small for this to pay (or desc is invalid);
  * with workspace == NULL, or fewer bytes than that, the call behaves exactly like mwu_gemm.
  * The workspace holds nothing between calls and may be shared by calls on the same stream.
