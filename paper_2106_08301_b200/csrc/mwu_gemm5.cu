@@ -252,8 +252,9 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
         const int chalf = (warp - 2) >> 2;                  // which 128 columns
         unsigned char *stg = stage_buf + (warp - 2) * boxes * R_EPI_BYTES;
         unsigned k = 0;
-        bool any = false;
+        bool any = false, dead = false;
         long long ncol0 = 0;
+        // A warp that ran out of time goes on without touching an accumulator, so that the barriers of the decode stay matched.
         for_tiles([&](unsigned nt) {
             const unsigned live = live_of(nt);
             const int nrec = nt * 2u + 1u < (unsigned long long)p.n_rec_tiles ? 2 : 1;
@@ -271,9 +272,11 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
             if (lane == 0) mbar_arrive(smem_u32(&sm->wfull));
             return true;
         }, [&](unsigned mt) {
+            if (dead) return true;
             const unsigned buf = k & 1u;
             const bool ok = mbar_wait(smem_u32(&sm->tfull[buf]), (k >> 1) & 1u, abort);
-            if (!__all_sync(0xffffffffu, ok)) return false;
+            dead = !__all_sync(0xffffffffu, ok);
+            if (dead) return true;
             ++k;
             tc_fence_after();
             const long long mrow0 = (long long)mt * BMH + quarter * 32;
