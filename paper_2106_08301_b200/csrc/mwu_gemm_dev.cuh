@@ -46,7 +46,6 @@ struct Params {
     void *Y;
     long long ldy;
     int y_fp32;
-    int resident;                       // pair kernel: a CTA pair keeps one weight tile (see mwu_gemm2.cu)
     int stage_epi;                      // single-CTA GEMM: 16 KB of shared memory is there for store_chunk_staged
     int y_tma;                          // two-operand GEMM: bf16 output leaves through TMA stores (a tensor map of Y exists)
     int bw;                             // block width the descriptor names (checked against the packed header)
