@@ -97,8 +97,7 @@ constexpr int D_A_BYTES = AH_BYTES;                  // this CTA's 128 activatio
 constexpr int D_B_BYTES = REC_BYTES;                 // this CTA's 128 weight rows
 constexpr int D_STAGE_BYTES = D_A_BYTES + D_B_BYTES;
 constexpr int D_BAND = 8;                            // activation row tiles per band of the tile order
-constexpr int D_EPI_BUFS = 1;                        // staging buffers per epilogue warp (2 with one slot fewer measured no faster)
-constexpr int D_EPI_BYTES = 4096 * D_EPI_BUFS;       // each buffer: 32 rows x 64 bf16 columns
+constexpr int D_EPI_BYTES = 4096;                    // per epilogue warp: 32 rows x 64 bf16 columns (two, with one slot fewer, measured no faster)
 
 constexpr int D_LIVE_TAB = 512;                      // live masks of all weight tiles, when they fit (short reductions)
 
@@ -376,18 +375,16 @@ mwu_dense_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_c
                 for (int h = 0; h < 2; ++h) {
                     const int c0 = 64 * h;
                     if (ncol0 + c0 >= p.N || mrow0 >= p.M) break;
-                    unsigned char *sbuf = stg + (D_EPI_BUFS == 2 ? h * 4096 : 0);
-                    // the last store out of this buffer has read it
-                    if (lane == 0) { if (D_EPI_BUFS == 2) bulk_wait_read_1(); else bulk_wait_read(); }
+                    if (lane == 0) bulk_wait_read();        // the last store has read the buffer
                     __syncwarp();
                     unsigned w[32];
                     pack_bf16(v[2 * h], w);
                     pack_bf16(v[2 * h + 1], w + 16);
-                    stage_row64(w, sbuf, lane);
+                    stage_row64(w, stg, lane);
                     fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) {
-                        tma_store_2d(&tmap_y, smem_u32(sbuf), (int)(ncol0 + c0), (int)mrow0);
+                        tma_store_2d(&tmap_y, smem_u32(stg), (int)(ncol0 + c0), (int)mrow0);
                         bulk_commit();
                     }
                 }

@@ -250,7 +250,11 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
         const unsigned t0 = (unsigned)e % R_DEC;
         const int quarter = warp & 3;                       // tensor-memory lanes (activation rows) this warp may read
         const int chalf = (warp - 2) >> 2;                  // which 128 columns
-        unsigned char *stg = stage_buf + (warp - 2) * boxes * R_EPI_BYTES;
+        unsigned char *const stg = stage_buf + (warp - 2) * boxes * R_EPI_BYTES;
+        // Place of the next store's box.  Two boxes alternate from store to store, whichever tiles those belong to: a tile may
+        // have an odd number of them (weight rows that end inside a box), and bulk_wait_read_1 leaves the latest store unwaited for.
+        unsigned box_at = 0;
+        const unsigned box_flip = boxes == 2 ? R_EPI_BYTES : 0;
         unsigned k = 0;
         bool any = false, dead = false;
         long long ncol0 = 0;
@@ -293,9 +297,10 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&sm->tempty[buf]));
             };
-            // 32 rows of 128 bytes leave through the warp's box (i: its how manieth of this tile); the tensor map clips them
-            auto store_box = [&](const unsigned (&w)[32], int i, int col, int row) {
-                unsigned char *box = stg + (boxes == 2 ? (i & 1) * R_EPI_BYTES : 0);
+            // 32 rows of 128 bytes leave through a box of the warp; the tensor map clips them
+            auto store_box = [&](const unsigned (&w)[32], int col, int row) {
+                unsigned char *box = stg + box_at;
+                box_at ^= box_flip;
                 if (lane == 0) { if (boxes == 2) bulk_wait_read_1(); else bulk_wait_read(); }      // the last store out of it has read it
                 __syncwarp();
                 stage_row64(w, box, lane);
@@ -319,7 +324,7 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     if (ncol0 + 64 * h >= p.N || mrow0 >= p.M) break;
-                    store_box(w[h], h, (int)(ncol0 + 64 * h), (int)mrow0);
+                    store_box(w[h], (int)(ncol0 + 64 * h), (int)mrow0);
                 }
             } else {
                 // boxes of 32 columns
@@ -330,7 +335,7 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
                     tmem_ld_wait(v);
                     if (q == 3) hand_back();
                     if (ncol0 + 32 * q >= p.N || mrow0 >= p.M) continue;
-                    store_box(v, q, (int)(ncol0 + 32 * q), (int)mrow0);
+                    store_box(v, (int)(ncol0 + 32 * q), (int)mrow0);
                 }
             }
             return true;

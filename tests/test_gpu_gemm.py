@@ -332,6 +332,35 @@ def test_gemm_short_reduction(rows, cols, b, M):
         assert errors(Y[:, :rows].float().cpu().numpy(), ref)[0] <= tol
 
 
+@pytest.mark.parametrize("rows,cols,M,fp32", [(64, 64, 100352, 0),        # one store a tile
+                                              (192, 192, 40000, 0),       # one in the second half of a tile
+                                              (2248, 128, 17000, 0),      # weight rows end 8 columns into a box of 64
+                                              (200, 192, 38000, 1),       # three stores of 32 columns, the last of 8
+                                              (1064, 128, 12000, 1),      # two, the second of 8
+                                              (1056, 128, 12000, 1)])     # one
+def test_gemm_short_reduction_odd_stores(rows, cols, M, fp32):
+    """Output that leaves through two boxes of shared memory, an odd number of stores to a tile: every value, several times."""
+    b = 8
+    W = inputs.normal_weights(rows, cols, 0.02, 900 + rows)
+    Mb = W.numel() // b
+    desc, bufs, packed, p = project_and_pack(W, b, Mb // 2, Mb // 4)
+    X = inputs.normal_activations_bf16((M, cols), 901 + rows)
+    What = O.decoded_weights(p, b)
+    Xf = X.to(torch.float64).numpy()
+    ref = O.gemm(Xf, What)
+    # rounding to bf16, 2^-8 of the value, and what each of `cols` fp32 additions may drop, 2^-23 of the sum's magnitude
+    bound = (0.0 if fp32 else 2.0 ** -8) * np.abs(ref) + cols * 2.0 ** -22 * O.gemm(np.abs(Xf), np.abs(What))
+    Xd, first = X.cuda(), None
+    for _ in range(5):
+        Y = torch.full((M, rows), float("nan"), dtype=torch.float32 if fp32 else torch.bfloat16, device="cuda")
+        B.mwu_gemm(desc, packed, Xd, M, cols, Y, rows, fp32, bufs.dev_status)
+        assert int(bufs.dev_status.item()) == 0
+        if first is None:
+            first = Y
+            assert (np.abs(Y.double().cpu().numpy() - ref) <= bound).all()
+        assert torch.equal(Y, first)
+
+
 @pytest.mark.parametrize("filters,cin,h,w,k,stride,pad,n,b", [(128, 64, 13, 11, 3, 2, 1, 2, 4),    # four planes, odd sizes
                                                               (136, 128, 9, 9, 3, 1, 1, 1, 8),     # two chunks over a cluster, ragged filters
                                                               (256, 64, 30, 29, 3, 1, 1, 24, 16),  # several tiles to a CTA, two filter tiles

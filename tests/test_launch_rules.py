@@ -67,3 +67,14 @@ def test_the_question_for_clusters_names_their_shared_memory():
     body = body[:body.index("\n}\n")]
     ask = body.index("cudaOccupancyMaxActiveClusters")
     assert "dynamicSmemBytes" in body[:ask] and "cudaFuncAttributeMaxDynamicSharedMemorySize" in body[:ask]
+
+
+def test_boxes_alternate_over_all_stores_of_a_warp():
+    # bulk_wait_read_1 lets the latest store go on reading its box, so the next box must be the other one, whichever tile the
+    # store belongs to: its place is kept across tiles and flipped at every store, not derived from the store's number in a tile
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        text = _strip_comments(open(path).read())
+        for m in re.finditer(r"bulk_wait_read_1\(\)", text):
+            start = text.rindex("unsigned char *box", 0, m.start())
+            assert re.match(r"unsigned char \*box = stg \+ box_at;\s*box_at \^= box_flip;", text[start:]), path
+            assert len(re.findall(r"box_at\s*[\^+*|&-]?=(?!=)", text)) == 2, path      # set once, flipped in one place
