@@ -165,14 +165,30 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
         // ---------------- TMA producer ----------------
         unsigned slot = 0, phase = 0, issued = 0, live = 0;
         unsigned column = 0;
+        // Stages that the L2 prefetch below brings: those that some weight tile multiplies, the first 1024 records asked (a stage
+        // at a time is 103 MB in the product named there: everything pruned 106 us with all of them fetched, 90 by expanding).
+        const bool ahead_too = n_tiles >= (unsigned)n_stages;
+        const unsigned all = (1u << n_stages) - 1u, n_rec = (unsigned)p.n_rec_tiles * (unsigned)n_stages;
+        unsigned wanted = ahead_too ? 0u : all;
+#pragma unroll 1
+        for (unsigned i0 = 0; wanted != all && i0 < n_rec; i0 += 128) {
+            if (i0 == 1024) { wanted = all; break; }
+            unsigned l = 0;
+#pragma unroll
+            for (unsigned k = 0; k < 4; ++k) {
+                const unsigned i = i0 + 32u * k + (unsigned)lane;
+                if (i < n_rec && (__ldg(&recs[i].w) & 0xFu)) l |= 1u << (i % (unsigned)n_stages);
+            }
+            wanted |= __reduce_or_sync(0xffffffffu, l);
+        }
         for_tiles([&](unsigned nt) { live = live_of(nt); column = nt; return true; }, [&](unsigned mt) {
             // The column's next tile to L2, a stage of it by one CTA of the columns that take it at the same time: the slots here do not
             // cover a trip to DRAM behind the output (200704 x 256 x 1024: 121 us without, so 107; two tiles ahead 111).
             const unsigned ahead = mt + runs;
-            if (n_tiles >= (unsigned)n_stages && ahead < m_tiles) {
+            if (ahead_too && ahead < m_tiles) {
                 unsigned who = ahead * (unsigned)n_stages % n_tiles;
                 for (int ks = 0; ks < n_stages; ++ks) {
-                    if (who == column && elect_one()) tma_prefetch_2d(&tmap_x, ks * BK, (int)(ahead * BMH));
+                    if (who == column && ((wanted >> ks) & 1u) && elect_one()) tma_prefetch_2d(&tmap_x, ks * BK, (int)(ahead * BMH));
                     __syncwarp();
                     if (++who == n_tiles) who = 0;
                 }

@@ -361,6 +361,25 @@ def test_gemm_short_reduction_odd_stores(rows, cols, M, fp32):
         assert torch.equal(Y, first)
 
 
+@pytest.mark.parametrize("rows,cols,M,first_live", [(1024, 256, 12000, 1024),     # two stages dead everywhere
+                                                    (1024, 256, 12000, 256),      # ... dead in the first weight tile only
+                                                    (5000, 256, 2000, 4864),      # ... alive in the 153rd record and later
+                                                    (33000, 256, 390, 33000),     # dead everywhere, more than 1024 records
+                                                    (520, 192, 13000, 0)])        # everything pruned
+def test_gemm_short_reduction_dead_stages(rows, cols, M, first_live):
+    """Stages that no weight tile multiplies, or only some do."""
+    b = 16
+    W = inputs.normal_weights(rows, cols, 0.02, 950)
+    W[:first_live, 64:192] = 0.0
+    Mb = W.numel() // b
+    zero = first_live * 128 // b
+    desc, bufs, packed, p = project_and_pack(W, b, zero + (Mb - zero) // 2 if first_live else Mb, zero if first_live else Mb)
+    X = inputs.normal_activations_bf16((M, cols), 951)
+    ref = O.gemm(X.to(torch.float64).numpy(), O.decoded_weights(p, b))
+    assert errors(run_gemm(desc, bufs, packed, X, 0), ref)[0] <= 2e-3
+    assert errors(run_gemm(desc, bufs, packed, X, 1), ref)[0] <= 1e-5
+
+
 @pytest.mark.parametrize("filters,cin,h,w,k,stride,pad,n,b", [(128, 64, 13, 11, 3, 2, 1, 2, 4),    # four planes, odd sizes
                                                               (136, 128, 9, 9, 3, 1, 1, 1, 8),     # two chunks over a cluster, ragged filters
                                                               (256, 64, 30, 29, 3, 1, 1, 24, 16),  # several tiles to a CTA, two filter tiles

@@ -78,3 +78,9 @@ def test_boxes_alternate_over_all_stores_of_a_warp():
             start = text.rindex("unsigned char *box", 0, m.start())
             assert re.match(r"unsigned char \*box = stg \+ box_at;\s*box_at \^= box_flip;", text[start:]), path
             assert len(re.findall(r"box_at\s*[\^+*|&-]?=(?!=)", text)) == 2, path      # set once, flipped in one place
+
+
+def test_the_short_reduction_kernel_brings_only_stages_that_are_multiplied_to_l2():
+    text = _strip_comments(open(os.path.join(CSRC, "mwu_gemm5.cu")).read())
+    lines = [l for l in text.splitlines() if "tma_prefetch_2d(" in l]
+    assert lines and all("(wanted >> ks) & 1u" in l for l in lines)
