@@ -380,6 +380,20 @@ def test_gemm_short_reduction_dead_stages(rows, cols, M, first_live):
     assert errors(run_gemm(desc, bufs, packed, X, 1), ref)[0] <= 1e-5
 
 
+@pytest.mark.parametrize("b", [2, 4, 8, 16])
+@pytest.mark.parametrize("pr,un", [(0, 0), (0, 10), (3, 6)])
+def test_gemm_short_reduction_uneven_records(b, pr, un):
+    """Records of every filling, several rounds of either list or of both: all dense, all unified, and a mixture of empty, nearly
+    empty and full ones (pr, un in tenths)."""
+    rows, cols, M = 904, 192, 9600
+    gen = torch.Generator().manual_seed(b + pr)
+    W = torch.randn(rows, cols, generator=gen) * 0.02
+    if pr:
+        W *= torch.tensor([0.0001, 1.0, 30.0, 0.01])[torch.randint(0, 4, (8, 3), generator=gen)].repeat_interleave(128, 0)[:rows].repeat_interleave(64, 1)
+    Mb = W.numel() // b
+    check_gemm(W, b, Mb * un // 10, Mb * pr // 10, M, seed=70 + b)
+
+
 @pytest.mark.parametrize("filters,cin,h,w,k,stride,pad,n,b", [(128, 64, 13, 11, 3, 2, 1, 2, 4),    # four planes, odd sizes
                                                               (136, 128, 9, 9, 3, 1, 1, 1, 8),     # two chunks over a cluster, ragged filters
                                                               (256, 64, 30, 29, 3, 1, 1, 24, 16),  # several tiles to a CTA, two filter tiles
