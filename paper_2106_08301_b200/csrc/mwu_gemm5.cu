@@ -47,8 +47,9 @@ __device__ __forceinline__ void decode_record(unsigned char *tile, const uint4 a
     constexpr unsigned OFF_MASK = DecodeCfg<BW, R_DEC>::OFF_MASK;
     constexpr int WORDS = BW / 2;
     constexpr unsigned BATCH = BW == 16 ? 4 : BW == 8 ? 6 : BW == 4 ? 9 : 11;
-    // ranges that do not lie inside the sections: not touched
-    const bool bad = a.x > b.x || b.x > p.n_unified || a.y > b.y || b.y > p.n_dense;
+    // ranges that do not lie inside the sections, or hold more than a record: not touched
+    const bool bad = a.x > b.x || b.x > p.n_unified || a.y > b.y || b.y > p.n_dense ||
+                     (b.x - a.x) + (b.y - a.y) > (unsigned)(kTileRows * BK / BW);
     const unsigned n_u = bad ? 0u : b.x - a.x, n_d = bad ? 0u : b.y - a.y, most = max(n_u, n_d);
     const uint2 *ul = reinterpret_cast<const uint2 *>(p.packed + p.off_ulist) + (bad ? 0u : a.x);
     const unsigned short *dpos = reinterpret_cast<const unsigned short *>(p.packed + p.off_dpos) + (bad ? 0u : a.y);

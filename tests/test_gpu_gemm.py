@@ -394,6 +394,25 @@ def test_gemm_short_reduction_uneven_records(b, pr, un):
     check_gemm(W, b, Mb * un // 10, Mb * pr // 10, M, seed=70 + b)
 
 
+@pytest.mark.parametrize("M", [40, 38000])       # the streaming kernel, the one that keeps the weights
+@pytest.mark.parametrize("b", [2, 4, 8, 16])
+def test_gemm_record_with_more_blocks_than_it_has(b, M):
+    """A damaged record table whose ranges stay inside the lists: a record that claims its neighbour's blocks too is reported."""
+    W = inputs.normal_weights(256, 192, 0.02, 980 + b)
+    Mb = W.numel() // b
+    desc, bufs, packed, _ = project_and_pack(W, b, Mb, 0)              # all unified: every record is full
+    rec = F.records(packed.cpu().numpy())
+    at = F.parse_header(packed.cpu().numpy())["off_rec"]
+    words = packed[at:at + rec.size * 4].view(torch.int32).view(-1, 4)
+    assert words[1, 0] == rec[1, 0] == 128 * 64 // b
+    words[1, 0] = int(rec[2, 0])
+    Y = torch.zeros((M, 256), dtype=torch.bfloat16, device="cuda")
+    X = inputs.normal_activations_bf16((M, 192), 981).cuda()
+    B.mwu_gemm(desc, packed, X, M, 192, Y, 256, 0, bufs.dev_status)
+    torch.cuda.synchronize()
+    assert int(bufs.dev_status.item()) == B.MWU_DEV_BOUNDS
+
+
 @pytest.mark.parametrize("filters,cin,h,w,k,stride,pad,n,b", [(128, 64, 13, 11, 3, 2, 1, 2, 4),    # four planes, odd sizes
                                                               (136, 128, 9, 9, 3, 1, 1, 1, 8),     # two chunks over a cluster, ragged filters
                                                               (256, 64, 30, 29, 3, 1, 1, 24, 16),  # several tiles to a CTA, two filter tiles
