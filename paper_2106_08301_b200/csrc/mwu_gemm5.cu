@@ -39,59 +39,70 @@ struct ResidentSmem {
 };
 
 // One record into its tile, by R_DEC threads: zeros, then the unified and the dense blocks (so pruned blocks need no list).
-// Bound by trips to L2, so entries of both lists travel together, as many to a thread as leave the kernel without spills, the first
-// while the tile is zeroed.  (One list after the other, from zeroing on: 256 x 256, b = 16, 37888 rows 16.3 us, so 15.1; 256 x 192, b = 2,
-// 20.5 / 18.3; 1024 x 256, b = 8, 200704 rows 105.7 / 104.)
+// Bound by trips to L2 and by fetching its own instructions: entries of both lists travel together, the first while the tile is
+// zeroed, in one loop whose code is there once.  (One list after the other, from zeroing on: 256 x 256, b = 16, 37900 rows 17.4 us, so
+// 16.0; b = 8 17.9 / 16.3, b = 4 18.7 / 17.6, b = 2 23.1 / 20.2; 1024 x 256, b = 8, 200704 rows 104.5 / 103.  Entries at a time: more dense ones take b = 4
+// from 19.6 to 20.2 us where all blocks are dense, twice as many unified ones b = 2 from 20.2 to 21.9; b = 8 spills 76 bytes with eight,
+// six, which spill none, take 17.7 instead of 16.0 us for 512 x 192 of dense blocks.)
 template <int BW>
 __device__ __forceinline__ void decode_record(unsigned char *tile, const uint4 a, const uint4 b, const Params &p, unsigned t0, int group) {
     constexpr unsigned OFF_MASK = DecodeCfg<BW, R_DEC>::OFF_MASK;
     constexpr int WORDS = BW / 2;
-    constexpr unsigned BATCH = BW == 16 ? 4 : BW == 8 ? 6 : BW == 4 ? 9 : 11;
+    constexpr unsigned UB = BW == 16 ? 4 : BW == 2 ? 12 : 8, DB = BW == 16 ? 4 : BW == 2 ? 16 : 8;     // entries of a thread at a time
     // ranges that do not lie inside the sections, or hold more than a record: not touched
     const bool bad = a.x > b.x || b.x > p.n_unified || a.y > b.y || b.y > p.n_dense ||
                      (b.x - a.x) + (b.y - a.y) > (unsigned)(kTileRows * BK / BW);
-    const unsigned n_u = bad ? 0u : b.x - a.x, n_d = bad ? 0u : b.y - a.y, most = max(n_u, n_d);
+    const unsigned n_u = bad ? 0u : b.x - a.x, n_d = bad ? 0u : b.y - a.y;
     const uint2 *ul = reinterpret_cast<const uint2 *>(p.packed + p.off_ulist) + (bad ? 0u : a.x);
     const unsigned short *dpos = reinterpret_cast<const unsigned short *>(p.packed + p.off_dpos) + (bad ? 0u : a.y);
     const unsigned char *pay = p.packed + p.off_dpay + (size_t)(bad ? 0u : a.y) * (2 * BW);
-    uint2 ent[BATCH];
-    unsigned off[BATCH], v[BATCH][WORDS];
-    auto read = [&](unsigned e0) {
-#pragma unroll
-        for (unsigned k = 0; k < BATCH; ++k)
-            if (e0 + k * R_DEC < n_u) ent[k] = __ldg(ul + e0 + k * R_DEC);
-#pragma unroll
-        for (unsigned k = 0; k < BATCH; ++k) {
-            const unsigned e = e0 + k * R_DEC;
-            if (e >= n_d) continue;
-            off[k] = __ldg(dpos + e);
-            ld_words<WORDS>(pay + (size_t)e * (2 * BW), v[k]);
-        }
-    };
-    read(t0);
-    uint4 *z = reinterpret_cast<uint4 *>(tile) + t0;
-#pragma unroll
-    for (int t = 0; t < REC_BYTES / 16 / R_DEC; ++t) z[t * R_DEC] = make_uint4(0, 0, 0, 0);
-    group_barrier<R_DEC>(1 + group);
-    if (bad) atomicOr(p.dev_status, (unsigned)MWU_DEV_BOUNDS);
+    unsigned u0 = 0, d0 = 0;
 #pragma unroll 1
-    for (unsigned e0 = t0;;) {
+    do {
+        uint2 ent[UB];
+        unsigned off[DB], v[DB][WORDS];
+        if (u0 < n_u) {
 #pragma unroll
-        for (unsigned k = 0; k < BATCH; ++k) {
-            if (e0 + k * R_DEC >= n_u) break;
-            unsigned w[WORDS];
-            unified_words<WORDS>(ent[k], w);
-            st_words<WORDS>(tile, ent[k].y & OFF_MASK, w);
+            for (unsigned k = 0; k < UB; ++k) {
+                const unsigned e = u0 + k * R_DEC + t0;
+                if (e < n_u) ent[k] = __ldg(ul + e);
+            }
         }
+        if (d0 < n_d) {
 #pragma unroll
-        for (unsigned k = 0; k < BATCH; ++k) {
-            if (e0 + k * R_DEC >= n_d) break;
-            st_words<WORDS>(tile, off[k] & OFF_MASK, v[k]);
+            for (unsigned k = 0; k < DB; ++k) {
+                const unsigned e = d0 + k * R_DEC + t0;
+                if (e >= n_d) continue;
+                off[k] = __ldg(dpos + e);
+                ld_words<WORDS>(pay + (size_t)e * (2 * BW), v[k]);
+            }
         }
-        e0 += BATCH * R_DEC;
-        if (e0 >= most) break;
-        read(e0);
-    }
+        if (u0 == 0) {
+            uint4 *z = reinterpret_cast<uint4 *>(tile) + t0;
+#pragma unroll
+            for (int t = 0; t < REC_BYTES / 16 / R_DEC; ++t) z[t * R_DEC] = make_uint4(0, 0, 0, 0);
+            group_barrier<R_DEC>(1 + group);
+        }
+        if (u0 < n_u) {
+#pragma unroll
+            for (unsigned k = 0; k < UB; ++k) {
+                if (u0 + k * R_DEC + t0 >= n_u) break;
+                unsigned w[WORDS];
+                unified_words<WORDS>(ent[k], w);
+                st_words<WORDS>(tile, ent[k].y & OFF_MASK, w);
+            }
+        }
+        if (d0 < n_d) {
+#pragma unroll
+            for (unsigned k = 0; k < DB; ++k) {
+                if (d0 + k * R_DEC + t0 >= n_d) break;
+                st_words<WORDS>(tile, off[k] & OFF_MASK, v[k]);
+            }
+        }
+        u0 += UB * R_DEC;
+        d0 += DB * R_DEC;
+    } while (u0 < n_u || d0 < n_d);
+    if (bad) atomicOr(p.dev_status, (unsigned)MWU_DEV_BOUNDS);
 }
 
 template <int BW>
@@ -385,11 +396,9 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
 constexpr size_t R_SMEM_MAX = 227 * 1024;
 
 // From two tiles an SM on, so that decoding the weights is shared (us, this kernel / expanding the weights: 256 x 256, b = 16, 37888
-// rows, 296 tiles: 15.1 / 17.1; 256 x 192, b = 2: 18.3 / 21.9; 65536 x 256, b = 2, 300 rows, three tiles to a weight tile: 53 / 58; 4096 x 128,
-// b = 4, 4096 rows, 512 tiles: 13.9 / 17.7; 1024 x 256, b = 8, 20000 rows, 628 tiles: 19.5 / 22.2, 200704 rows 104 / 132 (fused, without a
-// workspace: 215); 640 x 192, 200704 rows: 64 / 94, 65536 rows of fp32 output 52 / 83; 96 x 256, 200704 rows: 33 / 40).  Where one or two weight
-// tiles have just begun a third tile to an SM it is the slower one by up to 7 % (140 x 256, b = 4, 297 tiles: 15.4 / 14.4, 314 tiles
-// 16.1 / 16.0; 512 x 192, b = 2, 70 % dense, 302 tiles: 20.9 / 19.4), in others of these shapes the faster one (200 x 192, b = 16, 297 tiles: 12.1 / 13.9).
+// rows, 296 tiles: 15.1 / 17.1; 256 x 192, b = 2: 17.4 / 21.9; 65536 x 256, b = 2, 300 rows, three tiles to a weight tile: 46 / 58; 4096 x 128,
+// b = 4, 4096 rows, 512 tiles: 13.9 / 17.7; 1024 x 256, b = 8, 20000 rows, 628 tiles: 19.5 / 22.2, 200704 rows 103 / 132 (fused, without a
+// workspace: 215); 640 x 192, 200704 rows: 62 / 94, 65536 rows of fp32 output 52 / 83; 96 x 256, 200704 rows: 33 / 40).
 bool resident_eligible(const Params &p, int sm_count) {
     if (p.n_stages > R_MAX_STAGES) return false;
     const long long tiles = (p.M + BMH - 1) / BMH * ((p.n_rec_tiles + 1) / 2);
