@@ -38,9 +38,10 @@ cudaError_t launch_stream(int bw, const CUtensorMap &tmap_x, const Params &p, in
 bool halo_eligible(int h, int w, int kh, int kw, int stride, int pad);
 int run_conv_halo(const Params &g, const void *X, int n, int c, int h, int w, int kh, int kw, int stride, int pad, int sm_count,
                   cudaStream_t st);
-// decode-once path, defined in mwu_gemm3.cu
-bool resident_eligible(const Params &p, int sm_count);
+// short reductions, defined in mwu_gemm5.cu
+bool resident_eligible(const Params &p, int sm_count, bool can_expand);
 cudaError_t launch_resident(int bw, const CUtensorMap &tmap_x, const CUtensorMap &tmap_y, const Params &p, int sm_count, cudaStream_t st);
+// decode-once path, defined in mwu_gemm3.cu
 cudaError_t launch_decode(int bw, const Params &p, __nv_bfloat16 *Wd, long long ldw, cudaStream_t st);
 cudaError_t launch_dense(const CUtensorMap &tmap_x, const CUtensorMap &tmap_w, const CUtensorMap &tmap_y,
                          const Params &p, int sm_count,
@@ -647,7 +648,7 @@ extern "C" int mwu_gemm_ws(const mwu_proj_desc *desc, const void *packed, const 
     }
 
     // a short reduction: the weights stay in shared memory
-    if (resident_eligible(p, sm_count)) {
+    if (resident_eligible(p, sm_count, can_expand)) {
         CUtensorMap tmap_x, tmap_y;
         if (!encode_bf16_2d(encode, &tmap_x, X, desc->cols, M, ldx, BMH) ||
             !encode_2d(encode, &tmap_y, y_dtype != 0, Y, desc->rows, M, ldy, 32)) return MWU_ERR_CUDA;

@@ -399,9 +399,20 @@ constexpr size_t R_SMEM_MAX = 227 * 1024;
 // rows, 296 tiles: 15.1 / 17.1; 256 x 192, b = 2: 17.4 / 21.9; 65536 x 256, b = 2, 300 rows, three tiles to a weight tile: 46 / 58; 4096 x 128,
 // b = 4, 4096 rows, 512 tiles: 13.9 / 17.7; 1024 x 256, b = 8, 20000 rows, 628 tiles: 19.5 / 22.2, 200704 rows 103 / 132 (fused, without a
 // workspace: 215); 640 x 192, 200704 rows: 62 / 94, 65536 rows of fp32 output 52 / 83; 96 x 256, 200704 rows: 33 / 40).
-bool resident_eligible(const Params &p, int sm_count) {
+// Narrow blocks that are mostly in one list take many trips to L2.  Where the weights could be expanded, few weight tiles (whose
+// activations are not brought to L2 ahead) then need more than four tiles an SM, and more weight tiles than SMs more than five tiles each:
+// 256 x 256, all dense, b = 4, 297 tiles 19.6 / 17.7, 592 tiles 24.8 / 24.2, 740 tiles 27.9 / 27.5; b = 2 22.9 / 20.3, 27.9 / 26.0, 31.1 / 29.5; 65536 x 256, b = 4,
+// all dense, four tiles to a weight tile 47 / 41, seven 59.4 / 59.1.  Not so with 70 % of the blocks dense and b = 2 (256 x 256, 297 tiles 21.7 / 23.5),
+// half of them and b = 4 (17.6 / 17.9), four weight tiles (1024 x 256, b = 4, all dense, 372 tiles 18.2 / 18.3) or two stages (40000 x 128, b = 4, all
+// dense, three tiles to a weight tile 20.9 / 24.6).
+bool resident_eligible(const Params &p, int sm_count, bool can_expand) {
     if (p.n_stages > R_MAX_STAGES) return false;
-    const long long tiles = (p.M + BMH - 1) / BMH * ((p.n_rec_tiles + 1) / 2);
+    const long long n_tiles = (p.n_rec_tiles + 1) / 2, tiles = (p.M + BMH - 1) / BMH * n_tiles;
+    if (can_expand && !p.y_fp32 && p.n_stages >= 3) {
+        const long long blocks = p.n_rec_tiles * p.n_stages * (kTileRows * BK / p.bw), longest = p.n_unified > p.n_dense ? p.n_unified : p.n_dense;
+        const bool one_list = p.bw == 2 ? 4ll * p.n_dense > 3 * blocks : p.bw == 4 && 5 * longest > 3 * blocks;
+        if (one_list && (n_tiles < p.n_stages ? tiles <= 4ll * sm_count : n_tiles > sm_count && tiles <= 5 * n_tiles)) return false;
+    }
     return tiles >= 2ll * sm_count;
 }
 

@@ -83,6 +83,28 @@ def test_gemm_ws_block_widths_and_ragged_shapes(b):
     check_gemm_ws(W, b, Mb * 6 // 10, Mb * 3 // 10, 1100, seed=b)
 
 
+@pytest.mark.parametrize("b,ku,kp,fp32,M,launches", [(4, 0, 0, 0, 38016, 2),        # one long list, three tiles an SM: expanded
+                                                     (4, 0, 0, 1, 38016, 1),
+                                                     (4, 0, 0, 0, 75800, 1),        # more than four tiles an SM
+                                                     (4, 10, 0, 0, 38016, 2),
+                                                     (4, 5, 2, 0, 38016, 1),
+                                                     (2, 1, 0, 0, 38016, 2),
+                                                     (2, 3, 0, 0, 38016, 1),
+                                                     (8, 0, 0, 0, 38016, 1)])
+def test_gemm_ws_short_reduction_of_hardly_compressed_weights(b, ku, kp, fp32, M, launches):
+    """With a workspace such weights are expanded (two launches) unless enough tiles share their decoding (ku, kp in tenths)."""
+    assert torch.cuda.get_device_properties(0).multi_processor_count == 148
+    W = inputs.normal_weights(256, 192, 0.02, 7050 + b)
+    Mb = W.numel() // b
+    desc, bufs, packed, p = project_and_pack(W, b, Mb * ku // 10, Mb * kp // 10)
+    X = inputs.normal_activations_bf16((M, 192), 7051)
+    before = B.mwu_kernel_launches()
+    Y = run_gemm_ws(desc, bufs, packed, X, fp32)
+    assert B.mwu_kernel_launches() - before == launches
+    ref = O.gemm(X.to(torch.float64).numpy(), O.decoded_weights(p, b))
+    assert errors(Y, ref)[0] <= (1e-5 if fp32 else 2e-3)
+
+
 def test_gemm_ws_many_tiles_per_pair_and_long_reduction():
     """More tiles than CTA pairs (both accumulator buffers are reused several times) and a
     reduction longer than the six-slot ring."""
@@ -211,9 +233,10 @@ def test_gemm_ws_short_reduction_many_rows(N, K, M, b):
     check_gemm_ws(W, b, Mb * 7 // 10, Mb * 4 // 10, M, seed=N)
 
 
-def test_gemm_ws_short_reduction_dead_stage():
+@pytest.mark.parametrize("K", [256, 384])               # the kernel that keeps the weights, the two-operand kernel
+def test_gemm_ws_short_reduction_dead_stage(K):
     """A 64-column stage that is pruned in every row is skipped (short reduction, many rows)."""
-    N, K, b, M = 512, 256, 16, 40000
+    N, b, M = 512, 16, 40000
     W = inputs.normal_weights(N, K, 0.02, 7100)
     W[:, 64:128] = 0.0
     Mb = N * K // b

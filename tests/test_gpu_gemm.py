@@ -247,19 +247,18 @@ def test_conv_config2():
 
 
 @pytest.mark.parametrize("b", [2, 4, 8, 16])
-def test_gemm_pair_tiles(b):
-    """Shapes that take the two-CTA path: M > 256, an even number of 128-row weight tiles, N a
-    multiple of 256; M = 900 leaves a ragged last 512-row tile, K = 320 gives five stages (more
-    than the four pipeline slots)."""
+def test_gemm_few_stages(b):
+    """The streaming kernel: M = 900 leaves a ragged last tile of eight, K = 320 gives five stages."""
     W = inputs.normal_weights(512, 320, 0.02, 80 + b)
     Mb = W.numel() // b
     check_gemm(W, b, Mb * 7 // 10, Mb * 4 // 10, 900, seed=20 + b)
 
 
-def test_gemm_pair_tiles_dead_stages_and_all_pruned():
+def test_gemm_dead_stages_and_all_pruned():
+    """The streaming kernel over several tiles of activation rows."""
     W = inputs.normal_weights(512, 512, 0.02, 90)
     W[:, 128:256] = 0.0                 # stages 2 and 3 dead in every record
-    W[:256, 448:464] = 0.0              # one dead slice in the first pair tile only
+    W[:256, 448:464] = 0.0              # one dead slice in the first two weight tiles only
     b = 16
     Mb = W.numel() // b
     n_zero = int((W.reshape(-1, b).abs().sum(dim=1) == 0).sum())
@@ -268,11 +267,44 @@ def test_gemm_pair_tiles_dead_stages_and_all_pruned():
     check_gemm(W, b, 0, 0, 513)         # everything dense
 
 
+def assert_fused(rows, cols, M):
+    """Too many record decodes for the streaming kernel (nine an SM), too long a reduction for the one that keeps the weights:
+    without a workspace the fused kernels multiply."""
+    assert cols > 256 and M > 640
+    assert -(-rows // 128) * -(-M // 128) * (cols // 64) > 9 * torch.cuda.get_device_properties(0).multi_processor_count
+
+
+@pytest.mark.parametrize("b", [2, 4, 8, 16])
+@pytest.mark.parametrize("rows,cols,M", [(512, 320, 9000),       # pairs of CTAs: five stages (more than the four slots), a ragged last tile
+                                         (512, 1024, 2900),      # ... sixteen stages
+                                         (640, 1024, 2300),      # a CTA to a tile: an odd number of record tiles
+                                         (1000, 1024, 2100),     # ... weight rows that end inside a tile
+                                         (128, 1024, 11000)])    # ... one record tile
+def test_gemm_fused_tiles(rows, cols, M, b):
+    assert_fused(rows, cols, M)
+    W = inputs.normal_weights(rows, cols, 0.02, 80 + b)
+    Mb = W.numel() // b
+    check_gemm(W, b, Mb * 7 // 10, Mb * 4 // 10, M, seed=20 + b)
+
+
+@pytest.mark.parametrize("rows,M", [(512, 5500), (640, 4500)])         # pairs of CTAs, a CTA to a tile
+def test_gemm_fused_tiles_dead_stages_and_all_pruned(rows, M):
+    assert_fused(rows, 512, M)
+    W = inputs.normal_weights(rows, 512, 0.02, 90)
+    W[:, 128:256] = 0.0                 # stages 2 and 3 dead in every record
+    W[:256, 448:464] = 0.0              # one dead slice in the first tile only
+    b = 16
+    Mb = W.numel() // b
+    n_zero = int((W.reshape(-1, b).abs().sum(dim=1) == 0).sum())
+    check_gemm(W, b, n_zero + 700, n_zero, M)
+    check_gemm(W, b, Mb, Mb, M)         # everything pruned: zeros, no MMA issued at all
+    check_gemm(W, b, 0, 0, M)           # everything dense
+
+
 @pytest.mark.parametrize("K,b", [(256, 8), (192, 16)])
-def test_gemm_pair_tiles_resident_weights(K, b):
-    """Small reduction, many activation rows: a CTA pair keeps one weight tile in shared memory and
-    walks the activation tiles (K = 256 fills the four slots exactly, so decode is skipped after
-    the first tile; K = 192 takes the same tile order but re-decodes)."""
+def test_gemm_short_reduction_two_weight_tiles(K, b):
+    """Small reduction, many activation rows: half of the CTAs keep one weight tile, half the other, and walk the activation
+    tiles (K = 256: one store box a warp, K = 192: two)."""
     W = inputs.normal_weights(512, K, 0.02, 95 + b)
     Mb = W.numel() // b
     check_gemm(W, b, Mb * 3 // 4, Mb // 2, 77000 + 37, seed=31 + b)
@@ -294,17 +326,36 @@ def test_gemm_few_rows(b, rows, cols, M, ku, kp):
     check_gemm(W, b, Mb * ku // 10, Mb * kp // 10, M, seed=40 + b)
 
 
+def uneven_weights(rows, cols, seed, balanced=False):
+    """Each run of 64 columns on a scale of its own, from 1e-4 to 30; balanced: a quarter of them on each."""
+    gen = torch.Generator().manual_seed(seed)
+    W = torch.randn(rows, cols, generator=gen) * 0.02
+    which = torch.randperm(cols // 64, generator=gen) % 4 if balanced else torch.randint(0, 4, (cols // 64,), generator=gen)
+    return W * torch.tensor([0.0001, 1.0, 30.0, 0.01])[which].repeat_interleave(64)[None, :]
+
+
 @pytest.mark.parametrize("b,M,pr,un", [(16, 20, 4, 7), (16, 3, 1, 2), (16, 100, 6, 9), (8, 20, 4, 7), (4, 5, 3, 6), (2, 17, 3, 6)])
 def test_gemm_few_rows_uneven_records(b, M, pr, un):
-    """A run of more than 32 stages whose records differ: dead ones, nearly empty ones, all-dense and all-unified ones that
-    need several batches, so that every way of clearing a tile follows every other (pr, un in tenths)."""
+    """Records that differ, in runs of nine stages or less: dead ones, nearly empty ones, all-dense and all-unified ones that
+    need several batches (pr, un in tenths)."""
     rows, cols = 296, 64 * 70
-    gen = torch.Generator().manual_seed(b * 100 + M)
-    W = torch.randn(rows, cols, generator=gen) * 0.02
-    scale = torch.tensor([0.0001, 1.0, 30.0, 0.01])[torch.randint(0, 4, (cols // 64,), generator=gen)]
-    W = W * scale.repeat_interleave(64)[None, :]
+    W = uneven_weights(rows, cols, b * 100 + M)
     Mb = W.numel() // b
     check_gemm(W, b, Mb * un // 10, Mb * pr // 10, M)
+
+
+@pytest.mark.parametrize("b,M,pr,un", [(16, 20, 4, 7), (16, 100, 5, 8), (8, 20, 4, 7), (4, 5, 3, 6), (2, 128, 3, 6)])
+def test_gemm_few_rows_long_runs(b, M, pr, un):
+    """Runs of 65 stages: fp32 results of more than 6912 columns are summed in two pieces at most.  Dead stages among the
+    first 32 and behind them, so that the list of the live ones is closed up over several rounds, and at least six records to a
+    decode group, so that every way of clearing a tile follows every other."""
+    rows, cols = 296, 64 * 130
+    W = uneven_weights(rows, cols, b * 100 + M, balanced=True)
+    Mb = W.numel() // b
+    _, _, packed, _ = check_gemm(W, b, Mb * un // 10, Mb * pr // 10, M)
+    live = F.records(packed.cpu().numpy())[:3 * 130, 3].reshape(3, 2, 65) != 0
+    assert (live.sum(axis=2) >= 6 * 5).all()
+    assert not live[:, :, :32].all(axis=2).any() and not live[:, :, 32:].all(axis=2).any()
 
 
 @pytest.mark.parametrize("rows,cols,b,M", [(96, 128, 8, 37900),          # one record tile: half a tile of outputs (fp32: the streaming kernel)
