@@ -464,9 +464,14 @@ int stream_box_rows(const Params &p, int sm_count) { return plan_of(p, sm_count,
 // 256 x 256, 16384 rows, 256 tiles: 14.2 / 11.1; 128 x 192, b = 16, 32768 rows, 256 tiles: 11.5 / 12.7; 4096 x 256, 777 rows, 224 tiles: 11.5 / 12.0;
 // without a workspace 512 x 256, 8192 rows, 256 tiles: 14.1 / 18.8, 128 x 192, 256 tiles: 11.0 / 10.6).  Nor where a reduction of less
 // than 1024 has to be split to two CTAs an SM (512 x 512, b = 4, 4096 rows: 15.9 / 12.0; 2048 x 512, 300 rows: 12.1 / 13.4).
-// fp32 results, which the other paths store in pieces of a row, stay (1024 x 64, 8192 rows: 19.2 / 20.3; 512 x 512, 2048 rows: 13.1 / 15.4).
+// fp32 results, which the paths that expand store in pieces of a row, stay (512 x 512, 2048 rows: 13.1 / 15.4), but not where the kernel
+// of the short reductions takes over, whose fp32 output leaves through TMA (from two tiles of 128 x 256 outputs an SM, this kernel / that one:
+// 256 x 64, b = 4, 37900 rows 20.7 / 14.7, 128 x 64, 38000 rows 11.0 / 10.2, 80000 rows 21.9 / 15.5; 16384 x 64, 1024 rows 33.6 / 18.0; 640 x 128, 12801 rows
+// 21.6 / 15.5; 128 x 256, 38000 rows 24.9 / 15.7; b = 16 18.4 / 13.7, 10.4 / 9.9, 19.4 / 15.3, 28.9 / 17.4, 19.4 / 14.5, 20.0 / 14.9).
 // Where it may not split as it would (128 x 7168, 55 rows, fp32: 16 us in eight pieces, 43 in two, 41 expanding), the
 // other path is taken if the caller's workspace allows it (can_expand).
+bool resident_eligible(const Params &p, int sm_count, bool can_expand);      // mwu_gemm5.cu
+
 bool stream_eligible(const Params &p, int sm_count, bool can_expand) {
     const StreamPlan s = plan_of(p, sm_count, most_pieces(p));
     if (can_expand && most_pieces(p) < 8 && 2 * s.cost > 3 * plan_of(p, sm_count, 8).cost) return false;
@@ -478,7 +483,7 @@ bool stream_eligible(const Params &p, int sm_count, bool can_expand) {
                        : 2 * wide * ((p.M + 511) / 512) <= pairs) return true;
     }
     if (tiles * p.n_stages > 9ll * sm_count) return false;
-    if (p.y_fp32) return true;
+    if (p.y_fp32) return !resident_eligible(p, sm_count, can_expand);
     if (can_expand && p.n_stages < 16 && s.q.split > 1 && s.grid > sm_count && p.M > 512) return false;
     const bool two = can_expand ? p.n_rec_tiles == 1 || s.q.m_tiles <= 8 : p.n_rec_tiles > 1 || p.n_stages > 1;
     return tiles <= (two ? 2ll : 1ll) * sm_count;

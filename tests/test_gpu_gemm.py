@@ -358,10 +358,11 @@ def test_gemm_few_rows_long_runs(b, M, pr, un):
     assert not live[:, :, :32].all(axis=2).any() and not live[:, :, 32:].all(axis=2).any()
 
 
-@pytest.mark.parametrize("rows,cols,b,M", [(96, 128, 8, 37900),          # one record tile: half a tile of outputs (fp32: the streaming kernel)
+@pytest.mark.parametrize("rows,cols,b,M", [(96, 128, 8, 37900),          # one record tile: half a tile of outputs
                                            (640, 192, 4, 12801),         # five record tiles, a ragged last row, two boxes a warp
                                            (1000, 256, 2, 9604),         # ragged weight rows; one box a warp
                                            (16384, 64, 16, 620),         # 64 weight tiles: CTAs change weights on the way
+                                           (128, 64, 4, 37888),          # exactly two tiles an SM, the fewest
                                            (264, 256, 16, 20000)])
 def test_gemm_short_reduction(rows, cols, b, M):
     """Weights kept in shared memory: at least two tiles of 128 x 256 outputs an SM, with dead stages and slices where there is room."""
