@@ -186,7 +186,7 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
         unsigned column = 0;
         // Stages that the L2 prefetch below brings: those that some weight tile multiplies, the first 1024 records asked (a stage
         // at a time is 103 MB in the product named there: everything pruned 106 us with all of them fetched, 90 by expanding).
-        const bool ahead_too = n_tiles >= (unsigned)n_stages;
+        const bool ahead_too = n_tiles >= (unsigned)(p.y_fp32 || n_stages == 1 ? n_stages : 2);
         const unsigned all = (1u << n_stages) - 1u, n_rec = (unsigned)p.n_rec_tiles * (unsigned)n_stages;
         unsigned wanted = ahead_too ? 0u : all;
 #pragma unroll 1
@@ -202,7 +202,9 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
         }
         for_tiles([&](unsigned nt) { live = live_of(nt); column = nt; return true; }, [&](unsigned mt) {
             // The column's next tile to L2, a stage of it by one CTA of the columns that take it at the same time: the slots here do not
-            // cover a trip to DRAM behind the output (200704 x 256 x 1024: 121 us without, so 107; two tiles ahead 111).
+            // cover a trip to DRAM behind the output (200704 rows, b = 8, us without and so: 1024 x 256 133 / 107, 768 x 256 92 / 82, 512 x 256 69 / 64,
+            // 512 x 192 62 / 59, 2304 x 192 228 / 185; one weight tile: 256 x 192 38.5 / 39.0, 128 x 256 32.9 / 33.2, but 64 x 64 17.7 / 17.0; fp32 with fewer weight
+            // tiles than stages: 768 x 256 136 / 139, 512 x 256 110 / 113).  Two tiles ahead 111 where one took 107.
             const unsigned ahead = mt + runs;
             if (ahead_too && ahead < m_tiles) {
                 unsigned who = ahead * (unsigned)n_stages % n_tiles;
