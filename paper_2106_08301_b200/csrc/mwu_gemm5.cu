@@ -3,16 +3,18 @@
 // A 1x1 convolution as a product (256 weight columns, 1024 rows, 200704 pixels) has four k stages to a tile of outputs, so what
 // happens between two tiles counts as much as the multiplication.  The two-operand kernel brought both operands of every tile
 // from L2 (822 MB for that product) and passed each accumulator between the two CTAs of a pair, whose messages queue
-// behind the outgoing output: 2.2 us a tile of 256 x 256 against 1.1 of tensor time, 132 us with expanding the weights.
+// behind the outgoing output: 2.2 us a tile of 256 x 256 against 1.1 of tensor time, 132 us with expanding the weights (150 where the
+// activations are new in every call).
 // Here a CTA works alone on tiles of 128 activation rows x 256 weight rows.  It decodes the weights of its tile column once,
-// straight from the packed form (no expansion, no workspace), and then only activations stream in: 411 MB, 106 us.
+// straight from the packed form (no expansion, no workspace), and then only activations stream in: 411 MB of output, 103 to 118 us
+// (the longer the row of calls the slower, as of the other kernel), 125 with new activations.
 // What bounds it: activations in (through four slots for K = 256) and output out at the same time; with the stores left out 81
-// us, with the loads left out 88, stores alone 81; the DRAM traffic alone (457 MB) would take 73.
+// us, with the loads left out 88, the epilogue and its stores alone 81; the DRAM traffic alone (457 MB) would take 73.
 //
 // The tiles of a weight tile column follow one another in the list that is dealt out, in equal shares, to the CTAs, so a CTA meets
 // one weight tile or two.  In a column neighbouring CTAs take neighbouring activation tiles at the same time, and so do the
-// CTAs of the other columns: L2 holds the activations, and whole rows of the output are written at a time (output alone: 68 us
-// so, 78 with a run of consecutive activation tiles to a CTA).
+// CTAs of the other columns: L2 holds the activations, and whole rows of the output are written at a time (filling 411 MB in this
+// order takes 68 us, 78 with a run of consecutive activation tiles to a CTA).
 // Roles: warp 0 TMA producer (activation stages), warp 1 tensor memory and MMAs, warps 2 to 9 decode the weights and
 // then are the epilogue (two warps to a 32-lane quarter, 128 columns each; accumulators double-buffered in tensor memory; the
 // output leaves through TMA stores of 32 rows x 128 bytes).
@@ -28,7 +30,7 @@ constexpr int R_THREADS = 32 * (2 + R_EPI_WARPS);
 constexpr int R_MAX_STAGES = 4;
 constexpr int R_W_STAGE = 2 * REC_BYTES;                // 256 weight rows of a k stage
 constexpr int R_EPI_BYTES = 4096;                       // of a warp: 32 rows x 64 bf16 columns
-constexpr int R_MAX_SLOTS = 10;                         // activation stages in flight
+constexpr int R_MAX_SLOTS = 8;                          // activation stages in flight: what fits beside one stage of weights
 constexpr int R_DEC = 64;                               // threads that decode a record together
 
 struct ResidentSmem {
@@ -396,6 +398,8 @@ mwu_gemm_resident_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
 // host
 // ------------------------------------------------------------------------------------------
 constexpr size_t R_SMEM_MAX = 227 * 1024;
+static_assert((R_SMEM_MAX - 1024 - R_W_STAGE - 2 * R_EPI_WARPS * R_EPI_BYTES - sizeof(ResidentSmem)) / AH_BYTES <= R_MAX_SLOTS,
+              "one stage of weights leaves most slots");
 
 // From two tiles an SM on, so that decoding the weights is shared (us, this kernel / expanding the weights: 256 x 256, b = 16, 37888
 // rows, 296 tiles: 15.1 / 17.1; 256 x 192, b = 2: 17.4 / 21.9; 65536 x 256, b = 2, 300 rows, three tiles to a weight tile: 46 / 58; 4096 x 128,
@@ -425,8 +429,7 @@ static cudaError_t launch_resident_bw(const CUtensorMap &tmap_x, const CUtensorM
     // 116 / 107, 200704 x 192 x 640 78 / 73; with two boxes and two stages for K = 256, 200704 x 256 x 1024: 138).
     const int boxes = p.n_stages <= 3 ? 2 : 1;
     const size_t fixed = 1024 + (size_t)p.n_stages * R_W_STAGE + (size_t)(R_EPI_WARPS * boxes * R_EPI_BYTES) + sizeof(ResidentSmem);
-    int slots = (int)((R_SMEM_MAX - fixed) / AH_BYTES);
-    if (slots > R_MAX_SLOTS) slots = R_MAX_SLOTS;
+    const int slots = (int)((R_SMEM_MAX - fixed) / AH_BYTES);
     const size_t smem = fixed + (size_t)slots * AH_BYTES;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R_SMEM_MAX);
     if (e != cudaSuccess) return e;

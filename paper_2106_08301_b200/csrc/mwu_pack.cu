@@ -307,12 +307,13 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(Params p, int counte
 
 constexpr unsigned OWN_THREADS = 512;
 // CTAs to an SM that the registers are cut to: enough warps to hide the gathers of W and u, few enough that their lines stay in
-// L1 until the neighbouring blocks' turn (16384 x 4096, 50 % / 25 %, b = 2: 160 us with 12; 181 with 8 and 317 with 16 where 12 took 175;
-// b = 4: 107; b = 8: 83 with 16, 88 with 8).  Without a scan: all 512 CTAs of 2048 x 2048 at once (three to an SM: 13.5 us instead of 12.9).
+// L1 until the neighbouring blocks' turn (16384 x 4096, 50 % / 25 %, b = 2: 158 us with 12; 181 with 8 and 317 with 16 where 12 took 175;
+// b = 4: 105; b = 8: 84 with 16, 88 with 8).  Without a scan: all 512 CTAs of 2048 x 2048 at once, for 8 bytes of spills (b = 8 11.7 us,
+// with three to an SM 13.2; b = 16 9.3 / 11.0).
 __host__ __device__ constexpr int fill_ctas(int b, bool own) { return own ? (b == 2 ? 3 : 4) : b <= 4 ? 12 : 16; }
 // Most blocks (padding rows included) of the form without a scan: every CTA reads on average half of the bitmaps.  Whole
-// mwu_pack calls, us, with it and without: 256 x 256, b = 4: 8.5 / 13.0; 1000 x 1216, b = 2: 13.7 / 17.0; 2048 x 2048, b = 8,
-// 524288 blocks: 12.5 / 15.1; 3072 x 2048, b = 8, 786432: 19.0 / 19.7; 1024 x 2048, b = 2, 1048576: 26.0 / 17.7.
+// mwu_pack calls, 50 % / 25 %, us, with it and without: 1024 x 1024, b = 8: 6.2 / 14.1; 1000 x 1216, b = 2: 11.8 / 14.9; 2048 x 1024, b = 4 and
+// 2048 x 2048, b = 8, 524288 blocks: 10.8 / 14.7 and 11.7 / 15.2; 3072 x 2048, b = 8, 786432: 17.7 / 19.6; 1024 x 2048, b = 2, 1048576: 23.5 / 15.9.
 constexpr long long OWN_BLOCKS = 655360;
 
 // row and block of a tile offset (the inverse of tile_offset)
@@ -347,7 +348,7 @@ __device__ __forceinline__ unsigned to_slots(unsigned w, unsigned r) {
 }
 
 // Bounded by instruction issue and latency (16384 x 4096, b = 16, 80 % / 60 %: 51 us the whole call with a ballot for each
-// (class, slot) and 64-bit addresses, 47 so; b = 2 175 / 160; 256 x 256, b = 4: 7.7 / 6.8).
+// (class, slot) and 64-bit addresses, 47.6 so; b = 2, 50 % / 25 %, 175 / 158; 1000 x 1216, b = 8: 7.9 / 6.9).
 // Bounded by latency where records are few (a chain of some dozen L2 round trips, out of a cold instruction cache).
 // OWN: the base of the record's lists is counted here too, from the bitmaps of everything before it: no record table, no
 // kernel before this one; the lists are then written by four times the threads.
