@@ -554,7 +554,7 @@ def run_gpu(args):
                         "frac": gbs / peaks["hbm_gbs"], "peak_source": peaks["source"] + " (copy)",
                         "algorithmic_bytes_per_launch": abytes["gemm"]}
             roof["kernel"] = ("mwu_conv_implicit" if is_conv else "mwu_gemm") + (
-                " (decode kernel + two-operand tensor-core kernel, timed together)" if ws_bytes else " (fused kernel)")
+                " (with a workspace: the kernels of the call, timed together)" if ws_bytes else " (fused kernel)")
             roof["roofline_ms"] = max(t_flops, t_bytes) * 1e3
             # DRAM bytes come from an ncu capture of this call, not from this run; null once the kernels changed
             roof["traffic"] = recorded_traffic(wl.name) if (ws_bytes and not args.m and not group) else None
